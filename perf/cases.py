@@ -98,17 +98,25 @@ def _randn(g, *shape):
 
 
 def _features(g, c):
-    """bf16 [B, n, D]: tokens N(0, 1) with the redundancy of the layout."""
+    """bf16 [B, n, D]: what a vision encoder yields -- patches of a few themes, each with a spread of its own, and the
+    redundancy of the layout.  (Independent patches would all be equally dense, and every decision of the clustering a tie
+    in the last bits.)"""
     B, n, D, layout = c["B"], c["n"], c["D"], c["layout"]
-    if layout == "video":                                  # frame t + 1 is frame t plus N(0, 0.05), 144 tokens a frame
-        frames = -(-n // 144)
-        cur = _randn(g, B, 144, D).bfloat16()
+    m = 144 if layout == "video" else n                    # tokens of a frame
+    themes = max(1, m // 20)
+    # runs of neighbouring patches share a theme; a patch's own part is half to twice as long as the theme's, mostly less
+    run = (torch.rand(B, m, generator=g, device="cuda") < 0.125).long().cumsum(1)
+    theme = torch.randint(0, themes, (B, m + 1), generator=g, device="cuda").gather(1, run)
+    f = _randn(g, B, themes, D).gather(1, theme[..., None].expand(-1, -1, D))
+    f += 0.5 * torch.exp(0.5 * _randn(g, B, m, 1)) * _randn(g, B, m, D)
+    if layout == "video":                                  # frame t + 1 is frame t plus N(0, 0.05) on the whole: some patches
+        frames = -(-n // 144)                              # move, others rest
+        cur = f.bfloat16()
         out = [cur]
         for _ in range(1, frames):
-            cur = (cur.float() + 0.05 * _randn(g, B, 144, D)).bfloat16()
+            cur = (cur.float() + 0.05 * torch.exp(_randn(g, B, 144, 1)) * _randn(g, B, 144, D)).bfloat16()
             out.append(cur)
         return torch.cat(out, 1)[:, :n].contiguous()
-    f = _randn(g, B, n, D)
     share = {"grid": 0.2, "anyres": 0.3, "long": 0.4}[layout]
     n_dup = int(share * n)
     if n_dup:                                              # near-duplicates: a clean token close by, plus N(0, 0.01)
@@ -120,7 +128,8 @@ def _features(g, c):
             at = torch.searchsorted(clean, dup) + torch.randint(0, 4, (B, n_dup), generator=g, device="cuda")
             at = at.clamp_(max=clean.shape[1] - 1)
         src = clean.gather(1, at)
-        rows = f.gather(1, src[..., None].expand(-1, -1, D)) + 0.01 * _randn(g, B, n_dup, D)
+        rows = f.gather(1, src[..., None].expand(-1, -1, D))
+        rows += 0.01 * torch.exp(_randn(g, B, n_dup, 1)) * _randn(g, B, n_dup, D)
         f.scatter_(1, dup[..., None].expand(-1, -1, D), rows)
     if layout == "long":                                   # a few outliers, ten times as long
         f.mul_(1.0 + 9.0 * (torch.rand(B, n, 1, generator=g, device="cuda") < 0.01))
