@@ -1304,6 +1304,7 @@ bool make_rowmajor_bf16_map(CUtensorMap* map, const void* base, int batches, int
 }
 
 unsigned long long gram_wait_limit_ns() { return g_wait_ns.load(); }
+int gram_expire_roles() { return g_expire_roles.load(); }
 
 void gram_set_wait_debug(unsigned long long limit_ns, int expire_roles) {
     g_wait_ns.store(limit_ns ? limit_ns : kWaitLimitNs);

@@ -71,6 +71,7 @@ bool gram_keeps_tiles(int B, int n);
 // Applies to launches made after the call.
 void gram_set_wait_debug(unsigned long long limit_ns, int expire_roles);
 unsigned long long gram_wait_limit_ns();
+int gram_expire_roles();
 
 // Tile width the sweeps use for a problem: wide tiles halve the operand traffic per flop, narrow tiles fill
 // the SMs when the problem is small.

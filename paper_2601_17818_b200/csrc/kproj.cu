@@ -4,16 +4,23 @@
 // that a stand-alone K-norm costs (the largest byte term of a pruning step) disappears.
 //
 //   A = hidden [B * N, Dh] (rows = tokens), B = W_k [H * d, Dh] (rows = output features, as a linear layer stores its
-//   weight): both K-major, so D = A * B^T needs no transposition.  Output tile 128 tokens x 256 features.
+//   weight): both K-major, so D = A * B^T needs no transposition.  Output tile 256 tokens x 256 features.
 //
-// One persistent CTA per SM, warp-specialised like the Gram sweep: warp 0 loads, one thread of warp 1 issues the
-// MMAs into one of two accumulators, 8 epilogue warps drain the other: a thread owns one token row (its TMEM lane),
-// the two warps of a lane quarter share the row's 256 columns.  Per 32-column chunk a thread rounds the values to
-// bf16 (round to nearest even), stores them (64 contiguous bytes of K[b, h, t, :]) and adds their squares -- of the
-// ROUNDED values, i.e. Eq. 4 of the K cache as written -- to the row's fp32 partial sum.  With rotary embedding the
-// chunks holding the two halves of a head are taken together and turned first.  Partial sums go to one slot per
-// column tile and are added by a second, tiny kernel in slot order (the same bits on every run).
-// Every wait is bounded; on expiry the CTA leaves in order and the call reports VITCOP_ERR_TIMEOUT.
+// Bound by the tensor cores at the clock that the power limit leaves.  Persistent clusters of two CTAs, one CTA per SM, each cluster on one tile at a time (tcgen05 cta_group::2): a CTA stages
+// its 128 token rows and its half of the weight rows, 32 KB per k-block where two CTAs working apart would each stage 48 KB,
+// so six k-blocks fit and a third of the operand traffic from the L2 goes (16 x 640 tokens x 4096 -> 4096 back to back,
+// rotary on: 304 us with CTAs working apart, 275 us so; cuBLAS in a sustained loop: 253).  Warp-specialised like the Gram sweep: warp 0
+// loads, one thread of the leader's warp 1 issues the MMAs into one of two accumulators, 8 epilogue warps of each CTA drain
+// the other: a thread owns one token row (its TMEM lane), the two warps of a lane quarter share the row's 256 columns.  Per
+// 32-column chunk a thread rounds the values to bf16 (round to nearest even), stores them (64 contiguous bytes of
+// K[b, h, t, :]) and adds their squares -- of the ROUNDED values, i.e. Eq. 4 of the K cache as written -- to the row's fp32
+// partial sum.  With rotary embedding the chunks holding the two halves of a head are taken together and turned first.
+// Partial sums go to one slot per 128 columns and are added by a second, tiny kernel in slot order (the same bits on every
+// run).
+// When the last round of tiles would occupy at most half of the clusters, its tiles are cut into two of 128 features each
+// (the MMA keeps its rate at N = 128 with two CTAs), so that the round takes half as long
+// (2 x 16512 tokens x 3584 -> 512: 3.5 rounds instead of 4; 121 us before, 113 now).
+// Every wait is bounded; on expiry both CTAs of the cluster leave in order and the call reports VITCOP_ERR_TIMEOUT.
 #include "async_copy.cuh"
 #include "gram.cuh"
 #include "tcgen05.cuh"
@@ -21,24 +28,28 @@
 namespace vitcop {
 namespace {
 
-constexpr int BM = 128, BN = 256;
-constexpr int kStages = 4;
-constexpr int kABytes = BM * BK * 2, kBBytes = BN * BK * 2, kStageBytes = kABytes + kBBytes;
+constexpr int BM = 128, BN = 256;                 // rows of one CTA, columns of the cluster's tile
+constexpr int kStages = 6;
+constexpr int kBoxRows = 64;                      // weight rows per load: a CTA stages one or two boxes
+constexpr int kABytes = BM * BK * 2, kBBytes = BN / 2 * BK * 2, kStageBytes = kABytes + kBBytes;
 constexpr int kEpiWarps = 8, kEpiThreads = kEpiWarps * 32, kThreads = 64 + kEpiThreads;
-constexpr int kSmemBytes = 1024 + kStages * kStageBytes + BM * 4 + 256;
+constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 256;
 
 struct KprojArgs {
     int B, N, Dh, H, d;
     int M, NO;                      // rows of A (B * N), output features (H * d)
-    int TI, TJ;                     // row tiles, column tiles
+    int TI, TJ;                     // tiles of 256 rows, of 256 columns
+    int n_full;                     // tiles taken whole; the others are cut into two column halves
     uint16_t* K_out;                // bf16 [B, H, N, d]
-    float* part;                    // [TJ, M] sum of squares of a token's values inside one column tile
+    float* part;                    // [2 TJ, M] sum of squares of a token's values inside 128 columns
     const float* cos_tab;           // [n_pos, d / 2] or null (no rotation)
     const float* sin_tab;
     const int32_t* position;        // [B, N] or null (token index)
     int n_pos;
     int* status;
     unsigned long long wait_ns;
+    int expire_roles;               // roles whose waits give up at once: 1 load warp, 2 MMA warp, 4 epilogue warps
+    __device__ __forceinline__ unsigned long long limit_of(int role) const { return (expire_roles & role) ? 0ull : wait_ns; }
 };
 
 __device__ __forceinline__ uint32_t pack_bf16_rne(float lo, float hi) {
@@ -67,21 +78,40 @@ __device__ __forceinline__ float round_store_sumsq(const float (&v)[32], uint16_
     return s0 + s1;
 }
 
+// Work item t of a cluster: row tile, first column, 128-column halves.
+struct KprojItem {
+    int ti, col0, halves;
+};
+__device__ __forceinline__ KprojItem decode_item(const KprojArgs& k, int t) {
+    const int x = t - k.n_full;
+    const int tile = x < 0 ? t : k.n_full + (x >> 1);
+    KprojItem it;
+    it.ti = tile / k.TJ;
+    it.col0 = (tile - it.ti * k.TJ) * BN + (x < 0 ? 0 : (x & 1) * (BN / 2));
+    it.halves = x < 0 ? 2 : 1;
+    return it;
+}
+
 template <bool ROPE>
-__global__ void __launch_bounds__(kThreads, 1)
-kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const KprojArgs k) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const KprojArgs k,
+             const int n_items) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;
     uint8_t* gen = smem_raw + (tiles - raw);
-    float* rowsum = reinterpret_cast<float*>(gen + kStages * kStageBytes);           // [BM] second slice's partial
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + kStages * kStageBytes + BM * 4);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + kStages * kStageBytes);
+    // The leader's full barriers count the bytes of both CTAs and its tempty barriers the epilogue warps of both; empty and
+    // tfull are signalled in both CTAs by the leader's commits.
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kStages;
     const uint32_t bar_tfull = bar_empty + 8 * kStages, bar_tempty = bar_tfull + 16, bar_drain = bar_tempty + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const uint32_t abort_addr = smem_u32(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t kTmemCols = 2 * BN;
+    const uint32_t rank = cluster_ctarank();
+    const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -90,7 +120,7 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(bar_tfull + 8 * a, 1);
-            mbar_init(bar_tempty + 8 * a, kEpiThreads);
+            mbar_init(bar_tempty + 8 * a, 2 * kEpiWarps);
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
@@ -98,13 +128,13 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
     }
-    if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+    if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();                                    // both CTAs' barriers and tensor memory are ready
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    const long long total = (long long)k.TI * k.TJ;
     const int KB = k.Dh / BK;
     uint32_t issued = 0, issued_parity = 0;                // thread 0, per stage: a load was issued / parity of its phase
 
@@ -113,72 +143,88 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 
     if (warp == 0) {
         if (lane == 0) {
+            const unsigned long long lim = k.limit_of(1);
             uint32_t stage = 0, phase = 0;
             bool ok = true;
-            for (long long t = blockIdx.x; ok && t < total; t += gridDim.x) {
-                const int ti = (int)(t / k.TJ), tj = (int)(t - (long long)ti * k.TJ);
+            for (int t = cluster; ok && t < n_items; t += n_clusters) {
+                const KprojItem it = decode_item(k, t);
+                const int row = (it.ti * 2 + (int)rank) * BM;
+                const int col = it.col0 + (int)rank * it.halves * kBoxRows;
+                const uint32_t bytes = 2u * (uint32_t)(kABytes + it.halves * (kBBytes / 2));      // both CTAs
                 for (int kb = 0; kb < KB; ++kb) {
-                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, k.wait_ns)) { ok = false; break; }
+                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
                     const uint32_t sa = tiles + stage * kStageBytes;
-                    mbar_expect_tx(bar_full + 8 * stage, kStageBytes);     // rows outside the tensors arrive as zeros
-                    tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, ti * BM, 0);
-                    tma_load_3d(sa + kABytes, &map_b, bar_full + 8 * stage, kb * BK, tj * BN, 0);
+                    const uint32_t full = cluster_map(bar_full + 8 * stage, 0);
+                    if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, bytes);    // rows outside the tensors arrive as zeros
+                    tma_load_3d_pair(sa, &map_a, full, kb * BK, row, 0);
+                    tma_load_3d_pair(sa + kABytes, &map_b, full, kb * BK, col, 0);
+                    if (it.halves == 2) tma_load_3d_pair(sa + kABytes + kBBytes / 2, &map_b, full, kb * BK, col + kBoxRows, 0);
                     issued |= 1u << stage;
                     issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
             }
+            // the leader's last commits must have reached this CTA's barriers before it goes away
+            for (int s = 0; ok && s < kStages; ++s) {
+                ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim);
+                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            }
+            if (!ok) raise_abort_pair(abort_addr, rank);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(BM, BN);
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc_full = umma_idesc_bf16(2 * BM, BN), idesc_half = umma_idesc_bf16(2 * BM, BN / 2);
+            const unsigned long long lim = k.limit_of(2);
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
-            for (long long t = blockIdx.x; ok && t < total; t += gridDim.x) {
-                if (!mbar_wait(bar_tempty + 8 * acc, acc_phase ^ 1u, abort_flag, k.wait_ns)) { ok = false; break; }
+            for (int t = cluster; ok && t < n_items; t += n_clusters) {
+                if (!mbar_wait(bar_tempty + 8 * acc, acc_phase ^ 1u, abort_flag, lim)) { ok = false; break; }
                 tc_fence_after();
+                const uint32_t idesc = decode_item(k, t).halves == 2 ? idesc_full : idesc_half;
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 for (int kb = 0; kb < KB; ++kb) {
-                    if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, k.wait_ns)) { ok = false; break; }
+                    if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t sa = tiles + stage * kStageBytes;
                     const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + kABytes);
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
-                                    (kb > 0 || kk > 0) ? 1u : 0u);
-                    tc_commit(bar_empty + 8 * stage);
+                        tc_mma_bf16_pair(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
+                                         (kb > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit_pair(bar_empty + 8 * stage);
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                tc_commit(bar_tfull + 8 * acc);
+                tc_commit_pair(bar_tfull + 8 * acc);
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
             if (!ok) {
-                tc_commit(bar_drain);
+                raise_abort_pair(abort_addr, rank);
+                tc_commit_pair(bar_drain);
                 mbar_drain(bar_drain, 0);
             }
         }
     } else {
         // ------------------------------------------------------------------ epilogue
-        const int quarter = warp & 3, slice = (warp - 2) >> 2;     // TMEM lane quarter; which chunks of the row
+        const int quarter = warp & 3, slice = (warp - 2) >> 2;     // TMEM lane quarter; which half of the columns
         const int rl = quarter * 32 + lane;
         const int half32 = k.d / 64;                               // chunks in half a head (rotation only)
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        for (long long t = blockIdx.x; t < total; t += gridDim.x) {
-            const int ti = (int)(t / k.TJ), tj = (int)(t - (long long)ti * k.TJ);
-            const int m = ti * BM + rl;                            // token row of this thread
+        for (int t = cluster; ok && t < n_items; t += n_clusters) {
+            const KprojItem it = decode_item(k, t);
+            const int m = (it.ti * 2 + (int)rank) * BM + rl;       // token row of this thread
             const bool row_valid = m < k.M;
             const int b = row_valid ? m / k.N : 0, tok = row_valid ? m - b * k.N : 0;
-            if (ok) ok = mbar_wait(bar_tfull + 8 * acc, acc_phase, abort_flag, k.wait_ns);
+            ok = mbar_wait(bar_tfull + 8 * acc, acc_phase, abort_flag, k.limit_of(4));
             ok = __all_sync(0xffffffffu, ok);
-            float ssq = 0.f;
-            if (ok) {
-                tc_fence_after();
+            if (!ok) break;
+            tc_fence_after();
+            if (slice < it.halves) {                               // (a column half has work for one slice only)
+                float ssq = 0.f;
                 const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16);
                 auto dst_of = [&](int chunk) -> uint16_t* {        // K[b, head, tok, e0 ..] of a 32-column chunk
-                    const int col = tj * BN + chunk * 32;
+                    const int col = it.col0 + chunk * 32;
                     const int head = col / k.d, e0 = col - head * k.d;
                     return k.K_out + (((size_t)b * k.H + head) * k.N + tok) * k.d + e0;
                 };
@@ -188,7 +234,7 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                         const int chunk = slice * 4 + c;
                         float v[32];
                         tmem_ld32(taddr + chunk * 32, v);
-                        const bool write = row_valid && tj * BN + chunk * 32 < k.NO;
+                        const bool write = row_valid && it.col0 + chunk * 32 < k.NO;
                         ssq += round_store_sumsq(v, dst_of(chunk), write);
                     }
                 } else {
@@ -202,7 +248,7 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                         float x[32], y[32];
                         tmem_ld32(taddr + lo * 32, x);
                         tmem_ld32(taddr + hi * 32, y);
-                        const int e0 = (tj * BN + lo * 32) % k.d;                  // first of the 32 rotation angles
+                        const int e0 = (it.col0 + lo * 32) % k.d;                  // first of the 32 rotation angles
                         const float4* ct = reinterpret_cast<const float4*>(k.cos_tab + (size_t)pos * (k.d / 2) + e0);
                         const float4* st = reinterpret_cast<const float4*>(k.sin_tab + (size_t)pos * (k.d / 2) + e0);
 #pragma unroll
@@ -216,46 +262,54 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                                 y[4 * u4 + r] = fmaf(bb, cv[r], a * sv[r]);
                             }
                         }
-                        const bool write = row_valid && tj * BN + hi * 32 < k.NO;
+                        const bool write = row_valid && it.col0 + hi * 32 < k.NO;
                         ssq += round_store_sumsq(x, dst_of(lo), write);
                         ssq += round_store_sumsq(y, dst_of(hi), write);
                     }
                 }
-                tc_fence_before();
-                mbar_arrive(bar_tempty + 8 * acc);
+                if (row_valid) k.part[(size_t)(it.col0 / (BN / 2) + slice) * k.M + m] = ssq;
             }
-            // the row's two slices meet in shared memory; slice 0 writes the tile's partial sum
-            if (slice == 1) rowsum[rl] = ssq;
-            epi_bar_sync<kEpiThreads>();
-            if (ok && slice == 0 && row_valid) k.part[(size_t)tj * k.M + m] = ssq + rowsum[rl];
-            if (epi_bar_or<kEpiThreads>(!ok)) break;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_map(bar_tempty + 8 * acc, 0));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
+        if (!ok && lane == 0) raise_abort_pair(abort_addr, rank);
     }
 
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) {
+        // Some role gave up, so loads issued here may never have been consumed: give the copies still in flight into this
+        // CTA's shared memory time to land before the CTA goes away.  (The other CTA's land on the leader's barriers.)
+        if (rank == 0) {
+            for (int s = 0; s < kStages; ++s)
+                if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
+        } else if (issued) {
+            const unsigned long long t0 = global_ns();
+            while (global_ns() - t0 < kDrainLimitNs) {}
+        }
+        if (k.status) atomicMax(k.status, VITCOP_ERR_TIMEOUT);
+    }
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();                                    // neither CTA leaves while the other may reach into it
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
-    }
-    if (threadIdx.x == 0 && *abort_flag) {
-        for (int s = 0; s < kStages; ++s)
-            if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
-        if (k.status) atomicMax(k.status, VITCOP_ERR_TIMEOUT);
+        tmem_dealloc_pair(tmem_base, kTmemCols);
     }
     grid_dependency_launch_dependents();
 }
 
-// score[b, i] = sqrt( sum over the column tiles, in order, of the partial sums of token vis_start + i ).
-__global__ void kproj_score_kernel(const float* __restrict__ part, int M, int TJ, int N, int vis_start, int Nv,
+// score[b, i] = sqrt( sum over the slots, in order, of the partial sums of token vis_start + i ).
+__global__ void kproj_score_kernel(const float* __restrict__ part, int M, int slots, int N, int vis_start, int Nv,
                                    float* __restrict__ score) {
     grid_dependency_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (i >= Nv) return;
     const size_t m = (size_t)b * N + vis_start + i;
     float s = 0.f;
-    for (int tj = 0; tj < TJ; ++tj) s += part[(size_t)tj * M + m];
+#pragma unroll 8
+    for (int q = 0; q < slots; ++q) s += part[(size_t)q * M + m];
     score[(size_t)b * Nv + i] = sqrtf(s);
 }
 
@@ -263,7 +317,7 @@ __global__ void kproj_score_kernel(const float* __restrict__ part, int M, int TJ
 
 size_t kproj_workspace_bytes(int B, int N, int H, int d) {
     const size_t TJ = ((size_t)H * d + BN - 1) / BN;
-    return kStatusBytes + align_up(TJ * (size_t)B * N * sizeof(float), 256);
+    return kStatusBytes + align_up(2 * TJ * (size_t)B * N * sizeof(float), 256);
 }
 
 int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, int H, int d, const float* cos_tab,
@@ -272,31 +326,38 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     KprojArgs k = {};
     k.B = B; k.N = N; k.Dh = Dh; k.H = H; k.d = d;
     k.M = B * N; k.NO = H * d;
-    k.TI = (k.M + BM - 1) / BM; k.TJ = (k.NO + BN - 1) / BN;
+    k.TI = (k.M + 2 * BM - 1) / (2 * BM); k.TJ = (k.NO + BN - 1) / BN;
     k.K_out = static_cast<uint16_t*>(K_out);
     k.part = reinterpret_cast<float*>(static_cast<char*>(workspace) + kStatusBytes);
     k.cos_tab = cos_tab; k.sin_tab = sin_tab; k.position = position; k.n_pos = n_pos;
     k.status = static_cast<int*>(workspace);
     k.wait_ns = gram_wait_limit_ns();
+    k.expire_roles = gram_expire_roles();
     const long long total = (long long)k.TI * k.TJ;
     if (total <= 0) return VITCOP_OK;
     CUtensorMap ma, mb;
-    if (!make_rowmajor_bf16_map(&ma, hidden, 1, k.M, Dh, BM) || !make_rowmajor_bf16_map(&mb, W, 1, k.NO, Dh, BN))
+    if (!make_rowmajor_bf16_map(&ma, hidden, 1, k.M, Dh, BM) || !make_rowmajor_bf16_map(&mb, W, 1, k.NO, Dh, kBoxRows))
         return VITCOP_ERR_CUDA;
     const bool rope = cos_tab != nullptr;
     auto kern = rope ? kproj_kernel<true> : kproj_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return record_cuda(e);
     cudaLaunchConfig_t cfg = {};
-    const int sms = gram_num_sms();
-    cfg.gridDim = dim3((unsigned)(total < sms ? total : sms));
+    const long long pairs = gram_num_sms() / 2 > 0 ? gram_num_sms() / 2 : 1;
+    if (2 * total > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
+    // (a rotated head of 256 columns cannot be cut: its halves are turned together)
+    const long long last = total % pairs;
+    const long long cut = (2 * last <= pairs && !(rope && d > BN / 2)) ? last : 0;
+    k.n_full = (int)(total - cut);
+    const int n_items = (int)(total + cut);
+    cfg.gridDim = dim3((unsigned)(2 * (n_items < pairs ? n_items : pairs)));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
     int rc;
     {
         KernelTimeScope timed("kproj_kernel", stream);
-        rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
+        rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k, n_items));
     }
     if (rc != VITCOP_OK || Nv <= 0 || !score) return rc;
     cudaLaunchAttribute attr[1];
@@ -309,7 +370,7 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     c2.attrs = attr;
     c2.numAttrs = pdl_allowed(true) ? 1 : 0;
     KernelTimeScope timed("kproj_score_kernel", stream);
-    return record_cuda(cudaLaunchKernelEx(&c2, kproj_score_kernel, (const float*)k.part, k.M, k.TJ, N, vis_start, Nv,
+    return record_cuda(cudaLaunchKernelEx(&c2, kproj_score_kernel, (const float*)k.part, k.M, 2 * k.TJ, N, vis_start, Nv,
                                           score));
 }
 

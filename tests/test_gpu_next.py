@@ -236,6 +236,13 @@ def test_kproj_knorm_small(B, N, Dh, H, d, rope):
     _kproj_case(B, N, Dh, H, d, rope, vis_start=min(5, N - 1), Nv=max(1, N - 9), seed=N)
 
 
+# Few tiles are all cut into column halves (every case above); these leave the tiles whole, or cut the last few of many.
+@pytest.mark.parametrize("B,N,Dh,H,d,rope", [(2, 2500, 64, 8, 64, True), (1, 9700, 64, 3, 64, False),
+                                              (1, 19500, 64, 4, 64, True), (1, 10300, 64, 2, 256, True)])
+def test_kproj_knorm_tile_split(B, N, Dh, H, d, rope):
+    _kproj_case(B, N, Dh, H, d, rope, vis_start=7, Nv=N - 19, rows=40, seed=N)
+
+
 def test_kproj_knorm_identity_weights_and_text_only_span():
     # W = I: K is the hidden row cut into heads, bit for bit, and the score is Eq. 4 of the input
     rng = np.random.default_rng(3)

@@ -114,3 +114,27 @@ def test_one_call_step_reports_timeout_and_recovers():
             assert torch.equal(got[key], ref[key]), key
         for key in ("ho", "Ko", "Vo"):
             assert torch.equal(got[key].view(torch.int16), ref[key].view(torch.int16)), key
+
+
+@pytest.mark.parametrize("roles", [ROLE_EPILOGUE, ROLE_MMA, ROLE_LOAD])
+def test_kproj_reports_timeout_and_recovers(roles):
+    """The key projection's pairs of CTAs: whichever role gives up, both CTAs leave."""
+    B, N, H, d, Dh = 1, 10300, 4, 128, 512
+    g = torch.Generator(device=DEV).manual_seed(3)
+    hid = torch.randn((B, N, Dh), generator=g, device=DEV).to(torch.bfloat16)
+    Wk = torch.randn((H * d, Dh), generator=g, device=DEV).to(torch.bfloat16)
+    ws = vb.alloc_workspace(vb.OP_KPROJ, B=B, H=H, N=N, d=d)
+
+    def run():
+        K = torch.zeros((B, H, N, d), dtype=torch.bfloat16, device=DEV)
+        score = torch.zeros((B, N), dtype=torch.float32, device=DEV)
+        vb.vitcop_kproj_knorm(hid, Wk, H, d, K, ws, score=score)
+        return vb.vitcop_poll_status(ws), K, score
+
+    st, K0, s0 = run()
+    assert st == vb.OK
+    vb.vitcop_set_wait_limit(0, roles)
+    assert run()[0] == vb.ERR_TIMEOUT
+    vb.vitcop_set_wait_limit(0, 0)
+    st, K1, s1 = run()
+    assert st == vb.OK and torch.equal(K0.view(torch.int16), K1.view(torch.int16)) and torch.equal(s0, s1)
