@@ -1,5 +1,5 @@
 // Shared-memory barriers (mbarrier), bounded waits on them and bulk asynchronous copies into shared memory: the
-// plumbing shared by the kernels that stage data through shared memory with the copy engine (gram.cu, delta_pass.cu).
+// plumbing shared by the kernels that stage data through shared memory with the copy engine (gram.cu, density.cu, kproj.cu).
 // Every wait is bounded: when the limit runs out the caller's CTA-wide abort flag is raised and the wait returns
 // false; the kernel then leaves in an orderly way and reports VITCOP_ERR_TIMEOUT.
 #pragma once

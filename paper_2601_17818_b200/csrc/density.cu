@@ -1,0 +1,550 @@
+// Density sweep (Algorithm 2, step 1 and Eq. 2) of problems too large for the one-kernel sweep: every Gram value of the
+// symmetric half on the tensor cores, partial sums of Eq. 2, and what the search of Eq. 3 needs (density.cuh: Gram values and
+// block minima).
+//
+// Persistent clusters of two CTAs, one CTA per SM, each cluster on one 256 x 256 tile at a time (tcgen05 cta_group::2): a CTA
+// stages its 128 row tokens and half of the column tokens, 32 KB per k-block instead of the 48 KB that a 128 x 256 tile of
+// its own would take, so six k-blocks are in flight and the operand traffic from the L2, which bounds the main loop next to the
+// tensor cores, falls by a third.  Warp 0 loads, one thread of the leader's warp 1 issues the MMAs into one of two
+// accumulators, 16 epilogue warps per CTA drain the other, in two roles; warp (q, h) of either takes rows 32 q .. + 31 of the CTA
+// and columns 128 h .. + 127, in four blocks of 32 x 32 pairs:
+//   column warps   keep the Gram values, the block minima of both sides and the column sums of Eq. 2.  They read the accumulator
+//                  in the 16-lanes x 256-bit shape: a thread holds 4 rows x 8 columns of a block, so that both sides reduce
+//                  mostly inside the thread and only 4 and 8 values a thread go through shuffles.  (With one row per thread, as
+//                  the 32-lane shape gives it, every column costs a butterfly or a redux over 32 lanes.)
+//   row warps      the row sums of Eq. 2, one row per thread, column by column: that order of the sums is part of the result.
+//
+// Measured with sixteen warps of one role: 8 x 2880 x 1024 70 us, 60 us with an empty epilogue; 2 x 16384 x 1280 517 us, 484 us
+// without the stores of the Gram values, 433 us with an empty epilogue (0.69 Tflop at the rate cuBLAS reaches in a burst).  The
+// sweep before this one, without the minima: 68 and 549 us.
+//
+// A last round of tiles that would occupy at most half of the clusters is cut into tiles of 128 columns.
+// Every wait is bounded; on expiry both CTAs of the cluster leave in order and the call reports VITCOP_ERR_TIMEOUT.
+#include "async_copy.cuh"
+#include "density.cuh"
+#include "tcgen05.cuh"
+
+namespace vitcop {
+namespace {
+
+constexpr int BM = kGramBM, BN = kSweepTile;
+constexpr int kBoxRows = 64;                      // column tokens per load: a CTA stages one or two boxes
+constexpr int kABytes = BM * BK * 2, kBBytes = BN / 2 * BK * 2, kStageBytes = kABytes + kBBytes;
+constexpr int kHalfBlks = BM / kBlk;              // blocks of a warp: 128 columns
+constexpr int kEpiWarps = 16, kEpiThreads = kEpiWarps * 32, kThreads = 64 + kEpiThreads;
+constexpr float kInf = __builtin_huge_valf();
+constexpr int kRoleLoad = 1, kRoleMma = 2, kRoleEpi = 4;
+
+// Epilogue scratch: column factors per warp; per parity of the tile, sums and minima of the columns per row quarter, and the
+// row minima of the block on the diagonal.
+template <int METRIC>
+struct EpiSmem {
+    float w[kEpiWarps][BM], a[METRIC == 1 ? kEpiWarps : 1][BM];
+    float colsum[2][4][BN], colmin[2][4][BN];
+    float rowmin[2][BM][4];
+};
+template <int METRIC>
+__host__ __device__ constexpr int stages() { return METRIC == 1 ? 5 : 6; }       // (what shared memory holds)
+template <int METRIC>
+__host__ __device__ constexpr int smem_bytes() { return 1024 + stages<METRIC>() * kStageBytes + (int)sizeof(EpiSmem<METRIC>) + 256; }
+static_assert(smem_bytes<0>() <= 227 * 1024 && smem_bytes<1>() <= 227 * 1024, "shared memory of an SM");
+
+struct KernelArgs {
+    SweepArgs g;
+    int n_full, n_items;           // tiles taken whole; work items (the other tiles count twice)
+    unsigned long long wait_ns;
+    int expire_roles;
+    __device__ __forceinline__ unsigned long long limit_of(int role) const { return (expire_roles & role) ? 0ull : wait_ns; }
+};
+
+// Work item: row tile tp against column tile tj of sample b, or the 128 columns of it that start at `half`.
+struct Item {
+    int b, tp, tj, half, halves;
+    __device__ __forceinline__ bool one_operand() const { return tp == tj && halves == 2; }   // rows and columns are the same tokens
+};
+__device__ __forceinline__ Item decode_item(const KernelArgs& k, int t) {
+    const int x = t - k.n_full;
+    const int tile = x < 0 ? t : k.n_full + (x >> 1);
+    Item it;
+    it.halves = x < 0 ? 2 : 1;
+    it.half = x < 0 ? 0 : (x & 1);
+    it.b = tile / k.g.t.tiles_per_b;
+    const int r = tile - it.b * k.g.t.tiles_per_b;
+    int q = (int)((sqrtf(8.f * (float)r + 1.f) - 1.f) * 0.5f);
+    while (q > 0 && q * (q + 1) / 2 > r) --q;
+    while ((q + 1) * (q + 2) / 2 <= r) ++q;
+    it.tj = q;
+    it.tp = r - q * (q + 1) / 2;
+    return it;
+}
+
+// Two fp32 operations in one instruction (each half rounded like the scalar instruction).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 o;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(v));
+    return o;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// 2^x for x <= 0 (results below the normal range flush to zero); relative error about 2^-22.
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 16 lanes x 32 columns of the accumulator: register 4 k + 2 p + r holds row T / 4 + 8 p, column 8 k + 2 (T % 4) + r.
+__device__ __forceinline__ void tmem_ld_16x32_issue(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+// Completes the loads issued so far; names their registers, so that no use of them can be moved in front of it.
+__device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                   "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 :
+                 : "memory");
+}
+
+template <bool MIN>
+__device__ __forceinline__ float join(float a, float b) { return MIN ? fminf(a, b) : a + b; }
+// Four values per thread, one per row T / 4 + 8 m: afterwards the thread holds the minimum over its group of four lanes of
+// value m = T % 4.
+__device__ __forceinline__ float reduce_rows_min(const float (&v)[4], int lane) {
+    const bool u2 = lane & 2, u1 = lane & 1;
+    const float a0 = fminf(u2 ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, u2 ? v[0] : v[2], 2));
+    const float a1 = fminf(u2 ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, u2 ? v[1] : v[3], 2));
+    return fminf(u1 ? a1 : a0, __shfl_xor_sync(0xffffffffu, u1 ? a0 : a1, 1));
+}
+// Eight values per thread, value 2 k + r for column 8 k + 2 (T % 4) + r: afterwards the thread holds the total over the eight
+// lanes with its T % 4 of column column_of(T), joined as a tree over the bits of T / 4, highest first.
+template <bool MIN>
+__device__ __forceinline__ float reduce_columns(const float (&v)[8], int lane) {
+    const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
+    float a[4], b[2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        a[q] = join<MIN>(u16 ? v[q + 4] : v[q], __shfl_xor_sync(0xffffffffu, u16 ? v[q] : v[q + 4], 16));
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        b[q] = join<MIN>(u8 ? a[q + 2] : a[q], __shfl_xor_sync(0xffffffffu, u8 ? a[q] : a[q + 2], 8));
+    return join<MIN>(u4 ? b[1] : b[0], __shfl_xor_sync(0xffffffffu, u4 ? b[0] : b[1], 4));
+}
+__device__ __forceinline__ int column_of(int lane) {
+    return 8 * (((lane >> 4) & 1) * 2 + ((lane >> 3) & 1)) + 2 * (lane & 3) + ((lane >> 2) & 1);
+}
+
+template <int METRIC>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                     const __grid_constant__ KernelArgs k) {
+    constexpr int kStages = stages<METRIC>();
+    const SweepArgs& g = k.g;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t tiles = (raw + 1023u) & ~1023u;                 // 1024-byte aligned for the 128B swizzle
+    uint8_t* gen = smem_raw + (tiles - raw);
+    EpiSmem<METRIC>& sm = *reinterpret_cast<EpiSmem<METRIC>*>(gen + kStages * kStageBytes);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + kStages * kStageBytes + sizeof(EpiSmem<METRIC>));
+    // The leader's full barriers count the bytes of both CTAs and its tempty barriers the epilogue warps of both; empty and
+    // tfull are signalled in both CTAs by the leader's commits.
+    const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kStages;
+    const uint32_t bar_tfull = bar_empty + 8 * kStages, bar_tempty = bar_tfull + 16, bar_drain = bar_tempty + 16;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const uint32_t abort_addr = smem_u32(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr uint32_t kTmemCols = 2 * BN;
+    const uint32_t rank = cluster_ctarank();
+    const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(bar_full + 8 * s, 1);
+            mbar_init(bar_empty + 8 * s, 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(bar_tfull + 8 * a, 1);
+            mbar_init(bar_tempty + 8 * a, 2 * kEpiWarps);
+        }
+        mbar_init(bar_drain, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
+    }
+    if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                                    // both CTAs' barriers and tensor memory are ready
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    // The kernels that follow on the stream may be scheduled from here on; they wait for this grid to complete
+    // before they touch anything it writes.
+    grid_dependency_launch_dependents();
+
+    const int KB = g.D / BK;
+    uint32_t issued = 0, issued_parity = 0;                // thread 0, per stage: a load was issued / parity of its phase
+
+    if (warp == 0) {
+        // ------------------------------------------------------------------ TMA producer
+        // The features are an input of the whole call (never written by the kernel before this one), so
+        // the loads need not wait for the preceding grid.
+        if (lane == 0) {
+            const unsigned long long lim = k.limit_of(kRoleLoad);
+            uint32_t stage = 0, phase = 0;
+            bool ok = true;
+            for (int t = cluster; ok && t < k.n_items; t += n_clusters) {
+                const Item it = decode_item(k, t);
+                const int row = (it.tp * 2 + (int)rank) * BM;
+                const int col = it.tj * BN + it.half * BM + (int)rank * it.halves * kBoxRows;
+                const bool one = it.one_operand();
+                const uint32_t bytes = 2u * (uint32_t)(kABytes + (one ? 0 : it.halves * (kBBytes / 2)));      // both CTAs
+                for (int kb = 0; kb < KB; ++kb) {
+                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
+                    const uint32_t sa = tiles + stage * kStageBytes;
+                    const uint32_t full = cluster_map(bar_full + 8 * stage, 0);
+                    if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, bytes);    // rows outside the tensor arrive as zeros
+                    tma_load_3d_pair(sa, &map_a, full, kb * BK, row, it.b);
+                    if (!one) {
+                        tma_load_3d_pair(sa + kABytes, &map_b, full, kb * BK, col, it.b);
+                        if (it.halves == 2)
+                            tma_load_3d_pair(sa + kABytes + kBBytes / 2, &map_b, full, kb * BK, col + kBoxRows, it.b);
+                    }
+                    issued |= 1u << stage;
+                    issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                }
+            }
+            // the leader's last commits must have reached this CTA's barriers before it goes away
+            for (int s = 0; ok && s < kStages; ++s) {
+                ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim);
+                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            }
+            if (!ok) raise_abort_pair(abort_addr, rank);
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer (leader)
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc_full = umma_idesc_bf16(2 * BM, BN), idesc_half = umma_idesc_bf16(2 * BM, BN / 2);
+            const unsigned long long lim = k.limit_of(kRoleMma);
+            uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
+            bool ok = true;
+            for (int t = cluster; ok && t < k.n_items; t += n_clusters) {
+                if (!mbar_wait(bar_tempty + 8 * acc, acc_phase ^ 1u, abort_flag, lim)) { ok = false; break; }
+                tc_fence_after();
+                const Item it = decode_item(k, t);
+                const uint32_t idesc = it.halves == 2 ? idesc_full : idesc_half;
+                const uint32_t b_at = it.one_operand() ? 0u : (uint32_t)kABytes;
+                const uint32_t d_tmem = tmem_base + acc * BN;
+                for (int kb = 0; kb < KB; ++kb) {
+                    if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t sa = tiles + stage * kStageBytes;
+                    const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + b_at);
+#pragma unroll
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                        tc_mma_bf16_pair(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
+                                         (kb > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit_pair(bar_empty + 8 * stage);
+                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                }
+                if (!ok) break;
+                tc_commit_pair(bar_tfull + 8 * acc);
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+            if (!ok) {
+                // leaving early: let the MMAs already issued finish before TMEM is released
+                raise_abort_pair(abort_addr, rank);
+                tc_commit_pair(bar_drain);
+                mbar_drain(bar_drain, 0);
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue (warps 2 .. 17)
+        const int quarter = warp & 3, ew = warp - 2, e = threadIdx.x - 64;
+        const int h = (ew >> 2) & 1;                               // which 128 columns
+        const bool row_role = ew >= kEpiWarps / 2;
+        const int lrow = lane >> 2, lcol = 2 * (lane & 3);         // column warps: rows lrow + 8 m, columns lcol + 8 k, + 1
+        const int TI = g.t.TI, nb = g.t.n_blk();
+        const unsigned long long lim = k.limit_of(kRoleEpi);
+        const f32x2 two2 = pack2(2.f, 2.f), c22 = pack2(g.c2, g.c2);
+        uint32_t acc = 0, acc_phase = 0, parity = 0;
+        bool ok = true;
+
+        grid_dependency_wait();                            // w, a and the bounding boxes come from the preceding kernel
+        for (int t = cluster; t < k.n_items; t += n_clusters, parity ^= 1u) {
+            const Item it = decode_item(k, t);
+            const size_t bo = (size_t)it.b * g.n;
+            const int R = 2 * it.tp + (int)rank;           // 128-token block of the CTA's rows ...
+            const int C0 = 2 * it.tj + it.half;            // ... and of its first 128 columns
+            const int C = C0 + h;                          // this warp's
+            const bool work = h < it.halves && R <= C && C < TI;           // (R > C: below the diagonal)
+            const int i0 = R * BM + quarter * kBlk;
+            const int rb = R * 4 + quarter;                                // the warp's rows as a block of 32
+            const int step = row_role ? 0 : 8;                             // rows of the thread: first, first + step, ..
+            const int first = i0 + (row_role ? lane : lrow);
+            float m2w[4], ai[4];
+            bool far = false;
+            if (work) {
+                // this warp's column factors, its rows' factors, and whether its pairs all lie beyond the spatial radius
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = C * BM + u * 32 + lane;
+                    sm.w[ew][u * 32 + lane] = j < g.n ? g.w[bo + j] : 0.f;
+                    if (METRIC == 1) sm.a[ew][u * 32 + lane] = j < g.n ? g.a[bo + j] : 0.f;
+                    const int i = first + u * step;
+                    m2w[u] = i < g.n ? -2.f * g.w[bo + i] : 0.f;
+                    ai[u] = (METRIC == 1 && i < g.n) ? g.a[bo + i] : 0.f;
+                }
+                if (g.bbox && !row_role)
+                    far = blocks_outside_radius(g.bbox[(size_t)it.b * TI + R], g.bbox[(size_t)it.b * TI + C], g.tau2);
+                __syncwarp();
+            }
+            if (ok) ok = mbar_wait(bar_tfull + 8 * acc, acc_phase, abort_flag, lim);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) tc_fence_after();
+            const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16) + h * BM;
+            if (ok && work && row_role) {
+                // ---- Eq. 2, row side: exp(-d^2 / d_c^2) of this thread's row, added column by column
+                const int i = first;
+                const f32x2 m2w2 = pack2(m2w[0], m2w[0]), ai2 = pack2(ai[0], ai[0]);
+                float sum = 0.f;
+#pragma unroll 1
+                for (int c = 0; c < kHalfBlks; ++c) {
+                    const int cb = C * 4 + c;
+                    if (cb < rb) continue;                         // (blocks below the diagonal hold no pair i < j)
+                    float v[32];
+                    tmem_ld32(taddr + c * kBlk, v);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const float4 cw = *reinterpret_cast<const float4*>(&sm.w[ew][c * kBlk + 4 * q]);
+                        float4 ca = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (METRIC == 1) ca = *reinterpret_cast<const float4*>(&sm.a[ew][c * kBlk + 4 * q]);
+#pragma unroll
+                        for (int p = 0; p < 2; ++p) {              // two neighbouring columns at a time
+                            const int u = 4 * q + 2 * p;
+                            const f32x2 x = mul2(pack2(v[u], v[u + 1]), p ? pack2(cw.z, cw.w) : pack2(cw.x, cw.y));
+                            const f32x2 base = METRIC == 0 ? two2 : add2(ai2, p ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y));
+                            const float2 d = unpack2(fma2(x, m2w2, base));
+                            const float2 arg = unpack2(mul2(pack2(fmaxf(d.x, 0.f), fmaxf(d.y, 0.f)), c22));
+                            v[u] = ex2_approx(arg.x);
+                            v[u + 1] = ex2_approx(arg.y);
+                        }
+                    }
+                    if (cb == rb || (cb + 1) * kBlk > g.n) {       // pairs that are none: j <= i, tokens past the sample
+#pragma unroll
+                        for (int u = 0; u < 32; ++u) {
+                            const int j = cb * kBlk + u;
+                            v[u] = (j > i && j < g.n) ? v[u] : 0.f;
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) sum += v[u];
+                }
+                if (i < g.n) g.part[((size_t)it.b * g.t.slots() + C) * g.t.n_pad + i] = sum;
+            }
+            if (ok && work && !row_role) {
+                float* const blocks = g.gram + (size_t)it.b * g.t.tiles_per_b * kSweepTileFloats;
+                float rblk[kHalfBlks] = {kInf, kInf, kInf, kInf};  // minimum of this thread's row over each of the four blocks
+#pragma unroll
+                for (int c = 0; c < kHalfBlks; ++c) {
+                    const int cb = C * 4 + c;
+                    float csum = 0.f, cmin = kInf;
+                    if (cb >= rb) {
+                        uint32_t r[32];
+                        tmem_ld_16x32_issue(taddr + c * kBlk, r);
+                        tmem_ld_16x32_issue(taddr + c * kBlk + (16u << 16), r + 16);
+                        tmem_ld_wait32(r);
+                        if (!far) {
+                            float4* dst = reinterpret_cast<float4*>(blocks + gram_block_offset(rb, cb)) + lane;
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                __stcs(dst + q * 32, make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                                                                 __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3])));
+                        }
+                        // ---- squared distances
+                        float d[32];                               // [m][k][r]: row lrow + 8 m, column 8 k + lcol + r
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 cw = *reinterpret_cast<const float2*>(&sm.w[ew][c * kBlk + 8 * q + lcol]);
+                            float2 ca = make_float2(0.f, 0.f);
+                            if (METRIC == 1) ca = *reinterpret_cast<const float2*>(&sm.a[ew][c * kBlk + 8 * q + lcol]);
+                            const f32x2 cw2 = pack2(cw.x, cw.y), ca2 = pack2(ca.x, ca.y);
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                const int at = (m >> 1) * 16 + q * 4 + (m & 1) * 2;
+                                const f32x2 x = mul2(pack2(__uint_as_float(r[at]), __uint_as_float(r[at + 1])), cw2);
+                                const f32x2 base = METRIC == 0 ? two2 : add2(pack2(ai[m], ai[m]), ca2);
+                                const float2 o = unpack2(fma2(x, pack2(m2w[m], m2w[m]), base));
+                                d[m * 8 + q * 2] = fmaxf(o.x, 0.f);
+                                d[m * 8 + q * 2 + 1] = fmaxf(o.y, 0.f);
+                            }
+                        }
+                        const bool edge = cb == rb || (cb + 1) * kBlk > g.n;
+                        if (edge) {                                // pairs that are none lie infinitely far apart
+#pragma unroll
+                            for (int u = 0; u < 32; ++u) {
+                                const int i = i0 + lrow + 8 * (u >> 3), j = cb * kBlk + 8 * ((u >> 1) & 3) + lcol + (u & 1);
+                                d[u] = (j > i && j < g.n) ? d[u] : kInf;
+                            }
+                        }
+                        // ---- block minima of both sides (none where the block lies beyond the spatial radius)
+                        if (!far) {
+                            float rm[4], cm[8];
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                const float* x = d + m * 8;
+                                rm[m] = fminf(fminf(fminf(x[0], x[1]), fminf(x[2], x[3])), fminf(fminf(x[4], x[5]), fminf(x[6], x[7])));
+                            }
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) cm[q] = fminf(fminf(d[q], d[8 + q]), fminf(d[16 + q], d[24 + q]));
+                            rblk[c] = reduce_rows_min(rm, lane);
+                            cmin = reduce_columns<true>(cm, lane);
+                        }
+                        // ---- Eq. 2, column side: the sum of 32 rows as a tree over the bits of the row, highest first
+#pragma unroll
+                        for (int u = 0; u < 32; u += 2) {
+                            const float2 x = unpack2(mul2(pack2(d[u], d[u + 1]), c22));
+                            if (edge) {
+                                d[u] = d[u] == kInf ? 0.f : ex2_approx(x.x);
+                                d[u + 1] = d[u + 1] == kInf ? 0.f : ex2_approx(x.y);
+                            } else {
+                                d[u] = ex2_approx(x.x);
+                                d[u + 1] = ex2_approx(x.y);
+                            }
+                        }
+                        float cs[8];
+#pragma unroll
+                        for (int q = 0; q < 8; q += 2) {
+                            const f32x2 even = add2(pack2(d[q], d[q + 1]), pack2(d[16 + q], d[17 + q]));
+                            const f32x2 odd = add2(pack2(d[8 + q], d[9 + q]), pack2(d[24 + q], d[25 + q]));
+                            const float2 o = unpack2(add2(even, odd));
+                            cs[q] = o.x;
+                            cs[q + 1] = o.y;
+                        }
+                        csum = reduce_columns<false>(cs, lane);
+                    }
+                    const int at = h * BM + c * kBlk + column_of(lane);
+                    sm.colsum[parity][quarter][at] = csum;
+                    sm.colmin[parity][quarter][at] = cmin;
+                }
+                // ---- row minima of row lrow + 8 (T % 4); those of the block on the diagonal are joined with the column side below
+                const int row = quarter * kBlk + lrow + 8 * (lane & 3), i = R * BM + row;
+                const float4 mins = make_float4(rblk[0], rblk[1], rblk[2], rblk[3]);
+                if (R == C) *reinterpret_cast<float4*>(sm.rowmin[parity][row]) = mins;
+                else if (i < g.n) *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + i) * nb + 4 * C) = mins;
+            }
+            // this warp has read all it needs from the accumulator
+            if (ok) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(cluster_map(bar_tempty + 8 * acc, 0));
+            }
+            if (epi_bar_or<kEpiThreads>(!ok)) { ok = false; break; }
+            // ---- column side, one column per thread: the sums of the four row quarters in order, the minima as they are.  (The
+            //      arrays of the other parity are free for the next tile meanwhile.)
+            const int half = e / BM, cc = C0 + half, j = cc * BM + e % BM;
+            if (e < BN && half < it.halves && R <= cc && j < g.n) {
+                const float(*cs)[BN] = sm.colsum[parity];
+                const float(*cm)[BN] = sm.colmin[parity];
+                const int slot = R == cc ? TI : R;                 // (slot R of the own block holds the row side)
+                g.part[((size_t)it.b * g.t.slots() + slot) * g.t.n_pad + j] = ((cs[0][e] + cs[1][e]) + cs[2][e]) + cs[3][e];
+                float4 m = make_float4(cm[0][e], cm[1][e], cm[2][e], cm[3][e]);
+                if (R == cc) {                                     // both sides speak about the same blocks
+                    const float4 o = *reinterpret_cast<const float4*>(sm.rowmin[parity][e % BM]);
+                    m = make_float4(fminf(m.x, o.x), fminf(m.y, o.y), fminf(m.z, o.z), fminf(m.w, o.w));
+                }
+                *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + j) * nb + 4 * R) = m;
+            }
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        }
+        if (!ok && lane == 0) raise_abort_pair(abort_addr, rank);
+    }
+
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) {
+        // Some role gave up, so loads issued here may never have been consumed: give the copies still in flight into this
+        // CTA's shared memory time to land before the CTA goes away.  (The other CTA's land on the leader's barriers.)
+        if (rank == 0) {
+            for (int s = 0; s < kStages; ++s)
+                if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
+        } else if (issued) {
+            const unsigned long long t0 = global_ns();
+            while (global_ns() - t0 < kDrainLimitNs) {}
+        }
+        if (g.status) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                                    // neither CTA leaves while the other may reach into it
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, kTmemCols);
+    }
+}
+
+}  // namespace
+
+int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cudaStream_t stream, bool pdl) {
+    KernelArgs k;
+    k.g = args;
+    k.wait_ns = gram_wait_limit_ns();
+    k.expire_roles = gram_expire_roles();
+    const long long total = (long long)args.B * args.t.tiles_per_b;
+    if (total <= 0) return VITCOP_OK;
+    if (2 * total > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
+    const long long pairs = gram_num_sms() / 2 > 0 ? gram_num_sms() / 2 : 1;
+    const long long last = total % pairs, cut = 2 * last <= pairs ? last : 0;
+    k.n_full = (int)(total - cut);
+    k.n_items = (int)(total + cut);
+    CUtensorMap ma, mb;
+    if (!make_rowmajor_bf16_map(&ma, feat, args.B, args.n, args.D, BM) ||
+        !make_rowmajor_bf16_map(&mb, feat, args.B, args.n, args.D, kBoxRows))
+        return VITCOP_ERR_CUDA;
+    const int smem = metric == 1 ? smem_bytes<1>() : smem_bytes<0>();
+    auto kern = metric == 1 ? density_sweep_kernel<1> : density_sweep_kernel<0>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return record_cuda(e);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * (k.n_items < pairs ? k.n_items : pairs)));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl_allowed(pdl) ? 1 : 0;
+    KernelTimeScope timed("density_sweep_kernel", stream);
+    return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
+}
+
+}  // namespace vitcop

@@ -2,19 +2,20 @@
 //
 // Pipeline (one stream, no host synchronisation; consecutive kernels overlap through programmatic dependent
 // launch, each waiting for its predecessor before it reads what that one wrote):
-//   1. Gram sweep, GRAM_DIAG  the diagonal tiles only: g_ii -> per-token factors (cosine: 1/sqrt(g_ii);
-//                             euclid: g_ii), from the same tensor-core arithmetic as every g_ij
-//   2. Gram sweep, GRAM_RHO   Gram tiles on the tensor cores (gram.cu); the epilogue turns each tile into
-//                             squared distances, exp(-(d/d_c)^2) and partial sums of Eq. 2 per tile, and, for
-//                             long samples, keeps the tile's Gram values in the workspace
+//   1. Gram diagonal          the diagonal tiles only: g_ii -> per-token factors (cosine: 1/sqrt(g_ii);
+//                             euclid: g_ii), from the same tensor-core arithmetic as every g_ij (gram.cu)
+//   2. density_sweep_kernel   Gram tiles on the tensor cores (density.cu); the epilogue turns each tile into
+//                             squared distances, exp(-(d/d_c)^2) and partial sums of Eq. 2, keeps the Gram values in the
+//                             workspace and leaves the smallest distance of every token to every block of 32 tokens
 //   3. rho_reduce_kernel      fixed-order sum of the partials -> rho (bit-reproducible)
-//   4. delta_pass_kernel      (long samples) reads the tiles back (delta_pass.cu) and keeps, per token, the nearest
-//                             denser token inside the spatial radius (Eq. 3) as a packed (d^2, j) 64-bit minimum;
-//      Gram sweep, GRAM_DELTA (otherwise) the same tiles computed again, Eq. 3 in the epilogue
+//   4. nearest_denser_kernel  (nearest.cu) searches the few blocks that can hold it for each token's nearest denser
+//                             token inside the spatial radius (Eq. 3): packed (d^2, j)
+//   (2-4 run sample group by sample group where the Gram values of the whole batch would take more than 1.5 GB)
 //   5. vic_finalize_kernel    gamma = rho * delta, radix-select of the centres, pointer jumping over the
 //                             parent forest, orphan fallback, labels (Algorithm 2, steps 3-4)
 // Small problems replace 1-4 by gram_resident_kernel (gram.cu): one pass over the Gram tiles, accumulators kept in
 // tensor memory.
+#include "density.cuh"
 #include "gram.cuh"
 
 namespace vitcop {
@@ -23,101 +24,77 @@ namespace {
 // ------------------------------------------------------------------------------------------------
 // small kernels
 // ------------------------------------------------------------------------------------------------
-// rho[b,i] = sum of the partials of the tiles that hold token i, in a fixed order (reproducible bits): the row-side
-// slots of the column tiles that pair row tile i / 128 with later tokens, then the column-side slots of the row tiles
-// that pair column tile i / BN with earlier tokens -- one contiguous range of slots.  LANES neighbouring lanes share a
-// token: each adds its part of the range slot by slot (sixteen independent loads at a time), and the sums are added
-// in lane order.  A long sample has up to 190 slots per token, which one thread alone would fetch in a dozen
-// dependent rounds; for a few dozen slots one thread per token is the faster shape.
+// rho[b,i] = sum of the partials of the density sweep in a fixed order (reproducible bits): first the later tokens, 256 at a
+// time (a tile's columns: the sum of its two 128-token blocks), then the earlier ones, one 128-token block after the other, to
+// the end of the token's tile (blocks that hold none of them count as zero).  LANES neighbouring lanes share a token: each adds
+// its part of that list (sixteen independent loads at a time), and the sums are added in lane order.  A long sample has a list
+// of up to 190 entries, which one thread alone would fetch in a dozen dependent rounds; for a few dozen entries one
+// thread per token is the faster shape.  blk_rho[b,k]: bits of the largest density among the tokens of block k (densities are
+// not negative, their bit patterns order like the values).
 constexpr int kRhoLanesLong = 4;
-constexpr int kRhoLongSlots = 64;                          // samples with more slots than this take kRhoLanesLong lanes
+constexpr int kRhoLongEntries = 64;                        // samples with longer lists than this take kRhoLanesLong lanes
+constexpr int kRhoThreads = 256;
 template <int LANES>
-__global__ void rho_reduce_kernel(const float* __restrict__ part, int n, GramTiling t, float* __restrict__ rho,
-                                  float* __restrict__ rho_user) {
+__global__ void __launch_bounds__(kRhoThreads)
+rho_reduce_kernel(const float* __restrict__ part, int n, SweepTiling t, float* __restrict__ rho,
+                  float* __restrict__ rho_user, uint32_t* __restrict__ blk_rho) {
+    constexpr int kBlocks = kRhoThreads / LANES / kBlk;    // blocks of 32 tokens per CTA
+    __shared__ uint32_t top[kBlocks];
     grid_dependency_launch_dependents();
     grid_dependency_wait();
+    if (threadIdx.x < kBlocks) top[threadIdx.x] = 0u;
+    __syncthreads();
     const int q = threadIdx.x % LANES;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+    const int local = threadIdx.x / LANES;
+    const int i = blockIdx.x * (kRhoThreads / LANES) + local;
     const int b = blockIdx.y;
     const bool valid = i < n;                              // (all lanes stay for the shuffles)
     float s = 0.f;
     if (valid) {
-        const int ti = i / kGramBM, tj = i / t.BN;
-        const int cap = t.R * (tj + 1);
-        const int first = ti / t.R, last = t.TJ + (t.TI < cap ? t.TI : cap);
-        const int per = (last - first + LANES - 1) / LANES;
-        const int c0 = first + q * per, c1 = min(last, c0 + per);
+        const int own = i / kGramBM, tile = own / 2;
+        const int rows = t.T - tile;                       // entries on the row side, then min(TI, 2 (tile + 1)) more
+        const int entries = rows + min(t.TI, 2 * (tile + 1));
+        const int per = (entries + LANES - 1) / LANES;
+        const int c0 = q * per, c1 = min(entries, c0 + per);
         const float* p = part + (size_t)b * t.slots() * t.n_pad + i;
-        for (int c = c0; c < c1; c += 16) {
-            float v[16];
+        auto slot = [&](int k) { return p[(size_t)k * t.n_pad]; };
+        for (int c = c0; c < c1; c += 8) {
+            float v[8], v2[8];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = (c + u < c1) ? p[(size_t)(c + u) * t.n_pad] : 0.f;
+            for (int u = 0; u < 8; ++u) {
+                const int e = c + u;
+                v[u] = v2[u] = 0.f;
+                if (e < c1) {
+                    if (e < rows) {
+                        const int k = 2 * (tile + e);
+                        if (k >= own) v[u] = slot(k);
+                        if (k + 1 >= own && k + 1 < t.TI) v2[u] = slot(k + 1);
+                    } else {
+                        const int k = e - rows;
+                        if (k <= own) v[u] = slot(k == own ? t.TI : k);
+                    }
+                }
+            }
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
-                if (c + u < c1) s += v[u];
+            for (int u = 0; u < 8; ++u)
+                if (c + u < c1) s += v[u] + v2[u];
         }
     }
     float others[LANES];
 #pragma unroll
     for (int u = 1; u < LANES; ++u) others[u] = __shfl_down_sync(0xffffffffu, s, u);
-    if (!valid || q != 0) return;
 #pragma unroll
     for (int u = 1; u < LANES; ++u) s += others[u];
-    rho[(size_t)b * n + i] = s;
-    if (rho_user) rho_user[(size_t)b * n + i] = s;
-}
-
-// The tiles of the symmetric numbering that lie within the spatial radius (gram.cuh: tile_outside_radius), in
-// ascending order: list[0 .. *count).  One small CTA that fits on an SM beside a CTA of the density sweep: it is
-// queued behind that sweep, does its work while the sweep runs and only then waits for it, so that the kernels
-// queued behind see both complete.  Thread t tests the tiles [t E, (t + 1) E) of a round of 256 E tiles with all its
-// loads in flight; one scan per round places them.
-constexpr int kKeptThreads = 256;
-constexpr int kKeptPerThread = 16;
-__global__ void __launch_bounds__(kKeptThreads)
-kept_tiles_kernel(const float4* __restrict__ bbox, GramTiling t, long long total, float tau2, int32_t* __restrict__ list,
-                  int32_t* __restrict__ count) {
-    __shared__ uint32_t warp_sums[kKeptThreads / 32];
-    grid_dependency_launch_dependents();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t placed = 0;
-    for (long long base = 0; base < total; base += (long long)kKeptThreads * kKeptPerThread) {
-        uint32_t keep = 0;
-#pragma unroll
-        for (int e = 0; e < kKeptPerThread; ++e) {
-            const long long tile = base + (long long)threadIdx.x * kKeptPerThread + e;
-            if (tile < total) {
-                int b, ti, tj;
-                decode_sym_tile(t, tile, b, ti, tj);
-                if (!tile_outside_radius(bbox + (size_t)b * t.TI, t, ti, tj, tau2)) keep |= 1u << e;
-            }
-        }
-        // exclusive prefix of the per-thread counts over the CTA, in thread order
-        const uint32_t mine = __popc(keep);
-        uint32_t incl = mine;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += o;
-        }
-        __syncthreads();                                   // (the previous round's sums have been read)
-        if (lane == 31) warp_sums[warp] = incl;
-        __syncthreads();
-        uint32_t before = 0, round_total = 0;
-#pragma unroll
-        for (int w = 0; w < kKeptThreads / 32; ++w) {
-            const uint32_t v = warp_sums[w];
-            if (w < warp) before += v;
-            round_total += v;
-        }
-        uint32_t pos = placed + before + incl - mine;
-#pragma unroll
-        for (int e = 0; e < kKeptPerThread; ++e)
-            if (keep >> e & 1u) list[pos++] = (int32_t)(base + (long long)threadIdx.x * kKeptPerThread + e);
-        placed += round_total;
+    const bool mine = valid && q == 0;
+    if (mine) {
+        rho[(size_t)b * n + i] = s;
+        if (rho_user) rho_user[(size_t)b * n + i] = s;
     }
-    if (threadIdx.x == 0) *count = (int32_t)placed;
-    grid_dependency_wait();
+    const uint32_t m = __reduce_max_sync(0xffffffffu, mine ? __float_as_uint(s) : 0u);
+    if ((threadIdx.x & 31) == 0) atomicMax(&top[local / kBlk], m);
+    __syncthreads();
+    const int k = blockIdx.x * kBlocks + threadIdx.x;
+    if (threadIdx.x < kBlocks && k < t.n_blk()) blk_rho[(size_t)b * t.n_blk() + k] = top[threadIdx.x];
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -367,12 +344,12 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
 // host side
 // ------------------------------------------------------------------------------------------------
 // Workspace of the filter: status block | row-block flags [B, ceil(n / 128)] | w | a | rho | best |
-// rho partials [B, slots, n_pad] (sized for either tile width) | bounding boxes of the row blocks' positions |
-// count and list of the tiles within the spatial radius | Gram tiles of the density sweep (problems too large
-// for the one-kernel sweep: 4 bytes per pair of the symmetric half, tile padding included).  The status block and the
+// rho partials [B, slots, n_pad] (sized for either sweep) | bounding boxes of the row blocks' positions | and, for
+// problems too large for the one-kernel sweep, of one group of samples: block densities, block minima, Gram values of
+// the density sweep (4 bytes per pair of the symmetric half, tile padding included).  The status block and the
 // flags are zeroed at the start of every call.  Words of the status block: 0 status, 2 grid barrier.
 struct FilterWs {
-    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_kept, off_tiles, total;
+    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_blk_rho, off_blk_min, off_gram, total;
     FilterWs(int B, int n) {
         size_t o = kStatusBytes;
         const size_t bn = (size_t)B * n;
@@ -381,16 +358,16 @@ struct FilterWs {
         off_a = o;    o += align_up(bn * 4, 256);
         off_rho = o;  o += align_up(bn * 4, 256);
         off_best = o; o += align_up(bn * 8, 256);
-        const GramTiling t = make_gram_tiling(n, 128);           // the narrow tiling has the most slots
+        const GramTiling t = make_gram_tiling(n, 128);           // (two slots per block: never fewer than the density sweep's)
         off_part = o; o += align_up((size_t)B * t.slots() * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
-        off_kept = off_tiles = o;
-        if (gram_keeps_tiles(B, n)) {
-            const int bn = gram_pick_bn(B, n);
-            const size_t tiles = (size_t)B * make_gram_tiling(n, bn).tiles_per_b;
-            o += align_up((tiles + 1) * sizeof(int32_t), 256);    // count, then the list of kept tiles
-            off_tiles = o;
-            o += align_up(tiles * gram_tile_floats(bn) * 4, 256);
+        off_blk_rho = off_blk_min = off_gram = o;
+        if (B > 0 && n > 0 && !gram_fits_resident(B, n)) {
+            const SweepTiling s = make_sweep_tiling(n);
+            const size_t group = (size_t)sweep_group_samples(B, n);
+            o += align_up(group * s.n_blk() * 4, 256);
+            off_blk_min = o; o += align_up(group * s.n_blk() * s.n_pad * 4, 256);
+            off_gram = o;    o += align_up(group * s.tiles_per_b * kSweepTileFloats * 4, 256);
         }
         total = o;
     }
@@ -433,7 +410,6 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     unsigned long long* best = reinterpret_cast<unsigned long long*>(ws + l.off_best);
     float* part = reinterpret_cast<float*>(ws + l.off_part);
 
-    const GramTiling tiling = make_gram_tiling(n, gram_pick_bn(B, n));
     GramArgs g = {};
     g.B = B; g.n = n; g.D = D; g.row0 = 0; g.row_end = n; g.metric = p.metric;
     g.c2 = -1.4426950408889634f / (p.d_c * p.d_c);
@@ -464,58 +440,42 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
         rc = launch_gram_resident(feat, g, make_gram_tiling(n, 128), stream);
         if (rc != VITCOP_OK) return rc;
     } else {
-        const bool keep_tiles = gram_keeps_tiles(B, n);
-        g.gram_tiles = keep_tiles ? reinterpret_cast<float*>(ws + l.off_tiles) : nullptr;
-        // with a spatial radius, tiles beyond it are neither kept nor read back (gram.cuh: tile_outside_radius)
-        g.bbox = (keep_tiles && g.tau2 >= 0.f) ? reinterpret_cast<float4*>(ws + l.off_bbox) : nullptr;
-        rc = launch_gram_sweep(GRAM_DIAG, feat, g, make_gram_tiling(n, 128), stream, false);
+        // with a spatial radius, blocks beyond it are neither kept nor looked into (density.cuh: blocks_outside_radius)
+        g.bbox = g.tau2 >= 0.f ? reinterpret_cast<float4*>(ws + l.off_bbox) : nullptr;
+        g.best = nullptr;                                  // (the search writes every token's entry)
+        rc = launch_gram_sweep(GRAM_DIAG, feat, g, stream, false);
         if (rc != VITCOP_OK) return rc;
-        rc = launch_gram_sweep(GRAM_RHO, feat, g, tiling, stream, true);
-        if (rc != VITCOP_OK) return rc;
-        if (g.bbox) {
-            // which tiles the delta pass will read: one small CTA beside the density sweep (the boxes come from the
-            // diagonal sweep, complete since the density sweep's epilogues started)
-            int32_t* cnt = reinterpret_cast<int32_t*>(ws + l.off_kept);
-            const long long tiles = (long long)B * tiling.tiles_per_b;
-            if (tiles > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
-            cudaLaunchConfig_t cfg;
-            cudaLaunchAttribute attr[1];
-            pdl_config(cfg, attr, dim3(1), dim3(kKeptThreads), 0, stream, true);
-            KernelTimeScope timed("kept_tiles_kernel", stream);
-            rc = record_cuda(cudaLaunchKernelEx(&cfg, kept_tiles_kernel, (const float4*)g.bbox, tiling, tiles, g.tau2, cnt + 1,
-                                                cnt));
+        const SweepTiling tiling = make_sweep_tiling(n);
+        const int group = sweep_group_samples(B, n);
+        for (int b0 = 0; b0 < B; b0 += group) {
+            const size_t at = (size_t)b0 * n;
+            SweepArgs s = {};
+            s.B = B - b0 < group ? B - b0 : group;
+            s.n = n; s.D = D; s.c2 = g.c2; s.tau2 = g.tau2;
+            s.w = w + at; s.a = a + at; s.rho = rho + at; s.best = best + at;
+            s.pos = pos ? pos + 2 * at : nullptr;
+            s.bbox = g.bbox ? g.bbox + (size_t)b0 * tiling.TI : nullptr;
+            s.part = part + (size_t)b0 * tiling.slots() * tiling.n_pad;
+            s.blk_rho = reinterpret_cast<uint32_t*>(ws + l.off_blk_rho);
+            s.blk_min = reinterpret_cast<float*>(ws + l.off_blk_min);
+            s.gram = reinterpret_cast<float*>(ws + l.off_gram);
+            s.status = g.status;
+            s.t = tiling;
+            rc = launch_density_sweep(static_cast<const uint16_t*>(feat) + at * D, s, p.metric, stream, true);
             if (rc != VITCOP_OK) return rc;
-            g.kept = cnt + 1;
-            g.n_kept = cnt;
-        }
-        {
-            cudaLaunchConfig_t cfg;
-            cudaLaunchAttribute attr[1];
-            const int lanes = tiling.slots() > kRhoLongSlots ? kRhoLanesLong : 1;
-            pdl_config(cfg, attr, dim3((n * lanes + 255) / 256, B), dim3(256), 0, stream, true);
-            KernelTimeScope timed("rho_reduce_kernel", stream);
-            rc = record_cuda(cudaLaunchKernelEx(&cfg, lanes == 1 ? rho_reduce_kernel<1> : rho_reduce_kernel<kRhoLanesLong>,
-                                                (const float*)part, n, tiling, rho, rho_user));
+            {
+                cudaLaunchConfig_t cfg;
+                cudaLaunchAttribute attr[1];
+                const int lanes = tiling.T + tiling.TI > kRhoLongEntries ? kRhoLanesLong : 1;
+                pdl_config(cfg, attr, dim3((n * lanes + kRhoThreads - 1) / kRhoThreads, s.B), dim3(kRhoThreads), 0, stream, true);
+                KernelTimeScope timed("rho_reduce_kernel", stream);
+                rc = record_cuda(cudaLaunchKernelEx(&cfg, lanes == 1 ? rho_reduce_kernel<1> : rho_reduce_kernel<kRhoLanesLong>,
+                                                    (const float*)s.part, n, tiling, rho + at,
+                                                    rho_user ? rho_user + at : nullptr, s.blk_rho));
+                if (rc != VITCOP_OK) return rc;
+            }
+            rc = launch_nearest_denser(s, p.metric, stream, true);
             if (rc != VITCOP_OK) return rc;
-        }
-        if (!keep_tiles) {
-            rc = launch_gram_sweep(GRAM_DELTA, feat, g, tiling, stream, true);
-            if (rc != VITCOP_OK) return rc;
-        }
-        // The delta pass is bound by ALU issue and by the read of the tiles, the K-norm by the read of K: given one,
-        // the pass leaves a quarter of every SM free and the K-norm, which depends on nothing in this call, runs
-        // beside it (it still waits for the pass before it ends, so the kernels behind it see both complete).
-        const bool knorm_beside = keep_tiles && knorm != nullptr;
-        if (keep_tiles) {
-            rc = launch_delta_pass(g, tiling, stream, true, knorm_beside);
-            if (rc != VITCOP_OK) return rc;
-        }
-        if (knorm_beside) {
-            rc = launch_knorm(knorm->K, knorm->B, knorm->H, knorm->d, (int64_t)knorm->H * knorm->N * knorm->d,
-                              (int64_t)knorm->N * knorm->d, knorm->d, knorm->vis_start, nullptr, knorm->Nv, knorm->score,
-                              knorm->Nv, stream, true);
-            if (rc != VITCOP_OK) return rc;
-            knorm_in_sweep = knorm->B;                     // nothing left for the launch behind vic_finalize_kernel
         }
     }
 
@@ -558,9 +518,9 @@ int launch_similarity_rows(const void* feat, int B, int n, int D, int metric, in
     g.B = B; g.n = n; g.D = D; g.row0 = row_begin; g.row_end = row_end; g.metric = metric;
     g.c2 = 0.f; g.tau2 = -1.f;
     g.w = w; g.a = a; g.w_out = w; g.a_out = a; g.sim_out = out; g.status = reinterpret_cast<int*>(ws);
-    int rc = launch_gram_sweep(GRAM_DIAG, feat, g, make_gram_tiling(n, 128), stream, false);
+    int rc = launch_gram_sweep(GRAM_DIAG, feat, g, stream, false);
     if (rc != VITCOP_OK) return rc;
-    return launch_gram_sweep(GRAM_SIM, feat, g, make_gram_tiling(n, 128), stream, true);
+    return launch_gram_sweep(GRAM_SIM, feat, g, stream, true);
 }
 
 }  // namespace vitcop

@@ -1,21 +1,19 @@
-// Tensor-core sweep over the Gram matrix of the visual-token features (Algorithm 2, step 1) with the
-// per-pair work of Eq. 2 (density) or Eq. 3 (nearest denser neighbour) fused into the epilogue.
+// Tensor-core work on the Gram matrix of the visual-token features (Algorithm 2, step 1): its diagonal (per-token factors), rows
+// of it (similarity), and, for small problems, the whole of Eq. 2 (density) and Eq. 3 (nearest denser neighbour) in one kernel.
+// Larger problems take density.cu and nearest.cu for the two equations.
 //
 // The Gram matrix f_I . f_J^T is taken on the RAW bf16 features (bf16 x bf16 products are exact in fp32) by
-// tcgen05.mma with fp32 accumulators in tensor memory; the L2 normalisation enters as fp32 factors in the
-// epilogue.  Nothing of size n^2 is ever written: the density sweep and the delta sweep each recompute the
-// tiles they need.
+// tcgen05.mma with fp32 accumulators in tensor memory; the L2 normalisation enters as fp32 factors in the epilogue.
 //
-// Symmetry: d_ij = d_ji, so the two sweeps visit only tiles that hold a pair i < j.  Such a pair serves its
+// Symmetry: d_ij = d_ji, so the one-kernel sweep visits only tiles that hold a pair i < j.  Such a pair serves its
 // row token i (a per-thread accumulation along the row) and its column token j (a reduction over the 128
 // rows of the tile: inside each warp a shuffle butterfly for the sums of Eq. 2 and one redux.sync per column for
 // the minima of Eq. 3, then a fixed-order combination of the four warps that share a column range).
 //
 // One persistent CTA per SM, warp-specialised:
-//   warp 0      TMA producer: feature tiles [128 x 64] and [BN x 64] (128-byte swizzle) into a ring of stages
-//   warp 1      one thread issues tcgen05.mma (M = 128, N = BN, K = 16) into one of two TMEM accumulators
-//   warps 2..   epilogue (8 warps for the density sweep, 16 for the delta sweep): warp w reads TMEM lanes
-//               32 * (w % 4) .. + 31 (its rows) and one slice of the columns
+//   warp 0      TMA producer: feature tiles [128 x 64] (128-byte swizzle) into a ring of stages
+//   warp 1      one thread issues tcgen05.mma into one of two TMEM accumulators
+//   warps 2..   epilogue: warp w reads TMEM lanes 32 * (w % 4) .. + 31 (its rows) and one slice of the columns
 // Every wait is bounded; on expiry the CTA raises an abort flag, all roles leave, TMEM is released and
 // VITCOP_ERR_TIMEOUT is written to the status word.
 #include <cuda.h>
@@ -196,7 +194,6 @@ struct EpiCall {
     bool rho_from_part;            // GRAM_DELTA: sum rho from the density partials (and publish it from diagonal tiles)
     volatile int* abort_flag;
     unsigned long long limit_ns;   // time limit of the wait for the accumulator
-    float* store;                  // GRAM_RHO: where this tile's Gram values go (gram.cuh: layout), or null
 };
 
 // Returns true when the CTA must give up (a bounded wait expired somewhere).
@@ -354,14 +351,6 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                     }
                 }
             } else if (MODE == GRAM_RHO) {
-                if (call.store) {
-                    // keep the Gram values for the delta pass: four columns of this thread's row per store, the
-                    // warp's 32 rows side by side
-                    float4* dst = reinterpret_cast<float4*>(call.store) + (size_t)(cl0 >> 2) * BM + rl;
-#pragma unroll
-                    for (int q4 = 0; q4 < GW / 4; ++q4)
-                        __stcs(dst + (size_t)q4 * BM, make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]));
-                }
                 // e_ij = exp(-d_ij^2 / d_c^2), Eq. 2
 #pragma unroll
                 for (int q4 = 0; q4 < GW / 4; ++q4) {
@@ -607,9 +596,6 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t bar_drain = bar_tempty + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S::kStages + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    // (the last words of the barrier block hold the epilogue's mask of tiles that are not kept)
-    static_assert((2 * S::kStages + 5) * 8 + 8 + (NS * 128 / 32) * 4 <= S::kBarBytes, "barrier block too small");
-
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t kTmemCols = 2 * BN;
 
@@ -635,11 +621,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t tmem_base = *tmem_slot;
 
     // The kernels that follow on the stream may be scheduled from here on; they wait for this grid to complete
-    // before they touch anything it writes.  A density sweep that has a kernel running beside it (filter.cu: the list
-    // of tiles within the spatial radius) releases them only once its own predecessors are complete, so that the
-    // neighbour may rely on their results without a wait of its own.
-    const bool release_late = MODE == GRAM_RHO && g.bbox != nullptr;
-    if (!release_late) grid_dependency_launch_dependents();
+    // before they touch anything it writes.
+    grid_dependency_launch_dependents();
 
     const long long total_tiles = k.total_tiles;
     const int KB = g.D / BK;
@@ -709,12 +692,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // ------------------------------------------------------------------ epilogue (warps 2 ..)
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        const bool skip_far = MODE == GRAM_RHO && g.gram_tiles && g.bbox;
-        uint32_t* far_mask = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(bars) + S::kBarBytes) - kEpiThreads / 32;
-        long long kt = 0;                                  // tiles this CTA has taken
-
         grid_dependency_wait();                            // w, a, rho, best come from the preceding kernels
-        if (release_late) grid_dependency_launch_dependents();
 
         for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
             EpiCall c;
@@ -726,27 +704,6 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             c.rho_from_part = false;
             c.abort_flag = abort_flag;
             c.limit_ns = k.limit_of(kRoleEpi);
-            c.store = (MODE == GRAM_RHO && g.gram_tiles) ? g.gram_tiles + (size_t)t * gram_tile_floats(BN) : nullptr;
-            if (skip_far) {
-                // a tile beyond the spatial radius is of no use to Eq. 3 and is not kept (gram.cuh:
-                // tile_outside_radius); the CTA's next kEpiThreads tiles are tested together, one per thread
-                const int kk = (int)(kt % kEpiThreads);
-                if (kk == 0) {
-                    epi_bar_sync<kEpiThreads>();               // (the previous mask has been read by everyone)
-                    const long long mine = t + (long long)(threadIdx.x - 64) * gridDim.x;
-                    bool far = false;
-                    if (mine < total_tiles) {
-                        int fb, fti, ftj;
-                        decode_tile<BN, SYM, DIAG>(k, mine, fb, fti, ftj);
-                        far = tile_outside_radius(g.bbox + (size_t)fb * k.t.TI, k.t, fti, ftj, g.tau2);
-                    }
-                    const uint32_t bal = __ballot_sync(0xffffffffu, far);
-                    if (lane == 0) far_mask[warp - 2] = bal;
-                    epi_bar_sync<kEpiThreads>();
-                }
-                if (far_mask[kk >> 5] >> (kk & 31) & 1u) c.store = nullptr;
-            }
-            ++kt;
             if (epi_tile<BN, MODE, METRIC, SPATIAL, NS>(k, sm, c, ok)) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -1099,7 +1056,6 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             c.rho_from_part = rho_from_part;
             c.abort_flag = abort_flag;
             c.limit_ns = lim;
-            c.store = nullptr;
             return c;
         };
 
@@ -1239,38 +1195,9 @@ int launch_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(pdl) ? 1 : 0;
-    KernelTimeScope timed(MODE == GRAM_RHO ? "gram_tc_kernel<rho>"
-                          : MODE == GRAM_DELTA ? "gram_tc_kernel<delta>"
-                          : MODE == GRAM_DIAG ? "gram_tc_kernel<diag>" : "gram_tc_kernel<sim>",
-                          stream);
+    KernelTimeScope timed(MODE == GRAM_DIAG ? "gram_tc_kernel<diag>" : "gram_tc_kernel<sim>", stream);
     return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
 }
-
-template <int BN>
-int launch_bn(int mode, const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream,
-              bool pdl) {
-    const bool euclid = k.g.metric == 1;
-    const bool spatial = k.g.tau2 >= 0.f && k.g.pos != nullptr;
-    switch (mode) {
-        case GRAM_RHO:
-            return euclid ? launch_one<BN, GRAM_RHO, 1, false>(ma, mb, k, stream, pdl)
-                          : launch_one<BN, GRAM_RHO, 0, false>(ma, mb, k, stream, pdl);
-        case GRAM_DELTA:
-            if (spatial)
-                return euclid ? launch_one<BN, GRAM_DELTA, 1, true>(ma, mb, k, stream, pdl)
-                              : launch_one<BN, GRAM_DELTA, 0, true>(ma, mb, k, stream, pdl);
-            return euclid ? launch_one<BN, GRAM_DELTA, 1, false>(ma, mb, k, stream, pdl)
-                          : launch_one<BN, GRAM_DELTA, 0, false>(ma, mb, k, stream, pdl);
-        case GRAM_DIAG:
-            if (BN != BM) return VITCOP_ERR_INVALID_ARG;
-            return euclid ? launch_one<BM, GRAM_DIAG, 1, false>(ma, mb, k, stream, pdl)
-                          : launch_one<BM, GRAM_DIAG, 0, false>(ma, mb, k, stream, pdl);
-        default:
-            return euclid ? launch_one<BN, GRAM_SIM, 1, false>(ma, mb, k, stream, pdl)
-                          : launch_one<BN, GRAM_SIM, 0, false>(ma, mb, k, stream, pdl);
-    }
-}
-
 
 template <int METRIC, bool SPATIAL>
 int launch_resident_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream) {
@@ -1311,31 +1238,19 @@ void gram_set_wait_debug(unsigned long long limit_ns, int expire_roles) {
     g_expire_roles.store(expire_roles & 7);
 }
 
-bool gram_keeps_tiles(int B, int n) {
-    return B > 0 && n >= kKeepTilesFromTokens && !gram_fits_resident(B, n) && gram_pick_bn(B, n) == 256;
-}
-
-int gram_pick_bn(int B, int n) {
-    const long long ti = (n + BM - 1) / BM;
-    const long long tiles128 = (long long)B * ti * (ti + 1) / 2;
-    return tiles128 >= 4LL * num_sms() ? 256 : 128;
-}
-
-int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream,
-                      bool pdl) {
+int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStream_t stream, bool pdl) {
+    if (mode != GRAM_DIAG && mode != GRAM_SIM) return VITCOP_ERR_INVALID_ARG;
     KernelArgs k;
     k.g = args;
-    k.t = tiling;
+    k.t = make_gram_tiling(args.n, BM);
     if (mode == GRAM_SIM) {
         // plain rectangle: rows [row0, row_end) x all columns
-        const int rows = args.row_end - args.row0;
-        k.t.TI = (rows + BM - 1) / BM;
-        k.t.TJ = (args.n + tiling.BN - 1) / tiling.BN;
+        k.t.TI = (args.row_end - args.row0 + BM - 1) / BM;
         k.t.tiles_per_b = k.t.TI * k.t.TJ;
     } else {
         k.g.row0 = 0;
         k.g.row_end = args.n;
-        if (mode == GRAM_DIAG) k.t.tiles_per_b = k.t.TI;        // one tile per 128-row block (tiling.BN == 128)
+        k.t.tiles_per_b = k.t.TI;                              // one tile per 128-row block
     }
     k.total_tiles = (long long)args.B * k.t.tiles_per_b;
     k.extra_units_per_b = 0;
@@ -1343,11 +1258,14 @@ int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, const Gr
     k.expire_roles = g_expire_roles.load();
     if (k.total_tiles <= 0) return VITCOP_OK;
     CUtensorMap ma, mb;
-    if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) ||
-        !make_feat_map(&mb, feat, args.B, args.n, args.D, tiling.BN))
+    if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) || !make_feat_map(&mb, feat, args.B, args.n, args.D, BM))
         return VITCOP_ERR_CUDA;
-    return tiling.BN == 256 ? launch_bn<256>(mode, ma, mb, k, stream, pdl)
-                            : launch_bn<128>(mode, ma, mb, k, stream, pdl);
+    const bool euclid = args.metric == 1;
+    if (mode == GRAM_DIAG)
+        return euclid ? launch_one<BM, GRAM_DIAG, 1, false>(ma, mb, k, stream, pdl)
+                      : launch_one<BM, GRAM_DIAG, 0, false>(ma, mb, k, stream, pdl);
+    return euclid ? launch_one<BM, GRAM_SIM, 1, false>(ma, mb, k, stream, pdl)
+                  : launch_one<BM, GRAM_SIM, 0, false>(ma, mb, k, stream, pdl);
 }
 
 bool gram_fits_resident(int B, int n) {

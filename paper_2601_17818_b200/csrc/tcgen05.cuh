@@ -1,5 +1,5 @@
 // tcgen05 (fifth-generation tensor core) and TMA plumbing in inline PTX, shared by the kernels that run a bf16 GEMM
-// with fp32 accumulators in tensor memory (gram.cu, kproj.cu).
+// with fp32 accumulators in tensor memory (gram.cu, density.cu, kproj.cu).
 #pragma once
 
 #include <cuda.h>
@@ -107,8 +107,10 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+// (Relaxed: what it announces is that tensor memory has been read, which tcgen05.wait::ld has completed; a release would
+// also wait for the thread's global stores to land.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_in_cluster) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_in_cluster) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_in_cluster) : "memory");
 }
 // As tma_load_3d into this CTA's shared memory, the bytes counted on a barrier of either CTA of the pair.
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar_in_cluster, int c0, int c1,

@@ -470,6 +470,43 @@ def test_filter_long_samples_scattered_positions():
         check_vic_sample(f[b], p[b], 0, w.d_c, 0.3, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
 
 
+# Too many tiles for the one-kernel sweep: pairs of CTAs on 256 x 256 tiles (ragged ends, an odd number of 128-token blocks, the
+# last tiles cut into column halves or not), block minima, the search.  Half of the last sample's tokens are one token plus
+# noise (plain copies would tie in every distance, and the oracle's report excuses ties): the densest of them have neighbours
+# in half of the blocks and none is denser, so the search hands them to the whole CTA.
+@pytest.mark.parametrize("B,n,metric,tau", [(16, 1153, 0, 0.6), (16, 1279, 1, -1.0), (17, 1281, 0, 0.1), (300, 127, 0, 0.6),
+                                             (80, 257, 1, 0.3)])
+def test_filter_sweep_and_search_edges(B, n, metric, tau):
+    w = dataclasses.replace(W.workload("tiny"), B=B, D=64, dup_rate=0.3)
+    f = W.make_features(w, n=n, B=B).copy()
+    rng = np.random.default_rng(n)
+    spread = 0.3 * np.exp(0.5 * rng.standard_normal((n - n // 2, 1)))
+    f[-1, n // 2:] = W.f32_to_bf16_bits(W.bf16_bits_to_f32(f[-1, 0]) + spread * rng.standard_normal((n - n // 2, 64)))
+    p = np.ascontiguousarray(np.broadcast_to(W.make_positions(w, n)[:1], (B, n, 2)))
+    d_c = w.d_c if metric == 0 else 8.0
+    nc = max(1, n // 20)
+    g = gpu_filter(f, p, metric, d_c, tau, nc)
+    assert g.status == vb.OK and np.all(g.n_clusters == nc)
+    for b in (0, B - 1):
+        check_vic_sample(f[b], p[b], metric, d_c, tau, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
+
+
+def test_filter_sample_groups():
+    """More Gram values than the workspace keeps at a time: the samples go through the sweep and the search in groups, and
+    give what each gives by itself."""
+    n = 16384
+    w = dataclasses.replace(W.workload("c4"), B=3, D=64, dup_rate=0.3)
+    f = W.make_features(w, n=n, B=3)
+    p = W.make_positions(dataclasses.replace(w, B=3), n)
+    nc = n // 20
+    g = gpu_filter(f, p, 0, w.d_c, w.tau, nc)
+    assert g.status == vb.OK
+    for b in range(3):
+        one = gpu_filter(f[b:b + 1], p[b:b + 1], 0, w.d_c, w.tau, nc)
+        for key in ("rho", "delta2", "parent", "label"):
+            assert np.array_equal(getattr(g, key)[b], getattr(one, key)[0]), key
+
+
 def test_filter_edge_cases():
     w = W.workload("tiny")
     # identical tokens: one cluster led by token 0
