@@ -8,11 +8,12 @@
 // tensor cores, falls by a third.  Warp 0 loads, one thread of the leader's warp 1 issues the MMAs into one of two
 // accumulators, 16 epilogue warps per CTA drain the other, in two roles; warp (q, h) of either takes rows 32 q .. + 31 of the CTA
 // and columns 128 h .. + 127, in four blocks of 32 x 32 pairs:
-//   column warps   keep the Gram values, the block minima of both sides and the column sums of Eq. 2.  They read the accumulator
-//                  in the 16-lanes x 256-bit shape: a thread holds 4 rows x 8 columns of a block, so that both sides reduce
-//                  mostly inside the thread and only 4 and 8 values a thread go through shuffles.  (With one row per thread, as
-//                  the 32-lane shape gives it, every column costs a butterfly or a redux over 32 lanes.)
-//   row warps      the row sums of Eq. 2, one row per thread, column by column: that order of the sums is part of the result.
+//   row warps      one row per thread: store the Gram values, take the row tokens' block minima and their sums of Eq. 2, column
+//                  by column (that order of the sums is part of the result).
+//   column warps   the column tokens' block minima and sums.  They read the accumulator in the 16-lanes x 256-bit shape: a
+//                  thread holds 4 rows x 8 columns of a block, so that columns reduce partly inside the thread and only 8 values
+//                  go through shuffles.  (With one row per thread every column costs a butterfly or a redux over 32 lanes.)
+// Distances and exponentials are computed by both, which is cheaper than passing them on.
 //
 // Measured with sixteen warps of one role: 8 x 2880 x 1024 70 us, 60 us with an empty epilogue; 2 x 16384 x 1280 517 us, 484 us
 // without the stores of the Gram values, 433 us with an empty epilogue (0.69 Tflop at the rate cuBLAS reaches in a burst).  The
@@ -52,6 +53,7 @@ static_assert(smem_bytes<0>() <= 227 * 1024 && smem_bytes<1>() <= 227 * 1024, "s
 struct KernelArgs {
     SweepArgs g;
     int n_full, n_items;           // tiles taken whole; work items (the other tiles count twice)
+    float inv_tiles;               // 1 / tiles_per_b
     unsigned long long wait_ns;
     int expire_roles;
     __device__ __forceinline__ unsigned long long limit_of(int role) const { return (expire_roles & role) ? 0ull : wait_ns; }
@@ -68,11 +70,16 @@ __device__ __forceinline__ Item decode_item(const KernelArgs& k, int t) {
     Item it;
     it.halves = x < 0 ? 2 : 1;
     it.half = x < 0 ? 0 : (x & 1);
-    it.b = tile / k.g.t.tiles_per_b;
-    const int r = tile - it.b * k.g.t.tiles_per_b;
-    int q = (int)((sqrtf(8.f * (float)r + 1.f) - 1.f) * 0.5f);
-    while (q > 0 && q * (q + 1) / 2 > r) --q;
-    while ((q + 1) * (q + 2) / 2 <= r) ++q;
+    // (every warp decodes every item, so without divisions: the estimates are off by one at most)
+    const int per = k.g.t.tiles_per_b;
+    int b = (int)((float)tile * k.inv_tiles);
+    int r = tile - b * per;
+    if (r < 0) { --b; r += per; }
+    if (r >= per) { ++b; r -= per; }
+    int q = (int)((__fsqrt_rn(8.f * (float)r + 1.f) - 1.f) * 0.5f);
+    if (q * (q + 1) / 2 > r) --q;
+    if ((q + 1) * (q + 2) / 2 <= r) ++q;
+    it.b = b;
     it.tj = q;
     it.tp = r - q * (q + 1) / 2;
     return it;
@@ -112,6 +119,12 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // 16 lanes x 32 columns of the accumulator: register 4 k + 2 p + r holds row T / 4 + 8 p, column 8 k + 2 (T % 4) + r.
 __device__ __forceinline__ void tmem_ld_16x32_issue(uint32_t taddr, uint32_t* r) {
     asm volatile(
@@ -134,14 +147,6 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
 
 template <bool MIN>
 __device__ __forceinline__ float join(float a, float b) { return MIN ? fminf(a, b) : a + b; }
-// Four values per thread, one per row T / 4 + 8 m: afterwards the thread holds the minimum over its group of four lanes of
-// value m = T % 4.
-__device__ __forceinline__ float reduce_rows_min(const float (&v)[4], int lane) {
-    const bool u2 = lane & 2, u1 = lane & 1;
-    const float a0 = fminf(u2 ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, u2 ? v[0] : v[2], 2));
-    const float a1 = fminf(u2 ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, u2 ? v[1] : v[3], 2));
-    return fminf(u1 ? a1 : a0, __shfl_xor_sync(0xffffffffu, u1 ? a0 : a1, 1));
-}
 // Eight values per thread, value 2 k + r for column 8 k + 2 (T % 4) + r: afterwards the thread holds the total over the eight
 // lanes with its T % 4 of column column_of(T), joined as a tree over the bits of T / 4, highest first.
 template <bool MIN>
@@ -309,8 +314,7 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             const bool work = h < it.halves && R <= C && C < TI;           // (R > C: below the diagonal)
             const int i0 = R * BM + quarter * kBlk;
             const int rb = R * 4 + quarter;                                // the warp's rows as a block of 32
-            const int step = row_role ? 0 : 8;                             // rows of the thread: first, first + step, ..
-            const int first = i0 + (row_role ? lane : lrow);
+            const int first = i0 + (row_role ? lane : lrow);               // rows of the thread: first (, first + 8, ..)
             float m2w[4], ai[4];
             bool far = false;
             if (work) {
@@ -320,11 +324,18 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                     const int j = C * BM + u * 32 + lane;
                     sm.w[ew][u * 32 + lane] = j < g.n ? g.w[bo + j] : 0.f;
                     if (METRIC == 1) sm.a[ew][u * 32 + lane] = j < g.n ? g.a[bo + j] : 0.f;
-                    const int i = first + u * step;
-                    m2w[u] = i < g.n ? -2.f * g.w[bo + i] : 0.f;
-                    ai[u] = (METRIC == 1 && i < g.n) ? g.a[bo + i] : 0.f;
                 }
-                if (g.bbox && !row_role)
+                m2w[0] = first < g.n ? -2.f * g.w[bo + first] : 0.f;
+                ai[0] = (METRIC == 1 && first < g.n) ? g.a[bo + first] : 0.f;
+                if (!row_role) {
+#pragma unroll
+                    for (int m = 1; m < 4; ++m) {
+                        const int i = first + 8 * m;
+                        m2w[m] = i < g.n ? -2.f * g.w[bo + i] : 0.f;
+                        ai[m] = (METRIC == 1 && i < g.n) ? g.a[bo + i] : 0.f;
+                    }
+                }
+                if (g.bbox)
                     far = blocks_outside_radius(g.bbox[(size_t)it.b * TI + R], g.bbox[(size_t)it.b * TI + C], g.tau2);
                 __syncwarp();
             }
@@ -336,13 +347,21 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                 // ---- Eq. 2, row side: exp(-d^2 / d_c^2) of this thread's row, added column by column
                 const int i = first;
                 const f32x2 m2w2 = pack2(m2w[0], m2w[0]), ai2 = pack2(ai[0], ai[0]);
+                float* const blocks = g.gram + (size_t)it.b * g.t.tiles_per_b * kSweepTileFloats;
                 float sum = 0.f;
+                float4 mins = make_float4(kInf, kInf, kInf, kInf); // of the row over each of the four blocks
 #pragma unroll 1
                 for (int c = 0; c < kHalfBlks; ++c) {
                     const int cb = C * 4 + c;
                     if (cb < rb) continue;                         // (blocks below the diagonal hold no pair i < j)
                     float v[32];
                     tmem_ld32(taddr + c * kBlk, v);
+                    if (!far) {
+                        float4* dst = reinterpret_cast<float4*>(blocks + gram_block_offset(rb, cb)) + lane;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            __stcs(dst + q * 32, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+                    }
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         const float4 cw = *reinterpret_cast<const float4*>(&sm.w[ew][c * kBlk + 4 * q]);
@@ -354,12 +373,43 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                             const f32x2 x = mul2(pack2(v[u], v[u + 1]), p ? pack2(cw.z, cw.w) : pack2(cw.x, cw.y));
                             const f32x2 base = METRIC == 0 ? two2 : add2(ai2, p ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y));
                             const float2 d = unpack2(fma2(x, m2w2, base));
-                            const float2 arg = unpack2(mul2(pack2(fmaxf(d.x, 0.f), fmaxf(d.y, 0.f)), c22));
-                            v[u] = ex2_approx(arg.x);
-                            v[u + 1] = ex2_approx(arg.y);
+                            v[u] = d.x;
+                            v[u + 1] = d.y;
                         }
                     }
-                    if (cb == rb || (cb + 1) * kBlk > g.n) {       // pairs that are none: j <= i, tokens past the sample
+                    const bool edge = cb == rb || (cb + 1) * kBlk > g.n;
+                    if (edge) {                                    // pairs that are none (j <= i, tokens past the sample): far apart
+#pragma unroll
+                        for (int u = 0; u < 32; ++u) {
+                            const int j = cb * kBlk + u;
+                            v[u] = (j > i && j < g.n) ? v[u] : kInf;
+                        }
+                    }
+                    float mn = min3(v[0], v[1], v[2]), mn2 = min3(v[3], v[4], v[5]);
+#pragma unroll
+                    for (int u = 6; u < 30; u += 4) {
+                        mn = min3(mn, v[u], v[u + 1]);
+                        mn2 = min3(mn2, v[u + 2], v[u + 3]);
+                    }
+                    mn = min3(min3(mn, v[30], v[31]), mn2, kInf);
+                    // (rounding can leave a near-duplicate's d^2 below zero: rare, so looked for before all are clamped)
+                    if (__any_sync(0xffffffffu, mn < 0.f)) {
+#pragma unroll
+                        for (int u = 0; u < 32; ++u) v[u] = fmaxf(v[u], 0.f);
+                        mn = fmaxf(mn, 0.f);
+                    }
+                    if (far) mn = kInf;                            // (a block beyond the spatial radius has no minima)
+                    if (c == 0) mins.x = mn;
+                    if (c == 1) mins.y = mn;
+                    if (c == 2) mins.z = mn;
+                    if (c == 3) mins.w = mn;
+#pragma unroll
+                    for (int u = 0; u < 32; u += 2) {
+                        const float2 arg = unpack2(mul2(pack2(v[u], v[u + 1]), c22));
+                        v[u] = ex2_approx(arg.x);
+                        v[u + 1] = ex2_approx(arg.y);
+                    }
+                    if (edge) {
 #pragma unroll
                         for (int u = 0; u < 32; ++u) {
                             const int j = cb * kBlk + u;
@@ -370,11 +420,12 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                     for (int u = 0; u < 32; ++u) sum += v[u];
                 }
                 if (i < g.n) g.part[((size_t)it.b * g.t.slots() + C) * g.t.n_pad + i] = sum;
+                // (the block on the diagonal: joined with the column side below)
+                if (R == C) *reinterpret_cast<float4*>(sm.rowmin[parity][quarter * kBlk + lane]) = mins;
+                else if (i < g.n) *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + i) * nb + 4 * C) = mins;
             }
             if (ok && work && !row_role) {
-                float* const blocks = g.gram + (size_t)it.b * g.t.tiles_per_b * kSweepTileFloats;
-                float rblk[kHalfBlks] = {kInf, kInf, kInf, kInf};  // minimum of this thread's row over each of the four blocks
-#pragma unroll
+#pragma unroll 1
                 for (int c = 0; c < kHalfBlks; ++c) {
                     const int cb = C * 4 + c;
                     float csum = 0.f, cmin = kInf;
@@ -383,13 +434,6 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                         tmem_ld_16x32_issue(taddr + c * kBlk, r);
                         tmem_ld_16x32_issue(taddr + c * kBlk + (16u << 16), r + 16);
                         tmem_ld_wait32(r);
-                        if (!far) {
-                            float4* dst = reinterpret_cast<float4*>(blocks + gram_block_offset(rb, cb)) + lane;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                __stcs(dst + q * 32, make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                                                 __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3])));
-                        }
                         // ---- squared distances
                         float d[32];                               // [m][k][r]: row lrow + 8 m, column 8 k + lcol + r
 #pragma unroll
@@ -404,8 +448,8 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                                 const f32x2 x = mul2(pack2(__uint_as_float(r[at]), __uint_as_float(r[at + 1])), cw2);
                                 const f32x2 base = METRIC == 0 ? two2 : add2(pack2(ai[m], ai[m]), ca2);
                                 const float2 o = unpack2(fma2(x, pack2(m2w[m], m2w[m]), base));
-                                d[m * 8 + q * 2] = fmaxf(o.x, 0.f);
-                                d[m * 8 + q * 2 + 1] = fmaxf(o.y, 0.f);
+                                d[m * 8 + q * 2] = o.x;
+                                d[m * 8 + q * 2 + 1] = o.y;
                             }
                         }
                         const bool edge = cb == rb || (cb + 1) * kBlk > g.n;
@@ -416,29 +460,29 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                                 d[u] = (j > i && j < g.n) ? d[u] : kInf;
                             }
                         }
-                        // ---- block minima of both sides (none where the block lies beyond the spatial radius)
-                        if (!far) {
-                            float rm[4], cm[8];
+                        // ---- block minima (none where the block lies beyond the spatial radius); clamping as in the row warps
+                        float cm[8];
 #pragma unroll
-                            for (int m = 0; m < 4; ++m) {
-                                const float* x = d + m * 8;
-                                rm[m] = fminf(fminf(fminf(x[0], x[1]), fminf(x[2], x[3])), fminf(fminf(x[4], x[5]), fminf(x[6], x[7])));
-                            }
+                        for (int q = 0; q < 8; ++q) cm[q] = min3(fminf(d[q], d[8 + q]), d[16 + q], d[24 + q]);
+                        cmin = reduce_columns<true>(cm, lane);
+                        if (__any_sync(0xffffffffu, cmin < 0.f)) {
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) cm[q] = fminf(fminf(d[q], d[8 + q]), fminf(d[16 + q], d[24 + q]));
-                            rblk[c] = reduce_rows_min(rm, lane);
-                            cmin = reduce_columns<true>(cm, lane);
+                            for (int u = 0; u < 32; ++u) d[u] = fmaxf(d[u], 0.f);
+                            cmin = fmaxf(cmin, 0.f);
                         }
+                        if (far) cmin = kInf;
                         // ---- Eq. 2, column side: the sum of 32 rows as a tree over the bits of the row, highest first
 #pragma unroll
                         for (int u = 0; u < 32; u += 2) {
                             const float2 x = unpack2(mul2(pack2(d[u], d[u + 1]), c22));
-                            if (edge) {
-                                d[u] = d[u] == kInf ? 0.f : ex2_approx(x.x);
-                                d[u + 1] = d[u + 1] == kInf ? 0.f : ex2_approx(x.y);
-                            } else {
-                                d[u] = ex2_approx(x.x);
-                                d[u + 1] = ex2_approx(x.y);
+                            d[u] = ex2_approx(x.x);
+                            d[u + 1] = ex2_approx(x.y);
+                        }
+                        if (edge) {
+#pragma unroll
+                            for (int u = 0; u < 32; ++u) {
+                                const int i = i0 + lrow + 8 * (u >> 3), j = cb * kBlk + 8 * ((u >> 1) & 3) + lcol + (u & 1);
+                                d[u] = (j > i && j < g.n) ? d[u] : 0.f;
                             }
                         }
                         float cs[8];
@@ -456,11 +500,6 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                     sm.colsum[parity][quarter][at] = csum;
                     sm.colmin[parity][quarter][at] = cmin;
                 }
-                // ---- row minima of row lrow + 8 (T % 4); those of the block on the diagonal are joined with the column side below
-                const int row = quarter * kBlk + lrow + 8 * (lane & 3), i = R * BM + row;
-                const float4 mins = make_float4(rblk[0], rblk[1], rblk[2], rblk[3]);
-                if (R == C) *reinterpret_cast<float4*>(sm.rowmin[parity][row]) = mins;
-                else if (i < g.n) *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + i) * nb + 4 * C) = mins;
             }
             // this warp has read all it needs from the accumulator
             if (ok) {
@@ -520,11 +559,12 @@ int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cu
     k.expire_roles = gram_expire_roles();
     const long long total = (long long)args.B * args.t.tiles_per_b;
     if (total <= 0) return VITCOP_OK;
-    if (2 * total > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
+    if (total >= 1 << 22) return VITCOP_ERR_UNSUPPORTED;   // (group sizes keep it far below; decode_item's estimates hold to there)
     const long long pairs = gram_num_sms() / 2 > 0 ? gram_num_sms() / 2 : 1;
     const long long last = total % pairs, cut = 2 * last <= pairs ? last : 0;
     k.n_full = (int)(total - cut);
     k.n_items = (int)(total + cut);
+    k.inv_tiles = 1.f / (float)args.t.tiles_per_b;
     CUtensorMap ma, mb;
     if (!make_rowmajor_bf16_map(&ma, feat, args.B, args.n, args.D, BM) ||
         !make_rowmajor_bf16_map(&mb, feat, args.B, args.n, args.D, kBoxRows))

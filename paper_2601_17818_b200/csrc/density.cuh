@@ -8,7 +8,7 @@ namespace vitcop {
 // The symmetric half of a sample's Gram matrix is cut into tiles of 256 x 256, numbered column-tile major: column tile tj
 // holds the row tiles 0 .. tj and starts at tj (tj + 1) / 2.  The sweep keeps every Gram value it computes, in blocks of
 // 32 x 32 pairs: block (rb, cb), rb <= cb, of a sample sits at gram_block_offset floats, its element (r, c) at
-// gram_elem_offset inside it (the order in which the sweep's threads hold it in registers).
+// gram_elem_offset inside it.
 //
 // Beside the values it leaves a summary of every block: for each of the block's 64 tokens the smallest squared distance to a
 // token of the other side (blk_min).  Eq. 3 asks for the nearest DENSER token, and densities are known only when the sweep is
@@ -41,12 +41,9 @@ __host__ __device__ inline size_t gram_block_offset(int rb, int cb) {
     return (size_t)(tj * (tj + 1) / 2 + tp) * kSweepTileFloats +
            (size_t)((rb % kSweepBlks) * kSweepBlks + cb % kSweepBlks) * (kBlk * kBlk);
 }
-// Element (r, c) of a block: thread T of the warp that read the block from tensor memory (16 lanes x 256 bits at a time)
-// holds rows T / 4 + 8 m and columns 2 (T % 4) + 8 k, + 1; it stores four values (two rows of a 16-row half, two columns)
-// per instruction.
-__host__ __device__ inline int gram_elem_offset(int r, int c) {
-    return (((r >> 4) * 4 + (c >> 3)) * 32 + (r & 7) * 4 + ((c >> 1) & 3)) * 4 + ((r >> 3) & 1) * 2 + (c & 1);
-}
+// Groups of four columns, inside a group row by row: the 32 threads of a warp, one row each, store 512 contiguous bytes per
+// instruction.
+__host__ __device__ inline int gram_elem_offset(int r, int c) { return ((c >> 2) * kBlk + r) * 4 + (c & 3); }
 
 // Samples whose Gram values are kept at one time: the sweep and the search run group by group, so that the workspace
 // stays bounded whatever the batch.
@@ -71,6 +68,8 @@ struct SweepArgs {
     float* blk_min;             // [B, n_pad, n_blk]: entry (t, k) = smallest d^2 between token t and the other tokens of
                                 // block k (32 k ..), +inf where the blocks lie beyond the spatial radius
     uint32_t* blk_rho;          // [B, n_blk] bits of the largest density in a block of 32 tokens
+    int32_t* left;              // tokens (b n + i) that one warp's share of the search did not settle, and their number
+    int32_t* n_left;
     unsigned long long* best;   // [B, n] packed (d^2 bits << 32 | index) of the nearest denser token, ~0 = none
     int* status;                // device status word
     SweepTiling t;

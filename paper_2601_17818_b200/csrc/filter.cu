@@ -9,7 +9,7 @@
 //                             workspace and leaves the smallest distance of every token to every block of 32 tokens
 //   3. rho_reduce_kernel      fixed-order sum of the partials -> rho (bit-reproducible)
 //   4. nearest_denser_kernel  (nearest.cu) searches the few blocks that can hold it for each token's nearest denser
-//                             token inside the spatial radius (Eq. 3): packed (d^2, j)
+//      nearest_left_kernel    token inside the spatial radius (Eq. 3): packed (d^2, j)
 //   (2-4 run sample group by sample group where the Gram values of the whole batch would take more than 1.5 GB)
 //   5. vic_finalize_kernel    gamma = rho * delta, radix-select of the centres, pointer jumping over the
 //                             parent forest, orphan fallback, labels (Algorithm 2, steps 3-4)
@@ -26,75 +26,65 @@ namespace {
 // ------------------------------------------------------------------------------------------------
 // rho[b,i] = sum of the partials of the density sweep in a fixed order (reproducible bits): first the later tokens, 256 at a
 // time (a tile's columns: the sum of its two 128-token blocks), then the earlier ones, one 128-token block after the other, to
-// the end of the token's tile (blocks that hold none of them count as zero).  LANES neighbouring lanes share a token: each adds
-// its part of that list (sixteen independent loads at a time), and the sums are added in lane order.  A long sample has a list
-// of up to 190 entries, which one thread alone would fetch in a dozen dependent rounds; for a few dozen entries one
-// thread per token is the faster shape.  blk_rho[b,k]: bits of the largest density among the tokens of block k (densities are
-// not negative, their bit patterns order like the values).
-constexpr int kRhoLanesLong = 4;
-constexpr int kRhoLongEntries = 64;                        // samples with longer lists than this take kRhoLanesLong lanes
+// the end of the token's tile (blocks that hold none of them count as zero).  Up to 64 entries are added one by one; longer
+// lists (up to 192 on the longest samples) in four equal parts, whose sums are then added.  One CTA per 32 tokens: its warps
+// fetch the entries, all of them in one trip to memory, and the sums are taken from shared memory.  (One thread per token
+// walking its list paid a trip for every sixteen entries.)
+// blk_rho[b,k]: bits of the largest density among the tokens of block k (densities are not negative, their bit patterns order
+// like the values).
 constexpr int kRhoThreads = 256;
-template <int LANES>
+constexpr int kRhoOneByOne = 64;
+constexpr int kRhoEntries = 3 * VITCOP_MAX_VISUAL_TOKENS / kSweepTile;       // longest list
 __global__ void __launch_bounds__(kRhoThreads)
 rho_reduce_kernel(const float* __restrict__ part, int n, SweepTiling t, float* __restrict__ rho,
-                  float* __restrict__ rho_user, uint32_t* __restrict__ blk_rho) {
-    constexpr int kBlocks = kRhoThreads / LANES / kBlk;    // blocks of 32 tokens per CTA
-    __shared__ uint32_t top[kBlocks];
+                  float* __restrict__ rho_user, uint32_t* __restrict__ blk_rho, int32_t* __restrict__ n_left) {
+    constexpr int kWarps = kRhoThreads / 32;
+    __shared__ float entry[kRhoEntries][kBlk];
+    __shared__ float parts[4][kBlk];
     grid_dependency_launch_dependents();
     grid_dependency_wait();
-    if (threadIdx.x < kBlocks) top[threadIdx.x] = 0u;
-    __syncthreads();
-    const int q = threadIdx.x % LANES;
-    const int local = threadIdx.x / LANES;
-    const int i = blockIdx.x * (kRhoThreads / LANES) + local;
-    const int b = blockIdx.y;
-    const bool valid = i < n;                              // (all lanes stay for the shuffles)
-    float s = 0.f;
-    if (valid) {
-        const int own = i / kGramBM, tile = own / 2;
-        const int rows = t.T - tile;                       // entries on the row side, then min(TI, 2 (tile + 1)) more
-        const int entries = rows + min(t.TI, 2 * (tile + 1));
-        const int per = (entries + LANES - 1) / LANES;
-        const int c0 = q * per, c1 = min(entries, c0 + per);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int blk = blockIdx.x, b = blockIdx.y, i = blk * kBlk + lane;
+    if (blk == 0 && b == 0 && threadIdx.x == 0) *n_left = 0;         // for the search behind this kernel
+    const int own = blk * kBlk / kGramBM, tile = own / 2;
+    const int rows = t.T - tile;                           // entries on the row side, then min(TI, 2 (tile + 1)) more
+    const int entries = rows + min(t.TI, 2 * (tile + 1));
+    if (i < n) {
         const float* p = part + (size_t)b * t.slots() * t.n_pad + i;
         auto slot = [&](int k) { return p[(size_t)k * t.n_pad]; };
-        for (int c = c0; c < c1; c += 8) {
-            float v[8], v2[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int e = c + u;
-                v[u] = v2[u] = 0.f;
-                if (e < c1) {
-                    if (e < rows) {
-                        const int k = 2 * (tile + e);
-                        if (k >= own) v[u] = slot(k);
-                        if (k + 1 >= own && k + 1 < t.TI) v2[u] = slot(k + 1);
-                    } else {
-                        const int k = e - rows;
-                        if (k <= own) v[u] = slot(k == own ? t.TI : k);
-                    }
-                }
+#pragma unroll 6
+        for (int e = warp; e < entries; e += kWarps) {
+            float v = 0.f, v2 = 0.f;
+            if (e < rows) {
+                const int k = 2 * (tile + e);
+                if (k >= own) v = slot(k);
+                if (k + 1 >= own && k + 1 < t.TI) v2 = slot(k + 1);
+            } else {
+                const int k = e - rows;
+                if (k <= own) v = slot(k == own ? t.TI : k);
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (c + u < c1) s += v[u] + v2[u];
+            entry[e][lane] = v + v2;
         }
     }
-    float others[LANES];
-#pragma unroll
-    for (int u = 1; u < LANES; ++u) others[u] = __shfl_down_sync(0xffffffffu, s, u);
-#pragma unroll
-    for (int u = 1; u < LANES; ++u) s += others[u];
-    const bool mine = valid && q == 0;
-    if (mine) {
+    __syncthreads();
+    const int nparts = t.T + t.TI > kRhoOneByOne ? 4 : 1;
+    if (warp < nparts) {
+        const int per = (entries + nparts - 1) / nparts, e1 = min(entries, (warp + 1) * per);
+        float s = 0.f;
+#pragma unroll 8
+        for (int e = warp * per; e < e1; ++e) s += entry[e][lane];
+        parts[warp][lane] = s;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    float s = parts[0][lane];
+    for (int q = 1; q < nparts; ++q) s += parts[q][lane];
+    if (i < n) {
         rho[(size_t)b * n + i] = s;
         if (rho_user) rho_user[(size_t)b * n + i] = s;
     }
-    const uint32_t m = __reduce_max_sync(0xffffffffu, mine ? __float_as_uint(s) : 0u);
-    if ((threadIdx.x & 31) == 0) atomicMax(&top[local / kBlk], m);
-    __syncthreads();
-    const int k = blockIdx.x * kBlocks + threadIdx.x;
-    if (threadIdx.x < kBlocks && k < t.n_blk()) blk_rho[(size_t)b * t.n_blk() + k] = top[threadIdx.x];
+    const uint32_t m = __reduce_max_sync(0xffffffffu, i < n ? __float_as_uint(s) : 0u);
+    if (lane == 0) blk_rho[(size_t)b * t.n_blk() + blk] = m;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -345,11 +335,11 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
 // ------------------------------------------------------------------------------------------------
 // Workspace of the filter: status block | row-block flags [B, ceil(n / 128)] | w | a | rho | best |
 // rho partials [B, slots, n_pad] (sized for either sweep) | bounding boxes of the row blocks' positions | and, for
-// problems too large for the one-kernel sweep, of one group of samples: block densities, block minima, Gram values of
+// problems too large for the one-kernel sweep, of one group of samples: count and list of the search's leftovers, block densities, block minima, Gram values of
 // the density sweep (4 bytes per pair of the symmetric half, tile padding included).  The status block and the
 // flags are zeroed at the start of every call.  Words of the status block: 0 status, 2 grid barrier.
 struct FilterWs {
-    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_blk_rho, off_blk_min, off_gram, total;
+    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_left, off_blk_rho, off_blk_min, off_gram, total;
     FilterWs(int B, int n) {
         size_t o = kStatusBytes;
         const size_t bn = (size_t)B * n;
@@ -361,11 +351,12 @@ struct FilterWs {
         const GramTiling t = make_gram_tiling(n, 128);           // (two slots per block: never fewer than the density sweep's)
         off_part = o; o += align_up((size_t)B * t.slots() * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
-        off_blk_rho = off_blk_min = off_gram = o;
+        off_left = off_blk_rho = off_blk_min = off_gram = o;
         if (B > 0 && n > 0 && !gram_fits_resident(B, n)) {
             const SweepTiling s = make_sweep_tiling(n);
             const size_t group = (size_t)sweep_group_samples(B, n);
-            o += align_up(group * s.n_blk() * 4, 256);
+            o += align_up((group * n + 1) * 4, 256);
+            off_blk_rho = o; o += align_up(group * s.n_blk() * 4, 256);
             off_blk_min = o; o += align_up(group * s.n_blk() * s.n_pad * 4, 256);
             off_gram = o;    o += align_up(group * s.tiles_per_b * kSweepTileFloats * 4, 256);
         }
@@ -456,6 +447,8 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             s.pos = pos ? pos + 2 * at : nullptr;
             s.bbox = g.bbox ? g.bbox + (size_t)b0 * tiling.TI : nullptr;
             s.part = part + (size_t)b0 * tiling.slots() * tiling.n_pad;
+            s.n_left = reinterpret_cast<int32_t*>(ws + l.off_left);
+            s.left = s.n_left + 1;
             s.blk_rho = reinterpret_cast<uint32_t*>(ws + l.off_blk_rho);
             s.blk_min = reinterpret_cast<float*>(ws + l.off_blk_min);
             s.gram = reinterpret_cast<float*>(ws + l.off_gram);
@@ -466,12 +459,10 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             {
                 cudaLaunchConfig_t cfg;
                 cudaLaunchAttribute attr[1];
-                const int lanes = tiling.T + tiling.TI > kRhoLongEntries ? kRhoLanesLong : 1;
-                pdl_config(cfg, attr, dim3((n * lanes + kRhoThreads - 1) / kRhoThreads, s.B), dim3(kRhoThreads), 0, stream, true);
+                pdl_config(cfg, attr, dim3((n + kBlk - 1) / kBlk, s.B), dim3(kRhoThreads), 0, stream, true);
                 KernelTimeScope timed("rho_reduce_kernel", stream);
-                rc = record_cuda(cudaLaunchKernelEx(&cfg, lanes == 1 ? rho_reduce_kernel<1> : rho_reduce_kernel<kRhoLanesLong>,
-                                                    (const float*)s.part, n, tiling, rho + at,
-                                                    rho_user ? rho_user + at : nullptr, s.blk_rho));
+                rc = record_cuda(cudaLaunchKernelEx(&cfg, rho_reduce_kernel, (const float*)s.part, n, tiling, rho + at,
+                                                    rho_user ? rho_user + at : nullptr, s.blk_rho, s.n_left));
                 if (rc != VITCOP_OK) return rc;
             }
             rc = launch_nearest_denser(s, p.metric, stream, true);
