@@ -13,7 +13,9 @@
 //   column warps   the column tokens' block minima and sums.  They read the accumulator in the 16-lanes x 256-bit shape: a
 //                  thread holds 4 rows x 8 columns of a block, so that columns reduce partly inside the thread and only 8 values
 //                  go through shuffles.  (With one row per thread every column costs a butterfly or a redux over 32 lanes.)
-// Distances and exponentials are computed by both, which is cheaper than passing them on.
+// Distances and exponentials are computed by both, which is cheaper than passing them on.  Two more warps fetch the factors of the
+// next tile's tokens and join the column warps' parts of the previous one, so that neither the trip to the L2 nor the joining
+// stands between two tiles.
 //
 // Measured with sixteen warps of one role: 8 x 2880 x 1024 70 us, 60 us with an empty epilogue; 2 x 16384 x 1280 517 us, 484 us
 // without the stores of the Gram values, 433 us with an empty epilogue (0.69 Tflop at the rate cuBLAS reaches in a burst).  The
@@ -32,22 +34,25 @@ constexpr int BM = kGramBM, BN = kSweepTile;
 constexpr int kBoxRows = 64;                      // column tokens per load: a CTA stages one or two boxes
 constexpr int kABytes = BM * BK * 2, kBBytes = BN / 2 * BK * 2, kStageBytes = kABytes + kBBytes;
 constexpr int kHalfBlks = BM / kBlk;              // blocks of a warp: 128 columns
-constexpr int kEpiWarps = 16, kEpiThreads = kEpiWarps * 32, kThreads = 64 + kEpiThreads;
+constexpr int kEpiWarps = 16, kEpiThreads = kEpiWarps * 32, kAuxThreads = 64;
+constexpr int kThreads = 64 + kEpiThreads + kAuxThreads;
+constexpr int kTileThreads = kEpiThreads + kAuxThreads;   // meet once per tile
 constexpr float kInf = __builtin_huge_valf();
 constexpr int kRoleLoad = 1, kRoleMma = 2, kRoleEpi = 4;
 
-// Epilogue scratch: column factors per warp; per parity of the tile, sums and minima of the columns per row quarter, and the
-// row minima of the block on the diagonal.
+// Epilogue scratch, per parity of the tile: the factors of its tokens, which of its two 128-column halves lie beyond the spatial
+// radius, sums and minima of the columns per row quarter, and the row minima of the block on the diagonal.
 template <int METRIC>
 struct EpiSmem {
-    float w[kEpiWarps][BM], a[METRIC == 1 ? kEpiWarps : 1][BM];
+    float colw[2][BN], rowm2w[2][BM];             // w_j; -2 w_i
+    float cola[2][METRIC == 1 ? BN : 4], rowa[2][METRIC == 1 ? BM : 4];
     float colsum[2][4][BN], colmin[2][4][BN];
     float rowmin[2][BM][4];
+    int far[2][4];
 };
+constexpr int kStages = 6;
 template <int METRIC>
-__host__ __device__ constexpr int stages() { return METRIC == 1 ? 5 : 6; }       // (what shared memory holds)
-template <int METRIC>
-__host__ __device__ constexpr int smem_bytes() { return 1024 + stages<METRIC>() * kStageBytes + (int)sizeof(EpiSmem<METRIC>) + 256; }
+__host__ __device__ constexpr int smem_bytes() { return 1024 + kStages * kStageBytes + (int)sizeof(EpiSmem<METRIC>) + 256; }
 static_assert(smem_bytes<0>() <= 227 * 1024 && smem_bytes<1>() <= 227 * 1024, "shared memory of an SM");
 
 struct KernelArgs {
@@ -169,7 +174,6 @@ template <int METRIC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      const __grid_constant__ KernelArgs k) {
-    constexpr int kStages = stages<METRIC>();
     const SweepArgs& g = k.g;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -293,60 +297,110 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             }
         }
     } else {
-        // ------------------------------------------------------------------ epilogue (warps 2 .. 17)
-        const int quarter = warp & 3, ew = warp - 2, e = threadIdx.x - 64;
-        const int h = (ew >> 2) & 1;                               // which 128 columns
-        const bool row_role = ew >= kEpiWarps / 2;
-        const int lrow = lane >> 2, lcol = 2 * (lane & 3);         // column warps: rows lrow + 8 m, columns lcol + 8 k, + 1
+        // ------------------------------------------------------------------ epilogue (warps 2 .. 17), auxiliary warps
         const int TI = g.t.TI, nb = g.t.n_blk();
+        const int quarter = warp & 3, ew = warp - 2;
+        const int h = (ew >> 2) & 1;                               // which 128 columns
+        const bool row_role = ew >= kEpiWarps / 2, aux = ew >= kEpiWarps;
+        const int lrow = lane >> 2, lcol = 2 * (lane & 3);         // column warps: rows lrow + 8 m, columns lcol + 8 k, + 1
         const unsigned long long lim = k.limit_of(kRoleEpi);
         const f32x2 two2 = pack2(2.f, 2.f), c22 = pack2(g.c2, g.c2);
         uint32_t acc = 0, acc_phase = 0, parity = 0;
         bool ok = true;
 
-        grid_dependency_wait();                            // w, a and the bounding boxes come from the preceding kernel
-        for (int t = cluster; t < k.n_items; t += n_clusters, parity ^= 1u) {
+        // auxiliary warps: the factors of item t's tokens and whether its halves lie beyond the spatial radius
+        auto stage_factors = [&](int t, uint32_t par) {
             const Item it = decode_item(k, t);
             const size_t bo = (size_t)it.b * g.n;
+            const int R = 2 * it.tp + (int)rank, C0 = 2 * it.tj + it.half, l = threadIdx.x - 64 - kEpiThreads;
+            const int j0 = C0 * BM + l, i0 = R * BM + l;
+            float wj[BN / kAuxThreads], aj[BN / kAuxThreads], wi[BM / kAuxThreads], ai[BM / kAuxThreads];
+#pragma unroll
+            for (int u = 0; u < BN / kAuxThreads; ++u) {
+                const int j = j0 + u * kAuxThreads;
+                wj[u] = j < g.n ? g.w[bo + j] : 0.f;
+                aj[u] = (METRIC == 1 && j < g.n) ? g.a[bo + j] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < BM / kAuxThreads; ++u) {
+                const int i = i0 + u * kAuxThreads;
+                wi[u] = i < g.n ? -2.f * g.w[bo + i] : 0.f;
+                ai[u] = (METRIC == 1 && i < g.n) ? g.a[bo + i] : 0.f;
+            }
+            if (l < 2) {
+                const int C = C0 + l;
+                const float4* box = g.bbox + (size_t)it.b * TI;
+                sm.far[par][l] = g.bbox && R < TI && C < TI && blocks_outside_radius(box[R], box[C], g.tau2);
+            }
+#pragma unroll
+            for (int u = 0; u < BN / kAuxThreads; ++u) {
+                sm.colw[par][l + u * kAuxThreads] = wj[u];
+                if (METRIC == 1) sm.cola[par][l + u * kAuxThreads] = aj[u];
+            }
+#pragma unroll
+            for (int u = 0; u < BM / kAuxThreads; ++u) {
+                sm.rowm2w[par][l + u * kAuxThreads] = wi[u];
+                if (METRIC == 1) sm.rowa[par][l + u * kAuxThreads] = ai[u];
+            }
+        };
+        // auxiliary warps: column side of item t, one column at a time: the sums of the four row quarters in order, the minima as
+        // they are
+        auto join_columns = [&](int t, uint32_t par) {
+            const Item it = decode_item(k, t);
+            const int R = 2 * it.tp + (int)rank, C0 = 2 * it.tj + it.half;
+            const float(*cs)[BN] = sm.colsum[par];
+            const float(*cm)[BN] = sm.colmin[par];
+#pragma unroll
+            for (int u = 0; u < BN / kAuxThreads; ++u) {
+                const int e = (int)threadIdx.x - 64 - kEpiThreads + u * kAuxThreads;
+                const int half = e / BM, cc = C0 + half, j = cc * BM + e % BM;
+                if (half < it.halves && R <= cc && j < g.n) {
+                    const int slot = R == cc ? TI : R;             // (slot R of the own block holds the row side)
+                    g.part[((size_t)it.b * g.t.slots() + slot) * g.t.n_pad + j] = ((cs[0][e] + cs[1][e]) + cs[2][e]) + cs[3][e];
+                    float4 m = make_float4(cm[0][e], cm[1][e], cm[2][e], cm[3][e]);
+                    if (R == cc) {                                 // both sides speak about the same blocks
+                        const float4 o = *reinterpret_cast<const float4*>(sm.rowmin[par][e % BM]);
+                        m = make_float4(fminf(m.x, o.x), fminf(m.y, o.y), fminf(m.z, o.z), fminf(m.w, o.w));
+                    }
+                    *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + j) * nb + 4 * R) = m;
+                }
+            }
+        };
+
+        grid_dependency_wait();                            // w, a and the bounding boxes come from the preceding kernel
+        if (aux && cluster < k.n_items) stage_factors(cluster, 0);
+        epi_bar_sync<kTileThreads>();
+        for (int t = cluster; t < k.n_items; t += n_clusters, parity ^= 1u) {
+            if (aux) {
+                // between two meetings: join the previous tile, fetch the next one's factors.  (What the epilogue warps write
+                // meanwhile has this tile's parity.)
+                if (t != cluster) join_columns(t - n_clusters, parity ^ 1u);
+                if (t + n_clusters < k.n_items) stage_factors(t + n_clusters, parity ^ 1u);
+                if (epi_bar_or<kTileThreads>(false)) { ok = false; break; }
+                if (t + n_clusters >= k.n_items) join_columns(t, parity);
+                continue;
+            }
+            const Item it = decode_item(k, t);
             const int R = 2 * it.tp + (int)rank;           // 128-token block of the CTA's rows ...
             const int C0 = 2 * it.tj + it.half;            // ... and of its first 128 columns
             const int C = C0 + h;                          // this warp's
             const bool work = h < it.halves && R <= C && C < TI;           // (R > C: below the diagonal)
             const int i0 = R * BM + quarter * kBlk;
             const int rb = R * 4 + quarter;                                // the warp's rows as a block of 32
-            const int first = i0 + (row_role ? lane : lrow);               // rows of the thread: first (, first + 8, ..)
-            float m2w[4], ai[4];
-            bool far = false;
-            if (work) {
-                // this warp's column factors, its rows' factors, and whether its pairs all lie beyond the spatial radius
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int j = C * BM + u * 32 + lane;
-                    sm.w[ew][u * 32 + lane] = j < g.n ? g.w[bo + j] : 0.f;
-                    if (METRIC == 1) sm.a[ew][u * 32 + lane] = j < g.n ? g.a[bo + j] : 0.f;
-                }
-                m2w[0] = first < g.n ? -2.f * g.w[bo + first] : 0.f;
-                ai[0] = (METRIC == 1 && first < g.n) ? g.a[bo + first] : 0.f;
-                if (!row_role) {
-#pragma unroll
-                    for (int m = 1; m < 4; ++m) {
-                        const int i = first + 8 * m;
-                        m2w[m] = i < g.n ? -2.f * g.w[bo + i] : 0.f;
-                        ai[m] = (METRIC == 1 && i < g.n) ? g.a[bo + i] : 0.f;
-                    }
-                }
-                if (g.bbox)
-                    far = blocks_outside_radius(g.bbox[(size_t)it.b * TI + R], g.bbox[(size_t)it.b * TI + C], g.tau2);
-                __syncwarp();
-            }
+            const bool far = sm.far[parity][h] != 0;       // this warp's pairs all lie beyond the spatial radius
+            const float* const colw = sm.colw[parity] + h * BM;
+            const float* const cola = sm.cola[parity] + (METRIC == 1 ? h * BM : 0);
+            const float* const rowm2w = sm.rowm2w[parity] + quarter * kBlk;
+            const float* const rowa = sm.rowa[parity] + (METRIC == 1 ? quarter * kBlk : 0);
             if (ok) ok = mbar_wait(bar_tfull + 8 * acc, acc_phase, abort_flag, lim);
             ok = __all_sync(0xffffffffu, ok);
             if (ok) tc_fence_after();
             const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16) + h * BM;
             if (ok && work && row_role) {
                 // ---- Eq. 2, row side: exp(-d^2 / d_c^2) of this thread's row, added column by column
-                const int i = first;
-                const f32x2 m2w2 = pack2(m2w[0], m2w[0]), ai2 = pack2(ai[0], ai[0]);
+                const int i = i0 + lane;
+                const f32x2 m2w2 = pack2(rowm2w[lane], rowm2w[lane]);
+                const f32x2 ai2 = METRIC == 1 ? pack2(rowa[lane], rowa[lane]) : 0ull;
                 float* const blocks = g.gram + (size_t)it.b * g.t.tiles_per_b * kSweepTileFloats;
                 float sum = 0.f;
                 float4 mins = make_float4(kInf, kInf, kInf, kInf); // of the row over each of the four blocks
@@ -364,9 +418,9 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                     }
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
-                        const float4 cw = *reinterpret_cast<const float4*>(&sm.w[ew][c * kBlk + 4 * q]);
+                        const float4 cw = *reinterpret_cast<const float4*>(colw + c * kBlk + 4 * q);
                         float4 ca = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (METRIC == 1) ca = *reinterpret_cast<const float4*>(&sm.a[ew][c * kBlk + 4 * q]);
+                        if (METRIC == 1) ca = *reinterpret_cast<const float4*>(cola + c * kBlk + 4 * q);
 #pragma unroll
                         for (int p = 0; p < 2; ++p) {              // two neighbouring columns at a time
                             const int u = 4 * q + 2 * p;
@@ -425,6 +479,12 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                 else if (i < g.n) *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + i) * nb + 4 * C) = mins;
             }
             if (ok && work && !row_role) {
+                f32x2 m2w2[4], ai2[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    m2w2[m] = pack2(rowm2w[lrow + 8 * m], rowm2w[lrow + 8 * m]);
+                    ai2[m] = METRIC == 1 ? pack2(rowa[lrow + 8 * m], rowa[lrow + 8 * m]) : 0ull;
+                }
 #pragma unroll 1
                 for (int c = 0; c < kHalfBlks; ++c) {
                     const int cb = C * 4 + c;
@@ -438,16 +498,16 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                         float d[32];                               // [m][k][r]: row lrow + 8 m, column 8 k + lcol + r
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const float2 cw = *reinterpret_cast<const float2*>(&sm.w[ew][c * kBlk + 8 * q + lcol]);
+                            const float2 cw = *reinterpret_cast<const float2*>(colw + c * kBlk + 8 * q + lcol);
                             float2 ca = make_float2(0.f, 0.f);
-                            if (METRIC == 1) ca = *reinterpret_cast<const float2*>(&sm.a[ew][c * kBlk + 8 * q + lcol]);
+                            if (METRIC == 1) ca = *reinterpret_cast<const float2*>(cola + c * kBlk + 8 * q + lcol);
                             const f32x2 cw2 = pack2(cw.x, cw.y), ca2 = pack2(ca.x, ca.y);
 #pragma unroll
                             for (int m = 0; m < 4; ++m) {
                                 const int at = (m >> 1) * 16 + q * 4 + (m & 1) * 2;
                                 const f32x2 x = mul2(pack2(__uint_as_float(r[at]), __uint_as_float(r[at + 1])), cw2);
-                                const f32x2 base = METRIC == 0 ? two2 : add2(pack2(ai[m], ai[m]), ca2);
-                                const float2 o = unpack2(fma2(x, pack2(m2w[m], m2w[m]), base));
+                                const f32x2 base = METRIC == 0 ? two2 : add2(ai2[m], ca2);
+                                const float2 o = unpack2(fma2(x, m2w2[m], base));
                                 d[m * 8 + q * 2] = o.x;
                                 d[m * 8 + q * 2 + 1] = o.y;
                             }
@@ -507,22 +567,7 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(cluster_map(bar_tempty + 8 * acc, 0));
             }
-            if (epi_bar_or<kEpiThreads>(!ok)) { ok = false; break; }
-            // ---- column side, one column per thread: the sums of the four row quarters in order, the minima as they are.  (The
-            //      arrays of the other parity are free for the next tile meanwhile.)
-            const int half = e / BM, cc = C0 + half, j = cc * BM + e % BM;
-            if (e < BN && half < it.halves && R <= cc && j < g.n) {
-                const float(*cs)[BN] = sm.colsum[parity];
-                const float(*cm)[BN] = sm.colmin[parity];
-                const int slot = R == cc ? TI : R;                 // (slot R of the own block holds the row side)
-                g.part[((size_t)it.b * g.t.slots() + slot) * g.t.n_pad + j] = ((cs[0][e] + cs[1][e]) + cs[2][e]) + cs[3][e];
-                float4 m = make_float4(cm[0][e], cm[1][e], cm[2][e], cm[3][e]);
-                if (R == cc) {                                     // both sides speak about the same blocks
-                    const float4 o = *reinterpret_cast<const float4*>(sm.rowmin[parity][e % BM]);
-                    m = make_float4(fminf(m.x, o.x), fminf(m.y, o.y), fminf(m.z, o.z), fminf(m.w, o.w));
-                }
-                *reinterpret_cast<float4*>(g.blk_min + ((size_t)it.b * g.t.n_pad + j) * nb + 4 * R) = m;
-            }
+            if (epi_bar_or<kTileThreads>(!ok)) { ok = false; break; }
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (!ok && lane == 0) raise_abort_pair(abort_addr, rank);

@@ -5,7 +5,7 @@
 // A block can hold a token's answer only if its minimum is not above the best denser token found so far.  One warp per token:
 // every lane keeps the two smallest minima among its blocks (block % 32 = lane) and the warp looks into the blocks in
 // ascending order, two at a time (lane = token of the block: the Gram value, the factors, the density and the spatial test).
-// For nine tokens in ten two rounds are enough: their nearest neighbours include a denser token (half of all tokens need one
+// For nine tokens in ten two or three rounds are enough: their nearest neighbours include a denser token (half of all tokens need one
 // block).  The few tokens that are the densest of their surroundings may have to look into dozens of blocks; these are listed
 // and left to a second kernel, in which several warps share out a token's blocks, passing over those without a denser
 // token (largest density of the block): a warp alone would hold up everything behind it.  What is skipped could not have
@@ -20,7 +20,7 @@ namespace vitcop {
 namespace {
 
 constexpr int kNdThreads = 256, kNdWarps = kNdThreads / 32;
-constexpr int kNdRounds = 2;                               // rounds of two blocks that a warp does for its own token
+constexpr int kNdRounds = 3;                               // rounds of two blocks that a warp does for its own token
 constexpr uint32_t kInfBits = 0x7f800000u;
 // A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, i.e. a
 // bound up to 2^-14 too low.
@@ -237,9 +237,8 @@ int launch_nearest_denser(const SweepArgs& args, int metric, cudaStream_t stream
         rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, args));
         if (rc != VITCOP_OK) return rc;
     }
-    // about sixteen blocks a warp
-    int slices = 4;
-    while (slices * 16 < args.t.n_blk()) slices *= 2;
+    int slices = 2;                                        // at most 32 blocks a warp: one per lane
+    while (slices * 32 < args.t.n_blk()) slices *= 2;
     const long long most = ((long long)args.B * args.n * slices + kNdWarps - 1) / kNdWarps, ctas = 6LL * gram_num_sms();
     cfg.gridDim = dim3((unsigned)(most < ctas ? most : ctas));
     auto rest = metric == 1 ? (spatial ? nearest_left_kernel<1, true> : nearest_left_kernel<1, false>)
