@@ -21,6 +21,7 @@ namespace {
 
 constexpr int kNdThreads = 256, kNdWarps = kNdThreads / 32;
 constexpr int kNdRounds = 3;                               // rounds of two blocks that a warp does for its own token
+constexpr int kNdAhead = 4;                                // blocks a warp of the second kernel looks into at a time
 constexpr uint32_t kInfBits = 0x7f800000u;
 // A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, i.e. a
 // bound up to 2^-14 too low.
@@ -198,15 +199,21 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
             if (top < __float_as_uint(t.rho)) lo = kInfBits;
             uint32_t todo = __ballot_sync(0xffffffffu, can(lo, k));
             while (todo) {
-                const int b0 = k0 + (__ffs(todo) - 1) * slices;
-                todo &= todo - 1;
-                const auto p0 = s.fetch(i, b0, lane);
-                const int b1 = todo ? k0 + (__ffs(todo) - 1) * slices : -1;
-                todo &= todo - 1;
-                auto p1 = p0;
-                if (b1 >= 0) p1 = s.fetch(i, b1, lane);
-                s.finish(t, p0, b0, lane, best);
-                if (b1 >= 0) s.finish(t, p1, b1, lane, best);
+                typename Sample<METRIC, SPATIAL>::Pair p[kNdAhead];
+                int blk[kNdAhead];
+                int cnt = 0;
+#pragma unroll
+                for (int u = 0; u < kNdAhead; ++u) {
+                    if (todo) {
+                        blk[u] = k0 + (__ffs(todo) - 1) * slices;
+                        todo &= todo - 1;
+                        p[u] = s.fetch(i, blk[u], lane);
+                        cnt = u + 1;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kNdAhead; ++u)
+                    if (u < cnt) s.finish(t, p[u], blk[u], lane, best);
                 todo &= __ballot_sync(0xffffffffu, can(lo, k));
             }
         }
