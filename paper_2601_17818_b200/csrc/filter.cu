@@ -36,7 +36,7 @@ constexpr int kRhoThreads = 256;
 constexpr int kRhoOneByOne = 64;
 constexpr int kRhoEntries = 3 * VITCOP_MAX_VISUAL_TOKENS / kSweepTile;       // longest list
 __global__ void __launch_bounds__(kRhoThreads)
-rho_reduce_kernel(const float* __restrict__ part, int n, SweepTiling t, float* __restrict__ rho,
+rho_reduce_kernel(const float* part, int n, SweepTiling t, float* __restrict__ rho,
                   float* __restrict__ rho_user, uint32_t* __restrict__ blk_rho, int32_t* __restrict__ n_left) {
     constexpr int kWarps = kRhoThreads / 32;
     __shared__ float entry[kRhoEntries][kBlk];
@@ -51,7 +51,7 @@ rho_reduce_kernel(const float* __restrict__ part, int n, SweepTiling t, float* _
     const int entries = rows + min(t.TI, 2 * (tile + 1));
     if (i < n) {
         const float* p = part + (size_t)b * t.slots() * t.n_pad + i;
-        auto slot = [&](int k) { return p[(size_t)k * t.n_pad]; };
+        auto slot = [&](int k) { return __ldcg(p + (size_t)k * t.n_pad); };
 #pragma unroll 6
         for (int e = warp; e < entries; e += kWarps) {
             float v = 0.f, v2 = 0.f;
@@ -90,32 +90,44 @@ rho_reduce_kernel(const float* __restrict__ part, int n, SweepTiling t, float* _
 // ------------------------------------------------------------------------------------------------
 // Centres, forest roots and labels: one CTA per sample.
 // ------------------------------------------------------------------------------------------------
+// The CTA runs alone on its SM, so what counts is the number of dependent steps, not throughput: every thread holds its tokens'
+// keys in registers, all global loads are in flight together, the cut among the keys is found with one or two histogram
+// passes of 11 bits that start at the highest bit in which two keys differ, and what is left in the cut's bin is ranked by
+// counting.  (8-bit passes over the whole 64-bit key with ordered scans for ties and for the list of centres: 9.2 us on 576
+// tokens, 14 on 2880, 38 on 16384; the list is needed for surplus orphans only and is built when there are any.)
 constexpr int kFinThreads = 1024;
-constexpr int kFinIters = VITCOP_MAX_VISUAL_TOKENS / kFinThreads;      // tokens per thread at the largest sample
+constexpr int kFinBits = 11, kFinBins = 1 << kFinBits;
+constexpr int kFinRankLanes = 4;
+constexpr int kFinRank = kFinThreads / kFinRankLanes;      // bins of up to this many keys are ranked by counting
 
-// Shared memory: keys[n] (uint64; later reused as next[n] int32), isc[n] (uint8), centres[nc] (int32).
+// Dynamic shared memory: nxt[n] (uint16), isc[n] (uint8), centre list[nc] (uint16; surplus orphans).  E: tokens per thread.
+template <int E>
 __global__ void __launch_bounds__(kFinThreads)
-vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_centers, const float* __restrict__ rho,
-                    const unsigned long long* __restrict__ best, const float* __restrict__ w,
-                    const float* __restrict__ a, int32_t* __restrict__ label, int32_t* __restrict__ n_clusters,
+vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_centers, const float* rho, const unsigned long long* best,
+                    const float* w, const float* a, int32_t* __restrict__ label, int32_t* __restrict__ n_clusters,
                     float* __restrict__ delta2_user, int32_t* __restrict__ parent_user) {
     extern __shared__ __align__(16) uint8_t fin_smem[];
-    unsigned long long* keys = reinterpret_cast<unsigned long long*>(fin_smem);
-    int32_t* nxt = reinterpret_cast<int32_t*>(fin_smem);              // aliases keys after the selection
-    uint8_t* isc = fin_smem + (size_t)n * 8;
-    int32_t* centres = reinterpret_cast<int32_t*>(fin_smem + (size_t)n * 8 + (((size_t)n + 15) & ~(size_t)15));
-    __shared__ uint32_t hist[256];
+    const int n_al = (n + 15) & ~15;
+    uint16_t* nxt = reinterpret_cast<uint16_t*>(fin_smem);
+    uint8_t* isc = fin_smem + (size_t)n_al * 2;
+    uint16_t* centres = reinterpret_cast<uint16_t*>(fin_smem + (size_t)n_al * 3);
+    __shared__ uint32_t hist[kFinBins];
+    __shared__ unsigned long long cand_key[kFinRank];
+    __shared__ uint16_t cand_idx[kFinRank];
     __shared__ uint32_t warp_sums[32];
-    __shared__ uint32_t cnt[kFinIters * 32];               // one count per (iteration, warp)
-    __shared__ uint32_t s_digit, s_krem, s_whole;
+    __shared__ uint32_t s_lo, s_hi, s_digit, s_krem, s_count, s_cands;
     __shared__ unsigned long long orph_best[kFinThreads];
     __shared__ int orph_list[kFinThreads];
-    __shared__ int orph_cnt;
+    __shared__ int orph_cnt, centre_cnt;
 
+    const int tid = threadIdx.x, lane = tid & 31;
+    hist[tid] = 0;
+    hist[tid + kFinThreads] = 0;
+    if (tid == 0) { s_lo = 0xFFFFFFFFu; s_hi = 0u; s_cands = 0u; centre_cnt = 0; }
+    static_assert(kFinBins == 2 * kFinThreads, "two bins per thread");
     grid_dependency_launch_dependents();
     grid_dependency_wait();
     const int b = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     rho += (size_t)b * n;
     best += (size_t)b * n;
     w += (size_t)b * n;
@@ -126,163 +138,175 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
     if (parent_user) parent_user += (size_t)b * n;
     const int nc = min(n_centers, n);
 
-    // rank key, ascending = better centre candidate: ~( orphan ? (0xFFFFFFFF, rho) : (gamma, rho) )
-    for (int i = tid; i < n; i += kFinThreads) {
-        const unsigned long long p = best[i];
-        const bool orphan = p == ~0ull;
-        const float d2 = orphan ? __int_as_float(0x7f800000) : __uint_as_float((uint32_t)(p >> 32));
-        const int par = orphan ? -1 : (int)(uint32_t)(p & 0xFFFFFFFFull);
-        if (delta2_user) delta2_user[i] = d2;
-        if (parent_user) parent_user[i] = par;
-        const float r = rho[i];
-        const uint32_t hi = orphan ? 0xFFFFFFFFu : __float_as_uint(r * sqrtf(d2));
-        keys[i] = ~(((unsigned long long)hi << 32) | (unsigned long long)__float_as_uint(r));
+    // (Loads of what the preceding kernels wrote: pointers without __restrict__, so that nothing lets the compiler move one in
+    // front of the wait.)
+    // rank key, ascending = better centre candidate: ( ~( orphan ? 0xFFFFFFFF : gamma ), ~rho, index )
+    uint32_t hi[E];
+    {
+        unsigned long long p[E];
+        float r[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = e * kFinThreads + tid;
+            p[e] = i < n ? __ldcg(best + i) : 0ull;
+            r[e] = i < n ? __ldcg(rho + i) : 0.f;
+        }
+        uint32_t lo_k = 0xFFFFFFFFu, hi_k = 0u;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = e * kFinThreads + tid;
+            if (i < n) {
+                const bool orphan = p[e] == ~0ull;
+                const float d2 = orphan ? __int_as_float(0x7f800000) : __uint_as_float((uint32_t)(p[e] >> 32));
+                const int par = orphan ? -1 : (int)(uint32_t)(p[e] & 0xFFFFFFFFull);
+                if (delta2_user) delta2_user[i] = d2;
+                if (parent_user) parent_user[i] = par;
+                nxt[i] = (uint16_t)((par < 0 || par >= n) ? i : par);
+                hi[e] = ~(orphan ? 0xFFFFFFFFu : __float_as_uint(r[e] * sqrtf(d2)));
+                lo_k = min(lo_k, hi[e]);
+                hi_k = max(hi_k, hi[e]);
+            }
+        }
+        lo_k = __reduce_min_sync(0xffffffffu, lo_k);
+        hi_k = __reduce_max_sync(0xffffffffu, hi_k);
+        __syncthreads();                                   // (s_lo, s_hi and the histogram are set)
+        if (lane == 0 && lo_k <= hi_k) {
+            atomicMin(&s_lo, lo_k);
+            atomicMax(&s_hi, hi_k);
+        }
     }
     __syncthreads();
 
-    // ---- radix select of the nc smallest keys (8 passes of 8 bits), ties -> lower index
-    unsigned long long T = ~0ull;
-    uint32_t krem = 0;
-    if (nc > 0 && nc < n) {
-        unsigned long long prefix = 0;
-        krem = (uint32_t)nc;
-        for (int pass = 0; pass < 8; ++pass) {
-            const int shift = 56 - 8 * pass;
-            const unsigned long long hi_mask = pass == 0 ? 0ull : (~0ull << (shift + 8));
-            if (tid < 256) hist[tid] = 0;
-            __syncthreads();
-            for (int base = 0; base < n; base += kFinThreads) {
-                const int i = base + tid;
-                int dig = -1;
-                if (i < n) {
-                    const unsigned long long key = keys[i];
-                    if ((key & hi_mask) == prefix) dig = (int)((key >> shift) & 255ull);
-                }
-                const uint32_t peers = __match_any_sync(0xffffffffu, dig);
-                if (dig >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[dig], (uint32_t)__popc(peers));
-            }
-            __syncthreads();
-            const uint32_t c = tid < 256 ? hist[tid] : 0u;
-            uint32_t v = c;
+    // ---- the nc smallest keys.  `in`: tokens of this thread (bit e) that still are on the cut; `sel`: chosen ones.
+    uint32_t in = 0, sel = 0, ranked = 0;                  // ranked: how many of the listed candidates are wanted
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, v, off);
-                if (lane >= off) v += t;
-            }
-            if (lane == 31) warp_sums[warp] = v;
+    for (int e = 0; e < E; ++e)
+        if (e * kFinThreads + tid < n) in |= 1u << e;
+    if (nc >= n) {
+        sel = in;
+    } else if (nc > 0) {
+        uint32_t krem = (uint32_t)nc;
+        int word = 0, top = 32 - __clz(s_lo ^ s_hi);       // word of the key, bits of it not yet looked at
+        for (;;) {
+            while (top == 0) top = ++word == 2 ? 14 : 32;  // (indices differ: the last word settles everything)
+            const int shift = top > kFinBits ? top - kFinBits : 0;
+            auto digit = [&](int e) {
+                const int i = e * kFinThreads + tid;
+                const uint32_t k = word == 0 ? hi[e] : word == 1 ? ~__float_as_uint(__ldcg(rho + i)) : (uint32_t)i;
+                return (k >> shift) & ((1u << (top - shift)) - 1u);
+            };
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (in >> e & 1u) atomicAdd(&hist[digit(e)], 1u);
             __syncthreads();
-            if (tid < 256) {
-                uint32_t basew = 0;
-                for (int q = 0; q < warp; ++q) basew += warp_sums[q];
-                const uint32_t incl = basew + v, excl = incl - c;
-                if (excl < krem && krem <= incl) {
-                    s_digit = (uint32_t)tid;
-                    s_krem = krem - excl;
-                    s_whole = (c == krem - excl) ? 1u : 0u;         // the whole bin is wanted
+            const uint32_t h0 = hist[2 * tid], h1 = hist[2 * tid + 1];
+            uint32_t total;
+            const uint32_t before = block_exclusive_sum(h0 + h1, warp_sums, total);
+            if (before < krem && krem <= before + h0 + h1) {
+                const bool second = krem > before + h0;
+                s_digit = 2 * tid + (second ? 1 : 0);
+                s_krem = krem - before - (second ? h0 : 0u);
+                s_count = second ? h1 : h0;
+            }
+            hist[2 * tid] = 0;                             // for the next pass
+            hist[2 * tid + 1] = 0;
+            __syncthreads();
+            const uint32_t cut = s_digit, count = s_count;
+            krem = s_krem;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (in >> e & 1u) {
+                    const uint32_t d = digit(e);
+                    if (d < cut) sel |= 1u << e;
+                    if (d != cut) in &= ~(1u << e);
                 }
             }
-            __syncthreads();
-            prefix |= (unsigned long long)s_digit << shift;
-            krem = s_krem;
-            const bool whole = s_whole != 0;
-            __syncthreads();
-            if (whole) {
-                // every key that shares the prefix found so far is selected: no need to resolve lower digits
-                prefix |= (1ull << shift) - 1ull;
-                krem = 0xFFFFFFFFu;
+            top = shift;
+            if (count == krem) {                           // the whole bin is wanted
+                sel |= in;
                 break;
             }
-        }
-        T = prefix;
-    }
-    // ---- centre flags + ascending centre list.  Token i = it * 1024 + tid; ranks in index order come from one count
-    //      per (iteration, warp), scanned once for the whole sample, plus the lane's position in its warp's ballot:
-    //      first among the keys equal to the cut (ties -> lower index), then among the centres.
-    {
-        uint32_t eq_mask = 0, f_mask = 0;                  // bit it: this thread's token of iteration it is ... / is a centre
-        const int iters = (n + kFinThreads - 1) / kFinThreads;          // <= kFinIters
-        const uint32_t lane_below = (1u << lane) - 1u;
-        const bool cut = nc > 0 && nc < n;
-        if (cut) {
-            for (int it = 0; it < iters; ++it) {
-                const int i = it * kFinThreads + tid;
-                const bool eq = i < n && keys[i] == T;
-                const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-                if (eq) eq_mask |= 1u << it;
-                if (lane == 0) cnt[it * 32 + warp] = __popc(bal);
+            if (count <= (uint32_t)kFinRank) {
+                // few left: listed, and ranked below
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    if (in >> e & 1u) {
+                        const int i = e * kFinThreads + tid;
+                        const uint32_t at = atomicAdd(&s_cands, 1u);
+                        cand_key[at] = ((unsigned long long)hi[e] << 32) | (unsigned long long)~__float_as_uint(__ldcg(rho + i));
+                        cand_idx[at] = (uint16_t)i;
+                    }
+                }
+                ranked = krem;
+                break;
             }
-            __syncthreads();
-            uint32_t total;
-            const uint32_t excl = block_exclusive_sum(tid < iters * 32 ? cnt[tid] : 0u, warp_sums, total);
-            if (tid < iters * 32) cnt[tid] = excl;
-            __syncthreads();
-        }
-        for (int it = 0; it < iters; ++it) {
-            const int i = it * kFinThreads + tid;
-            bool f;
-            if (nc <= 0) f = false;
-            else if (nc >= n) f = i < n;
-            else {
-                const bool eq = (eq_mask >> it & 1u) != 0;
-                const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-                const uint32_t eq_rank = cnt[it * 32 + warp] + __popc(bal & lane_below);
-                f = i < n && (keys[i] < T || (eq && eq_rank < krem));
-            }
-            if (f) f_mask |= 1u << it;
-            if (i < n) isc[i] = f ? 1 : 0;
-        }
-        __syncthreads();                                   // cnt is reused
-        for (int it = 0; it < iters; ++it) {
-            const uint32_t bal = __ballot_sync(0xffffffffu, (f_mask >> it & 1u) != 0);
-            if (lane == 0) cnt[it * 32 + warp] = __popc(bal);
-        }
-        __syncthreads();
-        uint32_t total;
-        const uint32_t excl = block_exclusive_sum(tid < iters * 32 ? cnt[tid] : 0u, warp_sums, total);
-        if (tid < iters * 32) cnt[tid] = excl;
-        __syncthreads();
-        for (int it = 0; it < iters; ++it) {
-            const bool f = (f_mask >> it & 1u) != 0;
-            const uint32_t bal = __ballot_sync(0xffffffffu, f);
-            const uint32_t r = cnt[it * 32 + warp] + __popc(bal & lane_below);
-            if (f && r < (uint32_t)nc) centres[r] = it * kFinThreads + tid;
+            __syncthreads();                               // (s_digit .. are rewritten)
         }
     }
-    __syncthreads();   // keys are dead from here on; nxt aliases them
-
-    // ---- forest roots by pointer jumping: a centre or an orphan is its own root
-    for (int i = tid; i < n; i += kFinThreads) {
-        const unsigned long long p = best[i];
-        const int par = (p == ~0ull) ? -1 : (int)(uint32_t)(p & 0xFFFFFFFFull);
-        nxt[i] = (isc[i] || par < 0 || par >= n) ? i : par;
+    // ---- centres are roots; an orphan is one already
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = e * kFinThreads + tid;
+        if (i < n) {
+            const bool f = (sel >> e & 1u) != 0;
+            isc[i] = f ? 1 : 0;
+            if (f) nxt[i] = (uint16_t)i;
+        }
     }
     __syncthreads();
+    if (ranked > 0) {                                      // (uniform) four threads per candidate count the better ones
+        const int c = tid / kFinRankLanes, cands = (int)s_cands;
+        uint32_t rank = 0;
+        unsigned long long mine = 0ull;
+        int idx = 0;
+        if (c < cands) {
+            mine = cand_key[c];
+            idx = cand_idx[c];
+            for (int o = tid % kFinRankLanes; o < cands; o += kFinRankLanes)
+                rank += (cand_key[o] < mine || (cand_key[o] == mine && cand_idx[o] < idx)) ? 1u : 0u;
+        }
+#pragma unroll
+        for (int off = 1; off < kFinRankLanes; off <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
+        if (c < cands && tid % kFinRankLanes == 0 && rank < ranked) {
+            isc[idx] = 1;
+            nxt[idx] = (uint16_t)idx;
+        }
+        __syncthreads();
+    }
+    // ---- forest roots by pointer jumping: any value read is an ancestor, roots are fixed points
     for (int round = 0; round < 16; ++round) {
         int changed = 0;
-        for (int i = tid; i < n; i += kFinThreads) {
-            const int p = nxt[i];
-            const int q = nxt[p];
-            if (q != p) {
-                nxt[i] = q;       // any value read here is an ancestor of i, roots are fixed points
-                changed = 1;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = e * kFinThreads + tid;
+            if (i < n) {
+                int p = nxt[i];
+                const int q = nxt[p];
+                if (q != p) {
+                    p = nxt[q];
+                    nxt[i] = nxt[p];
+                    changed = 1;
+                }
             }
         }
         if (!__syncthreads_or(changed)) break;
     }
-
-    // ---- labels; a root that is an orphan but not a centre joins the nearest centre (feature distance)
-    for (int i = tid; i < n; i += kFinThreads) {
-        const int root = nxt[i];
-        label[i] = isc[root] ? root : -1 - root;
+    // ---- a root that is an orphan but not a centre joins the nearest centre (feature distance)
+    int any_surplus = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = e * kFinThreads + tid;
+        if (i < n && !isc[i] && nxt[i] == i) any_surplus = 1;
     }
-    __syncthreads();
-    int any_surplus = 0;                                   // a root that is neither a centre nor below one
-    for (int i = tid; i < n; i += kFinThreads) any_surplus |= (!isc[i] && nxt[i] == i) ? 1 : 0;
-    any_surplus = __syncthreads_or(any_surplus);
-    if (nc > 0 && any_surplus) {
-        // Surplus orphans (roots that are not centres) are rare but each needs its distance to every centre: they
-        // are listed, kFinThreads tokens at a time, and the (orphan, centre) pairs are spread over all warps; the
-        // nearest centre wins through a packed minimum (distance bits, then the lower centre rank).
+    if (nc > 0 && __syncthreads_or(any_surplus)) {
+        // Surplus orphans are rare but each needs its distance to every centre: they are listed, kFinThreads tokens at a time,
+        // and the (orphan, centre) pairs are spread over all warps; the nearest centre wins through a packed minimum
+        // (distance bits, then the lower centre).
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = e * kFinThreads + tid;
+            if (i < n && isc[i]) centres[atomicAdd(&centre_cnt, 1)] = (uint16_t)i;
+        }
         for (int base = 0; base < n; base += kFinThreads) {
             __syncthreads();                                        // the previous round's list has been consumed
             if (tid == 0) orph_cnt = 0;
@@ -295,7 +319,7 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
             }
             __syncthreads();
             const int pairs = orph_cnt * nc;
-            for (int pr = warp; pr < pairs; pr += kFinThreads / 32) {
+            for (int pr = tid >> 5; pr < pairs; pr += kFinThreads / 32) {
                 const int e = pr / nc, q = pr - e * nc;
                 const int oo = orph_list[e], c = centres[q];
                 const uint16_t* fo = feat + (size_t)oo * D;
@@ -311,20 +335,20 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
                 for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
                 const float d2 = fmaxf(0.f, fmaf(-2.f, (dot * w[oo]) * w[c], a[oo] + a[c]));
                 if (lane == 0)
-                    atomicMin(&orph_best[e], ((unsigned long long)__float_as_uint(d2) << 32) | (unsigned long long)q);
+                    atomicMin(&orph_best[e], ((unsigned long long)__float_as_uint(d2) << 32) | (unsigned long long)(uint32_t)c);
             }
             __syncthreads();
-            if (tid < orph_cnt)                                     // remember the adopted centre at the root
-                nxt[orph_list[tid]] = -1 - centres[(int)(orph_best[tid] & 0xFFFFFFFFull)];
+            if (tid < orph_cnt) nxt[orph_list[tid]] = (uint16_t)(orph_best[tid] & 0xFFFFFFFFull);   // the adopted centre
         }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = tid; i < n; i += kFinThreads) {
-        const int l = label[i];
-        if (l < 0) {
-            const int root = -1 - l;
-            const int adopted = nxt[root];
-            label[i] = adopted < 0 ? -1 - adopted : root;
+    // ---- labels
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = e * kFinThreads + tid;
+        if (i < n) {
+            const int root = nxt[i];
+            label[i] = isc[root] ? root : (int)nxt[root];           // (a surplus orphan's entry is the centre that adopted it)
         }
     }
     if (tid == 0) n_clusters[b] = nc;
@@ -471,9 +495,13 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     }
 
     const int nc = n_centers < n ? n_centers : n;
-    const size_t smem = (size_t)n * 8 + (((size_t)n + 15) & ~(size_t)15) + (size_t)(nc > 0 ? nc : 1) * 4 + 16;
-    if (smem > 32 * 1024) {                                // (the kernel's static arrays take part of the default 48 KB)
-        cudaError_t e = cudaFuncSetAttribute(vic_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = (((size_t)n + 15) & ~(size_t)15) * 3 + (size_t)(nc > 0 ? nc : 1) * 2 + 16;
+    auto fin = n <= kFinThreads       ? vic_finalize_kernel<1>
+               : n <= 4 * kFinThreads ? vic_finalize_kernel<4>
+               : n <= 8 * kFinThreads ? vic_finalize_kernel<8> : vic_finalize_kernel<16>;
+    static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kFinThreads, "tokens of the longest sample");
+    if (smem > 16 * 1024) {                                // (the kernel's static arrays take part of the default 48 KB)
+        cudaError_t e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return record_cuda(e);
     }
     cudaLaunchConfig_t cfg;
@@ -481,7 +509,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     pdl_config(cfg, attr, dim3(B), dim3(kFinThreads), smem, stream, true);
     {
         KernelTimeScope timed("vic_finalize_kernel", stream);
-        rc = record_cuda(cudaLaunchKernelEx(&cfg, vic_finalize_kernel, static_cast<const uint16_t*>(feat), n, D, nc,
+        rc = record_cuda(cudaLaunchKernelEx(&cfg, fin, static_cast<const uint16_t*>(feat), n, D, nc,
                                             (const float*)rho, (const unsigned long long*)best, (const float*)w,
                                             (const float*)a, label, n_clusters, delta2_user, parent_user));
         if (rc != VITCOP_OK) return rc;

@@ -491,6 +491,21 @@ def test_filter_sweep_and_search_edges(B, n, metric, tau):
         check_vic_sample(f[b], p[b], metric, d_c, tau, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
 
 
+# No token within the spatial radius of another: every token is an orphan, all keys of the centre selection agree in their first
+# word and the densities decide (cuts among more and among fewer tied keys than are ranked by counting, one to several tokens
+# per thread); the surplus orphans join the nearest centre.
+@pytest.mark.parametrize("n,nc", [(200, 40), (700, 699), (1100, 30), (4200, 64)])
+def test_filter_all_orphans(n, nc):
+    w = dataclasses.replace(W.workload("tiny"), B=1, D=64, dup_rate=0.3)
+    f = W.make_features(w, n=n, B=1)
+    p = np.stack([np.arange(n, dtype=np.float32), np.zeros(n, dtype=np.float32)], -1)[None]
+    g = gpu_filter(f, p, 0, w.d_c, 0.5, nc)
+    assert g.status == vb.OK and np.all(g.n_clusters == nc) and np.all(g.parent == -1)
+    check_vic_sample(f[0], p[0], 0, w.d_c, 0.5, nc, g.rho[0], g.delta2[0], g.parent[0], g.label[0], max_uncompared=1.0)
+    order = np.lexsort((np.arange(n), -g.rho[0].astype(np.float64)))
+    assert np.array_equal(np.unique(g.label[0]), np.sort(order[:nc]))
+
+
 def test_filter_sample_groups():
     """More Gram values than the workspace keeps at a time: the samples go through the sweep and the search in groups, and
     give what each gives by itself."""
