@@ -1,14 +1,18 @@
-"""Thin ctypes binding of ``libvitcop.so`` -- same entry-point names as ``include/vitcop.h``.
+"""Thin binding of ``libvitcop.so`` -- same entry-point names as ``include/vitcop.h``.
 
 Argument marshalling only: every function takes torch CUDA tensors (or ``None``), passes their
-``data_ptr()`` and the current CUDA stream to the C ABI and raises ``VitcopError`` on a non-zero
+data pointers and the current CUDA stream to the C ABI and raises ``VitcopError`` on a non-zero
 status.  No arithmetic of the method happens here, and there is no fallback: if the shared
-library is missing or fails to load, importing the functions raises.
+library is missing or fails to load, importing the functions raises.  The calls of a pruning step
+go through ``_call.so`` (csrc/call.cpp), the diagnostic and host-only ones through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
+import struct
 from dataclasses import dataclass
 from typing import Optional
 
@@ -16,6 +20,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libvitcop.so")
+CALL_PATH = os.path.join(_PKG, "_call.so")
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_BUDGET, ERR_CUDA, ERR_TIMEOUT = range(7)
 (OP_FILTER, OP_KNORM, OP_SELECT, OP_COMPACT, OP_PRUNE_STEP, OP_SIMILARITY, OP_SALIENCY, OP_MERGE, OP_COLLAB_STEP,
@@ -55,11 +60,17 @@ class SelectParams(C.Structure):
 
 
 _lib: Optional[C.CDLL] = None
+_native = None                                   # _call.so's function
+_address: dict = {}                              # entry point -> address
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# the parameter structs as bytes, laid out as the compiler does
+_filter_params = struct.Struct("@iffdi4x").pack
+_select_params = struct.Struct("@iii").pack
 
 
 def lib() -> C.CDLL:
     """Loads the shared library (once).  Fails loudly when it has not been built."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(f"{LIB_PATH} is missing: run `python -m paper_2601_17818_b200.build` first")
@@ -102,9 +113,25 @@ def lib() -> C.CDLL:
         L.vitcop_kernel_timing_begin.argtypes = []
         L.vitcop_kernel_timing_end.argtypes = [C.POINTER(KernelTime), i32, C.POINTER(C.c_int)]
         for name in EXPORTS:
-            getattr(L, name)
+            _address[name] = C.cast(getattr(L, name), C.c_void_p).value
+        if not os.path.exists(CALL_PATH):
+            raise ImportError(f"{CALL_PATH} is missing: run `python -m paper_2601_17818_b200.build` first")
+        loader = importlib.machinery.ExtensionFileLoader("_call", CALL_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_call", loader))
+        loader.exec_module(module)
+        _native = module.call
         _lib = L
     return _lib
+
+
+def _call(name: str, *args, scale: float = 0.0) -> None:
+    """Calls entry point ``name`` on the current stream (its last argument).  Tensors must be contiguous CUDA tensors;
+    ``scale`` is the entry point's float argument, if it has one."""
+    if _native is None:
+        lib()
+    rc = _native(_address[name], scale, *args, _raw_stream(_device()))
+    if rc != OK:
+        raise VitcopError(rc, name)
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -127,10 +154,10 @@ def _check(status: int, where: str):
 
 
 def _vis(vis_len):
-    """(device pointer or None, uniform length) from an int or an int32 CUDA tensor."""
+    """(device lengths or None, uniform length) from an int or an int32 CUDA tensor."""
     if isinstance(vis_len, torch.Tensor):
         assert vis_len.dtype == torch.int32
-        return _ptr(vis_len), 0
+        return vis_len, 0
     return None, int(vis_len)
 
 
@@ -157,9 +184,8 @@ def vitcop_knorm_score(K: torch.Tensor, vis_start: int, vis_len, score: torch.Te
     assert K.dtype == torch.bfloat16 and score.dtype == torch.float32 and K.dim() == 4 and K.stride(3) == 1
     B, H, N, d = K.shape
     vp, vu = _vis(vis_len)
-    rc = lib().vitcop_knorm_score(C.c_void_p(K.data_ptr()), B, H, N, d, K.stride(0), K.stride(1), K.stride(2),
-                                  vis_start, vp, vu, _ptr(score), score.shape[1], _stream())
-    _check(rc, "vitcop_knorm_score")
+    _call("vitcop_knorm_score", K.data_ptr(), B, H, N, d, K.stride(0), K.stride(1), K.stride(2), int(vis_start), vp, vu, score,
+          score.shape[1])
     return score
 
 
@@ -168,12 +194,10 @@ def vitcop_select(score: torch.Tensor, vis_len, budget: int, keep_idx: torch.Ten
                   keep_mask: Optional[torch.Tensor] = None, mode: Optional[int] = None):
     assert score.dtype == torch.float32 and keep_idx.dtype == torch.int32 and n_keep.dtype == torch.int32
     B, Nv_cap = score.shape
-    p = SelectParams((1 if label is not None else 0) if mode is None else mode, int(largest), int(budget))
+    p = _select_params((1 if label is not None else 0) if mode is None else int(mode), int(largest), int(budget))
     vp, vu = _vis(vis_len)
-    rc = lib().vitcop_select(_ptr(score), _ptr(label), B, vp, vu, Nv_cap, C.byref(p), _ptr(keep_idx),
-                             keep_idx.shape[1], _ptr(n_keep), _ptr(keep_mask), _ptr(workspace), workspace.numel(),
-                             _stream())
-    _check(rc, "vitcop_select")
+    _call("vitcop_select", score, label, B, vp, vu, Nv_cap, p, keep_idx, keep_idx.shape[1], n_keep, keep_mask, workspace,
+          workspace.numel())
     return keep_idx, n_keep
 
 
@@ -189,10 +213,8 @@ def vitcop_compact_kv(hidden, K, V, vis_start: int, vis_len, keep_idx, n_keep, h
         Ncap = hidden_out.shape[1]
     Dh = hidden.shape[2] if hidden is not None else 0
     vp, vu = _vis(vis_len)
-    rc = lib().vitcop_compact_kv(_ptr(hidden), _ptr(K), _ptr(V), B, H, N, d, Dh, _ptr(seq_len), vis_start, vp, vu,
-                                 _ptr(keep_idx), keep_idx.shape[1], _ptr(n_keep), _ptr(hidden_out), _ptr(K_out),
-                                 _ptr(V_out), Ncap, _ptr(kept_pos), _ptr(out_len), _stream())
-    _check(rc, "vitcop_compact_kv")
+    _call("vitcop_compact_kv", hidden, K, V, B, H, N, d, Dh, seq_len, int(vis_start), vp, vu, keep_idx, keep_idx.shape[1], n_keep,
+          hidden_out, K_out, V_out, Ncap, kept_pos, out_len)
     return out_len
 
 
@@ -203,11 +225,8 @@ def vitcop_prune_step(hidden, K, V, vis_start: int, vis_len, Nv_cap: int, budget
     Ncap = K_out.shape[2] if K_out is not None else hidden_out.shape[1]
     Dh = hidden.shape[2] if hidden is not None else 0
     vp, vu = _vis(vis_len)
-    rc = lib().vitcop_prune_step(_ptr(hidden), _ptr(K), _ptr(V), B, H, N, d, Dh, _ptr(seq_len), vis_start, vp, vu,
-                                 int(Nv_cap), _ptr(label), int(budget), _ptr(hidden_out), _ptr(K_out), _ptr(V_out),
-                                 Ncap, _ptr(kept_pos), _ptr(out_len), _ptr(score_out), _ptr(keep_idx_out),
-                                 _ptr(n_keep_out), _ptr(workspace), workspace.numel(), _stream())
-    _check(rc, "vitcop_prune_step")
+    _call("vitcop_prune_step", hidden, K, V, B, H, N, d, Dh, seq_len, int(vis_start), vp, vu, int(Nv_cap), label, int(budget),
+          hidden_out, K_out, V_out, Ncap, kept_pos, out_len, score_out, keep_idx_out, n_keep_out, workspace, workspace.numel())
     return out_len
 
 
@@ -224,11 +243,8 @@ def vitcop_prune_step_static(hidden, K, V, vis_start: int, vis_len, Nv_cap: int,
     Ncap = K_out.shape[2] if K_out is not None else hidden_out.shape[1]
     Dh = hidden.shape[2] if hidden is not None else 0
     vp, vu = _vis(vis_len)
-    rc = lib().vitcop_prune_step_static(_ptr(hidden), _ptr(K), _ptr(V), B, H, N, d, Dh, _ptr(seq_len), vis_start, vp,
-                                        vu, int(Nv_cap), _ptr(label), int(budget), _ptr(hidden_out), _ptr(K_out),
-                                        _ptr(V_out), Ncap, _ptr(kept_pos), _ptr(out_len), _ptr(score_out),
-                                        _ptr(keep_idx_out), _ptr(n_keep_out), _stream())
-    _check(rc, "vitcop_prune_step_static")
+    _call("vitcop_prune_step_static", hidden, K, V, B, H, N, d, Dh, seq_len, int(vis_start), vp, vu, int(Nv_cap), label,
+          int(budget), hidden_out, K_out, V_out, Ncap, kept_pos, out_len, score_out, keep_idx_out, n_keep_out)
     return out_len
 
 
@@ -241,13 +257,10 @@ def vitcop_collaborative_step(feat, pos, hidden, K, V, vis_start: int, budget: i
     _, H, N, d = K.shape
     Ncap = K_out.shape[2] if K_out is not None else hidden_out.shape[1]
     Dh = hidden.shape[2] if hidden is not None else 0
-    p = FilterParams(int(metric), float(d_c), float(tau), float(alpha), int(n_centers))
-    rc = lib().vitcop_collaborative_step(_ptr(feat), _ptr(pos), D, C.byref(p), _ptr(hidden), _ptr(K), _ptr(V), B, H, N,
-                                         d, Dh, vis_start, Nv, int(budget), _ptr(hidden_out), _ptr(K_out), _ptr(V_out),
-                                         Ncap, _ptr(kept_pos), _ptr(out_len), _ptr(label_out), _ptr(n_clusters_out),
-                                         _ptr(rho), _ptr(delta2), _ptr(parent), _ptr(score_out), _ptr(keep_idx_out), _ptr(n_keep_out), _ptr(workspace),
-                                         workspace.numel(), _stream())
-    _check(rc, "vitcop_collaborative_step")
+    p = _filter_params(int(metric), float(d_c), float(tau), float(alpha), int(n_centers))
+    _call("vitcop_collaborative_step", feat, pos, D, p, hidden, K, V, B, H, N, d, Dh, int(vis_start), Nv, int(budget), hidden_out,
+          K_out, V_out, Ncap, kept_pos, out_len, label_out, n_clusters_out, rho, delta2, parent, score_out, keep_idx_out,
+          n_keep_out, workspace, workspace.numel())
     return out_len
 
 
@@ -258,19 +271,15 @@ def vitcop_merge_clusters(hidden, vis_start: int, vis_len, label, keep_mask, mer
     Nv_cap = label.shape[1]
     Mcap = merged_label.shape[1]
     vp, vu = _vis(vis_len)
-    rc = lib().vitcop_merge_clusters(_ptr(hidden), B, N, Dh, vis_start, vp, vu, Nv_cap, _ptr(label), _ptr(keep_mask),
-                                     _ptr(merged), _ptr(merged_f32), _ptr(merged_label), _ptr(merged_count),
-                                     _ptr(n_merged), Mcap, _ptr(workspace), workspace.numel(), _stream())
-    _check(rc, "vitcop_merge_clusters")
+    _call("vitcop_merge_clusters", hidden, B, N, Dh, int(vis_start), vp, vu, Nv_cap, label, keep_mask, merged, merged_f32,
+          merged_label, merged_count, n_merged, Mcap, workspace, workspace.numel())
     return n_merged
 
 
 def vitcop_cls_saliency(q_cls, K, scale: float, saliency, workspace, cls_self=None):
     """Eq. 1: q_cls bf16 [B,H,d], K bf16 [B,H,M,d] (key 0 = [CLS]) -> saliency fp32 [B, M-1]."""
     B, H, M, d = K.shape
-    rc = lib().vitcop_cls_saliency(_ptr(q_cls), _ptr(K), B, H, M, d, float(scale), _ptr(saliency), _ptr(cls_self),
-                                   _ptr(workspace), workspace.numel(), _stream())
-    _check(rc, "vitcop_cls_saliency")
+    _call("vitcop_cls_saliency", q_cls, K, B, H, M, d, saliency, cls_self, workspace, workspace.numel(), scale=scale)
     return saliency
 
 
@@ -281,10 +290,8 @@ def vitcop_kproj_knorm(hidden, W_k, H: int, d: int, K_out, workspace, vis_start:
     assert W_k.shape == (H * d, Dh) and K_out.shape == (B, H, N, d)
     Nv = 0 if score is None else score.shape[1]
     n_pos = 0 if rope_cos is None else rope_cos.shape[0]
-    rc = lib().vitcop_kproj_knorm(_ptr(hidden), _ptr(W_k), B, N, Dh, H, d, _ptr(rope_cos), _ptr(rope_sin),
-                                  _ptr(position_ids), n_pos, _ptr(K_out), int(vis_start), Nv, _ptr(score),
-                                  _ptr(workspace), workspace.numel(), _stream())
-    _check(rc, "vitcop_kproj_knorm")
+    _call("vitcop_kproj_knorm", hidden, W_k, B, N, Dh, H, d, rope_cos, rope_sin, position_ids, n_pos, K_out, int(vis_start), Nv,
+          score, workspace, workspace.numel())
     return K_out
 
 
@@ -317,20 +324,15 @@ def vitcop_redundancy_filter(feat: torch.Tensor, pos: Optional[torch.Tensor], la
                              parent=None):
     assert feat.dtype == torch.bfloat16 and feat.dim() == 3 and label.dtype == torch.int32
     B, n, D = feat.shape
-    p = FilterParams(int(metric), float(d_c), float(tau), float(alpha), int(n_centers))
-    rc = lib().vitcop_redundancy_filter(_ptr(feat), _ptr(pos), B, n, D, C.byref(p), _ptr(label), _ptr(n_clusters),
-                                        _ptr(rho), _ptr(delta2), _ptr(parent), _ptr(workspace), workspace.numel(),
-                                        _stream())
-    _check(rc, "vitcop_redundancy_filter")
+    p = _filter_params(int(metric), float(d_c), float(tau), float(alpha), int(n_centers))
+    _call("vitcop_redundancy_filter", feat, pos, B, n, D, p, label, n_clusters, rho, delta2, parent, workspace, workspace.numel())
     return label
 
 
 def vitcop_similarity_rows(feat: torch.Tensor, metric: int, row_begin: int, row_end: int, out: torch.Tensor,
                            workspace: torch.Tensor):
     B, n, D = feat.shape
-    rc = lib().vitcop_similarity_rows(_ptr(feat), B, n, D, int(metric), int(row_begin), int(row_end), _ptr(out),
-                                      _ptr(workspace), workspace.numel(), _stream())
-    _check(rc, "vitcop_similarity_rows")
+    _call("vitcop_similarity_rows", feat, B, n, D, int(metric), int(row_begin), int(row_end), out, workspace, workspace.numel())
     return out
 
 

@@ -1,4 +1,5 @@
-"""Builds ``libvitcop.so`` (sm_100a) in-tree with nvcc.  ``python -m paper_2601_17818_b200.build``."""
+"""Builds ``libvitcop.so`` (sm_100a, nvcc) and ``_call.so`` (the Python caller, g++) in-tree.
+``python -m paper_2601_17818_b200.build``."""
 from __future__ import annotations
 
 import concurrent.futures as cf
@@ -13,6 +14,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libvitcop.so")
+CALL = os.path.join(PKG, "_call.so")
 SOURCES = ["api.cu", "knorm.cu", "select.cu", "compact.cu", "filter.cu", "gram.cu", "density.cu", "nearest.cu", "kproj.cu", "merge.cu", "saliency.cu",
            "schedule.cu"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -32,12 +34,30 @@ def _digest() -> str:
     return h.hexdigest()
 
 
+def _build_caller() -> None:
+    """``_call.so``: a CPython extension that unpacks torch tensors (headers of the torch that imports it)."""
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    inc = [a for p in [*cpp_extension.include_paths(), sysconfig.get_paths()["include"]] for a in ("-I", p)]
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = CALL + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *inc, os.path.join(CSRC, "call.cpp"), "-o", tmp, "-L", libdir, "-lc10", "-ltorch_cpu", "-ltorch_python"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode:
+        sys.stderr.write(f"$ {' '.join(cmd)}\n{r.stdout}{r.stderr}")
+        raise RuntimeError("g++ failed on call.cpp")
+    os.replace(tmp, CALL)
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compile every translation unit for sm_100a and link the shared library; returns its path."""
     os.makedirs(BUILD_DIR, exist_ok=True)
     stamp = os.path.join(BUILD_DIR, "stamp")
     dig = _digest()
-    if not force and os.path.exists(LIB) and os.path.exists(stamp) and open(stamp).read() == dig:
+    if not force and os.path.exists(LIB) and os.path.exists(CALL) and os.path.exists(stamp) and open(stamp).read() == dig:
         return LIB
 
     def compile_one(src: str) -> str:
@@ -53,8 +73,10 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError(f"nvcc failed on {src}")
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        caller = ex.submit(_build_caller)
         objs = list(ex.map(compile_one, SOURCES))
+        caller.result()
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.check_call([_nvcc(), "-shared", "-gencode", "arch=compute_100a,code=sm_100a", *objs, "-o", tmp])
     os.replace(tmp, LIB)
