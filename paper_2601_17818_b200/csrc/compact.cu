@@ -1,9 +1,11 @@
 // Order-preserving compaction of hidden states and the K/V cache (bit-exact row gather).
 //
-// One CTA per (output row, sample).  The source position of the row comes from the ascending
-// keep list; the CTA then moves the hidden row and the row of every K and V head with 128-bit
+// A group of 32 to 256 threads per (output row, sample).  The source position of the row comes from the ascending
+// keep list; the group then moves the hidden row and the row of every K and V head with 128-bit
 // loads, up to eight of them issued before the first store and taken from all three tensors alike, so that
 // each thread keeps several independent 16-byte requests in flight.  Dropped rows are never read.
+// The group is the largest that leaves its threads four pieces each: a row of 1024 bf16 values alone (2 KB) moved by 256
+// threads kept one request per thread in flight on half of them (16 x 289 such rows 16 us).
 #include "internal.cuh"
 
 namespace vitcop {
@@ -28,7 +30,8 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
 // V (d8 pieces per head, heads head_in / head_out pieces apart).  The pieces of all three tensors form one index
 // space, so that a thread has up to eight loads from any of them in flight before its first store: the row costs
 // one round trip to memory, not one per tensor.  Null tensors are skipped.
-__device__ __forceinline__ void copy_token(const uint4* __restrict__ hid_src, uint4* __restrict__ hid_dst, int dh8,
+template <int G>
+__device__ __forceinline__ void copy_token(int lane, const uint4* __restrict__ hid_src, uint4* __restrict__ hid_dst, int dh8,
                                            const uint4* __restrict__ k_src, uint4* __restrict__ k_dst,
                                            const uint4* __restrict__ v_src, uint4* __restrict__ v_dst, int H, int d8,
                                            int d8_shift, int64_t head_in, int64_t head_out) {
@@ -37,12 +40,12 @@ __device__ __forceinline__ void copy_token(const uint4* __restrict__ hid_src, ui
     const int n_k = k_src ? n_kv : 0;
     const int total = n_hid + n_k + (v_src ? n_kv : 0);
     constexpr int kInFlight = 8;
-    for (int q0 = threadIdx.x; q0 < total; q0 += kInFlight * kCompactThreads) {
+    for (int q0 = lane; q0 < total; q0 += kInFlight * G) {
         uint4 v[kInFlight];
         uint4* d[kInFlight];
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) {
-            int q = q0 + u * kCompactThreads;
+            int q = q0 + u * G;
             d[u] = nullptr;
             if (q < total) {
                 if (q < n_hid) {
@@ -65,52 +68,56 @@ __device__ __forceinline__ void copy_token(const uint4* __restrict__ hid_src, ui
     }
 }
 
-__global__ void __launch_bounds__(kCompactThreads, 4)
+template <int G>
+__global__ void __launch_bounds__(kCompactThreads, G == kCompactThreads ? 4 : 3)
 compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, const uint4* __restrict__ V, int B, int H, int N,
-               int d8, int dh8, int d8_shift, const int32_t* __restrict__ seq_len, int vis_start,
-               const int32_t* __restrict__ vis_len, int vis_len_uniform, const int32_t* __restrict__ keep_idx,
-               int keep_stride, const int32_t* __restrict__ n_keep, uint4* __restrict__ hidden_out,
+               int d8, int dh8, int d8_shift, const int32_t* seq_len, int vis_start,
+               const int32_t* vis_len, int vis_len_uniform, const int32_t* keep_idx,
+               int keep_stride, const int32_t* n_keep, uint4* __restrict__ hidden_out,
                uint4* __restrict__ K_out, uint4* __restrict__ V_out, int Ncap, int32_t* __restrict__ kept_pos,
                int32_t* __restrict__ out_len) {
     // CTAs are handed out sample by sample within a row: all the rows in front of the visual span, which need not
     // wait for the selection, start before the rows that do
-    const int r = (int)(blockIdx.x / (unsigned)B);
-    const int b = (int)(blockIdx.x - (unsigned)r * (unsigned)B);
-    const int L = seq_len ? min(seq_len[b], N) : N;
+    const int rg = (int)(blockIdx.x / (unsigned)B);
+    const int b = (int)(blockIdx.x - (unsigned)rg * (unsigned)B);
+    // (uniform over the CTA where one row takes all of it)
+    const int r = G == kCompactThreads ? rg : rg * (kCompactThreads / G) + (int)threadIdx.x / G;
+    const int lane = G == kCompactThreads ? threadIdx.x : threadIdx.x % G;
+    const int L = seq_len ? min(__ldcg(seq_len + b), N) : N;
     const int64_t head_in = (int64_t)N * d8, head_out = (int64_t)Ncap * d8;
     // A row in front of the visual span keeps its place whatever the selection turns out to be: it is copied
     // before this kernel waits for the selection, while the kernels that produce it are still running.  (The
     // tensors copied here are inputs of the whole call, complete before its first kernel started.)
     const bool prefix_row = r < min(vis_start, L) && r < Ncap;
     if (prefix_row) {
-        copy_token(hidden ? hidden + ((int64_t)b * N + r) * dh8 : nullptr, hidden_out + ((int64_t)b * Ncap + r) * dh8, dh8,
+        copy_token<G>(lane, hidden ? hidden + ((int64_t)b * N + r) * dh8 : nullptr, hidden_out + ((int64_t)b * Ncap + r) * dh8, dh8,
                    K ? K + ((int64_t)b * H * N + r) * d8 : nullptr, K_out + ((int64_t)b * H * Ncap + r) * d8,
                    V ? V + ((int64_t)b * H * N + r) * d8 : nullptr, V_out + ((int64_t)b * H * Ncap + r) * d8, H, d8,
                    d8_shift, head_in, head_out);
-        if (kept_pos && threadIdx.x == 0) kept_pos[(int64_t)b * Ncap + r] = r;
+        if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = r;
         if (r != 0) return;                                // row 0 still reports the sample's new length
     }
     grid_dependency_wait();
-    int nv = vis_len ? vis_len[b] : vis_len_uniform;
+    int nv = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
     nv = max(0, min(nv, L - vis_start));
-    const int nk = max(0, min(n_keep[b], nv));
+    const int nk = max(0, min(__ldcg(n_keep + b), nv));
     const int olen = L - nv + nk;
-    if (r == 0 && threadIdx.x == 0) out_len[b] = olen;
+    if (r == 0 && lane == 0) out_len[b] = olen;
     if (r >= Ncap || prefix_row) return;
     if (r >= olen) {
-        if (kept_pos && threadIdx.x == 0) kept_pos[(int64_t)b * Ncap + r] = -1;
+        if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = -1;
         return;
     }
     int src_row;
     if (r < vis_start) src_row = r;
     else if (r < vis_start + nk) {
-        int ki = keep_idx[(int64_t)b * keep_stride + (r - vis_start)];
+        int ki = __ldcg(keep_idx + (int64_t)b * keep_stride + (r - vis_start));
         ki = max(0, min(ki, nv - 1));                     // a corrupt index can never leave the span
         src_row = vis_start + ki;
     } else src_row = r - nk + nv;
-    if (kept_pos && threadIdx.x == 0) kept_pos[(int64_t)b * Ncap + r] = src_row;
+    if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = src_row;
 
-    copy_token(hidden ? hidden + ((int64_t)b * N + src_row) * dh8 : nullptr, hidden_out + ((int64_t)b * Ncap + r) * dh8,
+    copy_token<G>(lane, hidden ? hidden + ((int64_t)b * N + src_row) * dh8 : nullptr, hidden_out + ((int64_t)b * Ncap + r) * dh8,
                dh8, K ? K + ((int64_t)b * H * N + src_row) * d8 : nullptr, K_out + ((int64_t)b * H * Ncap + r) * d8,
                V ? V + ((int64_t)b * H * N + src_row) * d8 : nullptr, V_out + ((int64_t)b * H * Ncap + r) * d8, H, d8,
                d8_shift, head_in, head_out);
@@ -130,7 +137,11 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
     cudaLaunchConfig_t cfg = {};
     // rows past min(N, Ncap) cannot exist; one extra CTA row keeps out_len written when Ncap == 0
     const int rows = Ncap > 0 ? Ncap : 1;
-    cfg.gridDim = dim3((unsigned)((long long)B * rows));
+    const long long pieces = (hidden ? Dh / 8 : 0) + (long long)H * d8 * ((K ? 1 : 0) + (V ? 1 : 0));
+    int G = kCompactThreads;
+    while (G > 32 && pieces < 4LL * G) G /= 2;
+    const int per_cta = kCompactThreads / G;
+    cfg.gridDim = dim3((unsigned)((long long)B * ((rows + per_cta - 1) / per_cta)));
     cfg.blockDim = dim3(kCompactThreads);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -139,8 +150,9 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(pdl) ? 1 : 0;
     KernelTimeScope timed("compact_kernel", stream);
+    auto kern = G == 256 ? compact_kernel<256> : G == 128 ? compact_kernel<128> : G == 64 ? compact_kernel<64> : compact_kernel<32>;
     return record_cuda(cudaLaunchKernelEx(
-        &cfg, compact_kernel, static_cast<const uint4*>(hidden), static_cast<const uint4*>(K),
+        &cfg, kern, static_cast<const uint4*>(hidden), static_cast<const uint4*>(K),
         static_cast<const uint4*>(V), B, H, N, d / 8, Dh / 8, d8_shift, seq_len, vis_start, vis_len, vis_len_uniform, keep_idx,
         keep_stride, n_keep, static_cast<uint4*>(hidden_out), static_cast<uint4*>(K_out), static_cast<uint4*>(V_out),
         Ncap, kept_pos, out_len));
