@@ -77,6 +77,7 @@ struct StepWs {
     }
 };
 
+// (Calls whose first kernel can do it clear the word there: a memset in front of a small kernel costs more than a microsecond.)
 int reset_status(void* ws, cudaStream_t s) { return record_cuda(cudaMemsetAsync(ws, 0, kStatusBytes, s)); }
 
 int check_span(int N, int vis_start, const int32_t* vis_len, int vis_len_uniform, int Nv_cap) {
@@ -253,10 +254,15 @@ int vitcop_select(const float* score, const int32_t* label, int B, const int32_t
     if (!workspace || workspace_bytes < kStatusBytes) return VITCOP_ERR_WORKSPACE;
     if (!aligned256(workspace)) return VITCOP_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int rc = reset_status(workspace, s);
-    if (rc != VITCOP_OK) return rc;
+    // (quota mode: any of the CTAs may set the word, so none of them can clear it)
+    int* const status = static_cast<int*>(workspace);
+    const bool in_kernel = p->mode == 0 && B > 0;
+    if (!in_kernel) {
+        const int rc = reset_status(workspace, s);
+        if (rc != VITCOP_OK) return rc;
+    }
     return launch_select(score, label, B, vis_len, vis_len_uniform, Nv_cap, p->mode, p->largest ? 1 : 0, p->budget,
-                         keep_idx, keep_stride, n_keep, keep_mask, static_cast<int*>(workspace), s, false);
+                         keep_idx, keep_stride, n_keep, keep_mask, status, s, false, in_kernel ? status : nullptr);
 }
 
 static int check_compact_args(const void* hidden, const void* K, const void* V, int B, int H, int N, int d, int Dh,
@@ -317,12 +323,14 @@ int vitcop_prune_step(const void* hidden, const void* K, const void* V, int B, i
     float* score = score_out ? score_out : reinterpret_cast<float*>(ws + lay.off_score);
     int32_t* keep = keep_idx_out ? keep_idx_out : reinterpret_cast<int32_t*>(ws + lay.off_keep);
     int32_t* nkeep = n_keep_out ? n_keep_out : reinterpret_cast<int32_t*>(ws + lay.off_nkeep);
-    rc = reset_status(workspace, s);
-    if (rc != VITCOP_OK) return rc;
     bool have_knorm = false;
     rc = launch_knorm(K, B, H, d, (int64_t)H * N * d, (int64_t)N * d, d, vis_start, vis_len, vis_len_uniform, score,
-                      Nv_cap, s, false, &have_knorm);
+                      Nv_cap, s, false, &have_knorm, reinterpret_cast<int*>(ws));
     if (rc != VITCOP_OK) return rc;
+    if (!have_knorm) {
+        rc = reset_status(workspace, s);
+        if (rc != VITCOP_OK) return rc;
+    }
     // The selection releases its dependents before it waits for its predecessor, and the compaction copies the rows
     // in front of the span before its own wait: that is safe only behind a kernel of this call that has itself
     // waited for everything queued before the call.  With an empty span there is no such kernel, so the selection
@@ -396,8 +404,7 @@ int vitcop_merge_clusters(const void* hidden, int B, int N, int Dh, int vis_star
     if (!workspace || workspace_bytes < merge_workspace_bytes(B, Nv_cap, Mcap) || !aligned256(workspace))
         return VITCOP_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    rc = reset_status(workspace, s);
-    if (rc != VITCOP_OK) return rc;
+    if (B == 0) return reset_status(workspace, s);
     return launch_merge(hidden, B, N, Dh, vis_start, vis_len, vis_len_uniform, Nv_cap, label, keep_mask, merged,
                         merged_f32, merged_label, merged_count, n_merged, Mcap, workspace, s);
 }
@@ -409,8 +416,7 @@ int vitcop_cls_saliency(const void* q_cls, const void* K, int B, int H, int M, i
     if (!workspace || workspace_bytes < saliency_workspace_bytes(B, H, M) || !aligned256(workspace))
         return VITCOP_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int rc = reset_status(workspace, s);
-    if (rc != VITCOP_OK) return rc;
+    if (B == 0 || H == 0 || M == 0) return reset_status(workspace, s);
     return launch_cls_saliency(q_cls, K, B, H, M, d, scale, saliency, cls_self, workspace, s);
 }
 

@@ -34,8 +34,9 @@ inline bool pdl_allowed(bool requested) { return requested && !kernel_timing_on(
 // ---- launchers (enqueue on `stream`, return VITCOP_OK or VITCOP_ERR_CUDA) -------------------------
 int launch_knorm(const void* K, int B, int H, int d, int64_t stride_b, int64_t stride_h, int64_t stride_n,
                  int vis_start, const int32_t* vis_len, int vis_len_uniform, float* score, int Nv_cap,
-                 cudaStream_t stream, bool late_wait = false, bool* launched = nullptr);
-// (`launched`, when given, tells whether a kernel was enqueued at all: an empty span needs none.)
+                 cudaStream_t stream, bool late_wait = false, bool* launched = nullptr, int* clear_status = nullptr);
+// (`launched`, when given, tells whether a kernel was enqueued at all: an empty span needs none.  `clear_status`: a status
+// word that the kernel sets to VITCOP_OK.)
 
 // K-norm to be enqueued in the middle of the filter's kernel chain (vitcop_collaborative_step): it does not depend
 // on the filter, so it runs beside the filter's sweep.
@@ -47,7 +48,9 @@ struct KnormJob {
 
 int launch_select(const float* score, const int32_t* label, int B, const int32_t* vis_len, int vis_len_uniform,
                   int Nv_cap, int mode, int largest, int budget, int32_t* keep_idx, int keep_stride,
-                  int32_t* n_keep, uint8_t* keep_mask, int* status_word, cudaStream_t stream, bool pdl);
+                  int32_t* n_keep, uint8_t* keep_mask, int* status_word, cudaStream_t stream, bool pdl,
+                  int* clear_status = nullptr);
+// (`clear_status`: plain mode sets this status word to VITCOP_OK on the way, in place of a memset in front of the kernel.)
 
 int launch_compact(const void* hidden, const void* K, const void* V, int B, int H, int N, int d, int Dh,
                    const int32_t* seq_len, int vis_start, const int32_t* vis_len, int vis_len_uniform,

@@ -16,15 +16,16 @@ constexpr int kKnormThreads = 128;
 template <int LPR, int UNROLL>
 __global__ void __launch_bounds__(kKnormThreads)
 knorm_kernel(const uint4* __restrict__ K, int H, int d8, int64_t sb, int64_t sh, int64_t sn, int vis_start,
-             const int32_t* __restrict__ vis_len, int vis_len_uniform, float* __restrict__ score, int Nv_cap,
-             int late_wait) {
+             const int32_t* vis_len, int vis_len_uniform, float* __restrict__ score, int Nv_cap,
+             int late_wait, int* __restrict__ clear_status) {
     // late_wait: K is known to be final already (the caller ordered its producer before the preceding grid), so
     // this grid may run beside the preceding one; it still waits for it before it ends, which keeps "this grid
     // has completed" meaning "everything before it has completed" for the kernels that follow.
     if (!late_wait) grid_dependency_wait();
+    if (clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear_status = VITCOP_OK;
     const int b = blockIdx.y;
     // a device-side length never reaches past the capacity of the score row (nor, the host has checked, of K)
-    const int nv = max(0, min(vis_len ? vis_len[b] : vis_len_uniform, Nv_cap));
+    const int nv = max(0, min(vis_len ? __ldcg(vis_len + b) : vis_len_uniform, Nv_cap));
     constexpr int kTok = kKnormThreads / LPR;
     const int sub = threadIdx.x % LPR;
     const int i = blockIdx.x * kTok + threadIdx.x / LPR;
@@ -46,7 +47,7 @@ knorm_kernel(const uint4* __restrict__ K, int H, int d8, int64_t sb, int64_t sh,
 
 int launch_knorm(const void* K, int B, int H, int d, int64_t stride_b, int64_t stride_h, int64_t stride_n,
                  int vis_start, const int32_t* vis_len, int vis_len_uniform, float* score, int Nv_cap,
-                 cudaStream_t stream, bool late_wait, bool* launched) {
+                 cudaStream_t stream, bool late_wait, bool* launched, int* clear_status) {
     if (launched) *launched = false;
     if (B <= 0 || Nv_cap <= 0 || H <= 0) return VITCOP_OK;
     const int d8 = d / 8;
@@ -69,7 +70,7 @@ int launch_knorm(const void* K, int B, int H, int d, int64_t stride_b, int64_t s
         cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
         KernelTimeScope timed("knorm_kernel", stream);
         rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, Kp, H, d8, sb, sh, sn, vis_start, vis_len, vis_len_uniform,
-                                            score, Nv_cap, late_wait ? 1 : 0));
+                                            score, Nv_cap, late_wait ? 1 : 0, clear_status));
     };
     if (d8 >= 16) go(knorm_kernel<16, 8>, 16);
     else if (d8 >= 8) go(knorm_kernel<8, 8>, 8);

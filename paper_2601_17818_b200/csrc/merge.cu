@@ -102,11 +102,13 @@ __global__ void __launch_bounds__(kPlanThreads)
 merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__ keep_mask,
                   const int32_t* __restrict__ vis_len, int vis_len_uniform, int Nv_cap, int Mcap,
                   int32_t* __restrict__ merged_label, int32_t* __restrict__ merged_count,
-                  int32_t* __restrict__ n_merged, uint16_t* __restrict__ members, int32_t* __restrict__ starts) {
+                  int32_t* __restrict__ n_merged, uint16_t* __restrict__ members, int32_t* __restrict__ starts,
+                  int* __restrict__ status) {
     extern __shared__ __align__(16) uint32_t smem_items[];   // two item buffers of Nv_cap (rounded up to 4), then the counters
     __shared__ uint32_t warp_sums[32];
     grid_dependency_wait();
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (b == 0 && tid == 0) *status = VITCOP_OK;
     const uint32_t lt = (1u << lane) - 1u;
     int n = vis_len ? vis_len[b] : vis_len_uniform;
     n = max(0, min(n, Nv_cap));
@@ -299,7 +301,8 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
         cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
         KernelTimeScope timed("merge_plan_kernel", stream);
         int rc = record_cuda(cudaLaunchKernelEx(&cfg, merge_plan_kernel, label, keep_mask, vis_len, vis_len_uniform,
-                                                Nv_cap, Mcap, merged_label, merged_count, n_merged, members, starts));
+                                                Nv_cap, Mcap, merged_label, merged_count, n_merged, members, starts,
+                                                static_cast<int*>(workspace)));
         if (rc != VITCOP_OK) return rc;
     }
     if (Mcap <= 0 || Dh <= 0 || (!merged_bf16 && !merged_f32)) return VITCOP_OK;

@@ -46,7 +46,7 @@ __device__ __forceinline__ void dot8(const uint4& k, const float* q, float& a0, 
 template <int LANES>
 __global__ void __launch_bounds__(kSalThreads)
 cls_logits_kernel(const uint4* __restrict__ q, const uint4* __restrict__ K, int H, int M, int d8, float scale_log2e,
-                  float* __restrict__ logit, float2* __restrict__ part) {
+                  float* __restrict__ logit, float2* __restrict__ part, int* __restrict__ status) {
     constexpr int kRowsPerPass = kSalThreads / LANES;
     constexpr int kPasses = kSalChunk / kRowsPerPass;      // == LANES
     constexpr int kInFlight = 4;                           // rows a lane requests before it reduces any
@@ -55,6 +55,7 @@ cls_logits_kernel(const uint4* __restrict__ q, const uint4* __restrict__ K, int 
     __shared__ float scratch[kSalWarps];
     grid_dependency_wait();
     const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+    if (chunk == 0 && h == 0 && b == 0 && tid == 0) *status = VITCOP_OK;
     const int chunks = gridDim.x;
     const int sub = tid % LANES, slot = tid / LANES;
     const uint4* qrow = q + ((size_t)b * H + h) * d8;
@@ -189,7 +190,7 @@ int launch_cls_saliency(const void* q, const void* K, int B, int H, int M, int d
         KernelTimeScope timed("cls_logits_kernel", stream);
         auto kern = d8 <= 8 ? cls_logits_kernel<8> : d8 <= 16 ? cls_logits_kernel<16> : cls_logits_kernel<32>;
         int rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, static_cast<const uint4*>(q), static_cast<const uint4*>(K),
-                                                H, M, d8, scale * 1.4426950408889634f, logit, part));
+                                                H, M, d8, scale * 1.4426950408889634f, logit, part, static_cast<int*>(workspace)));
         if (rc != VITCOP_OK) return rc;
     }
     cudaLaunchConfig_t cfg = {};
