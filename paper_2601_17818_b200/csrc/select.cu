@@ -176,15 +176,17 @@ select_plain_kernel(const float* score, const int32_t* vis_len, int vis_len_unif
 }
 
 // ------------------------------------------------------------------------------------------ quota
+// R CTAs (a thread-block cluster) per sequence.
+template <int R>
 __global__ void __launch_bounds__(kSelThreads)
-select_quota_kernel(const float* __restrict__ score, const int32_t* __restrict__ label,
-                    const int32_t* __restrict__ vis_len, int vis_len_uniform, int Nv_cap, int P_cap, int budget,
+select_quota_kernel(const float* score, const int32_t* label,
+                    const int32_t* vis_len, int vis_len_uniform, int Nv_cap, int P_cap, int budget,
                     int32_t* __restrict__ keep_idx, int keep_stride, int32_t* __restrict__ n_keep,
                     uint8_t* __restrict__ keep_mask, int* __restrict__ status_word) {
     grid_dependency_launch_dependents();                  // see select_plain_kernel
     grid_dependency_wait();
-    select_quota_body(score, label, vis_len, vis_len_uniform, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep,
-                      keep_mask, status_word, blockIdx.x);
+    select_quota_body<R>(score, label, vis_len, vis_len_uniform, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep,
+                         keep_mask, status_word, blockIdx.x / R);
 }
 
 }  // namespace
@@ -216,14 +218,30 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
     }
     int P = 0;
     const size_t smem = select_quota_smem(Nv_cap, &P);
-    if (smem > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(select_quota_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // CTAs per sequence: one up to 2048 tokens (the others would be done preparing when the first is done), four, and eight
+    // beyond 8192
+    const int R = Nv_cap <= 2 * kSelThreads ? 1 : Nv_cap <= 8 * kSelThreads ? 4 : 8;
+    auto kern = R == 1 ? select_quota_kernel<1> : R == 4 ? select_quota_kernel<4> : select_quota_kernel<8>;
+    if (smem > 40 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return record_cuda(e);
     }
+    cudaLaunchAttribute attrs[2];
+    attrs[0] = attr[0];
+    int n_attr = cfg.numAttrs;
+    if (R > 1) {
+        attrs[n_attr].id = cudaLaunchAttributeClusterDimension;
+        attrs[n_attr].val.clusterDim.x = R;
+        attrs[n_attr].val.clusterDim.y = 1;
+        attrs[n_attr].val.clusterDim.z = 1;
+        ++n_attr;
+    }
+    cfg.attrs = attrs;
+    cfg.numAttrs = n_attr;
+    cfg.gridDim = dim3((unsigned)(B * R));
     cfg.dynamicSmemBytes = smem;
     KernelTimeScope timed("select_quota_kernel", stream);
-    return record_cuda(cudaLaunchKernelEx(&cfg, select_quota_kernel, score, label, vis_len, vis_len_uniform, Nv_cap,
+    return record_cuda(cudaLaunchKernelEx(&cfg, kern, score, label, vis_len, vis_len_uniform, Nv_cap,
                                           P, budget, keep_idx, keep_stride, n_keep, keep_mask, status_word));
 }
 

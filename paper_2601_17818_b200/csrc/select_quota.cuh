@@ -1,7 +1,8 @@
-// Cluster-quota selection (Eq. 5 / Algorithm 3 up to the elite set) as a CTA-wide device routine, called by
+// Cluster-quota selection (Eq. 5 / Algorithm 3 up to the elite set) as a device routine of one to eight CTAs, called by
 // select_quota_kernel (select.cu).
 #pragma once
 
+#include "async_copy.cuh"
 #include "block_sort.cuh"
 #include "internal.cuh"
 
@@ -65,7 +66,10 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
 // pairs:
 //   rank   -- the tokens are scattered into per-cluster segments and every token counts the members of its own
 //             segment that precede it: sum of |C_c|^2 comparisons, taken when that sum is a small multiple of n
-//             (clusters of similar size, the usual outcome of Algorithm 2);
+//             (clusters of similar size, the usual outcome of Algorithm 2).  On longer samples this is most of the work, and
+//             the CTAs of a thread-block cluster share the segments out: each prepares everything for itself (a microsecond
+//             or two), ranks its part and sends every verdict to the CTA that will emit the token.  (One CTA per sample:
+//             10 us on 576 tokens, 16 on 2880, 47 on 16384.);
 //   radix  -- every cluster runs its own radix select (4-bit digits) for its q_c-th smallest pair, all clusters at
 //             once: one shared histogram row per cluster, one thread per cluster to pick the digit, O(n) work per
 //             pass whatever the sizes.  Pairs are unique, so ties need no extra pass; a cluster stops as soon as a
@@ -73,9 +77,7 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
 constexpr int kMaxSeg = 1024;
 constexpr int kSegTok = 16;                               // tokens per thread: VITCOP_MAX_VISUAL_TOKENS / kSelThreads
 constexpr uint32_t kSegDone = 0xFFFFFFFFu;
-constexpr int kRankWork = 64;                             // rank search when sum |C_c|^2 <= kRankWork * n ...
-constexpr int kRankWorkLong = 16;                         // ... (long samples: a CTA's 1024 threads share all of it) ...
-constexpr int kRankLongTokens = 8192;
+constexpr int kRankWork = 64;                             // rank search when sum |C_c|^2 <= kRankWork * n per CTA ...
 constexpr int kRankMaxSize = 2048;                        // ... and no searched cluster is larger than this
 constexpr int kRadixMinTokens = 4096;                     // below this a sort beats the radix passes (fewer barriers)
 
@@ -124,11 +126,15 @@ struct ClusterSelSmem {
 };
 
 // Returns false (having written nothing) when the sample has more than kMaxSeg clusters, or sizes that rule out
-// the rank search on a sample too short for the radix search to pay: the caller then sorts.
+// the rank search on a sample too short for the radix search to pay: the caller then sorts.  R CTAs of a thread-block
+// cluster call together with the same arguments and return the same; what the rank search does not take is left to the first.
+template <int R>
 __device__ __forceinline__ bool select_quota_by_cluster(const float* score, const int32_t* label, int n, int budget,
                                                         int32_t* keep_idx, int keep_stride, int32_t* n_keep_b,
                                                         uint8_t* keep_mask, int* status_word, uint8_t* smem,
                                                         uint32_t* warp_sums) {
+    __shared__ uint32_t range_kept[R];                     // tokens kept in every CTA's range
+    const int part = R > 1 ? (int)cluster_ctarank() : 0;
     const ClusterSelSmem L(n);
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
     unsigned long long* seg = reinterpret_cast<unsigned long long*>(smem);
@@ -143,7 +149,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
     const int tid = threadIdx.x;
 
     // ---- dense cluster ids in ascending label order
-    for (int i = tid; i < n; i += kSelThreads) id_of[i] = 0;
+    for (int i = tid; i < L.n_al / 8; i += kSelThreads) reinterpret_cast<uint4*>(id_of)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < kMaxSeg) csize[tid] = 0;
     if (tid == 0) {
         misc[0] = 0xFFFFFFFFu;
@@ -160,10 +166,10 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         const int i = k * kSelThreads + tid;
         comp[k] = 0;
         if (i < n) {
-            uint32_t lab = (uint32_t)label[i];
+            uint32_t lab = (uint32_t)__ldcg(label + i);
             if (lab >= (uint32_t)n) lab = (uint32_t)n - 1;          // out-of-range labels are clamped, never indexed
             id_of[lab] = 1;
-            const uint32_t key = order_key(score[i], 0);
+            const uint32_t key = order_key(__ldcg(score + i), 0);
             key_lo = min(key_lo, key);
             key_hi = max(key_hi, key);
             comp[k] = ((unsigned long long)lab << 48) | ((unsigned long long)key << 16);
@@ -176,15 +182,42 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         atomicMax(&misc[1], key_hi);
     }
     __syncthreads();
-    const int per = (n + kSelThreads - 1) / kSelThreads;
-    const int l0 = tid * per;
-    uint32_t cnt = 0;
-    for (int j = 0; j < per; ++j) cnt += (l0 + j < n && id_of[l0 + j]) ? 1u : 0u;
+    // (a thread takes a run of labels; of eight at a time, two flags to a word, on longer samples)
     uint32_t n_seg;
-    uint32_t next_id = block_exclusive_sum(cnt, warp_sums, n_seg);
-    if (n_seg > (uint32_t)kMaxSeg) return false;           // uniform over the CTA
-    for (int j = 0; j < per; ++j)
-        if (l0 + j < n && id_of[l0 + j]) id_of[l0 + j] = (uint16_t)next_id++;
+    if (n <= 2 * kSelThreads) {
+        const int l0 = 2 * tid;
+        const uint32_t pair = l0 < n ? *reinterpret_cast<const uint32_t*>(id_of + l0) : 0u;     // (id_of is padded to eight)
+        const uint32_t f0 = pair & 1u, f1 = (pair >> 16 & 1u) && l0 + 1 < n ? 1u : 0u;
+        const uint32_t next_id = block_exclusive_sum(f0 + f1, warp_sums, n_seg);
+        if (n_seg > (uint32_t)kMaxSeg) return false;       // uniform over the CTAs
+        if (l0 < n) *reinterpret_cast<uint32_t*>(id_of + l0) = next_id | (next_id + f0) << 16;
+    } else {
+        const int words = (n + kSelThreads * 8 - 1) / (kSelThreads * 8);        // of eight labels per thread: 1 or 2
+        uint4 w[2];
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int l = (tid * words + v) * 8;
+            w[v] = v < words && l < n ? *reinterpret_cast<const uint4*>(id_of + l) : make_uint4(0u, 0u, 0u, 0u);
+            cnt += __popc(w[v].x) + __popc(w[v].y) + __popc(w[v].z) + __popc(w[v].w);
+        }
+        uint32_t next_id = block_exclusive_sum(cnt, warp_sums, n_seg);
+        if (n_seg > (uint32_t)kMaxSeg) return false;       // uniform over the CTAs
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int l = (tid * words + v) * 8;
+            if (v < words && l < n) {
+                uint32_t* f = &w[v].x;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t lo = f[q] & 1u, hi = f[q] >> 16;
+                    f[q] = next_id | (next_id + lo) << 16;
+                    next_id += lo + hi;
+                }
+                *reinterpret_cast<uint4*>(id_of + l) = w[v];
+            }
+        }
+    }
     __syncthreads();
 
     // ---- cluster sizes (the atomic's return value is the token's slot inside its cluster) and quotas (Eq. 5)
@@ -199,6 +232,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
     __syncthreads();
     const long long b_elites = (long long)budget - (long long)n_seg;
     if (b_elites < 0) {
+        if (part != 0) return true;
         if (tid == 0 && status_word) atomicMax(status_word, VITCOP_ERR_BUDGET);
         for (int i = tid; i < n; i += kSelThreads) keepf[i] = 0;
         __syncthreads();
@@ -210,10 +244,11 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         uint32_t size = 0, work = 0, veto = 0;
         if (tid < (int)n_seg) {
             size = csize[tid];
-            const long long q = ((long long)size * b_elites) / (long long)n;
-            quota[tid] = (uint32_t)q;
-            const bool searched = q > 0 && q < (long long)size;      // none or all of a cluster: nothing to search
-            krem[tid] = searched ? (uint32_t)q : kSegDone;
+            // (a budget of n or more keeps every cluster whole, as n does: the product fits 32 bits)
+            const uint32_t q = size * (uint32_t)(b_elites < n ? b_elites : n) / (uint32_t)n;
+            quota[tid] = q;
+            const bool searched = q > 0 && q < size;                 // none or all of a cluster: nothing to search
+            krem[tid] = searched ? q : kSegDone;
             if (searched) {
                 veto = size > (uint32_t)kRankMaxSize ? 1u : 0u;
                 work = veto ? 0u : size * size;
@@ -229,10 +264,10 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         const uint32_t o = block_exclusive_sum(size, warp_sums, total);   // its barriers publish misc as well
         if (tid < (int)n_seg) offs[tid] = o;
     }
-    const bool by_rank = misc[3] == 0 && (unsigned long long)misc[2] <=
-                                             (unsigned long long)(n > kRankLongTokens ? kRankWorkLong : kRankWork) * (unsigned)n;
+    const bool by_rank = misc[3] == 0 && (unsigned long long)misc[2] <= (unsigned long long)(kRankWork * R) * (unsigned)n;
     const uint32_t range_lo = misc[0], range_hi = misc[1];
     if (!by_rank && n <= kRadixMinTokens) return false;    // uniform; nothing has been written yet
+    if (!by_rank && part != 0) return true;
     __syncthreads();
 
     if (by_rank) {
@@ -247,9 +282,18 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
             }
         }
         __syncthreads();
-        for (int p = tid; p < n; p += kSelThreads) {
+        const int range = (n + R - 1) / R;                 // segment positions a CTA ranks, tokens it emits
+        if (R > 1) cluster_sync_all();                     // every CTA of the cluster has started: its memory may be written
+        for (int p = part * range + tid; p < n; p += kSelThreads) {
             const unsigned long long mine = seg[p];
             const uint32_t c = (uint32_t)(mine >> 48);
+            if (R > 1) {
+                // a CTA takes the segments that start in its range, whole: inside a segment the members' order is its own
+                // (slots were handed out by atomics), only where segments start is common to all CTAs
+                const int at = (int)offs[c];
+                if (at < part * range) continue;
+                if (at >= (part + 1) * range) break;
+            }
             const uint32_t q = quota[c], size = csize[c];
             bool keep = q >= size;
             if (!keep && q > 0) {
@@ -265,7 +309,44 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
                 for (; m < size; ++m) before += members[m] < mine ? 1u : 0u;
                 keep = before < q;                        // same cluster bits: the order of (score key, index)
             }
-            keepf[(uint32_t)(mine & 0xFFFFull)] = keep ? 1 : 0;
+            const uint32_t i = (uint32_t)(mine & 0xFFFFull);
+            if (R == 1) keepf[i] = keep ? 1 : 0;
+            else
+                asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(cluster_map(smem_u32(keepf + i), i / (uint32_t)range)),
+                             "r"(keep ? 1u : 0u)
+                             : "memory");
+        }
+        if (R > 1) {
+            // ---- every CTA emits its range of tokens, behind the kept ones of the ranges in front of it
+            cluster_sync_all();
+            const int first = part * range, last = min(n, first + range);
+            const int per = (range + kSelThreads - 1) / kSelThreads, i0 = first + tid * per;
+            uint32_t cnt = 0;
+            for (int j = 0; j < per; ++j) cnt += (i0 + j < last && keepf[i0 + j]) ? 1u : 0u;
+            uint32_t total;
+            uint32_t r = block_exclusive_sum(cnt, warp_sums, total);
+            if (tid < R)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(smem_u32(range_kept + part), (uint32_t)tid)), "r"(total)
+                             : "memory");
+            cluster_sync_all();
+            uint32_t all = 0;
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                if (u < part) r += range_kept[u];
+                all += range_kept[u];
+            }
+            for (int j = 0; j < per; ++j) {
+                const int i = i0 + j;
+                if (i >= last) break;
+                const bool f = keepf[i] != 0;
+                if (f) {
+                    if (r < (uint32_t)keep_stride) keep_idx[r] = i;
+                    ++r;
+                }
+                if (keep_mask) keep_mask[i] = f ? 1 : 0;
+            }
+            if (part == 0 && tid == 0) *n_keep_b = (int32_t)all;
+            return true;
         }
     } else {
         // ---- per-cluster radix select of the quota-th smallest pair, 4 bits per pass from the top of the 48-bit
@@ -344,31 +425,33 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
 
 // ------------------------------------------------------------------------------------------ quota
 // Shared memory: comp[P] (uint64), cstart[n] and csize[n] (uint16, indexed by label value), keep[n] (uint8).
-// Cluster-quota selection of sample b by the whole CTA (kSelThreads threads); uses the dynamic shared memory.
+// Cluster-quota selection of sample b by R whole CTAs (kSelThreads threads each); uses the dynamic shared memory.
+template <int R>
 __device__ __forceinline__ void select_quota_body(const float* score, const int32_t* label,
-                                                  const int32_t* __restrict__ vis_len, int vis_len_uniform,
+                                                  const int32_t* vis_len, int vis_len_uniform,
                                                   int Nv_cap, int P_cap, int budget, int32_t* __restrict__ keep_idx,
                                                   int keep_stride, int32_t* __restrict__ n_keep,
                                                   uint8_t* __restrict__ keep_mask, int* __restrict__ status_word,
                                                   int b) {
-    extern __shared__ __align__(16) uint32_t smem_u32[];
-    unsigned long long* comp = reinterpret_cast<unsigned long long*>(smem_u32);
+    extern __shared__ __align__(16) uint32_t quota_smem[];
+    unsigned long long* comp = reinterpret_cast<unsigned long long*>(quota_smem);
     uint16_t* cstart = reinterpret_cast<uint16_t*>(comp + P_cap);
     uint16_t* csize = cstart + Nv_cap;
     uint8_t* keepf = reinterpret_cast<uint8_t*>(csize + Nv_cap);
     __shared__ uint32_t warp_sums[kSelWarps];
 
     const int tid = threadIdx.x;
-    int n = vis_len ? vis_len[b] : vis_len_uniform;
+    int n = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
     n = max(0, min(n, Nv_cap));
     score += (int64_t)b * Nv_cap;
     label += (int64_t)b * Nv_cap;
     keep_idx += (int64_t)b * keep_stride;
     if (keep_mask) keep_mask += (int64_t)b * Nv_cap;
 
-    if (select_quota_by_cluster(score, label, n, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
-                                reinterpret_cast<uint8_t*>(smem_u32), warp_sums))
+    if (select_quota_by_cluster<R>(score, label, n, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
+                                   reinterpret_cast<uint8_t*>(quota_smem), warp_sums))
         return;
+    if (R > 1 && cluster_ctarank() != 0) return;
     __syncthreads();
     // more clusters than the per-cluster searches handle, or a short sample with very uneven clusters: sort the
     // composites (label, score key, index)

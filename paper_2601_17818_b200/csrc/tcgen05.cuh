@@ -4,7 +4,7 @@
 
 #include <cuda.h>
 
-#include "internal.cuh"
+#include "async_copy.cuh"
 
 namespace vitcop {
 
@@ -93,20 +93,6 @@ __device__ __forceinline__ bool epi_bar_or(bool pred) {
 // ---- two CTAs of a cluster working on one tile (cta_group::2): the even-ranked CTA (the leader) issues the MMAs for both;
 //      each CTA stages its half of the A rows and of the B rows at the same shared-memory offsets and receives the
 //      accumulator rows of its A half in its own tensor memory.  No load is multicast: what both need is split, not copied.
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-// Address, in the cluster's shared window, of what sits at `addr` of this CTA in the CTA of rank `rank`.
-__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 // (Relaxed: what it announces is that tensor memory has been read, which tcgen05.wait::ld has completed; a release would
 // also wait for the thread's global stores to land.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_in_cluster) {
