@@ -80,6 +80,7 @@ struct KernelArgs {
     GramTiling t;
     long long total_tiles;         // the resident sweep counts its units here
     int extra_units_per_b;         // resident sweep: units of one sample that do not hold a diagonal tile
+    int unit_w;                    // resident sweep: column blocks of a unit, 1 or 2
     unsigned long long wait_ns;    // time limit of every bounded wait
     int expire_roles;              // roles whose waits give up at once: 1 load warp, 2 MMA warp, 4 epilogue warps
     __device__ __forceinline__ unsigned long long limit_of(int role) const {
@@ -728,7 +729,9 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 // ------------------------------------------------------------------------------------------------
 // the resident kernel: density and delta from ONE pass over the Gram tiles (small problems)
 // ------------------------------------------------------------------------------------------------
-// The unit of work is one row block (128 tokens) against two adjacent column blocks: one MMA of N = 256 per
+// The unit of work is one row block (128 tokens) against two adjacent column blocks -- against one where that still leaves
+// no more units than SMs: the epilogue of a unit is most of the kernel's time (one sample of 576 tokens on 15 CTAs instead of
+// 9: 30 -> 24 us).  Two column blocks: one MMA of N = 256 per
 // k-step, the row operand loaded once for both 128 x 128 tiles (a quarter less operand traffic than tile by tile,
 // and the tensor cores run N = 256 at twice the rate of N = 128).  Row block ti owns the column blocks ti .. TI - 1,
 // paired from the diagonal on; the last unit of a row is half empty when their number is odd (the rows of its
@@ -802,11 +805,11 @@ __device__ __forceinline__ bool resident_wait_flags(const unsigned int* fa, cons
 // by sample and row block by row block.
 struct ResidentUnit {
     int b, ti, tj0;        // sample, row block, first column block
-    int width;             // column blocks inside the tensor: 2, or 1 for the half-empty last unit of a row
+    int width;             // column blocks inside the tensor: unit_w, or fewer for the last unit of a row
 };
-__host__ __device__ inline int resident_extra_units(int TI) {
+__host__ __device__ inline int resident_extra_units(int TI, int unit_w) {
     int e = 0;
-    for (int ti = 0; ti < TI; ++ti) e += (TI - ti + 1) / 2 - 1;
+    for (int ti = 0; ti < TI; ++ti) e += (TI - ti + unit_w - 1) / unit_w - 1;
     return e;
 }
 __device__ __forceinline__ ResidentUnit decode_resident_unit(const KernelArgs& k, long long t) {
@@ -823,14 +826,14 @@ __device__ __forceinline__ ResidentUnit decode_resident_unit(const KernelArgs& k
         int r = (int)(x - (long long)u.b * k.extra_units_per_b);
         int ti = 0;
         for (; ti < TI; ++ti) {
-            const int m = (TI - ti + 1) / 2 - 1;           // units of row block ti beyond its first
+            const int m = (TI - ti + k.unit_w - 1) / k.unit_w - 1;             // units of row block ti beyond its first
             if (r < m) break;
             r -= m;
         }
         u.ti = ti;
-        u.tj0 = ti + 2 * (r + 1);
+        u.tj0 = ti + k.unit_w * (r + 1);
     }
-    u.width = u.tj0 + 1 < TI ? 2 : 1;
+    u.width = min(k.unit_w, TI - u.tj0);
     return u;
 }
 
@@ -990,7 +993,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                     if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
                     const uint32_t sa = tiles + stage * S::kStageBytes;
                     // rows of the box past the sample's last token are zero-filled and still count as received
-                    mbar_expect_tx(bar_full + 8 * stage, S::kStageBytes);
+                    mbar_expect_tx(bar_full + 8 * stage, S::kABytes + (uint32_t)k.unit_w * S::kABytes);
                     tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, I0, u.b);
                     tma_load_3d(sa + S::kABytes, &map_b, bar_full + 8 * stage, kb * BK, J0, u.b);
                     issued |= 1u << stage;
@@ -1002,7 +1005,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer: unit s of this CTA -> columns 256 s ..
         if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(BM, kResidentBN);
+            const uint32_t idesc = k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BM);
             const unsigned long long lim = k.limit_of(kRoleMma);
             uint32_t stage = 0, phase = 0;
             uint32_t slot = 0;
@@ -1254,6 +1257,7 @@ int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStre
     }
     k.total_tiles = (long long)args.B * k.t.tiles_per_b;
     k.extra_units_per_b = 0;
+    k.unit_w = 0;
     k.wait_ns = g_wait_ns.load();
     k.expire_roles = g_expire_roles.load();
     if (k.total_tiles <= 0) return VITCOP_OK;
@@ -1279,7 +1283,7 @@ bool gram_fits_resident(int B, int n) {
     }
     if (c != 1) return false;
     const int ti = (n + BM - 1) / BM;
-    const long long units = (long long)B * (ti + resident_extra_units(ti));
+    const long long units = (long long)B * (ti + resident_extra_units(ti, 2));
     return units > 0 && units <= (long long)kResidentUnits * num_sms();
 }
 
@@ -1296,7 +1300,8 @@ int launch_gram_resident(const void* feat, const GramArgs& args, const GramTilin
     k.t = tiling;
     k.g.row0 = 0;
     k.g.row_end = args.n;
-    k.extra_units_per_b = resident_extra_units(k.t.TI);
+    k.unit_w = (long long)args.B * k.t.TI * (k.t.TI + 1) / 2 <= num_sms() ? 1 : 2;
+    k.extra_units_per_b = resident_extra_units(k.t.TI, k.unit_w);
     k.total_tiles = (long long)args.B * (k.t.TI + k.extra_units_per_b);
     k.wait_ns = g_wait_ns.load();
     k.expire_roles = g_expire_roles.load();
@@ -1304,7 +1309,7 @@ int launch_gram_resident(const void* feat, const GramArgs& args, const GramTilin
     if (tiling.BN != BM || k.total_tiles > (long long)kResidentUnits * num_sms()) return VITCOP_ERR_INVALID_ARG;
     CUtensorMap ma, mb;
     if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) ||
-        !make_feat_map(&mb, feat, args.B, args.n, args.D, kResidentBN))
+        !make_feat_map(&mb, feat, args.B, args.n, args.D, BM * k.unit_w))
         return VITCOP_ERR_CUDA;
     const bool euclid = args.metric == 1;
     const bool spatial = args.tau2 >= 0.f && args.pos != nullptr;
