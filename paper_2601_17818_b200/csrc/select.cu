@@ -176,8 +176,8 @@ select_plain_kernel(const float* score, const int32_t* vis_len, int vis_len_unif
 }
 
 // ------------------------------------------------------------------------------------------ quota
-// R CTAs (a thread-block cluster) per sequence.
-template <int R>
+// R CTAs (a thread-block cluster) per sequence, E tokens per thread.
+template <int R, int E>
 __global__ void __launch_bounds__(kSelThreads)
 select_quota_kernel(const float* score, const int32_t* label,
                     const int32_t* vis_len, int vis_len_uniform, int Nv_cap, int P_cap, int budget,
@@ -185,7 +185,7 @@ select_quota_kernel(const float* score, const int32_t* label,
                     uint8_t* __restrict__ keep_mask, int* __restrict__ status_word) {
     grid_dependency_launch_dependents();                  // see select_plain_kernel
     grid_dependency_wait();
-    select_quota_body<R>(score, label, vis_len, vis_len_uniform, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep,
+    select_quota_body<R, E>(score, label, vis_len, vis_len_uniform, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep,
                          keep_mask, status_word, blockIdx.x / R);
 }
 
@@ -221,7 +221,11 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
     // CTAs per sequence: one up to 2048 tokens (the others would be done preparing when the first is done), four, and eight
     // beyond 8192
     const int R = Nv_cap <= 2 * kSelThreads ? 1 : Nv_cap <= 8 * kSelThreads ? 4 : 8;
-    auto kern = R == 1 ? select_quota_kernel<1> : R == 4 ? select_quota_kernel<4> : select_quota_kernel<8>;
+    auto kern = Nv_cap <= kSelThreads ? select_quota_kernel<1, 1>
+                : R == 1              ? select_quota_kernel<1, 2>
+                : Nv_cap <= 4 * kSelThreads ? select_quota_kernel<4, 4>
+                : R == 4              ? select_quota_kernel<4, 8> : select_quota_kernel<8, 16>;
+    static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kSelThreads, "tokens of the longest sample");
     if (smem > 40 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return record_cuda(e);

@@ -75,7 +75,6 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
 //             pass whatever the sizes.  Pairs are unique, so ties need no extra pass; a cluster stops as soon as a
 //             whole histogram bin is wanted, the loop when all clusters have stopped.
 constexpr int kMaxSeg = 1024;
-constexpr int kSegTok = 16;                               // tokens per thread: VITCOP_MAX_VISUAL_TOKENS / kSelThreads
 constexpr uint32_t kSegDone = 0xFFFFFFFFu;
 constexpr int kRankWork = 64;                             // rank search when sum |C_c|^2 <= kRankWork * n per CTA ...
 constexpr int kRankMaxSize = 2048;                        // ... and no searched cluster is larger than this
@@ -128,7 +127,9 @@ struct ClusterSelSmem {
 // Returns false (having written nothing) when the sample has more than kMaxSeg clusters, or sizes that rule out
 // the rank search on a sample too short for the radix search to pay: the caller then sorts.  R CTAs of a thread-block
 // cluster call together with the same arguments and return the same; what the rank search does not take is left to the first.
-template <int R>
+// E: tokens per thread (a CTA that runs once fetches every instruction cold: sixteen unrolled bodies where one is needed cost
+// 576 tokens more than two of nine microseconds).
+template <int R, int E>
 __device__ __forceinline__ bool select_quota_by_cluster(const float* score, const int32_t* label, int n, int budget,
                                                         int32_t* keep_idx, int keep_stride, int32_t* n_keep_b,
                                                         uint8_t* keep_mask, int* status_word, uint8_t* smem,
@@ -159,10 +160,10 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
     }
     __syncthreads();
     // per token: (cluster << 48) | (score key << 16) | low; low = slot inside the cluster first, then the index
-    unsigned long long comp[kSegTok];
+    unsigned long long comp[E];
     uint32_t key_lo = 0xFFFFFFFFu, key_hi = 0u;
 #pragma unroll
-    for (int k = 0; k < kSegTok; ++k) {
+    for (int k = 0; k < E; ++k) {
         const int i = k * kSelThreads + tid;
         comp[k] = 0;
         if (i < n) {
@@ -222,7 +223,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
 
     // ---- cluster sizes (the atomic's return value is the token's slot inside its cluster) and quotas (Eq. 5)
 #pragma unroll
-    for (int k = 0; k < kSegTok; ++k) {
+    for (int k = 0; k < E; ++k) {
         if (k * kSelThreads + tid < n) {
             const uint32_t c = id_of[(uint32_t)(comp[k] >> 48)];
             const uint32_t slot = atomicAdd(&csize[c], 1u);
@@ -274,7 +275,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         // ---- scatter into per-cluster segments; then the thread of segment position p ranks the token stored
         // there.  The lanes of a warp mostly sit in one cluster: equal trip counts and broadcast reads.
 #pragma unroll
-        for (int k = 0; k < kSegTok; ++k) {
+        for (int k = 0; k < E; ++k) {
             const int i = k * kSelThreads + tid;
             if (i < n) {
                 const uint32_t c = (uint32_t)(comp[k] >> 48);
@@ -353,7 +354,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         // (score key, index) value.  The digits above the first bit in which two score keys differ are the same
         // for every token and are skipped.
 #pragma unroll
-        for (int k = 0; k < kSegTok; ++k)
+        for (int k = 0; k < E; ++k)
             comp[k] = (comp[k] & ~0xFFFFull) | (unsigned long long)(k * kSelThreads + tid);
         const int same_bits = __clz((int)(range_lo ^ range_hi));                 // 32 when all scores are equal
         const int shift0 = ((47 - same_bits) / 4) * 4;
@@ -367,7 +368,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
             for (int h = tid; h < (int)n_seg * 16 * copies; h += kSelThreads) hist[h] = 0;
             __syncthreads();
 #pragma unroll
-            for (int k = 0; k < kSegTok; ++k) {
+            for (int k = 0; k < E; ++k) {
                 if (k * kSelThreads + tid < n) {
                     const uint32_t c = (uint32_t)(comp[k] >> 48);
                     if (krem[c] != kSegDone) {
@@ -407,7 +408,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
             if (!__syncthreads_or(open_left)) break;
         }
 #pragma unroll
-        for (int k = 0; k < kSegTok; ++k) {
+        for (int k = 0; k < E; ++k) {
             const int i = k * kSelThreads + tid;
             if (i < n) {
                 const uint32_t c = (uint32_t)(comp[k] >> 48);
@@ -426,7 +427,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
 // ------------------------------------------------------------------------------------------ quota
 // Shared memory: comp[P] (uint64), cstart[n] and csize[n] (uint16, indexed by label value), keep[n] (uint8).
 // Cluster-quota selection of sample b by R whole CTAs (kSelThreads threads each); uses the dynamic shared memory.
-template <int R>
+template <int R, int E>
 __device__ __forceinline__ void select_quota_body(const float* score, const int32_t* label,
                                                   const int32_t* vis_len, int vis_len_uniform,
                                                   int Nv_cap, int P_cap, int budget, int32_t* __restrict__ keep_idx,
@@ -448,7 +449,7 @@ __device__ __forceinline__ void select_quota_body(const float* score, const int3
     keep_idx += (int64_t)b * keep_stride;
     if (keep_mask) keep_mask += (int64_t)b * Nv_cap;
 
-    if (select_quota_by_cluster<R>(score, label, n, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
+    if (select_quota_by_cluster<R, E>(score, label, n, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
                                    reinterpret_cast<uint8_t*>(quota_smem), warp_sums))
         return;
     if (R > 1 && cluster_ctarank() != 0) return;
