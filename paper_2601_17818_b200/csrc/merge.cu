@@ -2,12 +2,10 @@
 // averaged into one representative row.
 //
 // Two kernels on one stream:
-//   merge_plan_kernel   one CTA per sample: gathers the non-elite tokens in token order and sorts them by label with
-//                       a stable radix sort in shared memory, which lays every cluster's members out contiguously
-//                       in ascending token order; the clusters that have members are numbered in ascending label
-//                       order (ordered ballot/popc compaction of the run heads) and the member list goes to the
-//                       workspace
-//   merge_rows_kernel   one CTA per (merged row, sample, 512-byte slice of the hidden row): its four warps stream
+//   merge_plan_kernel   one CTA per sample: lays every cluster's non-elite tokens out contiguously in ascending token order,
+//                       clusters in ascending label order.  Up to 256 clusters by one stable counting pass over dense cluster
+//                       numbers; more by a stable radix sort of the labels in shared memory.
+//   merge_rows_kernel   one CTA per (merged row, sample, 1024-byte slice of the hidden row): its four warps stream
 //                       the members' row slices with 128-bit loads (member r goes to warp r mod 4) and the four
 //                       fp32 partial sums are added in warp order, a fixed order (bit-reproducible).  Only rows
 //                       that are averaged are read.
@@ -21,6 +19,7 @@ namespace {
 constexpr int kPlanThreads = 1024;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr int kRowsThreads = 128;
+constexpr int kRowsPieces = 2;                             // 16-byte pieces of a row per lane
 constexpr int kPlanItems = VITCOP_MAX_VISUAL_TOKENS / kPlanThreads;   // rows of 32 entries a warp walks at most
 constexpr int kDigitBits = 7, kDigits = 1 << kDigitBits;
 static_assert(kDigits * kPlanWarps == 4 * kPlanThreads, "four counters per thread in the scan");
@@ -28,6 +27,16 @@ static_assert(kDigits * kPlanWarps == 4 * kPlanThreads, "four counters per threa
 // the four counters a thread scans (one digit, consecutive warps) both spread over the banks.
 constexpr int kCntStride = kDigits + 2;
 constexpr int kCntEntries = kPlanWarps * kCntStride;
+
+// What merge_rows_kernel needs to know of a merged row; count 0 past the last one.  The headers come in the order in which the
+// rows are to be worked on: those with many members first, as one of them takes several times as long as the others.
+struct __align__(16) MergeHeader {
+    int32_t count, start;                                 // its run in the member list
+    int32_t row, pad;                                     // the merged row
+    uint16_t first[4][4];                                 // member r < 16 at [r % 4][r / 4]
+};
+constexpr int kManyMembers = 32;
+static_assert(sizeof(MergeHeader) == 48, "three 16-byte words");
 
 // Every array of the planner is walked the same way: warp w owns the entries [w * 32 E, (w + 1) * 32 E), E =
 // ceil(count / 1024), and takes them 32 at a time, lane by lane (coalesced, no bank conflicts, and entry order is
@@ -98,11 +107,147 @@ __device__ uint32_t* sort_by_label(uint32_t* a, uint32_t* b, int m, int label_bi
     return a;
 }
 
+// The plan by one stable counting pass, for samples with up to kCountSeg clusters that have non-elite tokens: labels get dense
+// numbers (presence flags, one scan), every warp ranks its tokens inside their cluster (one match per 32 tokens and a counter
+// per (warp, cluster)), one scan over the counters turns ranks into positions.  Returns false, nothing written, when there are
+// more clusters.  E: rows of 32 tokens per warp.  smem: uint32 flags / numbers packed as uint16 [n], counters uint16
+// [32][kCountStride].
+constexpr int kCountSeg = 256, kCountStride = kCountSeg + 2;
+__host__ __device__ constexpr size_t plan_count_bytes(int Nv_cap) {
+    return ((size_t)((Nv_cap + 7) & ~7) + (size_t)kPlanWarps * kCountStride) * sizeof(uint16_t);
+}
+template <int E>
+__device__ __forceinline__ bool plan_by_count(const int32_t* label, const uint8_t* keep_mask, int n, int Mcap,
+                                              int32_t* merged_label, int32_t* merged_count, int32_t* n_merged_b,
+                                              uint16_t* members, MergeHeader* headers, uint16_t* smem, uint32_t* warp_sums) {
+    __shared__ uint16_t seg_start[kCountSeg], seg_slot[kCountSeg];   // slot: place of the cluster's header
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int n_al = (n + 7) & ~7;
+    uint16_t* const id_of = smem;                          // by label: 1 = present, then its dense number
+    uint16_t* const cnt = smem + n_al;
+    for (int i = tid; i < n_al / 8; i += kPlanThreads) reinterpret_cast<uint4*>(id_of)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < kPlanWarps * kCountStride / 2; i += kPlanThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0u;
+    // warp w owns the tokens [w * 32 rows, (w + 1) * 32 rows), row by row: entry order is (warp, row, lane) order
+    const int rows = (n + kPlanThreads - 1) / kPlanThreads;
+    uint32_t lab[E], take = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = (warp * rows + e) * 32 + lane;
+        lab[e] = 0;
+        if (e < rows && i < n) {
+            const uint32_t l = (uint32_t)label[i];
+            lab[e] = l >= (uint32_t)n ? (uint32_t)n - 1 : l;       // out-of-range labels are clamped, never indexed
+            if (!keep_mask[i]) take |= 1u << e;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (take >> e & 1u) id_of[lab[e]] = 1;
+    __syncthreads();
+    uint32_t n_seg;
+    {
+        const int words = (n + kPlanThreads * 8 - 1) / (kPlanThreads * 8);      // of eight labels per thread: 1 or 2
+        uint4 w[2];
+        uint32_t c = 0;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int l = (tid * words + v) * 8;
+            w[v] = v < words && l < n ? *reinterpret_cast<const uint4*>(id_of + l) : make_uint4(0u, 0u, 0u, 0u);
+            c += __popc(w[v].x) + __popc(w[v].y) + __popc(w[v].z) + __popc(w[v].w);
+        }
+        uint32_t next = block_exclusive_sum(c, warp_sums, n_seg);
+        if (n_seg > (uint32_t)kCountSeg) return false;     // uniform
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int l = (tid * words + v) * 8;
+            if (v < words && l < n && (w[v].x | w[v].y | w[v].z | w[v].w)) {
+                uint32_t* f = &w[v].x;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const uint32_t here = (q & 1) ? f[q >> 1] >> 16 : f[q >> 1] & 1u;
+                    if (here) {
+                        if (next < (uint32_t)Mcap) merged_label[next] = l + q;
+                        id_of[l + q] = (uint16_t)next++;
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    uint32_t at[E];                                        // cluster << 16 | rank among the warp's tokens of the cluster
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        at[e] = 0;
+        if (e < rows) {                                    // (uniform)
+            const bool mine = (take >> e & 1u) != 0;
+            const uint32_t c = mine ? id_of[lab[e]] : 0xFFFFu;
+            const uint32_t peers = __match_any_sync(0xffffffffu, c);
+            uint32_t before = 0;
+            if (mine) before = cnt[warp * kCountStride + c];
+            __syncwarp();
+            if (mine && lane == __ffs(peers) - 1) cnt[warp * kCountStride + c] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            at[e] = (c << 16) | (before + __popc(peers & lt));
+        }
+    }
+    __syncthreads();
+    {
+        // counters in (cluster, warp) order -> positions: four threads per cluster, eight warps each
+        const int c = tid >> 2, w0 = (tid & 3) * 8;
+        uint32_t v[8], sum = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            v[q] = cnt[(w0 + q) * kCountStride + c];
+            sum += v[q];
+        }
+        uint32_t m;
+        uint32_t pos = block_exclusive_sum(sum, warp_sums, m);
+        const uint32_t start = __shfl_sync(0xffffffffu, pos, lane & ~3);
+        const uint32_t end = __shfl_sync(0xffffffffu, pos + sum, lane | 3);
+        const bool row = (tid & 3) == 0 && c < (int)n_seg && c < Mcap, many = row && end - start >= (uint32_t)kManyMembers;
+        uint32_t totals;
+        const uint32_t before = block_exclusive_sum((row ? 1u : 0u) | (many ? 0x10000u : 0u), warp_sums, totals);
+        if ((tid & 3) == 0) {
+            seg_start[c] = (uint16_t)start;
+            seg_slot[c] = 0xFFFFu;
+            if (row) {
+                const uint32_t many_before = before >> 16, few_before = (before & 0xFFFFu) - many_before;
+                const uint32_t slot = many ? many_before : (totals >> 16) + few_before;
+                seg_slot[c] = (uint16_t)slot;
+                *reinterpret_cast<int4*>(headers + slot) = make_int4((int)(end - start), (int)start, c, 0);
+                merged_count[c] = (int32_t)(end - start);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            cnt[(w0 + q) * kCountStride + c] = (uint16_t)pos;
+            pos += v[q];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        if (take >> e & 1u) {
+            const uint32_t c = at[e] >> 16, p = cnt[warp * kCountStride + c] + (at[e] & 0xFFFFu), r = p - seg_start[c];
+            const uint16_t i = (uint16_t)((warp * rows + e) * 32 + lane);
+            members[p] = i;
+            if (r < 16 && seg_slot[c] != 0xFFFFu) headers[seg_slot[c]].first[r & 3][r >> 2] = i;
+        }
+    }
+    for (int c = (int)n_seg + tid; c < Mcap; c += kPlanThreads) headers[c].count = 0;
+    if (tid == 0) *n_merged_b = (int32_t)n_seg;
+    return true;
+}
+static_assert(kPlanThreads == 4 * kCountSeg && kPlanWarps == 32, "four threads per cluster, eight warps each");
+
+template <int E>
 __global__ void __launch_bounds__(kPlanThreads)
-merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__ keep_mask,
-                  const int32_t* __restrict__ vis_len, int vis_len_uniform, int Nv_cap, int Mcap,
+merge_plan_kernel(const int32_t* label, const uint8_t* keep_mask,
+                  const int32_t* vis_len, int vis_len_uniform, int Nv_cap, int Mcap,
                   int32_t* __restrict__ merged_label, int32_t* __restrict__ merged_count,
-                  int32_t* __restrict__ n_merged, uint16_t* __restrict__ members, int32_t* __restrict__ starts,
+                  int32_t* __restrict__ n_merged, uint16_t* members, MergeHeader* headers,
                   int* __restrict__ status) {
     extern __shared__ __align__(16) uint32_t smem_items[];   // two item buffers of Nv_cap (rounded up to 4), then the counters
     __shared__ uint32_t warp_sums[32];
@@ -110,7 +255,7 @@ merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (b == 0 && tid == 0) *status = VITCOP_OK;
     const uint32_t lt = (1u << lane) - 1u;
-    int n = vis_len ? vis_len[b] : vis_len_uniform;
+    int n = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
     n = max(0, min(n, Nv_cap));
     const int cap4 = (Nv_cap + 3) & ~3;
     uint32_t* buf0 = smem_items;
@@ -121,18 +266,24 @@ merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__
     merged_label += (size_t)b * Mcap;
     merged_count += (size_t)b * Mcap;
     members += (size_t)b * Nv_cap;
-    starts += (size_t)b * Mcap;
+    headers += (size_t)b * Mcap;
 
-    // ---- the non-elite tokens, in token order: count per warp, one scan, then place.  (Unrolled, unlike the walks
+    if (plan_by_count<E>(label, keep_mask, n, Mcap, merged_label, merged_count, n_merged + b, members, headers,
+                         reinterpret_cast<uint16_t*>(smem_items), warp_sums)) {
+        grid_dependency_launch_dependents();
+        return;
+    }
+    __syncthreads();
+    // ---- more clusters than that.  The non-elite tokens, in token order: count per warp, one scan, then place.  (Unrolled, unlike the walks
     //      over shared memory: all of a thread's global loads are in flight together.)
     uint32_t m;
     {
-        const int E = (n + kPlanThreads - 1) / kPlanThreads;
+        const int rows = (n + kPlanThreads - 1) / kPlanThreads;
         uint32_t it[kPlanItems], take = 0, mine = 0;
 #pragma unroll
         for (int e = 0; e < kPlanItems; ++e) {
-            const int i = (warp * E + e) * 32 + lane;
-            if (e < E && i < n) {
+            const int i = (warp * rows + e) * 32 + lane;
+            if (e < rows && i < n) {
                 uint32_t lab = (uint32_t)label[i];
                 if (lab >= (uint32_t)n) lab = (uint32_t)n - 1;     // out-of-range labels are clamped, never indexed
                 it[e] = (lab << 16) | (uint32_t)i;
@@ -154,11 +305,11 @@ merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__
     const uint32_t* items = sort_by_label(buf0, buf1, (int)m, n > 1 ? 32 - __clz(n - 1) : 0, cnt, warp_sums);
 
     // ---- run heads -> merged rows; run tails close them; the sorted indices are the member list
-    const int E = ((int)m + kPlanThreads - 1) / kPlanThreads;
+    const int rows = ((int)m + kPlanThreads - 1) / kPlanThreads;
     uint32_t wh = 0, wt = 0;
 #pragma unroll 1
-    for (int e = 0; e < E; ++e) {
-        const int p = (warp * E + e) * 32 + lane;
+    for (int e = 0; e < rows; ++e) {
+        const int p = (warp * rows + e) * 32 + lane;
         bool head = false, tail = false;
         if (p < (int)m) {
             const uint32_t c = items[p], lab = c >> 16;
@@ -175,8 +326,8 @@ merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__
     uint32_t hs = before & 0xFFFFu, ts = before >> 16;
     const uint32_t heads = totals & 0xFFFFu;
 #pragma unroll 1
-    for (int e = 0; e < E; ++e) {
-        const int p = (warp * E + e) * 32 + lane;
+    for (int e = 0; e < rows; ++e) {
+        const int p = (warp * rows + e) * 32 + lane;
         bool head = false, tail = false;
         uint32_t lab = 0;
         if (p < (int)m) {
@@ -188,14 +339,24 @@ merge_plan_kernel(const int32_t* __restrict__ label, const uint8_t* __restrict__
         const uint32_t h = hs + __popc(hb & lt), t = ts + __popc(tb & lt);
         if (head && h < (uint32_t)Mcap) {
             merged_label[h] = (int32_t)lab;
-            starts[h] = p;
+            headers[h].start = p;
         }
         if (tail && t < (uint32_t)Mcap) merged_count[t] = p;            // position of the run's last member for now
         hs += __popc(hb);
         ts += __popc(tb);
     }
     __syncthreads();
-    for (int mm = tid; mm < min((int)heads, Mcap); mm += kPlanThreads) merged_count[mm] = merged_count[mm] - starts[mm] + 1;
+    for (int mm = tid; mm < Mcap; mm += kPlanThreads) {
+        int count = 0;
+        if (mm < (int)heads) {
+            const int start = headers[mm].start;
+            count = merged_count[mm] - start + 1;
+            merged_count[mm] = count;
+            for (int r = 0; r < min(count, 16); ++r) headers[mm].first[r & 3][r >> 2] = (uint16_t)(items[start + r] & 0xFFFFu);
+        }
+        headers[mm].count = count;
+        headers[mm].row = mm;
+    }
     if (tid == 0) n_merged[b] = (int32_t)heads;
     grid_dependency_launch_dependents();
 }
@@ -205,67 +366,97 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ void add8(float (&a)[8], const uint4& v) {
-    a[0] += bf16lo(v.x); a[1] += bf16hi(v.x); a[2] += bf16lo(v.y); a[3] += bf16hi(v.y);
-    a[4] += bf16lo(v.z); a[5] += bf16hi(v.z); a[6] += bf16lo(v.w); a[7] += bf16hi(v.w);
+// a[q] += the bf16 pair q of v, both halves with one instruction (each rounded like a scalar addition).
+__device__ __forceinline__ void add8(unsigned long long (&a)[4], const uint4& v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        unsigned long long x;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(w[q] << 16), "r"(w[q] & 0xffff0000u));
+        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a[q]) : "l"(x));
+    }
 }
 
+// A CTA lives for its trips to memory, so the planner leaves, beside the member list, a header per merged row that holds the
+// run and its first sixteen members, four for each warp: one trip leads to the data.  (Run, member list and rows in three
+// dependent trips: 36 us for 121 MB of rows, 4 x 4608 tokens x 4096.)
 __global__ void __launch_bounds__(kRowsThreads)
-merge_rows_kernel(const uint4* __restrict__ hidden, int N, int dh8, int vis_start, int Nv_cap, int Mcap,
-                  const int32_t* __restrict__ merged_count, const int32_t* __restrict__ n_merged,
-                  const uint16_t* __restrict__ members, const int32_t* __restrict__ starts,
+merge_rows_kernel(const uint4* __restrict__ hidden, int B, int N, int dh8, int slices, int vis_start, int Nv_cap, int Mcap,
+                  const MergeHeader* headers, const uint16_t* members,
                   void* __restrict__ merged_bf16, float* __restrict__ merged_f32) {
     constexpr int G = kRowsThreads / 32;                  // warps sharing the members
-    __shared__ float partial[G][32][9];                   // padded against bank conflicts
+    static_assert(G == 4, "a header lists members for four warps");
+    __shared__ unsigned long long partial[kRowsPieces][G][32][5];      // padded against bank conflicts
     grid_dependency_wait();
-    const int m = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    // the three descriptors of the row are independent loads: issue them together
-    const int nm = n_merged[b];
-    const int count = merged_count[(size_t)b * Mcap + m];
-    const int start = starts[(size_t)b * Mcap + m];
-    if (m >= min(nm, Mcap)) return;
-    const uint16_t* mem = members + (size_t)b * Nv_cap + start;
-
-    const int g = tid >> 5, lane = tid & 31;
-    const int piece = blockIdx.z * 32 + lane;             // 16-byte piece of the hidden row this lane owns
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (piece < dh8) {
+    // slices of a row side by side, then the samples, then the rows in header order: the long ones of all samples come first
+    const int tid = threadIdx.x, g = tid >> 5, lane = tid & 31;
+    const int slice = (int)(blockIdx.x % (unsigned)slices), xb = (int)(blockIdx.x / (unsigned)slices);
+    const int b = xb % B, x = xb / B;
+    const MergeHeader* h = headers + (size_t)b * Mcap + x;
+    const int4 run = __ldcg(reinterpret_cast<const int4*>(h));
+    const uint2 four = __ldcg(reinterpret_cast<const uint2*>(h->first[g]));
+    const int count = run.x, m = run.z;
+    if (count == 0) return;                               // no such merged row
+    const uint16_t* mem = members + (size_t)b * Nv_cap + run.y;
+    const int piece = slice * (32 * kRowsPieces) + lane;      // 16-byte pieces of the hidden row this lane owns: + 32 p
+    unsigned long long acc[kRowsPieces][4];               // pairs of fp32 sums
+#pragma unroll
+    for (int p = 0; p < kRowsPieces; ++p)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[p][u] = 0ull;
+    {
         const uint4* src = hidden + ((size_t)b * N + vis_start) * dh8 + piece;
-        int r = g;
-        for (; r + 3 * G < count; r += 4 * G) {
-            uint4 v[4];
+        uint32_t idx[4] = {four.x & 0xFFFFu, four.x >> 16, four.y & 0xFFFFu, four.y >> 16};
+        for (int r = g; r < count; r += 4 * G) {
+            uint4 v[4][kRowsPieces];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = ld_stream(src + (size_t)mem[r + u * G] * dh8);
+            for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) add8(acc, v[u]);
+                for (int p = 0; p < kRowsPieces; ++p)
+                    if (r + u * G < count && piece + 32 * p < dh8) v[u][p] = ld_stream(src + (size_t)idx[u] * dh8 + 32 * p);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)                   // the next four travel with the data
+                if (r + (4 + u) * G < count) idx[u] = __ldcg(mem + r + (4 + u) * G);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int p = 0; p < kRowsPieces; ++p)
+                    if (r + u * G < count && piece + 32 * p < dh8) add8(acc[p], v[u][p]);
         }
-        for (; r < count; r += G) add8(acc, ld_stream(src + (size_t)mem[r] * dh8));
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) partial[g][lane][u] = acc[u];
+    for (int p = 0; p < kRowsPieces; ++p)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) partial[p][g][lane][u] = acc[p][u];
     __syncthreads();
-    const int pl = tid & 31;                              // this thread finishes elements tid / 32, + G, .. of piece pl
-    const int pcol = blockIdx.z * 32 + pl;
-    if (pcol >= dh8) return;
+    // each thread finishes a pair of elements of its lane's pieces: g, so that a row is written in 4- and 8-byte words
 #pragma unroll
-    for (int k = tid >> 5; k < 8; k += G) {
-        float sum = 0.f;
+    for (int p = 0; p < kRowsPieces; ++p) {
+        if (piece + 32 * p >= dh8) break;
+        float sum[2] = {0.f, 0.f};
 #pragma unroll
-        for (int q = 0; q < G; ++q) sum += partial[q][pl][k];   // warp order: fixed
-        sum = sum / (float)count;
-        const size_t o = (((size_t)b * Mcap + m) * dh8 + pcol) * 8 + k;
-        if (merged_f32) merged_f32[o] = sum;
-        if (merged_bf16) static_cast<__nv_bfloat16*>(merged_bf16)[o] = __float2bfloat16_rn(sum);
+        for (int q = 0; q < G; ++q) {                     // warp order: fixed
+            const unsigned long long pair = partial[p][q][lane][g];
+            sum[0] += __uint_as_float((uint32_t)pair);
+            sum[1] += __uint_as_float((uint32_t)(pair >> 32));
+        }
+        sum[0] = sum[0] / (float)count;
+        sum[1] = sum[1] / (float)count;
+        const size_t o = (((size_t)b * Mcap + m) * dh8 + piece + 32 * p) * 8 + 2 * g;
+        if (merged_f32) *reinterpret_cast<float2*>(merged_f32 + o) = make_float2(sum[0], sum[1]);
+        if (merged_bf16)
+            *reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(merged_bf16) + o) =
+                __nv_bfloat162(__float2bfloat16_rn(sum[0]), __float2bfloat16_rn(sum[1]));
     }
 }
 
-// Workspace: status | members uint16 [B, Nv_cap] | starts int32 [B, Mcap]
+// Workspace: status | members uint16 [B, Nv_cap] | headers [B, Mcap]
 struct MergeWs {
-    size_t off_members, off_starts, total;
+    size_t off_members, off_headers, total;
     MergeWs(int B, int Nv_cap, int Mcap) {
         size_t o = kStatusBytes;
         off_members = o; o += align_up((size_t)B * Nv_cap * sizeof(uint16_t), 256);
-        off_starts = o;  o += align_up((size_t)B * Mcap * sizeof(int32_t), 256);
+        off_headers = o; o += align_up((size_t)B * Mcap * sizeof(MergeHeader), 256);
         total = o;
     }
 };
@@ -282,14 +473,18 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
     const MergeWs lay(B, Nv_cap, Mcap);
     char* ws = static_cast<char*>(workspace);
     uint16_t* members = reinterpret_cast<uint16_t*>(ws + lay.off_members);
-    int32_t* starts = reinterpret_cast<int32_t*>(ws + lay.off_starts);
+    MergeHeader* headers = reinterpret_cast<MergeHeader*>(ws + lay.off_headers);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     {
-        const size_t smem = 2 * (size_t)((Nv_cap + 3) & ~3) * sizeof(uint32_t) + (size_t)kCntEntries * sizeof(uint16_t);
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(merge_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const size_t sort_bytes = 2 * (size_t)((Nv_cap + 3) & ~3) * sizeof(uint32_t) + (size_t)kCntEntries * sizeof(uint16_t);
+        const size_t smem = sort_bytes > plan_count_bytes(Nv_cap) ? sort_bytes : plan_count_bytes(Nv_cap);
+        auto kern = Nv_cap <= kPlanThreads       ? merge_plan_kernel<1>
+                    : Nv_cap <= 4 * kPlanThreads ? merge_plan_kernel<4>
+                    : Nv_cap <= 8 * kPlanThreads ? merge_plan_kernel<8> : merge_plan_kernel<16>;
+        if (smem > 40 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return record_cuda(e);
         }
         cudaLaunchConfig_t cfg = {};
@@ -300,23 +495,26 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
         cfg.attrs = attr;
         cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
         KernelTimeScope timed("merge_plan_kernel", stream);
-        int rc = record_cuda(cudaLaunchKernelEx(&cfg, merge_plan_kernel, label, keep_mask, vis_len, vis_len_uniform,
-                                                Nv_cap, Mcap, merged_label, merged_count, n_merged, members, starts,
+        int rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, label, keep_mask, vis_len, vis_len_uniform,
+                                                Nv_cap, Mcap, merged_label, merged_count, n_merged, members, headers,
                                                 static_cast<int*>(workspace)));
         if (rc != VITCOP_OK) return rc;
     }
     if (Mcap <= 0 || Dh <= 0 || (!merged_bf16 && !merged_f32)) return VITCOP_OK;
     const int dh8 = Dh / 8;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(Mcap, B, (dh8 + 31) / 32);
+    const int slices = (dh8 + 32 * kRowsPieces - 1) / (32 * kRowsPieces);
+    const long long ctas = (long long)Mcap * B * slices;
+    if (ctas > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
+    cfg.gridDim = dim3((unsigned)ctas);
     cfg.blockDim = dim3(kRowsThreads);
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
     KernelTimeScope timed("merge_rows_kernel", stream);
-    return record_cuda(cudaLaunchKernelEx(&cfg, merge_rows_kernel, static_cast<const uint4*>(hidden), N, dh8, vis_start,
-                                          Nv_cap, Mcap, (const int32_t*)merged_count, (const int32_t*)n_merged,
-                                          (const uint16_t*)members, (const int32_t*)starts, merged_bf16, merged_f32));
+    return record_cuda(cudaLaunchKernelEx(&cfg, merge_rows_kernel, static_cast<const uint4*>(hidden), B, N, dh8, slices,
+                                          vis_start, Nv_cap, Mcap, (const MergeHeader*)headers, (const uint16_t*)members, merged_bf16,
+                                          merged_f32));
 }
 
 }  // namespace vitcop
