@@ -262,7 +262,7 @@ int vitcop_select(const float* score, const int32_t* label, int B, const int32_t
         if (rc != VITCOP_OK) return rc;
     }
     return launch_select(score, label, B, vis_len, vis_len_uniform, Nv_cap, p->mode, p->largest ? 1 : 0, p->budget,
-                         keep_idx, keep_stride, n_keep, keep_mask, status, s, false, in_kernel ? status : nullptr);
+                         keep_idx, keep_stride, n_keep, keep_mask, status, s, in_kernel, in_kernel ? status : nullptr);
 }
 
 static int check_compact_args(const void* hidden, const void* K, const void* V, int B, int H, int N, int d, int Dh,
@@ -301,7 +301,7 @@ int vitcop_compact_kv(const void* hidden, const void* K, const void* V, int B, i
     if (rc != VITCOP_OK) return rc;
     return launch_compact(hidden, K, V, B, H, N, d, Dh, seq_len, vis_start, vis_len, vis_len_uniform, keep_idx,
                           keep_stride, n_keep, hidden_out, K_out, V_out, Ncap, kept_pos, out_len,
-                          static_cast<cudaStream_t>(stream), false);
+                          static_cast<cudaStream_t>(stream), /*early=*/false);
 }
 
 int vitcop_prune_step(const void* hidden, const void* K, const void* V, int B, int H, int N, int d, int Dh,

@@ -55,7 +55,9 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
 int launch_compact(const void* hidden, const void* K, const void* V, int B, int H, int N, int d, int Dh,
                    const int32_t* seq_len, int vis_start, const int32_t* vis_len, int vis_len_uniform,
                    const int32_t* keep_idx, int keep_stride, const int32_t* n_keep, void* hidden_out, void* K_out,
-                   void* V_out, int Ncap, int32_t* kept_pos, int32_t* out_len, cudaStream_t stream, bool pdl);
+                   void* V_out, int Ncap, int32_t* kept_pos, int32_t* out_len, cudaStream_t stream, bool early);
+// (`early`: the tensors are inputs of a whole call whose first kernel has waited for everything queued before it, so rows that
+// do not depend on the selection may be copied while the kernels in front are still running.)
 
 size_t filter_workspace_bytes(int B, int n, int D);
 // Leading bytes of the filter workspace that must be zero when launch_filter starts (status block and flags).
