@@ -60,13 +60,15 @@ struct SweepArgs {
     float tau2;                 // tau^2; < 0: no spatial test
     const float* w;             // [B, n] per-token factors of the distance, as in GramArgs
     const float* a;
-    const float* rho;           // [B, n]
+    float* rho;                 // [B, n]
     const float* pos;           // [B, n, 2] or nullptr
     const float4* bbox;         // [B, TI] bounding boxes of the 128-token blocks' positions, or nullptr
     float* part;                // [B, slots, n_pad] rho partials
     float* gram;                // [B, tiles_per_b, 256 x 256] Gram values
     float* blk_min;             // [B, n_pad, n_blk]: entry (t, k) = smallest d^2 between token t and the other tokens of
                                 // block k (32 k ..), +inf where the blocks lie beyond the spatial radius
+    float4* tok;                // [B, n_pad] what a pair needs of a token: (w or, for euclid, a; rho; position).  Tokens past
+                                // the sample's last one, to the end of its block of 32, have density 0
     uint32_t* blk_rho;          // [B, n_blk] bits of the largest density in a block of 32 tokens
     int32_t* left;              // tokens (b n + i) that one warp's share of the search did not settle, and their number
     int32_t* n_left;

@@ -31,26 +31,37 @@ namespace {
 // fetch the entries, all of them in one trip to memory, and the sums are taken from shared memory.  (One thread per token
 // walking its list paid a trip for every sixteen entries.)
 // blk_rho[b,k]: bits of the largest density among the tokens of block k (densities are not negative, their bit patterns order
-// like the values).
+// like the values).  tok[b,i]: what the search needs of a token, in one 16-byte load.
 constexpr int kRhoThreads = 256;
 constexpr int kRhoOneByOne = 64;
 constexpr int kRhoEntries = 3 * VITCOP_MAX_VISUAL_TOKENS / kSweepTile;       // longest list
 __global__ void __launch_bounds__(kRhoThreads)
-rho_reduce_kernel(const float* part, int n, SweepTiling t, float* __restrict__ rho,
-                  float* __restrict__ rho_user, uint32_t* __restrict__ blk_rho, int32_t* __restrict__ n_left) {
+rho_reduce_kernel(const __grid_constant__ SweepArgs g, int metric, float* __restrict__ rho_user) {
     constexpr int kWarps = kRhoThreads / 32;
     __shared__ float entry[kRhoEntries][kBlk];
     __shared__ float parts[4][kBlk];
     grid_dependency_launch_dependents();
     grid_dependency_wait();
+    const SweepTiling& t = g.t;
+    const int n = g.n;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int blk = blockIdx.x, b = blockIdx.y, i = blk * kBlk + lane;
-    if (blk == 0 && b == 0 && threadIdx.x == 0) *n_left = 0;         // for the search behind this kernel
+    const size_t at = (size_t)b * n + i;
+    float4 tok = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (warp == 0 && i < n) {
+        tok.x = __ldcg((metric == 1 ? g.a : g.w) + at);
+        if (g.pos && g.tau2 >= 0.f) {
+            const float2 p = *reinterpret_cast<const float2*>(g.pos + 2 * at);
+            tok.z = p.x;
+            tok.w = p.y;
+        }
+    }
+    if (blk == 0 && b == 0 && threadIdx.x == 0) *g.n_left = 0;       // for the search behind this kernel
     const int own = blk * kBlk / kGramBM, tile = own / 2;
     const int rows = t.T - tile;                           // entries on the row side, then min(TI, 2 (tile + 1)) more
     const int entries = rows + min(t.TI, 2 * (tile + 1));
     if (i < n) {
-        const float* p = part + (size_t)b * t.slots() * t.n_pad + i;
+        const float* p = g.part + (size_t)b * t.slots() * t.n_pad + i;
         auto slot = [&](int k) { return __ldcg(p + (size_t)k * t.n_pad); };
 #pragma unroll 6
         for (int e = warp; e < entries; e += kWarps) {
@@ -80,11 +91,13 @@ rho_reduce_kernel(const float* part, int n, SweepTiling t, float* __restrict__ r
     float s = parts[0][lane];
     for (int q = 1; q < nparts; ++q) s += parts[q][lane];
     if (i < n) {
-        rho[(size_t)b * n + i] = s;
-        if (rho_user) rho_user[(size_t)b * n + i] = s;
+        g.rho[at] = s;
+        if (rho_user) rho_user[at] = s;
+        tok.y = s;
     }
+    g.tok[(size_t)b * t.n_pad + i] = tok;
     const uint32_t m = __reduce_max_sync(0xffffffffu, i < n ? __float_as_uint(s) : 0u);
-    if (lane == 0) blk_rho[(size_t)b * t.n_blk() + blk] = m;
+    if (lane == 0) g.blk_rho[(size_t)b * t.n_blk() + blk] = m;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -359,11 +372,11 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
 // ------------------------------------------------------------------------------------------------
 // Workspace of the filter: status block | row-block flags [B, ceil(n / 128)] | w | a | rho | best |
 // rho partials [B, slots, n_pad] (sized for either sweep) | bounding boxes of the row blocks' positions | and, for
-// problems too large for the one-kernel sweep, of one group of samples: count and list of the search's leftovers, block densities, block minima, Gram values of
+// problems too large for the one-kernel sweep, of one group of samples: count and list of the search's leftovers, the tokens as the search reads them, block densities, block minima, Gram values of
 // the density sweep (4 bytes per pair of the symmetric half, tile padding included).  The status block and the
 // flags are zeroed at the start of every call.  Words of the status block: 0 status, 2 grid barrier.
 struct FilterWs {
-    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_left, off_blk_rho, off_blk_min, off_gram, total;
+    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_left, off_tok, off_blk_rho, off_blk_min, off_gram, total;
     FilterWs(int B, int n) {
         size_t o = kStatusBytes;
         const size_t bn = (size_t)B * n;
@@ -375,11 +388,12 @@ struct FilterWs {
         const GramTiling t = make_gram_tiling(n, 128);           // (two slots per block: never fewer than the density sweep's)
         off_part = o; o += align_up((size_t)B * t.slots() * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
-        off_left = off_blk_rho = off_blk_min = off_gram = o;
+        off_left = off_tok = off_blk_rho = off_blk_min = off_gram = o;
         if (B > 0 && n > 0 && !gram_fits_resident(B, n)) {
             const SweepTiling s = make_sweep_tiling(n);
             const size_t group = (size_t)sweep_group_samples(B, n);
             o += align_up((group * n + 1) * 4, 256);
+            off_tok = o;     o += align_up(group * s.n_pad * sizeof(float4), 256);
             off_blk_rho = o; o += align_up(group * s.n_blk() * 4, 256);
             off_blk_min = o; o += align_up(group * s.n_blk() * s.n_pad * 4, 256);
             off_gram = o;    o += align_up(group * s.tiles_per_b * kSweepTileFloats * 4, 256);
@@ -473,6 +487,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             s.part = part + (size_t)b0 * tiling.slots() * tiling.n_pad;
             s.n_left = reinterpret_cast<int32_t*>(ws + l.off_left);
             s.left = s.n_left + 1;
+            s.tok = reinterpret_cast<float4*>(ws + l.off_tok);
             s.blk_rho = reinterpret_cast<uint32_t*>(ws + l.off_blk_rho);
             s.blk_min = reinterpret_cast<float*>(ws + l.off_blk_min);
             s.gram = reinterpret_cast<float*>(ws + l.off_gram);
@@ -485,8 +500,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
                 cudaLaunchAttribute attr[1];
                 pdl_config(cfg, attr, dim3((n + kBlk - 1) / kBlk, s.B), dim3(kRhoThreads), 0, stream, true);
                 KernelTimeScope timed("rho_reduce_kernel", stream);
-                rc = record_cuda(cudaLaunchKernelEx(&cfg, rho_reduce_kernel, (const float*)s.part, n, tiling, rho + at,
-                                                    rho_user ? rho_user + at : nullptr, s.blk_rho, s.n_left));
+                rc = record_cuda(cudaLaunchKernelEx(&cfg, rho_reduce_kernel, s, (int)p.metric, rho_user ? rho_user + at : nullptr));
                 if (rc != VITCOP_OK) return rc;
             }
             rc = launch_nearest_denser(s, p.metric, stream, true);

@@ -2,18 +2,21 @@
 // density sweep left behind (density.cuh): every Gram value of the symmetric half, and per (token, block of 32 tokens) the
 // smallest squared distance.
 //
-// A block can hold a token's answer only if its minimum is not above the best denser token found so far.  One warp per token:
-// every lane keeps the two smallest minima among its blocks (block % 32 = lane) and the warp looks into the blocks in
-// ascending order, two at a time (lane = token of the block: the Gram value, the factors, the density and the spatial test).
-// For nine tokens in ten two or three rounds are enough: their nearest neighbours include a denser token (half of all tokens need one
-// block).  The few tokens that are the densest of their surroundings may have to look into dozens of blocks; these are listed
-// and left to a second kernel, in which several warps share out a token's blocks, passing over those without a denser
-// token (largest density of the block): a warp alone would hold up everything behind it.  What is skipped could not have
+// A block can hold a token's answer only if it has a denser token (largest density of the block) and its minimum is not above
+// the best denser token found so far.  One warp per token: every lane keeps the two smallest minima among its blocks
+// (block % 32 = lane) and the warp looks into the blocks in ascending order, two at a time (lane = token of the block: the
+// Gram value and one 16-byte record with factor, density and position).  For nine tokens in ten a few rounds are enough: their
+// nearest neighbours include a denser token (half of all tokens need one block).  The few tokens that are the densest of
+// their surroundings may have to look into dozens of blocks; these are listed and left to a second kernel, in which
+// several warps share out a token's blocks: a warp alone would hold up everything behind it.  What is skipped could not have
 // changed the minimum, and d^2 is recomputed from the stored value with the arithmetic of the sweep (and of the one-kernel
 // sweep), so the result has the same bits as a full pass over the pairs.
 //
-// Both kernels are bound by the latency of their dependent trips to memory (minima, blocks, blocks again), hence few registers
-// and as many warps as fit.
+// Both kernels are bound by instruction issue (0.73 and 0.57 per cycle; the data sits in L2), so a lane carries its own best pair
+// from block to block and the warp exchanges only the bound; the place of a value is one add and one select away from the
+// token's.  Measured on 8 x 2880 tokens, caches warm: 19.7 -> 15.1 us and 18.3 -> 13.9 us against a warp-wide minimum and ballot
+// per block and four separate loads per token.  Passing over blocks without a denser token in the first kernel too: 6 us less on
+// 4 x 4096 tokens.  Four rounds instead of three: 1 us less there, 20 us more on 2 x 16384 tokens.
 #include "density.cuh"
 
 namespace vitcop {
@@ -23,83 +26,74 @@ constexpr int kNdThreads = 256, kNdWarps = kNdThreads / 32;
 constexpr int kNdRounds = 3;                               // rounds of two blocks that a warp does for its own token
 constexpr int kNdAhead = 4;                                // blocks a warp of the second kernel looks into at a time
 constexpr uint32_t kInfBits = 0x7f800000u;
-// A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, i.e. a
-// bound up to 2^-14 too low.
+// A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, above it
+// one bit that marks a stand-in; i.e. a bound up to 2^-13 too low.
 constexpr uint32_t kBlkMask = VITCOP_MAX_VISUAL_TOKENS / kBlk - 1;
+constexpr uint32_t kStandIn = kBlkMask + 1, kKeyMask = kStandIn | kBlkMask;
 static_assert((kBlkMask & (kBlkMask + 1)) == 0 && kBlkMask < (1u << 10), "block numbers fit the low bits of a key");
+static_assert((size_t)(VITCOP_MAX_VISUAL_TOKENS / kSweepTile) * (VITCOP_MAX_VISUAL_TOKENS / kSweepTile + 1) / 2 * kSweepTileFloats <
+                  (1u << 31), "a sample's Gram values are indexed with 32 bits");
 
-// One sample as the search sees it.
+// One token's search as one lane sees it: the lane stands for one token of every block that the warp looks into, and keeps the
+// nearest denser one it has met (bits of d^2, block; none: kInfBits).
 template <int METRIC, bool SPATIAL>
-struct Sample {
-    const float *rho, *w, *a, *gram, *minima;
-    const float2* pos;
-    const uint32_t* top;                                   // largest density of every block
-    int n, nb, row;                                        // tokens, blocks that hold tokens, minima per token
+struct Search {
+    const float* gram;                                     // of the sample
+    const float4* tok;                                     // of the sample, from this lane on
+    int i, lane;
+    float4 t;                                              // (factor, density, position) of the token
+    float rho_next;                                        // the next density above the token's
     float tau2;
-    __device__ __forceinline__ Sample(const SweepArgs& g, int b) {
-        const size_t bo = (size_t)b * g.n;
-        rho = g.rho + bo;
-        w = g.w + bo;
-        a = g.a + bo;
-        pos = SPATIAL ? reinterpret_cast<const float2*>(g.pos) + bo : nullptr;
+    uint32_t base_col, base_row;                           // this lane's value of block (k, own) is at base_col + k * kRowStep ..
+    uint32_t best = kInfBits;
+    int best_blk = 0;
+    static constexpr uint32_t kRowStep = kSweepBlks * kBlk * kBlk;             // block (k, own) to block (k + 1, own)
+    __device__ __forceinline__ Search(const SweepArgs& g, int b, int i_, int lane_) : i(i_), lane(lane_), tau2(g.tau2) {
         gram = g.gram + (size_t)b * g.t.tiles_per_b * kSweepTileFloats;
-        row = g.t.n_blk();
-        minima = g.blk_min + (size_t)b * g.t.n_pad * row;
-        top = g.blk_rho + (size_t)b * row;
-        n = g.n;
-        nb = (n + kBlk - 1) / kBlk;
-        tau2 = g.tau2;
+        tok = g.tok + (size_t)b * g.t.n_pad;
+        t = tok[i];
+        tok += lane;
+        rho_next = __uint_as_float(__float_as_uint(t.y) + 1u);
+        const int own = i / kBlk, ri = i % kBlk;
+        base_col = (uint32_t)gram_block_offset(0, own) + (uint32_t)gram_elem_offset(lane, ri);
+        base_row = (uint32_t)own * kRowStep + (uint32_t)gram_elem_offset(ri, lane);
     }
-    struct Token {
-        int i;
-        float rho, w, a;
-        float2 pos;
+    struct Pair {                                          // of the pair (i, 32 blk + lane)
+        float gram;
+        float4 t;
     };
-    __device__ __forceinline__ Token token(int i) const {
-        Token t;
-        t.i = i;
-        t.rho = rho[i];
-        t.w = w[i];
-        t.a = METRIC == 1 ? a[i] : 1.f;
-        t.pos = SPATIAL ? pos[i] : make_float2(0.f, 0.f);
-        return t;
-    }
-    struct Pair {                                          // what a lane needs of the pair (i, 32 blk + lane)
-        float gram, w, rho, a;
-        float2 pos;
-    };
-    __device__ __forceinline__ Pair fetch(int i, int blk, int lane) const {
+    // (in front of the token: a column of block (blk, own), whose rows follow one another tile after tile)
+    __device__ __forceinline__ bool below(int blk) const { return blk * kBlk + lane < i; }
+    __device__ __forceinline__ Pair fetch(int blk) const {
+        const uint32_t tj = (uint32_t)blk / kSweepBlks;
+        const uint32_t row = base_row + tj * (tj + 1) / 2 * (uint32_t)kSweepTileFloats + (uint32_t)blk % kSweepBlks * (kBlk * kBlk);
         Pair p;
-        const int j = min(blk * kBlk + lane, n - 1), own = i / kBlk, ri = i % kBlk;
-        // the pair's lower index is its row (inside the own block: in either order)
-        const bool below = blk < own || (blk == own && lane < ri);
-        const int r = below ? lane : ri, c = below ? ri : lane;
-        p.gram = gram[gram_block_offset(min(blk, own), max(blk, own)) + gram_elem_offset(r, c)];
-        p.w = w[j];
-        p.rho = rho[j];
-        p.a = METRIC == 1 ? a[j] : 1.f;
-        p.pos = SPATIAL ? pos[j] : make_float2(0.f, 0.f);
+        p.gram = gram[below(blk) ? base_col + (uint32_t)blk * kRowStep : row];
+        p.t = tok[blk * kBlk];
         return p;
     }
-    // Folds the block's nearest denser token into `best` (packed as SweepArgs::best; uniform over the warp).
-    __device__ __forceinline__ void finish(const Token& t, const Pair& p, int blk, int lane, unsigned long long& best) const {
-        const int j = blk * kBlk + lane;
+    __device__ __forceinline__ void look(const Pair& p, int blk) {
+        const bool lower = below(blk);                     // this lane's token has the lower index
         // d^2 = a_i + a_j - 2 (g w_col) w_row, row the lower index: the operations and their order as in the sweep
-        const float w_row = t.i < j ? t.w : p.w, w_col = t.i < j ? p.w : t.w;
-        const float d2 = fmaxf(fmaf(p.gram * w_col, -2.f * w_row, METRIC == 0 ? 2.f : t.a + p.a), 0.f);
-        bool usable = j < n && (p.rho > t.rho || (p.rho == t.rho && j < t.i));     // denser: (rho desc, index asc)
+        float d2;
+        if (METRIC == 0) d2 = fmaf(p.gram * (lower ? t.x : p.t.x), -2.f * (lower ? p.t.x : t.x), 2.f);
+        else d2 = fmaf(p.gram, -2.f, t.x + p.t.x);
+        bool usable = p.t.y >= (lower ? t.y : rho_next);   // denser: (rho desc, index asc)
         if (SPATIAL) {
-            const float dx = p.pos.x - t.pos.x, dy = p.pos.y - t.pos.y;
+            const float dx = p.t.z - t.z, dy = p.t.w - t.w;
             usable = usable && fmaf(dx, dx, dy * dy) <= tau2;
         }
-        const uint32_t key = usable ? __float_as_uint(d2) : kInfBits;
-        const uint32_t m = __reduce_min_sync(0xffffffffu, key);
-        if (m < kInfBits) {                                // lowest index among the block's nearest
-            const uint32_t who = __ballot_sync(0xffffffffu, key == m);
-            const unsigned long long cand =
-                ((unsigned long long)m << 32) | (unsigned long long)(uint32_t)(blk * kBlk + __ffs(who) - 1);
-            best = cand < best ? cand : best;
+        const uint32_t key = __float_as_uint(fmaxf(d2, 0.f));
+        if (usable && (key < best || (key == best && blk < best_blk))) {
+            best = key;
+            best_blk = blk;
         }
+    }
+    // uniform over the warp: the smallest d^2 so far, and all of it packed as SweepArgs::best
+    __device__ __forceinline__ uint32_t bound() const { return __reduce_min_sync(0xffffffffu, best); }
+    __device__ __forceinline__ unsigned long long packed(uint32_t bound) const {
+        const uint32_t j = __reduce_min_sync(0xffffffffu, best == bound ? (uint32_t)(best_blk * kBlk + lane) : ~0u);
+        return bound < kInfBits ? ((unsigned long long)bound << 32) | j : ~0ull;       // (the lowest index among the nearest)
     }
 };
 
@@ -112,61 +106,56 @@ nearest_denser_kernel(const __grid_constant__ SweepArgs g) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.y, i = blockIdx.x * kNdWarps + warp;
     if (i >= g.n) return;                                  // (uniform)
-    const Sample<METRIC, SPATIAL> s(g, b);
-    const float* const row = s.minima + (size_t)i * s.row;
-    const auto t = s.token(i);
+    const int nb = (g.n + kBlk - 1) / kBlk, n_blk = g.t.n_blk();
+    const float* const row = g.blk_min + ((size_t)b * g.t.n_pad + i) * n_blk;
+    const uint32_t* const top = g.blk_rho + (size_t)b * n_blk;       // largest density of every block
+    Search<METRIC, SPATIAL> s(g, b, i, lane);
     uint32_t m1 = kInfBits, m2 = kInfBits;                 // this lane's two smallest keys
-    for (int k0 = lane; k0 < s.nb; k0 += 128) {
-        uint32_t v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = k0 + u * 32 < s.nb ? __float_as_uint(row[k0 + u * 32]) : kInfBits;
+    for (int k0 = lane; k0 < nb; k0 += 128) {
+        uint32_t v[4], dens[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const uint32_t key = v[u] >= kInfBits ? kInfBits : ((v[u] & ~kBlkMask) | (uint32_t)(k0 + u * 32));
+            v[u] = k0 + u * 32 < nb ? __float_as_uint(__ldcg(row + k0 + u * 32)) : kInfBits;
+            dens[u] = k0 + u * 32 < nb ? top[k0 + u * 32] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t key = v[u] >= kInfBits || dens[u] < __float_as_uint(s.t.y) ? kInfBits : ((v[u] & ~kKeyMask) | (uint32_t)(k0 + u * 32));
             m2 = min(m2, max(m1, key));
             m1 = min(m1, key);
         }
     }
-    const bool more = lane + 64 < s.nb;                    // this lane has blocks beyond the two it remembers
-    int taken = 0;                                         // blocks of this lane looked into
-    unsigned long long best = ~0ull;
-    // The smallest key left, or kInfBits if no block can hold a token below `best` any more.  A lane whose two blocks are
-    // taken stands for the rest of its blocks with the larger key (`known` false).
-    auto next = [&](bool& known) {
-        const uint32_t least = __reduce_min_sync(0xffffffffu, m1);
-        known = true;
-        if (least >= kInfBits || (least & ~kBlkMask) > (uint32_t)(best >> 32)) return kInfBits;
-        const bool mine = m1 == least;                     // (keys are distinct but for a lane's stand-in)
-        known = !__any_sync(0xffffffffu, mine && taken == 2);
-        if (known && mine) {
-            ++taken;
-            m1 = (taken == 2 && !more) ? kInfBits : m2;
+    // A lane whose two blocks are taken stands for the rest of its blocks, if it has any, with the larger key.
+    const uint32_t rest = lane + 64 < nb ? kStandIn : kInfBits;
+    uint32_t bound = kInfBits, least = __reduce_min_sync(0xffffffffu, m1);
+    auto can = [&](uint32_t key) { return key < kInfBits && (key & ~kKeyMask) <= bound; };       // may hold a nearer token
+    auto take = [&]() {                                    // `least` is looked into; the next one
+        if (m1 == least) {                                 // (keys are distinct)
+            m1 = m2;
+            m2 |= rest;
         }
-        return least;
+        least = __reduce_min_sync(0xffffffffu, m1);
     };
-    bool open = true;
 #pragma unroll 1
-    for (int round = 0; round < kNdRounds; ++round) {
-        bool known0, known1 = false;
-        const uint32_t k0 = next(known0);
-        open = k0 < kInfBits;
-        if (!open || !known0) break;
-        const uint32_t k1 = next(known1);
-        const int b0 = (int)(k0 & kBlkMask), b1 = (int)(k1 & kBlkMask);
-        const auto p0 = s.fetch(i, b0, lane);
-        const bool two = k1 < kInfBits && known1;          // (uniform)
+    for (int round = 0; round < kNdRounds && can(least) && !(least & kStandIn); ++round) {
+        const int b0 = (int)(least & kBlkMask);
+        const auto p0 = s.fetch(b0);
+        take();
+        const bool two = can(least) && !(least & kStandIn);
+        const int b1 = (int)(least & kBlkMask);
         auto p1 = p0;
-        if (two) p1 = s.fetch(i, b1, lane);
-        s.finish(t, p0, b0, lane, best);
-        if (two) s.finish(t, p1, b1, lane, best);
+        if (two) {
+            p1 = s.fetch(b1);
+            take();
+        }
+        s.look(p0, b0);
+        if (two) s.look(p1, b1);
+        bound = s.bound();
     }
-    if (open) {
-        const uint32_t least = __reduce_min_sync(0xffffffffu, m1);
-        open = least < kInfBits && (least & ~kBlkMask) <= (uint32_t)(best >> 32);
-    }
+    const unsigned long long best = s.packed(bound);
     if (lane == 0) {
         g.best[(size_t)b * g.n + i] = best;
-        if (open) g.left[atomicAdd(g.n_left, 1)] = b * g.n + i;
+        if (can(least)) g.left[atomicAdd(g.n_left, 1)] = b * g.n + i;
     }
 }
 
@@ -178,28 +167,30 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
     grid_dependency_launch_dependents();
     grid_dependency_wait();
     const int lane = threadIdx.x & 31;
+    const int nb = (g.n + kBlk - 1) / kBlk, n_blk = g.t.n_blk();
     const long long items = (long long)*g.n_left * slices;
     for (long long q = (long long)blockIdx.x * kNdWarps + (threadIdx.x >> 5); q < items; q += (long long)gridDim.x * kNdWarps) {
         const int at = g.left[q / slices], slice = (int)(q % slices), b = at / g.n, i = at - b * g.n;
-        const Sample<METRIC, SPATIAL> s(g, b);
-        const auto t = s.token(i);
+        const float* const row = g.blk_min + ((size_t)b * g.t.n_pad + i) * n_blk;
+        const uint32_t* const top = g.blk_rho + (size_t)b * n_blk;   // largest density of every block
+        Search<METRIC, SPATIAL> s(g, b, i, lane);
         const unsigned long long known = __ldcg(g.best + at);      // (other warps may be lowering it: a stale one is only looser)
         unsigned long long best = known;
         // Can block k, with minimum `lo`, hold a token below `best`?  (An equal distance at a lower index would win.)
         auto can = [&](uint32_t lo, int k) {
             return lo < kInfBits && (((unsigned long long)lo << 32) | (unsigned long long)(uint32_t)(k * kBlk)) < best;
         };
-        for (int k0 = slice; k0 < s.nb; k0 += 32 * slices) {
+        for (int k0 = slice; k0 < nb; k0 += 32 * slices) {
             const int k = k0 + lane * slices;
-            uint32_t lo = kInfBits, top = 0u;
-            if (k < s.nb) {
-                top = s.top[k];
-                lo = __float_as_uint(s.minima[(size_t)i * s.row + k]);
+            uint32_t lo = kInfBits, dens = 0u;
+            if (k < nb) {
+                dens = top[k];
+                lo = __float_as_uint(__ldcg(row + k));
             }
-            if (top < __float_as_uint(t.rho)) lo = kInfBits;
+            if (dens < __float_as_uint(s.t.y)) lo = kInfBits;
             uint32_t todo = __ballot_sync(0xffffffffu, can(lo, k));
             while (todo) {
-                typename Sample<METRIC, SPATIAL>::Pair p[kNdAhead];
+                typename Search<METRIC, SPATIAL>::Pair p[kNdAhead];
                 int blk[kNdAhead];
                 int cnt = 0;
 #pragma unroll
@@ -207,13 +198,15 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
                     if (todo) {
                         blk[u] = k0 + (__ffs(todo) - 1) * slices;
                         todo &= todo - 1;
-                        p[u] = s.fetch(i, blk[u], lane);
+                        p[u] = s.fetch(blk[u]);
                         cnt = u + 1;
                     }
                 }
 #pragma unroll
                 for (int u = 0; u < kNdAhead; ++u)
-                    if (u < cnt) s.finish(t, p[u], blk[u], lane, best);
+                    if (u < cnt) s.look(p[u], blk[u]);
+                const unsigned long long found = s.packed(s.bound());
+                best = found < best ? found : best;
                 todo &= __ballot_sync(0xffffffffu, can(lo, k));
             }
         }
@@ -225,7 +218,7 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
 
 int launch_nearest_denser(const SweepArgs& args, int metric, cudaStream_t stream, bool pdl) {
     if (args.B <= 0 || args.n <= 0) return VITCOP_OK;
-    if (!args.gram || !args.blk_min || !args.blk_rho || !args.best || !args.left || !args.n_left) return VITCOP_ERR_INVALID_ARG;
+    if (!args.gram || !args.blk_min || !args.blk_rho || !args.tok || !args.best || !args.left || !args.n_left) return VITCOP_ERR_INVALID_ARG;
     const bool spatial = args.tau2 >= 0.f && args.pos != nullptr;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((args.n + kNdWarps - 1) / kNdWarps), (unsigned)args.B);
