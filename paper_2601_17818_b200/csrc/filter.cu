@@ -370,17 +370,18 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-// Workspace of the filter: status block | row-block flags [B, ceil(n / 128)] | w | a | rho | best |
+// Workspace of the filter: status block | for the one-kernel sweep the tokens' published factors [B, n] | w | a | rho | best |
 // rho partials [B, slots, n_pad] (sized for either sweep) | bounding boxes of the row blocks' positions | and, for
 // problems too large for the one-kernel sweep, of one group of samples: count and list of the search's leftovers, the tokens as the search reads them, block densities, block minima, Gram values of
 // the density sweep (4 bytes per pair of the symmetric half, tile padding included).  The status block and the
-// flags are zeroed at the start of every call.  Words of the status block: 0 status, 2 grid barrier.
+// published factors are zeroed at the start of every call.  Words of the status block: 0 status, 2 grid barrier.
 struct FilterWs {
-    size_t off_flags, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_left, off_tok, off_blk_rho, off_blk_min, off_gram, total;
+    size_t off_ready, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_left, off_tok, off_blk_rho, off_blk_min, off_gram, total;
     FilterWs(int B, int n) {
         size_t o = kStatusBytes;
         const size_t bn = (size_t)B * n;
-        off_flags = o; o += align_up((size_t)B * ((n + kGramBM - 1) / kGramBM) * 4, 256);
+        const bool resident = gram_fits_resident(B, n);
+        off_ready = o; o += resident ? align_up(bn * 4, 256) : 0;
         off_w = o;    o += align_up(bn * 4, 256);
         off_a = o;    o += align_up(bn * 4, 256);
         off_rho = o;  o += align_up(bn * 4, 256);
@@ -389,7 +390,7 @@ struct FilterWs {
         off_part = o; o += align_up((size_t)B * t.slots() * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
         off_left = off_tok = off_blk_rho = off_blk_min = off_gram = o;
-        if (B > 0 && n > 0 && !gram_fits_resident(B, n)) {
+        if (B > 0 && n > 0 && !resident) {
             const SweepTiling s = make_sweep_tiling(n);
             const size_t group = (size_t)sweep_group_samples(B, n);
             o += align_up((group * n + 1) * 4, 256);
@@ -456,7 +457,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
         g.rho_out = rho;
         g.rho_user = rho_user;
         g.grid_sync = reinterpret_cast<unsigned int*>(ws) + 2;       // zeroed with the status word at the start of the call
-        g.diag_ready = reinterpret_cast<unsigned int*>(ws + l.off_flags);
+        g.ready = reinterpret_cast<uint32_t*>(ws + l.off_ready);
         if (knorm && gram_resident_takes_knorm(knorm->H, knorm->d)) {
             // The sweep's two idle warps take the K-norm of the first samples, about as many as they finish while
             // the epilogue warps work on the accumulators; the other samples follow beside vic_finalize_kernel.

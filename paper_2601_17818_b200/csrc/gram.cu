@@ -187,6 +187,39 @@ struct EpiSmem {
         rowy = rowx + BM;
     }
 };
+// A token's factor travels from the diagonal tile's CTA to the others as one word, bits + 1 (0: not there yet), so that value
+// and flag arrive in one trip.  (Behind a flag per row block, i.e. stores, fence, flag, poll, fence, loads: 3.9 us from the
+// accumulator of the diagonal tile to the factors in every other CTA, instead of 2.0.)
+__device__ __forceinline__ void publish_factor(uint32_t* p, float f) {
+    const uint32_t v = __float_as_uint(f) + 1u;
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v ? v : 0x80000000u) : "memory");     // (a NaN stays one)
+}
+// Bounded; gives up (sets the abort flag, returns false) when the limit is over or another role has given up.
+__device__ __forceinline__ bool wait_factor(const uint32_t* p, float& f, volatile int* abort_flag, unsigned long long limit_ns) {
+    auto load = [&]() {
+        uint32_t v;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        return v;
+    };
+    uint32_t v = load();
+    bool ok = true;
+    if (v == 0u) {
+        unsigned long long t0;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+        while ((v = load()) == 0u) {
+            unsigned long long now;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+            if (limit_ns == 0ull || now - t0 > limit_ns || *abort_flag) {
+                *abort_flag = 1;
+                ok = false;
+                break;
+            }
+        }
+    }
+    f = __uint_as_float(v - 1u);
+    return ok;
+}
+
 struct EpiCall {
     int b, ti, tj;                 // sample, row tile, column tile
     uint32_t tmem_tile;            // TMEM address (lane 0) of the tile's first accumulator column
@@ -235,8 +268,15 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
             const int ce = it, j = J0 + ce;
             const bool cv = j < g.n;
             // (L2 loads: another CTA may have written these factors after this SM last cached their line)
-            colw[ce] = cv ? __ldcg(g.w + bo + j) : 0.f;
-            if (METRIC == 1) cola[ce] = cv ? __ldcg(g.a + bo + j) : 0.f;
+            if (MODE == GRAM_RHO) {
+                float f = 0.f;
+                if (cv) ok = wait_factor(g.ready + bo + j, f, call.abort_flag, call.limit_ns) && ok;
+                colw[ce] = METRIC == 0 ? f : cv ? 1.f : 0.f;
+                if (METRIC == 1) cola[ce] = f;
+            } else {
+                colw[ce] = cv ? __ldcg(g.w + bo + j) : 0.f;
+                if (METRIC == 1) cola[ce] = cv ? __ldcg(g.a + bo + j) : 0.f;
+            }
         } else if (it < 2 * BN) {
             if (MODE == GRAM_DELTA) {
                 const int ce = it - BN, j = J0 + ce;
@@ -261,8 +301,15 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
         } else if (it < 2 * BN + BM) {
             const int r = it - 2 * BN, ir = I0 + r;
             const bool rv = SYM ? (ir < g.n) : (ir < g.row_end);
-            sm.roww[r] = rv ? __ldcg(g.w + bo + ir) : 0.f;
-            if (METRIC == 1) sm.rowa[r] = rv ? __ldcg(g.a + bo + ir) : 0.f;
+            if (MODE == GRAM_RHO) {
+                float f = 0.f;
+                if (rv) ok = wait_factor(g.ready + bo + ir, f, call.abort_flag, call.limit_ns) && ok;
+                sm.roww[r] = METRIC == 0 ? f : rv ? 1.f : 0.f;
+                if (METRIC == 1) sm.rowa[r] = f;
+            } else {
+                sm.roww[r] = rv ? __ldcg(g.w + bo + ir) : 0.f;
+                if (METRIC == 1) sm.rowa[r] = rv ? __ldcg(g.a + bo + ir) : 0.f;
+            }
         } else if (MODE == GRAM_DELTA) {
             const int r = it - 2 * BN - BM, ir = I0 + r;
             float rr = 0.f;
@@ -338,7 +385,9 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                     // The squared norm comes from the same tensor-core arithmetic as every g_ij, so the
                     // rounding of the accumulation cancels in s_ij = g_ij / sqrt(g_ii g_jj) where it
                     // matters: near-duplicates (s -> 1, d^2 = 2 - 2 s -> 0); exact duplicates give s = 1.
-                    g.w_out[bo + i] = METRIC == 0 ? (gii > 0.f ? 1.0f / sqrtf(gii) : 0.f) : 1.f;
+                    const float wi = METRIC == 0 ? (gii > 0.f ? 1.0f / sqrtf(gii) : 0.f) : 1.f;
+                    if (g.ready) publish_factor(g.ready + bo + i, METRIC == 0 ? wi : gii);
+                    g.w_out[bo + i] = wi;
                     g.a_out[bo + i] = METRIC == 0 ? 1.f : gii;
                     if (g.best) g.best[bo + i] = ~0ull;
                 }
@@ -739,13 +788,13 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 // kResidentUnits units and keeps their accumulators in tensor memory (2 x 256 of the 512 columns).  Units that
 // start with a diagonal tile are numbered first, so that these accumulators are the first to complete.
 // Phases of the epilogue warps, which treat a unit as two tiles of 128 x 128:
-//   0. the diagonal tiles yield g_ii -> per-token normalisation factors, published behind one flag per row block
-//   1. density epilogue of every tile (after the flags of its row and column block) -> rho partials;
+//   0. the diagonal tiles yield g_ii -> per-token normalisation factors, published token by token
+//   1. density epilogue of every tile (when the factors of its row and column block are there) -> rho partials;
 //      grid-wide barrier
 //   2. delta epilogue of every tile, re-reading the accumulators; rho of the tile's rows and columns is summed
 //      from the partials on the way (the diagonal tiles publish it)
-// The grid (at most one CTA per SM) is launched cooperatively, so all CTAs are resident together; flags and barrier
-// are words in global memory with bounded waits.  No wait can form a cycle: a flag is raised by a CTA that has
+// The grid (at most one CTA per SM) is launched cooperatively, so all CTAs are resident together; factors and barrier
+// are words in global memory with bounded waits.  No wait can form a cycle: a factor is published by a CTA that has
 // waited for nothing but its own tensor-core work.
 // The load warp and the MMA warp are idle once the CTA's last MMA is issued, and so are, a little later, the
 // operand buffers and -- for the rest of the kernel, which is arithmetic on the accumulators -- the memory system:
@@ -762,41 +811,17 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
 }
 
 // Barrier over all CTAs of the grid, called by the epilogue threads.  Returns true when the grid must give up.
-// One thread speaks for the CTA: the CTA barrier orders every epilogue thread's writes before that thread's fence
-// (and its fence before their later reads), so the other threads need none of their own.
+// One thread speaks for the CTA: the CTA barrier orders every epilogue thread's writes before that thread's release
+// (and its acquire before their later reads), so the other threads need none of their own.
 __device__ __forceinline__ bool resident_grid_barrier(unsigned int* counter, volatile int* abort_flag, bool aborted,
                                                       unsigned long long limit_ns) {
     epi_bar_sync<kResidentEpiThreads>();
     if (threadIdx.x == 64 && !aborted) {
-        __threadfence();
-        atomicAdd(counter, 1u);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
         const unsigned long long t0 = global_ns();
         while (ld_acquire_u32(counter) < gridDim.x) {
             if (limit_ns == 0ull || global_ns() - t0 > limit_ns) { *abort_flag = 1; break; }
         }
-        __threadfence();
-    }
-    return epi_bar_or<kResidentEpiThreads>(aborted || *abort_flag != 0);
-}
-
-// Raises a flag once every epilogue thread's global writes are visible device-wide.
-__device__ __forceinline__ void resident_publish(unsigned int* flag) {
-    epi_bar_sync<kResidentEpiThreads>();
-    if (threadIdx.x == 64) {
-        __threadfence();
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flag), "r"(1u) : "memory");
-    }
-}
-
-// Waits (bounded) until both flags are up.  Returns true when the grid must give up.
-__device__ __forceinline__ bool resident_wait_flags(const unsigned int* fa, const unsigned int* fb,
-                                                    volatile int* abort_flag, bool aborted, unsigned long long limit_ns) {
-    if (threadIdx.x == 64 && !aborted) {
-        const unsigned long long t0 = global_ns();
-        while (ld_acquire_u32(fa) == 0u || ld_acquire_u32(fb) == 0u) {
-            if (limit_ns == 0ull || global_ns() - t0 > limit_ns) { *abort_flag = 1; break; }
-        }
-        __threadfence();
     }
     return epi_bar_or<kResidentEpiThreads>(aborted || *abort_flag != 0);
 }
@@ -1069,7 +1094,6 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             if (u.ti != u.tj0) continue;                   // uniform over the CTA
             const EpiCall c = tile_call(u, slot, 0, true, false);
             stop = epi_tile<BN, GRAM_DIAG, METRIC, false, NS, 8>(k, sm, c, ok);
-            if (!stop) resident_publish(g.diag_ready + (size_t)u.b * k.t.TI + u.ti);
         }
         // ---- phase 1: density partials, tile by tile as soon as the factors of its row and column block exist
         slot = 0;
@@ -1077,10 +1101,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             const ResidentUnit u = decode_resident_unit(k, t);
             for (int s = 0; s < u.width && !stop; ++s) {
                 const EpiCall c = tile_call(u, slot, s, true, false);
-                if (c.ti != c.tj)
-                    stop = resident_wait_flags(g.diag_ready + (size_t)c.b * k.t.TI + c.ti,
-                                               g.diag_ready + (size_t)c.b * k.t.TI + c.tj, abort_flag, stop, lim);
-                if (!stop) stop = epi_tile<BN, GRAM_RHO, METRIC, false, NS, 8>(k, sm, c, ok);
+                stop = epi_tile<BN, GRAM_RHO, METRIC, false, NS, 8>(k, sm, c, ok);
             }
         }
         stop = resident_grid_barrier(g.grid_sync, abort_flag, stop, lim);

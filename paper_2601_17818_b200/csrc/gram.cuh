@@ -77,7 +77,8 @@ struct GramArgs {
     float* rho_out;             // [B, n] written by the resident sweep (same memory as rho)
     float* rho_user;            // [B, n] optional copy of rho for the caller
     unsigned int* grid_sync;    // zeroed counter for the resident sweep's grid-wide barrier
-    unsigned int* diag_ready;   // zeroed flags [B, ceil(n / 128)] of the resident sweep: factors of a row block written
+    uint32_t* ready;            // resident sweep, zeroed [B, n]: a token's factor (w, or for euclid a) once it is known, as its
+                                // bits + 1
     // Optional K-norm (Eq. 4) for the resident sweep's load and MMA warps to stream once their own work is issued:
     // K bf16 [kn_B, kn_H, kn_N, kn_d] dense, span [kn_vis_start, kn_vis_start + kn_Nv), score [kn_B, kn_Nv].
     // Only shapes gram_resident_takes_knorm accepts.
@@ -120,8 +121,8 @@ bool gram_fits_resident(int B, int n);
 bool gram_resident_takes_knorm(int H, int d);
 
 // One kernel for the norms, Eq. 2 and Eq. 3 on small problems: every CTA keeps the accumulators of its tiles in
-// tensor memory; the diagonal tiles publish the per-token factors of their row block behind a flag that the
-// density epilogues of the other tiles wait for, the grid synchronises once (bounded waits) after the density
+// tensor memory; the diagonal tiles publish the per-token factors, which the density epilogues of the other tiles wait for
+// value by value, the grid synchronises once (bounded waits) after the density
 // partials; the delta epilogue sums the partials it needs itself and re-reads the same accumulators.
 // `tiling` = make_gram_tiling(n, 128).
 int launch_gram_resident(const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream);

@@ -60,7 +60,7 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
 // do not depend on the selection may be copied while the kernels in front are still running.)
 
 size_t filter_workspace_bytes(int B, int n, int D);
-// Leading bytes of the filter workspace that must be zero when launch_filter starts (status block and flags).
+// Leading bytes of the filter workspace that must be zero when launch_filter starts (status block and published factors).
 size_t filter_zeroed_bytes(int B, int n);
 size_t similarity_workspace_bytes(int B, int n, int D);
 int launch_filter(const void* feat, const float* pos, int B, int n, int D, const vitcop_filter_params& p,
