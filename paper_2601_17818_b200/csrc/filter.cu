@@ -387,7 +387,8 @@ struct FilterWs {
         off_rho = o;  o += align_up(bn * 4, 256);
         off_best = o; o += align_up(bn * 8, 256);
         const GramTiling t = make_gram_tiling(n, 128);           // (two slots per block: never fewer than the density sweep's)
-        off_part = o; o += align_up((size_t)B * t.slots() * t.n_pad * 4, 256);
+        const size_t slots = resident && gram_resident_halves(B, n) ? 5 * (size_t)t.TI : (size_t)t.slots();
+        off_part = o; o += align_up((size_t)B * slots * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
         off_left = off_tok = off_blk_rho = off_blk_min = off_gram = o;
         if (B > 0 && n > 0 && !resident) {

@@ -158,6 +158,13 @@ struct GemmSmem {
     static constexpr int kBarBytes = 256;
     static constexpr int kTotal = 1024 /*alignment slack*/ + kTileBytes + kEpiBytes + kBarBytes;
 };
+// The one-kernel sweep's units of 64 columns: the operand memory of GemmSmem<256> in stages of 128 + 64 rows.
+struct HalfUnitSmem {
+    static constexpr int kStageBytes = (BM + 64) * BK * 2;
+    static constexpr int kStages = 8;
+    static constexpr int kEpiBytes = (5 + 4 + 4) * 64 * 4 + (3 + 3 + 5) * BM * 4 + 2 * 16 * BM * 4;
+    static_assert(kStages * kStageBytes <= GemmSmem<256>::kTileBytes, "stages");
+};
 
 constexpr float kInf = __builtin_huge_valf();
 
@@ -168,6 +175,7 @@ struct EpiSmem {
     float *colw, *cola, *colrho, *colx, *coly, *colred, *rowred;
     int *colidx, *rowidx;
     float *roww, *rowa, *rowrho, *rowx, *rowy;
+    float* half;                                                // [2][16][BM], units of 64 columns only
     // Carves the arrays out of GemmSmem<BN>::kEpiBytes bytes at `base`.
     template <int BN>
     __device__ __forceinline__ void carve(uint8_t* base) {
@@ -185,6 +193,7 @@ struct EpiSmem {
         rowrho = rowa + BM;
         rowx = rowrho + BM;
         rowy = rowx + BM;
+        half = rowy + BM;
     }
 };
 // A token's factor travels from the diagonal tile's CTA to the others as one word, bits + 1 (0: not there yet), so that value
@@ -239,6 +248,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
     static_assert(GW == 8 || GW == 32, "group width");
     constexpr bool SYM = MODE == GRAM_RHO || MODE == GRAM_DELTA;
     constexpr bool DIAG = MODE == GRAM_DIAG;
+    constexpr bool HALF = SYM && BN == 64;             // a unit of the one-kernel sweep: half a tile
     constexpr int kEpiThreads = NS * 128;
     constexpr int kSliceCols = BN / NS;
     constexpr int kGroups = kSliceCols / GW;           // column groups per warp, taken one by one in a rolled loop
@@ -262,7 +272,10 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
     //      column rho and position, row factors, row rho and position -- so that all the global loads of the tile
     //      are in flight together: one round trip to L2 instead of one per group.
     const float* part_b = (MODE == GRAM_DELTA && call.rho_from_part)
-                              ? g.part + (size_t)b * k.t.slots() * k.t.n_pad : nullptr;
+                              ? g.part + (size_t)b * (HALF ? 5 * k.t.TI : k.t.slots()) * k.t.n_pad : nullptr;
+    auto sum_rho = [&](int x) {
+        return HALF ? rho_from_half_partials(part_b, k.t, g.n, x) : rho_from_partials(part_b + x, k.t, x);
+    };
     for (int it = e; it < 2 * BN + 2 * BM && !DIAG; it += kEpiThreads) {
         if (it < BN) {
             const int ce = it, j = J0 + ce;
@@ -286,8 +299,8 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                 if (cv) {
                     if (SPATIAL) pj = *reinterpret_cast<const float2*>(g.pos + 2 * (bo + j));
                     if (call.rho_from_part) {
-                        rj = rho_from_partials(part_b + j, k.t, j);
-                        if (ti == tj) {                        // the diagonal tile of a row block publishes its tokens' rho
+                        rj = sum_rho(j);
+                        if (ti == (HALF ? tj / 2 : tj)) {                        // the diagonal tile of a row block publishes its tokens' rho
                             g.rho_out[bo + j] = rj;
                             if (g.rho_user) g.rho_user[bo + j] = rj;
                         }
@@ -316,7 +329,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
             float2 pr = make_float2(0.f, 0.f);
             if (ir < g.n) {
                 if (SPATIAL) pr = *reinterpret_cast<const float2*>(g.pos + 2 * (bo + ir));
-                rr = call.rho_from_part ? rho_from_partials(part_b + ir, k.t, ir) : g.rho[bo + ir];
+                rr = call.rho_from_part ? sum_rho(ir) : g.rho[bo + ir];
             }
             sm.rowrho[r] = rr;
             if (SPATIAL) { sm.rowx[r] = pr.x; sm.rowy[r] = pr.y; }
@@ -372,7 +385,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
             const float4* ca4 = reinterpret_cast<const float4*>(cola + cl0);
             if (MODE == GRAM_DIAG) {
                 // g_ii sits in column rl of row rl
-                if (cl0 == (rl & ~(GW - 1)) && row_valid) {
+                if (J0 + cl0 == I0 + (rl & ~(GW - 1)) && row_valid) {
                     // (selected with explicit selp: left to itself the compiler indexes the array in local
                     // memory, a cold round trip on the path every other tile waits for)
                     float gii = 0.f;
@@ -440,8 +453,13 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                         v[u] = (j > i && j < g.n && row_valid) ? v[u] : 0.f;
                     }
                 }
+                if (HALF && (slice & 1)) {             // the second half of a 32-column sum: added by the warp that holds the first
 #pragma unroll
-                for (int u = 0; u < GW; ++u) racc += v[u];
+                    for (int u = 0; u < GW; ++u) sm.half[((slice >> 1) * 16 + c * GW + u) * BM + rl] = v[u];
+                } else {
+#pragma unroll
+                    for (int u = 0; u < GW; ++u) racc += v[u];
+                }
                 const float cs = column_sums(v, lane);
                 if (lane < GW) colred[quarter * BN + cl0 + lane] = cs;
             } else {  // GRAM_DELTA, Eq. 3
@@ -565,14 +583,25 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
     }
     if (SYM) {
         // ---- combine the four column slices of every row and the four row quarters of every column
-        if (slice > 0) {
+        if (slice > 0 && !(HALF && MODE == GRAM_RHO)) {
             rowred[(slice - 1) * BM + rl] = MODE == GRAM_RHO ? racc : rbest;
             if (MODE == GRAM_DELTA) rowidx[(slice - 1) * BM + rl] = rbest_c;
         }
         epi_bar_sync<kEpiThreads>();
         if (ok) {
             const int slot_base = b * k.t.slots();
-            if (MODE == GRAM_RHO) {
+            if (HALF && MODE == GRAM_RHO) {
+                float* const part = g.part + (size_t)b * 5 * k.t.TI * k.t.n_pad;
+                if (!(slice & 1) && row_valid) {
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) racc += sm.half[((slice >> 1) * 16 + u) * BM + rl];
+                    part[((size_t)(tj / 2) * k.t.n_pad + i) * 4 + (tj & 1) * 2 + (slice >> 1)] = racc;
+                }
+                for (int ce = e; ce < BN; ce += kEpiThreads)
+                    if (J0 + ce < g.n)
+                        part[(size_t)(4 * k.t.TI + ti) * k.t.n_pad + J0 + ce] =
+                            ((colred[ce] + colred[BN + ce]) + colred[2 * BN + ce]) + colred[3 * BN + ce];
+            } else if (MODE == GRAM_RHO) {
                 if (slice == 0 && row_valid) {
 #pragma unroll
                     for (int q = 0; q < NS - 1; ++q) racc += rowred[q * BM + rl];       // fixed order
@@ -778,16 +807,19 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 // ------------------------------------------------------------------------------------------------
 // the resident kernel: density and delta from ONE pass over the Gram tiles (small problems)
 // ------------------------------------------------------------------------------------------------
-// The unit of work is one row block (128 tokens) against two adjacent column blocks -- against one where that still leaves
-// no more units than SMs: the epilogue of a unit is most of the kernel's time (one sample of 576 tokens on 15 CTAs instead of
-// 9: 30 -> 24 us).  Two column blocks: one MMA of N = 256 per
+// The unit of work is one row block (128 tokens) against two adjacent column blocks -- against one, or half of one, where that
+// still leaves no more units than SMs: the epilogue of a unit is most of the kernel's time (one sample of 576 tokens on 9, 15,
+// 25 CTAs: 30, 24, 15 us; the last with the factors' faster way to the other CTAs).  Two column blocks: one MMA of N = 256 per
 // k-step, the row operand loaded once for both 128 x 128 tiles (a quarter less operand traffic than tile by tile,
 // and the tensor cores run N = 256 at twice the rate of N = 128).  Row block ti owns the column blocks ti .. TI - 1,
 // paired from the diagonal on; the last unit of a row is half empty when their number is odd (the rows of its
 // missing column block lie outside the tensor and are zero-filled at no cost in traffic).  A CTA owns at most
 // kResidentUnits units and keeps their accumulators in tensor memory (2 x 256 of the 512 columns).  Units that
 // start with a diagonal tile are numbered first, so that these accumulators are the first to complete.
-// Phases of the epilogue warps, which treat a unit as two tiles of 128 x 128:
+// Half a column block: the sums over 32 columns that the other units form in one warp are handed from the warp with the
+// first 16 to the one with the rest, and the four of a tile are stored side by side and joined by the reader, so that every
+// unit gives the same bits.
+// Phases of the epilogue warps, which treat a unit as two tiles of 128 x 128 (or one of 128 x 64):
 //   0. the diagonal tiles yield g_ii -> per-token normalisation factors, published token by token
 //   1. density epilogue of every tile (when the factors of its row and column block are there) -> rho partials;
 //      grid-wide barrier
@@ -836,6 +868,32 @@ __host__ __device__ inline int resident_extra_units(int TI, int unit_w) {
     int e = 0;
     for (int ti = 0; ti < TI; ++ti) e += (TI - ti + unit_w - 1) / unit_w - 1;
     return e;
+}
+// Units of 64 columns (tj0 counts blocks of 64): block ti owns the column blocks from 2 ti on.
+__host__ __device__ inline int resident_half_units(int TI, int TJ) {
+    int e = 0;
+    for (int ti = 0; ti < TI; ++ti) e += TJ - 2 * ti;
+    return e;
+}
+__device__ __forceinline__ ResidentUnit decode_half_unit(const KernelArgs& k, long long t) {
+    const int TJ = (k.g.n + 63) / 64;
+    const long long n_diag = (long long)k.g.B * TJ;
+    ResidentUnit u;
+    u.width = 1;
+    if (t < n_diag) {
+        u.b = (int)(t / TJ);
+        u.tj0 = (int)(t - (long long)u.b * TJ);
+        u.ti = u.tj0 / 2;
+    } else {
+        const long long x = t - n_diag;
+        u.b = (int)(x / k.extra_units_per_b);
+        int r = (int)(x - (long long)u.b * k.extra_units_per_b);
+        int ti = 0;
+        for (int m = TJ - 2; r >= m; ++ti, m -= 2) r -= m;     // units of row block ti behind its diagonal ones
+        u.ti = ti;
+        u.tj0 = 2 * ti + 2 + r;
+    }
+    return u;
 }
 __device__ __forceinline__ ResidentUnit decode_resident_unit(const KernelArgs& k, long long t) {
     const int TI = k.t.TI;
@@ -954,13 +1012,19 @@ __device__ __forceinline__ void resident_knorm(const GramArgs& g, const uint8_t*
     }
 }
 
-template <int METRIC, bool SPATIAL>
+// BN: columns of the epilogue's tiles: 128, or 64 for units of half a tile.
+template <int METRIC, bool SPATIAL, int BN>
 __global__ void __launch_bounds__(64 + kResidentEpiThreads, 1)
 gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      const KernelArgs k) {
-    constexpr int BN = BM;                                 // the epilogue's tiles
+    constexpr bool HALF = BN == 64;
     constexpr int NS = 4;
     using S = GemmSmem<kResidentBN>;                       // stages of 128 + 256 operand rows
+    constexpr uint32_t kStages = HALF ? HalfUnitSmem::kStages : S::kStages;
+    constexpr uint32_t kStageBytes = HALF ? HalfUnitSmem::kStageBytes : S::kStageBytes;
+    constexpr int kEpiBytes = HALF ? HalfUnitSmem::kEpiBytes : S::kEpiBytes;
+    auto unit_of = [&](long long t) { return HALF ? decode_half_unit(k, t) : decode_resident_unit(k, t); };
+    auto on_diagonal = [](const ResidentUnit& u) { return u.ti == (HALF ? u.tj0 / 2 : u.tj0); };
     const GramArgs& g = k.g;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -968,22 +1032,22 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     uint8_t* gen = smem_raw + (tiles - raw);
     EpiSmem sm;
     sm.template carve<BN>(gen + S::kTileBytes);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + S::kTileBytes + S::kEpiBytes);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + S::kTileBytes + kEpiBytes);
     // barriers: full[kStages], empty[kStages], tmem_full[kResidentUnits], drain, knorm[kKnBuffers]
     const uint32_t bar_full = smem_u32(bars);
-    const uint32_t bar_empty = bar_full + 8 * S::kStages;
-    const uint32_t bar_tfull = bar_empty + 8 * S::kStages;
+    const uint32_t bar_empty = bar_full + 8 * kStages;
+    const uint32_t bar_tfull = bar_empty + 8 * kStages;
     const uint32_t bar_drain = bar_tfull + 8 * kResidentUnits;
     const uint32_t bar_kn = bar_drain + 8;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S::kStages + kResidentUnits + 1 + kKnBuffers);
-    static_assert((2 * S::kStages + kResidentUnits + 1 + kKnBuffers) * 8 + 8 <= S::kBarBytes, "barrier block too small");
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + kResidentUnits + 1 + kKnBuffers);
+    static_assert((2 * kStages + kResidentUnits + 1 + kKnBuffers) * 8 + 8 <= S::kBarBytes, "barrier block too small");
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t kTmemCols = kResidentUnits * kResidentBN;   // 512: the whole tensor memory of the SM
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S::kStages; ++s) {
+        for (uint32_t s = 0; s < kStages; ++s) {
             mbar_init(bar_full + 8 * s, 1);
             mbar_init(bar_empty + 8 * s, 1);
         }
@@ -1012,25 +1076,25 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             for (long long t = blockIdx.x; ok && t < total_units; t += gridDim.x) {
-                const ResidentUnit u = decode_resident_unit(k, t);
-                const int I0 = u.ti * BM, J0 = u.tj0 * BM;
+                const ResidentUnit u = unit_of(t);
+                const int I0 = u.ti * BM, J0 = u.tj0 * BN;
                 for (int kb = 0; kb < KB; ++kb) {
                     if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
-                    const uint32_t sa = tiles + stage * S::kStageBytes;
+                    const uint32_t sa = tiles + stage * kStageBytes;
                     // rows of the box past the sample's last token are zero-filled and still count as received
-                    mbar_expect_tx(bar_full + 8 * stage, S::kABytes + (uint32_t)k.unit_w * S::kABytes);
+                    mbar_expect_tx(bar_full + 8 * stage, HALF ? kStageBytes : S::kABytes + (uint32_t)k.unit_w * S::kABytes);
                     tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, I0, u.b);
                     tma_load_3d(sa + S::kABytes, &map_b, bar_full + 8 * stage, kb * BK, J0, u.b);
                     issued |= 1u << stage;
                     issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
+                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer: unit s of this CTA -> columns 256 s ..
         if (lane == 0) {
-            const uint32_t idesc = k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BM);
+            const uint32_t idesc = !HALF && k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BN);
             const unsigned long long lim = k.limit_of(kRoleMma);
             uint32_t stage = 0, phase = 0;
             uint32_t slot = 0;
@@ -1040,14 +1104,14 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                 for (int kb = 0; kb < KB; ++kb) {
                     if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t sa = tiles + stage * S::kStageBytes;
+                    const uint32_t sa = tiles + stage * kStageBytes;
                     const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + S::kABytes);
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk)
                         tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
                                     (kb > 0 || kk > 0) ? 1u : 0u);
                     tc_commit(bar_empty + 8 * stage);
-                    if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
+                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
                 tc_commit(bar_tfull + 8 * slot);
@@ -1090,15 +1154,15 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         // ---- phase 0: the diagonal tiles give g_ii, hence the per-token factors every other epilogue needs
         uint32_t slot = 0;
         for (long long t = blockIdx.x; t < total_units && !stop; t += gridDim.x, ++slot) {
-            const ResidentUnit u = decode_resident_unit(k, t);
-            if (u.ti != u.tj0) continue;                   // uniform over the CTA
+            const ResidentUnit u = unit_of(t);
+            if (!on_diagonal(u)) continue;                  // uniform over the CTA
             const EpiCall c = tile_call(u, slot, 0, true, false);
             stop = epi_tile<BN, GRAM_DIAG, METRIC, false, NS, 8>(k, sm, c, ok);
         }
         // ---- phase 1: density partials, tile by tile as soon as the factors of its row and column block exist
         slot = 0;
         for (long long t = blockIdx.x; t < total_units && !stop; t += gridDim.x, ++slot) {
-            const ResidentUnit u = decode_resident_unit(k, t);
+            const ResidentUnit u = unit_of(t);
             for (int s = 0; s < u.width && !stop; ++s) {
                 const EpiCall c = tile_call(u, slot, s, true, false);
                 stop = epi_tile<BN, GRAM_RHO, METRIC, false, NS, 8>(k, sm, c, ok);
@@ -1112,7 +1176,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         //      columns from the partials (fixed order: the same bits everywhere)
         slot = 0;
         for (long long t = blockIdx.x; t < total_units && !stop; t += gridDim.x, ++slot) {
-            const ResidentUnit u = decode_resident_unit(k, t);
+            const ResidentUnit u = unit_of(t);
             for (int s = 0; s < u.width && !stop; ++s) {
                 const EpiCall c = tile_call(u, slot, s, false, true);
                 stop = epi_tile<BN, GRAM_DELTA, METRIC, SPATIAL, NS, 8>(k, sm, c, ok);
@@ -1128,7 +1192,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     }
     if (threadIdx.x == 0 && *abort_flag) {
         // (see gram_tc_kernel: unconsumed operand loads must have landed before the CTA goes away)
-        for (int s = 0; s < S::kStages; ++s)
+        for (uint32_t s = 0; s < kStages; ++s)
             if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
         if (g.status) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
     }
@@ -1223,19 +1287,20 @@ int launch_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k
     return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
 }
 
-template <int METRIC, bool SPATIAL>
+template <int METRIC, bool SPATIAL, int BN>
 int launch_resident_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream) {
     using S = GemmSmem<kResidentBN>;
     static std::atomic<unsigned long long> attr_done{0};
-    auto kern = gram_resident_kernel<METRIC, SPATIAL>;
-    const int arc = allow_dynamic_smem(kern, S::kTotal, attr_done);
+    auto kern = gram_resident_kernel<METRIC, SPATIAL, BN>;
+    constexpr int kSmem = S::kTotal + (BN == 64 ? HalfUnitSmem::kEpiBytes - S::kEpiBytes : 0);
+    const int arc = allow_dynamic_smem(kern, kSmem, attr_done);
     if (arc != VITCOP_OK) return arc;
     const long long ctas = (k.total_tiles + kResidentUnits - 1) / kResidentUnits;
     cudaLaunchConfig_t cfg = {};
     // as many CTAs as there are SMs (never fewer than the units need): the shortest chain of units per CTA
     cfg.gridDim = dim3((unsigned)(k.total_tiles < num_sms() ? k.total_tiles : (ctas > num_sms() ? ctas : num_sms())));
     cfg.blockDim = dim3(64 + kResidentEpiThreads);
-    cfg.dynamicSmemBytes = S::kTotal;
+    cfg.dynamicSmemBytes = kSmem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;          // all CTAs resident together: they wait for one another
@@ -1308,6 +1373,14 @@ bool gram_fits_resident(int B, int n) {
     return units > 0 && units <= (long long)kResidentUnits * num_sms();
 }
 
+// Units of 64 columns where that still leaves one unit per SM at most: with more, a CTA's second unit would cost what the
+// shorter units save (a unit's epilogue is most of the kernel's time).  One sample of 576 tokens: 25 CTAs instead of 15,
+// the call 35.9 -> 33.8 us; beyond the line the units of 128 or 256 columns use every SM as well.
+bool gram_resident_halves(int B, int n) {
+    const long long units = resident_half_units((n + BM - 1) / BM, (n + 63) / 64);
+    return (long long)B * units <= num_sms();
+}
+
 bool gram_resident_takes_knorm(int H, int d) {
     // sixteen or more 16-byte pieces per row (the lane layout of the stand-alone kernel's widest variant), and at
     // least one chunk of eight tokens must fit the operand buffers
@@ -1321,22 +1394,33 @@ int launch_gram_resident(const void* feat, const GramArgs& args, const GramTilin
     k.t = tiling;
     k.g.row0 = 0;
     k.g.row_end = args.n;
+    const bool halves = gram_resident_halves(args.B, args.n);
     k.unit_w = (long long)args.B * k.t.TI * (k.t.TI + 1) / 2 <= num_sms() ? 1 : 2;
     k.extra_units_per_b = resident_extra_units(k.t.TI, k.unit_w);
     k.total_tiles = (long long)args.B * (k.t.TI + k.extra_units_per_b);
+    if (halves) {
+        const int TJ = (args.n + 63) / 64, units = resident_half_units(k.t.TI, TJ);
+        k.extra_units_per_b = units - TJ;
+        k.total_tiles = (long long)args.B * units;
+    }
     k.wait_ns = g_wait_ns.load();
     k.expire_roles = g_expire_roles.load();
     if (k.total_tiles <= 0) return VITCOP_OK;
     if (tiling.BN != BM || k.total_tiles > (long long)kResidentUnits * num_sms()) return VITCOP_ERR_INVALID_ARG;
     CUtensorMap ma, mb;
     if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) ||
-        !make_feat_map(&mb, feat, args.B, args.n, args.D, BM * k.unit_w))
+        !make_feat_map(&mb, feat, args.B, args.n, args.D, halves ? 64 : BM * k.unit_w))
         return VITCOP_ERR_CUDA;
     const bool euclid = args.metric == 1;
     const bool spatial = args.tau2 >= 0.f && args.pos != nullptr;
+    if (halves) {
+        if (spatial)
+            return euclid ? launch_resident_one<1, true, 64>(ma, mb, k, stream) : launch_resident_one<0, true, 64>(ma, mb, k, stream);
+        return euclid ? launch_resident_one<1, false, 64>(ma, mb, k, stream) : launch_resident_one<0, false, 64>(ma, mb, k, stream);
+    }
     if (spatial)
-        return euclid ? launch_resident_one<1, true>(ma, mb, k, stream) : launch_resident_one<0, true>(ma, mb, k, stream);
-    return euclid ? launch_resident_one<1, false>(ma, mb, k, stream) : launch_resident_one<0, false>(ma, mb, k, stream);
+        return euclid ? launch_resident_one<1, true, BM>(ma, mb, k, stream) : launch_resident_one<0, true, BM>(ma, mb, k, stream);
+    return euclid ? launch_resident_one<1, false, BM>(ma, mb, k, stream) : launch_resident_one<0, false, BM>(ma, mb, k, stream);
 }
 
 }  // namespace vitcop

@@ -112,6 +112,39 @@ __host__ __device__ inline float rho_from_partials(const float* p, const GramTil
     return s;
 }
 
+// The same sum in the same order where the one-kernel sweep works on units of 64 columns (gram_resident_halves): per sample
+// TI row-side slots of float4 {32-column sums of the tile}, then TI column-side slots.
+__device__ inline float rho_from_half_partials(const float* part_b, const GramTiling& t, int n, int i) {
+    const int ti = i / kGramBM;
+    const float4* const row = reinterpret_cast<const float4*>(part_b) + i;
+    const float* const col = part_b + (size_t)4 * t.TI * t.n_pad + i;
+    constexpr int kCols = 8, kRows = 6;
+    float cv[kCols];                                       // (travels with the first row-side entries)
+#pragma unroll
+    for (int u = 0; u < kCols; ++u) cv[u] = u <= ti ? col[(size_t)u * t.n_pad] : 0.f;
+    float s = 0.f;
+    for (int c = ti; c < t.TI; c += kRows) {
+        float4 v[kRows];
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) v[u] = c + u < t.TI ? row[(size_t)(c + u) * t.n_pad] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            if (c + u >= t.TI) continue;
+            float x = v[u].x + v[u].y;
+            if ((c + u) * kGramBM + kGramBM / 2 < n) x = (x + v[u].z) + v[u].w;        // (else there is no second unit)
+            s += x;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kCols; ++u)
+        if (u <= ti) s += cv[u];
+    for (int u = kCols; u <= ti; ++u) s += col[(size_t)u * t.n_pad];
+    return s;
+}
+
+// True when the one-kernel sweep cuts the problem into units of 64 columns instead of 128 or 256 (gram.cu).
+bool gram_resident_halves(int B, int n);
+
 // True when the whole symmetric sweep of the problem fits the tensor memory of one wave of CTAs (at most two units
 // of one row block against two column blocks per SM): density and delta can then share one pass over the Gram tiles
 // (launch_gram_resident).

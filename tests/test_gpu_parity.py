@@ -491,6 +491,28 @@ def test_filter_sweep_and_search_edges(B, n, metric, tau):
         check_vic_sample(f[b], p[b], metric, d_c, tau, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
 
 
+# The one-kernel sweep in units of 64 columns (few enough of them for one per SM: 148) and, with one sample more, of 128 or 256:
+# ends inside the first and the second half of a tile, one row block and many.  The same bits, whatever the unit.
+@pytest.mark.parametrize("n,metric,tau", [(1, 0, 0.6), (64, 0, 0.6), (65, 1, 0.6), (129, 0, -1.0), (193, 1, -1.0), (576, 0, 0.6),
+                                          (1025, 0, 0.3), (1472, 1, 0.6)])
+def test_filter_small_units(n, metric, tau):
+    blocks = -(-n // 64)
+    units = sum(blocks - 2 * r for r in range(-(-n // 128)))
+    few = 148 // units
+    w = dataclasses.replace(W.workload("tiny"), B=few + 1, D=128, dup_rate=0.3)
+    f = W.make_features(w, n=n, B=few + 1)
+    p = np.ascontiguousarray(np.broadcast_to(W.make_positions(w, n)[:1], (few + 1, n, 2)))
+    d_c = w.d_c if metric == 0 else 12.0
+    nc = max(1, n // 10)
+    g = gpu_filter(f[:few], p[:few], metric, d_c, tau, nc)
+    more = gpu_filter(f, p, metric, d_c, tau, nc)
+    assert g.status == vb.OK and more.status == vb.OK and np.all(g.n_clusters == nc)
+    for key in ("rho", "delta2", "parent", "label"):
+        assert np.array_equal(getattr(g, key), getattr(more, key)[:few]), key
+    check_vic_sample(f[few - 1], p[few - 1], metric, d_c, tau, nc, g.rho[few - 1], g.delta2[few - 1], g.parent[few - 1],
+                     g.label[few - 1])
+
+
 # No token within the spatial radius of another: every token is an orphan, all keys of the centre selection agree in their first
 # word and the densities decide (cuts among more and among fewer tied keys than are ranked by counting, one to several tokens
 # per thread); the surplus orphans join the nearest centre.
