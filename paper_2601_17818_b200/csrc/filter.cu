@@ -386,7 +386,7 @@ struct FilterWs {
         off_a = o;    o += align_up(bn * 4, 256);
         off_rho = o;  o += align_up(bn * 4, 256);
         off_best = o; o += align_up(bn * 8, 256);
-        const GramTiling t = make_gram_tiling(n, 128);           // (two slots per block: never fewer than the density sweep's)
+        const GramTiling t = make_gram_tiling(n);           // (two slots per block: never fewer than the density sweep's)
         const size_t slots = resident && gram_resident_halves(B, n) ? 5 * (size_t)t.TI : (size_t)t.slots();
         off_part = o; o += align_up((size_t)B * slots * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
@@ -468,7 +468,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
                 g.kn_H = knorm->H; g.kn_N = knorm->N; g.kn_d = knorm->d; g.kn_vis_start = knorm->vis_start; g.kn_Nv = knorm->Nv;
             }
         }
-        rc = launch_gram_resident(feat, g, make_gram_tiling(n, 128), stream);
+        rc = launch_gram_resident(feat, g, make_gram_tiling(n), stream);
         if (rc != VITCOP_OK) return rc;
     } else {
         // with a spatial radius, blocks beyond it are neither kept nor looked into (density.cuh: blocks_outside_radius)

@@ -29,10 +29,10 @@ namespace vitcop {
 namespace {
 
 constexpr int BM = kGramBM;
-// Column slices an output tile is cut into for the epilogue; every slice is served by four warps (one per
-// TMEM lane quarter).  The delta sweep's epilogue is the heavier one and gets twice the warps.
-__host__ __device__ constexpr int epi_slices(int mode) { return mode == GRAM_DELTA ? 4 : 2; }
-__host__ __device__ constexpr int gemm_threads(int mode) { return 64 + epi_slices(mode) * 128; }
+// Column slices an output tile of gram_tc_kernel is cut into for the epilogue; every slice is served by four warps (one per
+// TMEM lane quarter).
+constexpr int kEpiSlices = 2;
+constexpr int kGemmThreads = 64 + kEpiSlices * 128;
 
 // ------------------------------------------------------------------------------------------------
 // PTX wrappers
@@ -89,12 +89,8 @@ struct KernelArgs {
 };
 constexpr int kRoleLoad = 1, kRoleMma = 2, kRoleEpi = 4;
 
-template <int BN, bool SYM, bool DIAG = false>
+template <bool DIAG>
 __device__ __forceinline__ void decode_tile(const KernelArgs& k, long long t, int& b, int& ti, int& tj) {
-    if (SYM) {
-        decode_sym_tile(k.t, t, b, ti, tj);
-        return;
-    }
     b = (int)(t / k.t.tiles_per_b);
     const int r = (int)(t - (long long)b * k.t.tiles_per_b);
     if (DIAG) {
@@ -108,40 +104,27 @@ __device__ __forceinline__ void decode_tile(const KernelArgs& k, long long t, in
 // ------------------------------------------------------------------------------------------------
 // warp butterflies: lane L ends up with the reduction over the 32 lanes of element L of the array
 // ------------------------------------------------------------------------------------------------
-template <int HALF, bool MIN>
+template <int HALF>
 __device__ __forceinline__ void butterfly_stage(float* v, bool up) {
 #pragma unroll
     for (int k = 0; k < HALF; ++k) {
         const float keep = up ? v[k + HALF] : v[k];
         const float send = up ? v[k] : v[k + HALF];
         const float recv = __shfl_xor_sync(0xffffffffu, send, HALF);
-        v[k] = MIN ? fminf(keep, recv) : keep + recv;
+        v[k] = keep + recv;
     }
 }
 // Eight columns held by every lane (one row each): afterwards every lane holds the sum over the 32 lanes of column
 // lane & 7, added in a fixed order.
 __device__ __forceinline__ float warp_column_sums8(float (&v)[8], int lane) {
-    butterfly_stage<4, false>(v, (lane & 4) != 0);
-    butterfly_stage<2, false>(v, (lane & 2) != 0);
-    butterfly_stage<1, false>(v, (lane & 1) != 0);
+    butterfly_stage<4>(v, (lane & 4) != 0);
+    butterfly_stage<2>(v, (lane & 2) != 0);
+    butterfly_stage<1>(v, (lane & 1) != 0);
     float s = v[0];
     s += __shfl_xor_sync(0xffffffffu, s, 8);
     s += __shfl_xor_sync(0xffffffffu, s, 16);
     return s;
 }
-__device__ __forceinline__ float column_sums(float (&v)[8], int lane) { return warp_column_sums8(v, lane); }
-template <bool MIN>
-__device__ __forceinline__ float warp_transpose_reduce(float (&v)[32], int lane) {
-    butterfly_stage<16, MIN>(v, (lane & 16) != 0);
-    butterfly_stage<8, MIN>(v, (lane & 8) != 0);
-    butterfly_stage<4, MIN>(v, (lane & 4) != 0);
-    butterfly_stage<2, MIN>(v, (lane & 2) != 0);
-    butterfly_stage<1, MIN>(v, (lane & 1) != 0);
-    return v[0];
-}
-
-__device__ __forceinline__ float column_sums(float (&v)[32], int lane) { return warp_transpose_reduce<false>(v, lane); }
-
 // ------------------------------------------------------------------------------------------------
 // shared memory
 // ------------------------------------------------------------------------------------------------
@@ -173,7 +156,7 @@ constexpr float kInf = __builtin_huge_valf();
 // ------------------------------------------------------------------------------------------------
 struct EpiSmem {
     float *colw, *cola, *colrho, *colx, *coly, *colred, *rowred;
-    int *colidx, *rowidx;
+    int *colidx, *rowidx;                                       // (colidx: the rows that attain colred, as a mask)
     float *roww, *rowa, *rowrho, *rowx, *rowy;
     float* half;                                                // [2][16][BM], units of 64 columns only
     // Carves the arrays out of GemmSmem<BN>::kEpiBytes bytes at `base`.
@@ -234,15 +217,13 @@ struct EpiCall {
     uint32_t tmem_tile;            // TMEM address (lane 0) of the tile's first accumulator column
     uint32_t wait_bar, wait_parity;   // mbarrier that completes when the accumulator is ready (0: it already is)
     uint32_t arrive_bar;           // mbarrier to arrive on once this thread has read the accumulator (0: none)
-    bool rho_from_part;            // GRAM_DELTA: sum rho from the density partials (and publish it from diagonal tiles)
     volatile int* abort_flag;
     unsigned long long limit_ns;   // time limit of the wait for the accumulator
 };
 
 // Returns true when the CTA must give up (a bounded wait expired somewhere).
-// GW: columns a warp takes from the accumulator at a time.  32 unrolls the whole arithmetic of a 32-column chunk
-// (fewest instructions; right where the code is reused tile after tile), 8 keeps it in a short rolled loop (right
-// where every tile is visited once and the instruction cache would otherwise miss all the way).
+// GW: columns a warp takes from the accumulator at a time: 8 in the one-kernel sweep, a short rolled loop, because every tile is
+// visited once and the instruction cache would otherwise miss all the way; 32 for the diagonal and the similarity rows.
 template <int BN, int MODE, int METRIC, bool SPATIAL, int NS, int GW = 32>
 __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm, const EpiCall& call, bool& ok) {
     static_assert(GW == 8 || GW == 32, "group width");
@@ -271,8 +252,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
     // ---- per-column and per-row constants.  One item per thread where the tile allows it -- column factors,
     //      column rho and position, row factors, row rho and position -- so that all the global loads of the tile
     //      are in flight together: one round trip to L2 instead of one per group.
-    const float* part_b = (MODE == GRAM_DELTA && call.rho_from_part)
-                              ? g.part + (size_t)b * (HALF ? 5 * k.t.TI : k.t.slots()) * k.t.n_pad : nullptr;
+    const float* const part_b = g.part + (size_t)b * (HALF ? 5 * k.t.TI : k.t.slots()) * k.t.n_pad;
     auto sum_rho = [&](int x) {
         return HALF ? rho_from_half_partials(part_b, k.t, g.n, x) : rho_from_partials(part_b + x, k.t, x);
     };
@@ -298,14 +278,10 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                 float2 pj = make_float2(0.f, 0.f);
                 if (cv) {
                     if (SPATIAL) pj = *reinterpret_cast<const float2*>(g.pos + 2 * (bo + j));
-                    if (call.rho_from_part) {
-                        rj = sum_rho(j);
-                        if (ti == (HALF ? tj / 2 : tj)) {                        // the diagonal tile of a row block publishes its tokens' rho
-                            g.rho_out[bo + j] = rj;
-                            if (g.rho_user) g.rho_user[bo + j] = rj;
-                        }
-                    } else {
-                        rj = g.rho[bo + j];
+                    rj = sum_rho(j);
+                    if (ti == (HALF ? tj / 2 : tj)) {          // the diagonal tile of a row block publishes its tokens' rho
+                        g.rho_out[bo + j] = rj;
+                        if (g.rho_user) g.rho_user[bo + j] = rj;
                     }
                 }
                 colrho[ce] = rj;
@@ -329,7 +305,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
             float2 pr = make_float2(0.f, 0.f);
             if (ir < g.n) {
                 if (SPATIAL) pr = *reinterpret_cast<const float2*>(g.pos + 2 * (bo + ir));
-                rr = call.rho_from_part ? sum_rho(ir) : g.rho[bo + ir];
+                rr = sum_rho(ir);
             }
             sm.rowrho[r] = rr;
             if (SPATIAL) { sm.rowx[r] = pr.x; sm.rowy[r] = pr.y; }
@@ -353,6 +329,9 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
     if (ok && call.wait_bar) ok = mbar_wait(call.wait_bar, call.wait_parity, call.abort_flag, call.limit_ns);
     ok = __all_sync(0xffffffffu, ok);
 
+    // GRAM_DELTA: the tile-local columns j of this row's pairs i < j < n
+    const int first_c = i + 1 - J0;
+    const uint32_t usable_c = row_valid ? (uint32_t)max(min(BN, g.n - J0) - first_c, 0) : 0u;
     float racc = 0.f;                              // GRAM_RHO: row-side sum
     float rbest = kInf;                            // GRAM_DELTA: row-side minimum and its tile-local column
     int rbest_c = -1;
@@ -383,7 +362,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
             const int cl0 = slice * kSliceCols + c * GW;       // tile-local first column of the group
             const float4* cw4 = reinterpret_cast<const float4*>(colw + cl0);
             const float4* ca4 = reinterpret_cast<const float4*>(cola + cl0);
-            if (MODE == GRAM_DIAG) {
+            if constexpr (MODE == GRAM_DIAG) {
                 // g_ii sits in column rl of row rl
                 if (J0 + cl0 == I0 + (rl & ~(GW - 1)) && row_valid) {
                     // (selected with explicit selp: left to itself the compiler indexes the array in local
@@ -404,7 +383,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                     g.a_out[bo + i] = METRIC == 0 ? 1.f : gii;
                     if (g.best) g.best[bo + i] = ~0ull;
                 }
-            } else if (MODE == GRAM_SIM) {
+            } else if constexpr (MODE == GRAM_SIM) {
                 if (row_valid) {
                     float* o = g.sim_out + ((size_t)b * rows_out + (i - g.row0)) * g.n;
 #pragma unroll
@@ -413,37 +392,24 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                         if (j < g.n) o[j] = METRIC == 0 ? (v[u] * w_i) * colw[cl0 + u] : v[u];
                     }
                 }
-            } else if (MODE == GRAM_RHO) {
+            } else if constexpr (MODE == GRAM_RHO) {
                 // e_ij = exp(-d_ij^2 / d_c^2), Eq. 2
 #pragma unroll
                 for (int q4 = 0; q4 < GW / 4; ++q4) {
                     const float4 cw = cw4[q4];
                     float4 ca = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (METRIC == 1) ca = ca4[q4];
-                    if constexpr (GW == 32) {
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {          // two neighbouring columns at a time
-                            const int u = 4 * q4 + 2 * h;
-                            const unsigned long long cw2 = h ? pack2(cw.z, cw.w) : pack2(cw.x, cw.y);
-                            const unsigned long long ca2 = h ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y);
-                            const unsigned long long x2 = mul2(pack2(v[u], v[u + 1]), cw2);
-                            const unsigned long long base2 = METRIC == 0 ? two2 : add2(ai2, ca2);
-                            const float2 d2 = unpack2(fma2(x2, m2w2, base2));
-                            const float2 arg = unpack2(mul2(pack2(fmaxf(d2.x, 0.f), fmaxf(d2.y, 0.f)), c22));
-                            v[u] = ex2_approx(arg.x);
-                            v[u + 1] = ex2_approx(arg.y);
-                        }
-                    } else {
-                        const float cwv[4] = {cw.x, cw.y, cw.z, cw.w};
-                        const float cav[4] = {ca.x, ca.y, ca.z, ca.w};
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const int u = 4 * q4 + r;
-                            const float x = v[u] * cwv[r];
-                            const float base = METRIC == 0 ? 2.f : a_i + cav[r];
-                            const float d2 = fmaxf(fmaf(x, m2w_i, base), 0.f);
-                            v[u] = ex2_approx(d2 * g.c2);
-                        }
+                    for (int h = 0; h < 2; ++h) {              // two neighbouring columns at a time
+                        const int u = 4 * q4 + 2 * h;
+                        const unsigned long long cw2 = h ? pack2(cw.z, cw.w) : pack2(cw.x, cw.y);
+                        const unsigned long long ca2 = h ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y);
+                        const unsigned long long x2 = mul2(pack2(v[u], v[u + 1]), cw2);
+                        const unsigned long long base2 = METRIC == 0 ? two2 : add2(ai2, ca2);
+                        const float2 d2 = unpack2(fma2(x2, m2w2, base2));
+                        const float2 arg = unpack2(mul2(pack2(fmaxf(d2.x, 0.f), fmaxf(d2.y, 0.f)), c22));
+                        v[u] = ex2_approx(arg.x);
+                        v[u + 1] = ex2_approx(arg.y);
                     }
                 }
                 if (!full) {
@@ -460,7 +426,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
 #pragma unroll
                     for (int u = 0; u < GW; ++u) racc += v[u];
                 }
-                const float cs = column_sums(v, lane);
+                const float cs = warp_column_sums8(v, lane);
                 if (lane < GW) colred[quarter * BN + cl0 + lane] = cs;
             } else {  // GRAM_DELTA, Eq. 3
                 const float4* cr4 = reinterpret_cast<const float4*>(colrho + cl0);
@@ -476,70 +442,54 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
                     if (SPATIAL) { cx = cx4[q4]; cy = cy4[q4]; }
                     const float crv[4] = {cr.x, cr.y, cr.z, cr.w};
                     float d2v[4], s2v[4];              // squared feature distance (unclamped), squared spatial distance
-                    if constexpr (GW == 32) {
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {          // two neighbouring columns at a time
-                            const int u = 4 * q4 + 2 * h;
-                            const unsigned long long cw2 = h ? pack2(cw.z, cw.w) : pack2(cw.x, cw.y);
-                            const unsigned long long ca2 = h ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y);
-                            const unsigned long long x2 = mul2(pack2(v[u], v[u + 1]), cw2);
-                            const unsigned long long base2 = METRIC == 0 ? two2 : add2(ai2, ca2);
-                            const float2 d2 = unpack2(fma2(x2, m2w2, base2));
-                            d2v[2 * h] = d2.x;
-                            d2v[2 * h + 1] = d2.y;
-                            if (SPATIAL) {
-                                const unsigned long long dx2 = add2(h ? pack2(cx.z, cx.w) : pack2(cx.x, cx.y), nxi2);
-                                const unsigned long long dy2 = add2(h ? pack2(cy.z, cy.w) : pack2(cy.x, cy.y), nyi2);
-                                const float2 s2 = unpack2(fma2(dx2, dx2, mul2(dy2, dy2)));
-                                s2v[2 * h] = s2.x;
-                                s2v[2 * h + 1] = s2.y;
-                            }
-                        }
-                    } else {
-                        const float cwv[4] = {cw.x, cw.y, cw.z, cw.w};
-                        const float cav[4] = {ca.x, ca.y, ca.z, ca.w};
-                        const float cxv[4] = {cx.x, cx.y, cx.z, cx.w};
-                        const float cyv[4] = {cy.x, cy.y, cy.z, cy.w};
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const float x = v[4 * q4 + r] * cwv[r];
-                            d2v[r] = fmaf(x, m2w_i, METRIC == 0 ? 2.f : a_i + cav[r]);
-                            if (SPATIAL) {
-                                const float dx = cxv[r] - x_i, dy = cyv[r] - y_i;
-                                s2v[r] = fmaf(dx, dx, dy * dy);
-                            }
+                    for (int h = 0; h < 2; ++h) {              // two neighbouring columns at a time
+                        const int u = 4 * q4 + 2 * h;
+                        const unsigned long long cw2 = h ? pack2(cw.z, cw.w) : pack2(cw.x, cw.y);
+                        const unsigned long long ca2 = h ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y);
+                        const unsigned long long x2 = mul2(pack2(v[u], v[u + 1]), cw2);
+                        const unsigned long long base2 = METRIC == 0 ? two2 : add2(ai2, ca2);
+                        const float2 d2 = unpack2(fma2(x2, m2w2, base2));
+                        d2v[2 * h] = d2.x;
+                        d2v[2 * h + 1] = d2.y;
+                        if (SPATIAL) {
+                            const unsigned long long dx2 = add2(h ? pack2(cx.z, cx.w) : pack2(cx.x, cx.y), nxi2);
+                            const unsigned long long dy2 = add2(h ? pack2(cy.z, cy.w) : pack2(cy.x, cy.y), nyi2);
+                            const float2 s2 = unpack2(fma2(dx2, dx2, mul2(dy2, dy2)));
+                            s2v[2 * h] = s2.x;
+                            s2v[2 * h + 1] = s2.y;
                         }
                     }
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
                         const int u = 4 * q4 + r;
-                        float d2 = fmaxf(d2v[r], 0.f);
-                        bool usable = true;        // the pair may serve as (child, parent) at all
-                        if (SPATIAL) usable = s2v[r] <= g.tau2;
-                        if (!full) {
-                            const int j = J0 + cl0 + u;
-                            usable = usable && j > i && j < g.n && row_valid;
-                        }
-                        if (SPATIAL || !full) d2 = usable ? d2 : kInf;
+                        const float d2 = fmaxf(d2v[r], 0.f);
+                        // the pair may serve as (child, parent) at all (one comparison, & and not &&: the branches a pair took
+                        // before cost the whole call 4 %, on 16 x 576 tokens 64.3 -> 61.9 us)
+                        bool usable = (uint32_t)(cl0 + u - first_c) < usable_c;
+                        if (SPATIAL) usable = usable & (s2v[r] <= g.tau2);
                         // with i < j: "j denser than i" is rho_j > rho_i, "i denser than j" is its complement
                         const bool jd = crv[r] > rho_i;
-                        const float kr = jd ? d2 : kInf;       // j as parent candidate of i (row side)
-                        kc[u] = __float_as_uint(jd ? kInf : d2);   // i as parent candidate of j (column side)
+                        const float kr = (usable & jd) ? d2 : kInf;     // j as parent candidate of i (row side)
+                        kc[u] = __float_as_uint((usable & !jd) ? d2 : kInf);   // i as parent candidate of j (column side)
                         if (kr < rbest) { rbest = kr; rbest_c = cl0 + u; }
                     }
                 }
-                // column side: minimum over this warp's 32 rows and the lowest row that attains it
-                uint32_t my_min = 0x7f800000u, my_rows = 0;
+                // column side: minimum over this warp's 32 rows and the rows that attain it
+                // (one lane stores what all lanes hold: selecting column u in lane u took three more instructions a column)
+                uint32_t m[GW], rows[GW];
 #pragma unroll
                 for (int u = 0; u < GW; ++u) {
-                    const uint32_t m = __reduce_min_sync(0xffffffffu, kc[u]);
-                    const uint32_t rows = __ballot_sync(0xffffffffu, kc[u] == m);
-                    if (lane == u) { my_min = m; my_rows = rows; }
+                    m[u] = __reduce_min_sync(0xffffffffu, kc[u]);
+                    rows[u] = __ballot_sync(0xffffffffu, kc[u] == m[u]);
                 }
-                if (lane < GW) {
-                    colred[quarter * BN + cl0 + lane] = __uint_as_float(my_min);
-                    colidx[quarter * BN + cl0 + lane] =
-                        my_min < 0x7f800000u ? I0 + quarter * 32 + (__ffs(my_rows) - 1) : -1;
+                if (lane == 0) {
+#pragma unroll
+                    for (int u = 0; u < GW; u += 4) {
+                        *reinterpret_cast<uint4*>(colred + quarter * BN + cl0 + u) = make_uint4(m[u], m[u + 1], m[u + 2], m[u + 3]);
+                        *reinterpret_cast<uint4*>(colidx + quarter * BN + cl0 + u) =
+                            make_uint4(rows[u], rows[u + 1], rows[u + 2], rows[u + 3]);
+                    }
                 }
             }
             if constexpr (GW == 8) {
@@ -632,7 +582,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {                                  // ascending rows: ties keep the lower row
                         const float kk = colred[q * BN + ce];
-                        if (kk < bk) { bk = kk; bi = colidx[q * BN + ce]; }
+                        if (kk < bk) { bk = kk; bi = I0 + q * 32 + __ffs(colidx[q * BN + ce]) - 1; }
                     }
                     if (bi >= 0) {
                         const unsigned long long packed =
@@ -650,14 +600,14 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
-template <int BN, int MODE, int METRIC, bool SPATIAL>
-__global__ void __launch_bounds__(gemm_threads(MODE), 1)
+// MODE: GRAM_DIAG or GRAM_SIM.
+template <int BN, int MODE, int METRIC>
+__global__ void __launch_bounds__(kGemmThreads, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const KernelArgs k) {
     using S = GemmSmem<BN>;
-    constexpr bool SYM = MODE == GRAM_RHO || MODE == GRAM_DELTA;
     constexpr bool DIAG = MODE == GRAM_DIAG;            // BN == BM: a diagonal tile multiplies the row block by itself
-    constexpr int NS = epi_slices(MODE);
+    constexpr int NS = kEpiSlices;
     constexpr int kEpiThreads = NS * 128;
     const GramArgs& g = k.g;
     extern __shared__ uint8_t smem_raw[];
@@ -717,7 +667,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             bool ok = true;
             for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
                 int b, ti, tj;
-                decode_tile<BN, SYM, DIAG>(k, t, b, ti, tj);
+                decode_tile<DIAG>(k, t, b, ti, tj);
                 const int I0 = g.row0 + ti * BM, J0 = tj * BN;
                 for (int kb = 0; kb < KB; ++kb) {
                     if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
@@ -775,15 +725,14 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
         for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
             EpiCall c;
-            decode_tile<BN, SYM, DIAG>(k, t, c.b, c.ti, c.tj);
+            decode_tile<DIAG>(k, t, c.b, c.ti, c.tj);
             c.tmem_tile = tmem_base + acc * BN;
             c.wait_bar = bar_tfull + 8 * acc;
             c.wait_parity = acc_phase;
             c.arrive_bar = bar_tempty + 8 * acc;
-            c.rho_from_part = false;
             c.abort_flag = abort_flag;
             c.limit_ns = k.limit_of(kRoleEpi);
-            if (epi_tile<BN, MODE, METRIC, SPATIAL, NS>(k, sm, c, ok)) break;
+            if (epi_tile<BN, MODE, METRIC, false, NS>(k, sm, c, ok)) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }
@@ -1136,7 +1085,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         const unsigned long long lim = k.limit_of(kRoleEpi);
         grid_dependency_wait();
         // tile s (0 or 1) of this CTA's unit number `slot`
-        auto tile_call = [&](const ResidentUnit& u, uint32_t slot, int s, bool wait_mma, bool rho_from_part) {
+        auto tile_call = [&](const ResidentUnit& u, uint32_t slot, int s, bool wait_mma) {
             EpiCall c;
             c.b = u.b;
             c.ti = u.ti;
@@ -1145,7 +1094,6 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             c.wait_bar = wait_mma ? bar_tfull + 8 * slot : 0;
             c.wait_parity = 0;
             c.arrive_bar = 0;
-            c.rho_from_part = rho_from_part;
             c.abort_flag = abort_flag;
             c.limit_ns = lim;
             return c;
@@ -1156,7 +1104,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         for (long long t = blockIdx.x; t < total_units && !stop; t += gridDim.x, ++slot) {
             const ResidentUnit u = unit_of(t);
             if (!on_diagonal(u)) continue;                  // uniform over the CTA
-            const EpiCall c = tile_call(u, slot, 0, true, false);
+            const EpiCall c = tile_call(u, slot, 0, true);
             stop = epi_tile<BN, GRAM_DIAG, METRIC, false, NS, 8>(k, sm, c, ok);
         }
         // ---- phase 1: density partials, tile by tile as soon as the factors of its row and column block exist
@@ -1164,7 +1112,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         for (long long t = blockIdx.x; t < total_units && !stop; t += gridDim.x, ++slot) {
             const ResidentUnit u = unit_of(t);
             for (int s = 0; s < u.width && !stop; ++s) {
-                const EpiCall c = tile_call(u, slot, s, true, false);
+                const EpiCall c = tile_call(u, slot, s, true);
                 stop = epi_tile<BN, GRAM_RHO, METRIC, false, NS, 8>(k, sm, c, ok);
             }
         }
@@ -1178,7 +1126,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         for (long long t = blockIdx.x; t < total_units && !stop; t += gridDim.x, ++slot) {
             const ResidentUnit u = unit_of(t);
             for (int s = 0; s < u.width && !stop; ++s) {
-                const EpiCall c = tile_call(u, slot, s, false, true);
+                const EpiCall c = tile_call(u, slot, s, false);
                 stop = epi_tile<BN, GRAM_DELTA, METRIC, SPATIAL, NS, 8>(k, sm, c, ok);
             }
         }
@@ -1266,16 +1214,16 @@ int allow_dynamic_smem(Kernel kern, int bytes, std::atomic<unsigned long long>& 
     return VITCOP_OK;
 }
 
-template <int BN, int MODE, int METRIC, bool SPATIAL>
+template <int BN, int MODE, int METRIC>
 int launch_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream, bool pdl) {
     using S = GemmSmem<BN>;
     static std::atomic<unsigned long long> attr_done{0};
-    auto kern = gram_tc_kernel<BN, MODE, METRIC, SPATIAL>;
+    auto kern = gram_tc_kernel<BN, MODE, METRIC>;
     const int arc = allow_dynamic_smem(kern, S::kTotal, attr_done);
     if (arc != VITCOP_OK) return arc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(k.total_tiles < num_sms() ? k.total_tiles : num_sms()));
-    cfg.blockDim = dim3(gemm_threads(MODE));
+    cfg.blockDim = dim3(kGemmThreads);
     cfg.dynamicSmemBytes = S::kTotal;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1331,7 +1279,7 @@ int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStre
     if (mode != GRAM_DIAG && mode != GRAM_SIM) return VITCOP_ERR_INVALID_ARG;
     KernelArgs k;
     k.g = args;
-    k.t = make_gram_tiling(args.n, BM);
+    k.t = make_gram_tiling(args.n);
     if (mode == GRAM_SIM) {
         // plain rectangle: rows [row0, row_end) x all columns
         k.t.TI = (args.row_end - args.row0 + BM - 1) / BM;
@@ -1352,10 +1300,10 @@ int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStre
         return VITCOP_ERR_CUDA;
     const bool euclid = args.metric == 1;
     if (mode == GRAM_DIAG)
-        return euclid ? launch_one<BM, GRAM_DIAG, 1, false>(ma, mb, k, stream, pdl)
-                      : launch_one<BM, GRAM_DIAG, 0, false>(ma, mb, k, stream, pdl);
-    return euclid ? launch_one<BM, GRAM_SIM, 1, false>(ma, mb, k, stream, pdl)
-                  : launch_one<BM, GRAM_SIM, 0, false>(ma, mb, k, stream, pdl);
+        return euclid ? launch_one<BM, GRAM_DIAG, 1>(ma, mb, k, stream, pdl)
+                      : launch_one<BM, GRAM_DIAG, 0>(ma, mb, k, stream, pdl);
+    return euclid ? launch_one<BM, GRAM_SIM, 1>(ma, mb, k, stream, pdl)
+                  : launch_one<BM, GRAM_SIM, 0>(ma, mb, k, stream, pdl);
 }
 
 bool gram_fits_resident(int B, int n) {
@@ -1406,7 +1354,7 @@ int launch_gram_resident(const void* feat, const GramArgs& args, const GramTilin
     k.wait_ns = g_wait_ns.load();
     k.expire_roles = g_expire_roles.load();
     if (k.total_tiles <= 0) return VITCOP_OK;
-    if (tiling.BN != BM || k.total_tiles > (long long)kResidentUnits * num_sms()) return VITCOP_ERR_INVALID_ARG;
+    if (k.total_tiles > (long long)kResidentUnits * num_sms()) return VITCOP_ERR_INVALID_ARG;
     CUtensorMap ma, mb;
     if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) ||
         !make_feat_map(&mb, feat, args.B, args.n, args.D, halves ? 64 : BM * k.unit_w))

@@ -11,45 +11,20 @@ constexpr int kGramBM = 128;   // rows of an output tile (UMMA M)
 // similarities.  GRAM_RHO and GRAM_DELTA are phases of the one-kernel sweep.
 enum GramMode { GRAM_RHO = 0, GRAM_DELTA = 1, GRAM_SIM = 2, GRAM_DIAG = 3 };
 
-// Tiling of the one-kernel sweep.  Only tiles that hold a pair (i, j) with i < j are
-// visited; a pair contributes to its row token i ("row side") and to its column token j ("column side").
-// Tiles are numbered column-tile major inside one sample: column tile tj holds the row tiles
-// 0 .. min(TI, R * (tj + 1)) - 1 with R = BN / kGramBM, and starts at offset R * tj * (tj + 1) / 2.
+// Tiling in row and column blocks of 128 tokens.
 struct GramTiling {
-    int BN;            // columns of an output tile: 128 or 256
-    int R;             // BN / kGramBM
-    int TI, TJ;        // row tiles, column tiles per sample
-    int tiles_per_b;   // visited tiles per sample
+    int TI, TJ;        // row blocks, column blocks per sample
+    int tiles_per_b;   // tiles gram_tc_kernel visits per sample
     int n_pad;         // padded token count of one partial-sum slot
     __host__ __device__ int slots() const { return TJ + TI; }   // rho partial slots per sample: TJ row-side + TI column-side
 };
 
-inline GramTiling make_gram_tiling(int n, int BN) {
+inline GramTiling make_gram_tiling(int n) {
     GramTiling t;
-    t.BN = BN;
-    t.R = BN / kGramBM;
-    t.TI = (n + kGramBM - 1) / kGramBM;
-    t.TJ = (n + BN - 1) / BN;
-    const int last = t.R * t.TJ < t.TI ? t.R * t.TJ : t.TI;
-    t.tiles_per_b = t.TJ > 0 ? t.R * (t.TJ - 1) * t.TJ / 2 + last : 0;
+    t.TI = t.TJ = (n + kGramBM - 1) / kGramBM;
+    t.tiles_per_b = t.TI * t.TJ;
     t.n_pad = t.TI * kGramBM;
     return t;
-}
-
-// Tile t of the symmetric numbering -> (sample, row tile, column tile).
-__host__ __device__ inline void decode_sym_tile(const GramTiling& tl, long long t, int& b, int& ti, int& tj) {
-    b = (int)(t / tl.tiles_per_b);
-    const int r = (int)(t - (long long)b * tl.tiles_per_b);
-    const int R = tl.R;
-#ifdef __CUDA_ARCH__
-    int q = (int)((sqrtf(8.f * (float)r / (float)R + 1.f) - 1.f) * 0.5f);
-#else
-    int q = 0;
-#endif
-    while (q > 0 && R * q * (q + 1) / 2 > r) --q;
-    while (R * (q + 1) * (q + 2) / 2 <= r) ++q;
-    tj = q;
-    ti = r - R * q * (q + 1) / 2;
 }
 
 // Bounded device waits of the Gram kernels: the time after which a wait gives up (0 = the default of 2 s) and, for
@@ -91,23 +66,20 @@ struct GramArgs {
 };
 
 // rho of token i of one sample from the partial sums of the tiles that hold it, in a fixed order (reproducible
-// bits): the row-side slots of the column tiles that pair row tile i / 128 with later tokens, then the column-side
-// slots of the row tiles that pair column tile i / BN with earlier tokens.  `p` points at the sample's slot 0, token i.
-__host__ __device__ inline float rho_from_partials(const float* p, const GramTiling& t, int i) {
-    const int ti = i / kGramBM, tj = i / t.BN;
-    const int cap = t.R * (tj + 1);
-    const int rows = t.TI < cap ? t.TI : cap;
-    // slots [c0, TJ) on the row side, then [TJ, TJ + rows) on the column side: one contiguous walk, loaded sixteen
-    // at a time (independent loads) and added one by one in slot order
-    const int first = ti / t.R, last = t.TJ + rows;
+// bits): the row-side slots ti .. TJ - 1 of the column blocks that pair its row block ti with later tokens, then the
+// column-side slots TJ .. TJ + ti of the row blocks that pair it with earlier ones.  One contiguous walk, as long for every
+// token, loaded sixteen at a time (independent loads: up to 1920 tokens one trip to L2).  `p` points at the sample's slot 0,
+// token i.
+__device__ __forceinline__ float rho_from_partials(const float* p, const GramTiling& t, int i) {
+    const float* const q = p + (size_t)(i / kGramBM) * t.n_pad;
+    const int entries = t.TJ + 1;
     float s = 0.f;
-    for (int c = first; c < last; c += 16) {
+    for (int c = 0; c < entries; c += 16) {
         float v[16];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = (c + u < last) ? p[(size_t)(c + u) * t.n_pad] : 0.f;
+        for (int u = 0; u < 16; ++u) v[u] = c + u < entries ? q[(c + u) * t.n_pad] : 0.f;
 #pragma unroll
-        for (int u = 0; u < 16; ++u)
-            if (c + u < last) s += v[u];
+        for (int u = 0; u < 16; ++u) s += v[u];            // (nothing is negative: adding 0 changes no bit)
     }
     return s;
 }
@@ -157,7 +129,7 @@ bool gram_resident_takes_knorm(int H, int d);
 // tensor memory; the diagonal tiles publish the per-token factors, which the density epilogues of the other tiles wait for
 // value by value, the grid synchronises once (bounded waits) after the density
 // partials; the delta epilogue sums the partials it needs itself and re-reads the same accumulators.
-// `tiling` = make_gram_tiling(n, 128).
+// `tiling` = make_gram_tiling(n).
 int launch_gram_resident(const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream);
 
 // Multiprocessors of the current device.
