@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2601_17818_b200 import binding as vb
 from paper_2601_17818_b200.build import build_library
@@ -52,6 +53,16 @@ def test_workspace_sizes():
     assert e.value.status == vb.ERR_INVALID_ARG
     with pytest.raises(vb.VitcopError):
         vb.vitcop_workspace_bytes(vb.OP_SELECT, B=-1)
+
+
+@pytest.mark.parametrize("arg,error", [(torch.zeros(4), ValueError), ("text", TypeError), (1.5, TypeError),
+                                       (2 ** 70, OverflowError)])
+def test_native_caller_rejects_what_it_cannot_pass(L, arg, error):
+    """A tensor that is not on the device, and whatever is neither a tensor nor an integer, never reaches the library."""
+    with pytest.raises(error):
+        vb._native(vb._address["vitcop_select"], 0.0, arg)
+    with pytest.raises(TypeError):
+        vb._native(vb._address["vitcop_select"], 0.0, *[0] * 40)
 
 
 def test_argument_validation_happens_on_the_host(L):

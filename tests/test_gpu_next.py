@@ -89,6 +89,20 @@ def test_merge_planner_sizes(n, clusters, keep_p):
     _check_merge(hid, vs, vl, label, keep, min(n, 900))
 
 
+# Up to 256 clusters the planner counts, beyond that it sorts: both sides of the line, where a segment of 256 tokens ends and
+# begins, and a sample without tokens.
+@pytest.mark.parametrize("n,clusters", [(255, 255), (256, 256), (257, 257), (4000, 256), (4000, 257), (513, 1)])
+def test_merge_planner_cluster_line(n, clusters):
+    rng = np.random.default_rng(n + clusters)
+    B, Dh, vs = 3, 64, 2
+    hid = W.f32_to_bf16_bits(rng.standard_normal((B, n + vs, Dh)).astype(np.float32))
+    ids = np.sort(rng.choice(n, size=clusters, replace=False)).astype(np.int32)
+    label = np.concatenate([np.broadcast_to(ids, (B, clusters)), ids[rng.integers(0, clusters, size=(B, n - clusters))]], 1)
+    label = rng.permuted(label, axis=1).astype(np.int32)
+    keep = (rng.random((B, n)) < 0.1).astype(np.uint8)
+    _check_merge(hid, vs, np.array([n, n, 0], dtype=np.int32), label, keep, min(n, 900))
+
+
 def test_merge_label_out_of_range_is_clamped():
     rng = np.random.default_rng(11)
     n, Dh = 100, 64

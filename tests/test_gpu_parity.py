@@ -143,6 +143,34 @@ def test_select_quota_exact(kind, skew):
             assert status == vb.ERR_BUDGET and np.all(nk == 0)
 
 
+# Spans around the sizes at which a sequence gets more tokens per thread or a larger cluster of CTAs; few large and many small
+# clusters.  The same scores on both sides, so the kept tokens are equal.
+@pytest.mark.parametrize("n", [1024, 1025, 2048, 2049, 4096, 4097, 8191, 8192, 8193])
+def test_select_quota_span_edges(n):
+    score = W.make_scores(n, 2, n, "ties")
+    for ncl, skew in ((1, 0.0), (61, 0.6), (n // 9, 0.0)):
+        label = W.make_labels(n, 2, n, ncl, skew=skew)
+        keeps, nk, _, status = gpu_select(score, (n + ncl) // 2, label=label)
+        assert status == vb.OK
+        for b in range(2):
+            want, _, _ = oracle.select_quota(score[b].astype(np.float64), label[b], (n + ncl) // 2)
+            assert np.array_equal(keeps[b], want), (n, ncl, skew)
+
+
+# Spans around the numbers of tokens per thread; more than 256 scores equal to the one at the cut, on either side of it.
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 4096, 4097, 8192, 8193, 16384])
+def test_select_plain_span_edges(n):
+    rng = np.random.default_rng(n)
+    score = rng.standard_normal((2, n)).astype(np.float32)
+    score[1, rng.permutation(n)[: n // 2]] = 0.25
+    for budget in (1, n // 2, n - 1):
+        for largest in (False, True):
+            keeps, _, _, status = gpu_select(score, budget, largest=largest)
+            assert status == vb.OK
+            for b in range(2):
+                assert np.array_equal(keeps[b], oracle.select_plain(score[b].astype(np.float64), budget, largest)), (n, budget)
+
+
 @pytest.mark.parametrize("n,ncl,skew", [(64, 5, 0.0), (600, 20, 0.7), (5000, 40, 0.0), (5000, 40, 0.7)])
 def test_select_quota_special_values(n, ncl, skew):
     """NaN (ranked after everything), infinities, signed zeros and many exact ties, through each search strategy."""
@@ -207,6 +235,22 @@ def test_compact_bit_exact(B, H, N, d, Dh, vs, nv):
         assert np.array_equal(ho[b, :L], o["hidden"][:L])
         assert np.array_equal(Ko[b, :, :L], o["K"][:, :L]) and np.array_equal(Vo[b, :, :L], o["V"][:, :L])
         assert np.all(ho[b, L:] == 0) and np.all(Ko[b, :, L:] == 0)      # rows past out_len are never written
+
+
+# Rows around the lengths (in pieces of 16 bytes) at which more threads move one: 128 64, 256 128, 512 256 and 1024 all of them.
+@pytest.mark.parametrize("pieces", [1, 127, 128, 255, 256, 511, 512, 1023, 1024])
+def test_compact_row_lengths(pieces):
+    rng = np.random.default_rng(pieces)
+    B, H, N, d, vs, nv = 2, 1, 37, 8, 5, 29
+    hid, K, V = _rand_bits(rng, (B, N, 8 * max(1, pieces - 2))), _rand_bits(rng, (B, H, N, d)), _rand_bits(rng, (B, H, N, d))
+    keeps = [np.sort(rng.permutation(nv)[: 11 + 7 * b]).astype(np.int32) for b in range(B)]
+    ho, Ko, Vo, pos, olen = _gpu_compact(hid, K, V, vs, nv, keeps, N)
+    for b in range(B):
+        o = oracle.compact(hid[b], K[b], V[b], N, vs, nv, keeps[b], N)
+        L = o["out_len"]
+        assert olen[b] == L and np.array_equal(pos[b], o["kept_pos"]) and np.array_equal(ho[b, :L], o["hidden"][:L])
+        assert np.array_equal(Ko[b, :, :L], o["K"][:, :L]) and np.array_equal(Vo[b, :, :L], o["V"][:, :L])
+        assert np.all(ho[b, L:] == 0)
 
 
 def test_compact_ragged_partial_tensors_and_small_capacity():
