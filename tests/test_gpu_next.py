@@ -90,8 +90,8 @@ def test_merge_planner_sizes(n, clusters, keep_p):
 
 
 # Up to 256 clusters the planner counts, beyond that it sorts: both sides of the line, where a segment of 256 tokens ends and
-# begins, and a sample without tokens.
-@pytest.mark.parametrize("n,clusters", [(255, 255), (256, 256), (257, 257), (4000, 256), (4000, 257), (513, 1)])
+# begins, a sample without tokens, and a span whose shared memory fits the default 48 KB only without the static arrays.
+@pytest.mark.parametrize("n,clusters", [(255, 255), (256, 256), (257, 257), (4000, 256), (4000, 257), (513, 1), (5100, 255)])
 def test_merge_planner_cluster_line(n, clusters):
     rng = np.random.default_rng(n + clusters)
     B, Dh, vs = 3, 64, 2
