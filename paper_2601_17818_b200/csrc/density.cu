@@ -17,9 +17,9 @@
 // next tile's tokens and join the column warps' parts of the previous one, so that neither the trip to the L2 nor the joining
 // stands between two tiles.
 //
-// Measured with sixteen warps of one role: 8 x 2880 x 1024 70 us, 60 us with an empty epilogue; 2 x 16384 x 1280 517 us, 484 us
-// without the stores of the Gram values, 433 us with an empty epilogue (0.69 Tflop at the rate cuBLAS reaches in a burst).  The
-// sweep before this one, without the minima: 68 and 549 us.
+// Measured: 8 x 2880 x 1024 75 us (60 us with an empty epilogue), 2 x 16384 x 1280 519 us (433 us with an empty epilogue:
+// 0.69 Tflop at the rate cuBLAS reaches in a burst; the stores of the Gram values are about 30 of the rest).  Sixteen warps of one role: 70 and 517 us, but another order of the sums.  A sweep of single SMs on 128 x 256 tiles,
+// without the minima: 68 and 549 us.
 //
 // A last round of tiles that would occupy at most half of the clusters is cut into tiles of 128 columns.
 // Every wait is bounded; on expiry both CTAs of the cluster leave in order and the call reports VITCOP_ERR_TIMEOUT.

@@ -69,7 +69,7 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
 //             (clusters of similar size, the usual outcome of Algorithm 2).  On longer samples this is most of the work, and
 //             the CTAs of a thread-block cluster share the segments out: each prepares everything for itself (a microsecond
 //             or two), ranks its part and sends every verdict to the CTA that will emit the token.  (One CTA per sample:
-//             10 us on 576 tokens, 16 on 2880, 47 on 16384.);
+//             10 us on 576 tokens, 16 on 2880, 47 on 16384; now 7.3, 11.7 and 32);
 //   radix  -- every cluster runs its own radix select (4-bit digits) for its q_c-th smallest pair, all clusters at
 //             once: one shared histogram row per cluster, one thread per cluster to pick the digit, O(n) work per
 //             pass whatever the sizes.  Pairs are unique, so ties need no extra pass; a cluster stops as soon as a
