@@ -161,6 +161,9 @@ nearest_denser_kernel(const __grid_constant__ SweepArgs g) {
 
 // The tokens left over, each shared out over `slices` warps: warp w of a token takes the blocks w, w + slices, .. that are
 // still open and hold a denser token.  (Those the first kernel has looked into already cannot improve on its result.)
+// Each warp in ascending order of its blocks' minima: in the order of their numbers it looked into more of them (2 x 16384 tokens
+// of no structure 128.6 -> 117.5 us; 4 x 4608 of a video, whole call, 212 -> 209).  Two or four times as many blocks per warp measured
+// the same or worse.
 template <int METRIC, bool SPATIAL>
 __global__ void __launch_bounds__(kNdThreads)
 nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
@@ -188,26 +191,29 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
                 lo = __float_as_uint(__ldcg(row + k));
             }
             if (dens < __float_as_uint(s.t.y)) lo = kInfBits;
-            uint32_t todo = __ballot_sync(0xffffffffu, can(lo, k));
-            while (todo) {
+            // in ascending order of the minima, several at a time: the first ones are the likeliest to hold the answer, and
+            // none behind the first that cannot hold it can
+            for (;;) {
                 typename Search<METRIC, SPATIAL>::Pair p[kNdAhead];
                 int blk[kNdAhead];
                 int cnt = 0;
 #pragma unroll
                 for (int u = 0; u < kNdAhead; ++u) {
-                    if (todo) {
-                        blk[u] = k0 + (__ffs(todo) - 1) * slices;
-                        todo &= todo - 1;
+                    const uint32_t m = __reduce_min_sync(0xffffffffu, lo);
+                    const int who = __ffs(__ballot_sync(0xffffffffu, lo == m)) - 1;
+                    blk[u] = k0 + who * slices;
+                    if (cnt == u && can(m, blk[u])) {
+                        if (lane == who) lo = kInfBits;
                         p[u] = s.fetch(blk[u]);
                         cnt = u + 1;
                     }
                 }
+                if (cnt == 0) break;
 #pragma unroll
                 for (int u = 0; u < kNdAhead; ++u)
                     if (u < cnt) s.look(p[u], blk[u]);
                 const unsigned long long found = s.packed(s.bound());
                 best = found < best ? found : best;
-                todo &= __ballot_sync(0xffffffffu, can(lo, k));
             }
         }
         if (lane == 0 && best < known) atomicMin(g.best + at, best);
