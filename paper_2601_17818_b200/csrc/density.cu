@@ -124,9 +124,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+// Smallest of the values, or NaN if one of them is none.
+__device__ __forceinline__ float min2(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 __device__ __forceinline__ float min3(float a, float b, float c) {
     float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
 
@@ -151,7 +157,7 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
 }
 
 template <bool MIN>
-__device__ __forceinline__ float join(float a, float b) { return MIN ? fminf(a, b) : a + b; }
+__device__ __forceinline__ float join(float a, float b) { return MIN ? min2(a, b) : a + b; }
 // Eight values per thread, value 2 k + r for column 8 k + 2 (T % 4) + r: afterwards the thread holds the total over the eight
 // lanes with its T % 4 of column column_of(T), joined as a tree over the bits of T / 4, highest first.
 template <bool MIN>
@@ -446,8 +452,9 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                         mn2 = min3(mn2, v[u + 2], v[u + 3]);
                     }
                     mn = min3(min3(mn, v[30], v[31]), mn2, kInf);
-                    // (rounding can leave a near-duplicate's d^2 below zero: rare, so looked for before all are clamped)
-                    if (__any_sync(0xffffffffu, mn < 0.f)) {
+                    // (rounding can leave a near-duplicate's d^2 below zero, and features without a finite norm give none at all,
+                    // which counts as zero in the search and in the one-kernel sweep: rare, so looked for before all are clamped)
+                    if (__any_sync(0xffffffffu, !(mn >= 0.f))) {
 #pragma unroll
                         for (int u = 0; u < 32; ++u) v[u] = fmaxf(v[u], 0.f);
                         mn = fmaxf(mn, 0.f);
@@ -523,9 +530,9 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                         // ---- block minima (none where the block lies beyond the spatial radius); clamping as in the row warps
                         float cm[8];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) cm[q] = min3(fminf(d[q], d[8 + q]), d[16 + q], d[24 + q]);
+                        for (int q = 0; q < 8; ++q) cm[q] = min3(min2(d[q], d[8 + q]), d[16 + q], d[24 + q]);
                         cmin = reduce_columns<true>(cm, lane);
-                        if (__any_sync(0xffffffffu, cmin < 0.f)) {
+                        if (__any_sync(0xffffffffu, !(cmin >= 0.f))) {
 #pragma unroll
                             for (int u = 0; u < 32; ++u) d[u] = fmaxf(d[u], 0.f);
                             cmin = fmaxf(cmin, 0.f);

@@ -535,6 +535,30 @@ def test_filter_sweep_and_search_edges(B, n, metric, tau):
         check_vic_sample(f[b], p[b], metric, d_c, tau, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
 
 
+# Tokens whose features have no finite norm: every path takes a distance that is not a number as zero.  The batch goes through
+# the density sweep and the search, a sample by itself through the one-kernel sweep.
+@pytest.mark.parametrize("B,n", [(300, 127), (64, 576)])
+@pytest.mark.parametrize("metric,bad", [(0, "nan"), (0, "huge"), (1, "nan"), (1, "huge")])
+def test_filter_tokens_without_norm(B, n, metric, bad):
+    w = dataclasses.replace(W.workload("tiny"), B=B, D=64, dup_rate=0.3)
+    f = W.make_features(w, n=n, B=B).copy()
+    if bad == "nan":
+        f[:, n // 3, 5] = 0x7FC0
+    else:                                                  # two rows of 3e38 and -3e38: their products overflow
+        f[:, [n // 3, n - 2]] = 0x7F62
+        f[:, n // 3, ::2] |= 0x8000
+    p = np.ascontiguousarray(np.broadcast_to(W.make_positions(w, n)[:1], (B, n, 2)))
+    d_c = w.d_c if metric == 0 else 8.0
+    nc = max(1, n // 20)
+    g = gpu_filter(f, p, metric, d_c, w.tau, nc)
+    for b in (0, B - 1):
+        one = gpu_filter(f[b:b + 1], p[b:b + 1], metric, d_c, w.tau, nc)
+        assert np.all(np.isfinite(one.rho))
+        np.testing.assert_allclose(g.rho[b], one.rho[0], rtol=2e-6)     # fp32 sums of up to 576 terms in another order
+        for key in ("delta2", "parent", "label"):
+            assert np.array_equal(getattr(g, key)[b], getattr(one, key)[0]), key
+
+
 # The one-kernel sweep in units of 64 columns (few enough of them for one per SM: 148) and, with one sample more, of 128 or 256:
 # ends inside the first and the second half of a tile, one row block and many.  The same bits, whatever the unit.
 @pytest.mark.parametrize("n,metric,tau", [(1, 0, 0.6), (64, 0, 0.6), (65, 1, 0.6), (129, 0, -1.0), (193, 1, -1.0), (576, 0, 0.6),
