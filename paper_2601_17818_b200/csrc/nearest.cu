@@ -177,7 +177,9 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
         const float* const row = g.blk_min + ((size_t)b * g.t.n_pad + i) * n_blk;
         const uint32_t* const top = g.blk_rho + (size_t)b * n_blk;   // largest density of every block
         Search<METRIC, SPATIAL> s(g, b, i, lane);
-        const unsigned long long known = __ldcg(g.best + at);      // (other warps may be lowering it: a stale one is only looser)
+        // (other warps may be lowering it: a stale one is only looser, but all lanes must go by the same one, as it decides which of
+        // them meet in the reductions below)
+        const unsigned long long known = __shfl_sync(0xffffffffu, lane == 0 ? __ldcg(g.best + at) : 0ull, 0);
         unsigned long long best = known;
         // Can block k, with minimum `lo`, hold a token below `best`?  (An equal distance at a lower index would win.)
         auto can = [&](uint32_t lo, int k) {

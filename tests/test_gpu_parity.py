@@ -514,6 +514,23 @@ def test_filter_long_samples_scattered_positions():
         check_vic_sample(f[b], p[b], 0, w.d_c, 0.3, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
 
 
+# Features without structure leave the most tokens to the search's second kernel, in which the warps that share a token lower its
+# entry while others read it: every run gives the same.
+@pytest.mark.parametrize("metric", [0, 1])
+def test_filter_search_shared_tokens(metric):
+    n, D = 12000, 64
+    feat = torch.randn((2, n, D), generator=torch.Generator(device=DEV).manual_seed(6), device=DEV).to(torch.bfloat16)
+    ws = vb.alloc_workspace(vb.OP_FILTER, B=2, Nv=n, D=D)
+    first = None
+    for _ in range(12):
+        o = [torch.zeros((2, n), dtype=t, device=DEV) for t in (torch.int32, torch.float32, torch.float32, torch.int32)]
+        vb.vitcop_redundancy_filter(feat, None, o[0], torch.zeros(2, dtype=torch.int32, device=DEV), ws, metric=metric,
+                                    d_c=0.5 if metric == 0 else 4.0, n_centers=600, rho=o[1], delta2=o[2], parent=o[3])
+        assert vb.vitcop_poll_status(ws) == vb.OK
+        first = first or o
+        assert all(torch.equal(a, b) for a, b in zip(o, first))
+
+
 # Too many tiles for the one-kernel sweep: pairs of CTAs on 256 x 256 tiles (ragged ends, an odd number of 128-token blocks, the
 # last tiles cut into column halves or not), block minima, the search.  Half of the last sample's tokens are one token plus
 # noise (plain copies would tie in every distance, and the oracle's report excuses ties): the densest of them have neighbours
