@@ -711,11 +711,10 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 tc_commit(bar_tfull + 8 * acc);            // accumulator complete
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-            if (!ok) {
-                // leaving early: let the MMAs already issued finish before TMEM is released
-                tc_commit(bar_drain);
-                mbar_drain(bar_drain, 0);
-            }
+            // let the MMAs issued finish before the operands and TMEM are released (the epilogue need not be waiting for them: it
+            // may have given up)
+            tc_commit(bar_drain);
+            mbar_drain(bar_drain, 0);
         }
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2 ..)
@@ -1065,10 +1064,8 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
                 if (!ok) break;
                 tc_commit(bar_tfull + 8 * slot);
             }
-            if (!ok) {
-                tc_commit(bar_drain);
-                mbar_drain(bar_drain, 0);
-            }
+            tc_commit(bar_drain);                          // (as in gram_tc_kernel)
+            mbar_drain(bar_drain, 0);
         }
     }
     if (warp < 2) {

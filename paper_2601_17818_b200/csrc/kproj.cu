@@ -198,11 +198,8 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 tc_commit_pair(bar_tfull + 8 * acc);
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-            if (!ok) {
-                raise_abort_pair(abort_addr, rank);
-                tc_commit_pair(bar_drain);
-                mbar_drain(bar_drain, 0);
-            }
+            if (!ok) raise_abort_pair(abort_addr, rank);
+            tc_commit_pair(bar_drain);                     // (waited for below)
         }
     } else {
         // ------------------------------------------------------------------ epilogue
@@ -278,6 +275,9 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     }
 
     __syncthreads();
+    // Another role may have given up behind the last MMA: operands and tensor memory stay until all of them have completed.
+    // (Otherwise they have; the wait costs nothing.)
+    if (threadIdx.x == 32) mbar_drain(bar_drain, 0);
     if (threadIdx.x == 0 && *abort_flag) {
         // Some role gave up, so loads issued here may never have been consumed: give the copies still in flight into this
         // CTA's shared memory time to land before the CTA goes away.  (The other CTA's land on the leader's barriers.)
