@@ -81,7 +81,8 @@ int vitcop_poll_status(const void* workspace, void* stream, int* device_status);
  * library remain usable).  This call sets the limit for launches made after it, process-wide:
  *   limit_ns      time after which a wait gives up; 0 restores the default of 2 s
  *   expire_roles  for failure-handling tests: waits of the named roles give up at once, whatever their state
- *                 (1 load warp, 2 tensor-core issue warp, 4 epilogue warps; 0 = none)
+ *                 (1 load warp, 2 tensor-core issue warp, 4 epilogue warps; 8, 16, 32 the same in the kernels that run
+ *                 on pairs of multiprocessors alone: density sweep, key projection; 0 = none)
  * Always returns VITCOP_OK. */
 int vitcop_set_wait_limit(unsigned long long limit_ns, int expire_roles);
 

@@ -607,7 +607,7 @@ int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cu
     KernelArgs k;
     k.g = args;
     k.wait_ns = gram_wait_limit_ns();
-    k.expire_roles = gram_expire_roles();
+    k.expire_roles = pair_expire_roles();
     const long long total = (long long)args.B * args.t.tiles_per_b;
     if (total <= 0) return VITCOP_OK;
     if (total >= 1 << 22) return VITCOP_ERR_UNSUPPORTED;   // (group sizes keep it far below; decode_item's estimates hold to there)

@@ -1265,11 +1265,14 @@ bool make_rowmajor_bf16_map(CUtensorMap* map, const void* base, int batches, int
 }
 
 unsigned long long gram_wait_limit_ns() { return g_wait_ns.load(); }
-int gram_expire_roles() { return g_expire_roles.load(); }
+int pair_expire_roles() {
+    const int r = g_expire_roles.load();
+    return (r | r >> 3) & 7;
+}
 
 void gram_set_wait_debug(unsigned long long limit_ns, int expire_roles) {
     g_wait_ns.store(limit_ns ? limit_ns : kWaitLimitNs);
-    g_expire_roles.store(expire_roles & 7);
+    g_expire_roles.store(expire_roles & 63);
 }
 
 int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStream_t stream, bool pdl) {
@@ -1290,7 +1293,7 @@ int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStre
     k.extra_units_per_b = 0;
     k.unit_w = 0;
     k.wait_ns = g_wait_ns.load();
-    k.expire_roles = g_expire_roles.load();
+    k.expire_roles = g_expire_roles.load() & 7;
     if (k.total_tiles <= 0) return VITCOP_OK;
     CUtensorMap ma, mb;
     if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) || !make_feat_map(&mb, feat, args.B, args.n, args.D, BM))
@@ -1349,7 +1352,7 @@ int launch_gram_resident(const void* feat, const GramArgs& args, const GramTilin
         k.total_tiles = (long long)args.B * units;
     }
     k.wait_ns = g_wait_ns.load();
-    k.expire_roles = g_expire_roles.load();
+    k.expire_roles = g_expire_roles.load() & 7;
     if (k.total_tiles <= 0) return VITCOP_OK;
     if (k.total_tiles > (long long)kResidentUnits * num_sms()) return VITCOP_ERR_INVALID_ARG;
     CUtensorMap ma, mb;

@@ -28,11 +28,12 @@ inline GramTiling make_gram_tiling(int n) {
 }
 
 // Bounded device waits of the Gram kernels: the time after which a wait gives up (0 = the default of 2 s) and, for
-// failure-handling tests, the roles whose waits give up at once (1 load warp, 2 MMA warp, 4 epilogue warps).
+// failure-handling tests, the roles whose waits give up at once (1 load warp, 2 MMA warp, 4 epilogue warps; times 8: in the
+// kernels on pairs of SMs alone).
 // Applies to launches made after the call.
 void gram_set_wait_debug(unsigned long long limit_ns, int expire_roles);
 unsigned long long gram_wait_limit_ns();
-int gram_expire_roles();
+int pair_expire_roles();                               // as the kernels on pairs of SMs take them
 
 struct GramArgs {
     int B, n, D;

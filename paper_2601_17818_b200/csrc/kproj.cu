@@ -332,7 +332,7 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     k.cos_tab = cos_tab; k.sin_tab = sin_tab; k.position = position; k.n_pos = n_pos;
     k.status = static_cast<int*>(workspace);
     k.wait_ns = gram_wait_limit_ns();
-    k.expire_roles = gram_expire_roles();
+    k.expire_roles = pair_expire_roles();
     const long long total = (long long)k.TI * k.TJ;
     if (total <= 0) return VITCOP_OK;
     CUtensorMap ma, mb;

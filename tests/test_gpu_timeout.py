@@ -34,7 +34,7 @@ def _filter_call(feat, pos, w, ws, out):
 
 
 # B = 2 runs the one-kernel sweep (accumulators resident in tensor memory, cooperative launch, flags between CTAs);
-# B = 80 exceeds what one wave of CTAs can keep resident and runs the diagonal / density / delta sweeps.
+# B = 80 exceeds what one wave of CTAs can keep resident and runs the diagonal, the density sweep and the search.
 @pytest.mark.parametrize("B,n", [(2, 200), (80, 300)])
 @pytest.mark.parametrize("roles", [ROLE_EPILOGUE, ROLE_MMA, ROLE_LOAD])
 def test_filter_reports_timeout_and_recovers(B, n, roles):
@@ -60,6 +60,32 @@ def test_filter_reports_timeout_and_recovers(B, n, roles):
     assert _filter_call(feat, pos, w, ws, got) == vb.OK                    # same workspace, next call is clean
     for key in ("label", "ncl", "rho", "d2", "par"):
         assert torch.equal(got[key], ref[key]), key
+
+
+# The density sweep's pairs of CTAs give up by themselves: the diagonal in front of them has its normal limit.
+@pytest.mark.parametrize("B,n", [(80, 300), (6, 1700)])
+@pytest.mark.parametrize("roles", [ROLE_EPILOGUE, ROLE_MMA, ROLE_LOAD])
+def test_density_sweep_reports_timeout_and_recovers(B, n, roles):
+    feat = torch.randn((B, n, 256), generator=torch.Generator(device=DEV).manual_seed(n), device=DEV).to(torch.bfloat16)
+    ws = vb.alloc_workspace(vb.OP_FILTER, B=B, Nv=n, D=256)
+
+    def run():
+        o = [torch.zeros((B, n), dtype=t, device=DEV) for t in (torch.int32, torch.float32, torch.float32, torch.int32)]
+        vb.vitcop_redundancy_filter(feat, None, o[0], torch.zeros(B, dtype=torch.int32, device=DEV), ws, n_centers=n // 20,
+                                    rho=o[1], delta2=o[2], parent=o[3])
+        return vb.vitcop_poll_status(ws), o
+
+    status, ref = run()
+    assert status == vb.OK
+    vb.vitcop_set_wait_limit(0, roles * 8)
+    assert run()[0] == vb.ERR_TIMEOUT
+    small = vb.alloc_workspace(vb.OP_FILTER, B=1, Nv=200, D=256)          # the one-kernel sweep is no pair kernel
+    vb.vitcop_redundancy_filter(feat[:1, :200].contiguous(), None, torch.zeros((1, 200), dtype=torch.int32, device=DEV),
+                                torch.zeros(1, dtype=torch.int32, device=DEV), small, n_centers=10)
+    assert vb.vitcop_poll_status(small) == vb.OK
+    vb.vitcop_set_wait_limit(0, 0)
+    status, got = run()
+    assert status == vb.OK and all(torch.equal(a, b) for a, b in zip(got, ref))
 
 
 def test_similarity_rows_reports_timeout_and_recovers():
