@@ -63,9 +63,23 @@ _lib: Optional[C.CDLL] = None
 _native = None                                   # _call.so's function
 _address: dict = {}                              # entry point -> address
 _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-# the parameter structs as bytes, laid out as the compiler does
-_filter_params = struct.Struct("@iffdi4x").pack
-_select_params = struct.Struct("@iii").pack
+
+
+# the parameter structs as bytes, laid out as the compiler does; values that a field cannot hold are converted as C does (a
+# radius of 1e300 is infinite), which struct refuses and ctypes, a microsecond slower, does
+def _packer(fmt: str, struct_type):
+    pack = struct.Struct(fmt).pack
+
+    def params(*values) -> bytes:
+        try:
+            return pack(*values)
+        except (struct.error, OverflowError):
+            return bytes(struct_type(*values))
+    return params
+
+
+_filter_params = _packer("@iffdi4x", FilterParams)
+_select_params = _packer("@iii", SelectParams)
 
 
 def lib() -> C.CDLL:

@@ -65,6 +65,15 @@ def test_native_caller_rejects_what_it_cannot_pass(L, arg, error):
         vb._native(vb._address["vitcop_select"], 0.0, *[0] * 40)
 
 
+@pytest.mark.parametrize("values", [(0, 0.5, 0.6, 0.05, 29), (1, 8.0, 1e300, 0.05, 0), (0, 1e39, -1e39, 2.0, 2 ** 31),
+                                    (0, float("inf"), float("nan"), 1e300, -2 ** 40)])
+def test_parameters_are_converted_as_c_does(values):
+    """Whatever the struct of the ABI takes, the binding passes: out of a field's range too."""
+    assert vb._filter_params(*values) == bytes(vb.FilterParams(*values))
+    ints = (0, 1, values[-1])
+    assert vb._select_params(*ints) == bytes(vb.SelectParams(*ints))
+
+
 def test_argument_validation_happens_on_the_host(L):
     """Every call below must return before any CUDA work (there may be no device at all)."""
     fake = C.c_void_p(0x1000)                       # 16-byte aligned, never dereferenced by the checks
