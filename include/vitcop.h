@@ -35,7 +35,7 @@ extern "C" {
 #define VITCOP_OK               0
 #define VITCOP_ERR_INVALID_ARG  1   /* NULL required pointer, negative size, span outside the sequence, aliasing */
 #define VITCOP_ERR_UNSUPPORTED  2   /* alignment / divisibility / size limit not met */
-#define VITCOP_ERR_WORKSPACE    3   /* workspace NULL or smaller than vitcop_workspace_bytes reports */
+#define VITCOP_ERR_WORKSPACE    3   /* workspace NULL or too small (vitcop_workspace_bytes reports what is enough) */
 #define VITCOP_ERR_BUDGET       4   /* quota mode with budget < number of clusters (device-side, via poll) */
 #define VITCOP_ERR_CUDA         5   /* a CUDA runtime call failed; see vitcop_last_cuda_error */
 #define VITCOP_ERR_TIMEOUT      6   /* a bounded device-side wait expired (device-side, via poll) */
@@ -64,7 +64,11 @@ int vitcop_last_cuda_error(void);
 
 /* Bytes of device workspace `op` needs for the given problem (arguments an op does not use are
  * ignored; pass 0).  Nv is the capacity of the visual span (max over samples), n == Nv for the
- * filter.  `bytes` is a host pointer.  The workspace must be 256-byte aligned. */
+ * filter.  `bytes` is a host pointer.  The workspace must be 256-byte aligned.
+ * For the filter and the one-call step the size never falls when B or Nv grows, so a workspace of the largest problem
+ * serves all smaller ones.  Up to 1.5 GB of it hold pairwise values of the samples that are worked on together (about
+ * 2 Nv^2 bytes each; 20 MB at 2880 tokens, 0.6 GB at 16384; small problems need none).  A caller that has less
+ * may pass less, down to one sample's: the samples then go through in smaller groups, with the same results, slower. */
 int vitcop_workspace_bytes(int op, int B, int H, int N, int d, int Nv, int D, int Dh, size_t* bytes);
 
 /* Synchronises `stream`, copies the device status word of `workspace` to `*device_status`

@@ -359,9 +359,11 @@ int vitcop_collaborative_step(const void* feat, const float* pos, int D, const v
     if (rc != VITCOP_OK) return rc;
     if (D % 64 || !aligned16(feat) || !aligned8(pos) || Nv > VITCOP_MAX_VISUAL_TOKENS || B > 65535)
         return VITCOP_ERR_UNSUPPORTED;
-    const size_t filter_bytes = align_up(filter_workspace_bytes(B, Nv, D), 256);
     const StepWs lay(B, Nv);
-    if (!workspace || workspace_bytes < filter_bytes + lay.total || !aligned256(workspace)) return VITCOP_ERR_WORKSPACE;
+    size_t filter_bytes = align_up(filter_workspace_bytes(B, Nv, D), 256);
+    if (!workspace || workspace_bytes < lay.total || !aligned256(workspace)) return VITCOP_ERR_WORKSPACE;
+    if (workspace_bytes - lay.total < filter_bytes) filter_bytes = (workspace_bytes - lay.total) / 256 * 256;
+    if (filter_bytes < filter_workspace_least_bytes(B, Nv)) return VITCOP_ERR_WORKSPACE;
     int nc = fp->n_centers;
     if (nc <= 0) {
         const double v = std::ceil((double)Nv * fp->alpha);
@@ -380,7 +382,7 @@ int vitcop_collaborative_step(const void* feat, const float* pos, int D, const v
     if (Nv > 0) {
         const KnormJob job = {K, B, H, N, d, vis_start, Nv, score};
         rc = launch_filter(feat, pos, B, Nv, D, *fp, nc, label_out, n_clusters_out, rho_out, delta2_out, parent_out,
-                           workspace, s, &job);
+                           workspace, filter_bytes, s, &job);
         if (rc != VITCOP_OK) return rc;
     }
     // (plain stream order when the filter was skipped: see vitcop_prune_step)
@@ -465,7 +467,7 @@ int vitcop_redundancy_filter(const void* feat, const float* pos, int B, int n, i
     if (!(p->d_c > 0.f)) return VITCOP_ERR_INVALID_ARG;
     if (D % 64 || !aligned16(feat) || !aligned8(pos) || n > VITCOP_MAX_VISUAL_TOKENS || B > 65535)
         return VITCOP_ERR_UNSUPPORTED;
-    if (!workspace || workspace_bytes < filter_workspace_bytes(B, n, D) || !aligned256(workspace))
+    if (!workspace || workspace_bytes < filter_workspace_least_bytes(B, n) || !aligned256(workspace))
         return VITCOP_ERR_WORKSPACE;
     int nc = p->n_centers;
     if (nc <= 0) {
@@ -477,7 +479,7 @@ int vitcop_redundancy_filter(const void* feat, const float* pos, int B, int n, i
     int rc = record_cuda(cudaMemsetAsync(workspace, 0, filter_zeroed_bytes(B, n), s));
     if (rc != VITCOP_OK) return rc;
     if (B == 0 || n == 0) return VITCOP_OK;
-    return launch_filter(feat, pos, B, n, D, *p, nc, label, n_clusters, rho, delta2, parent, workspace, s);
+    return launch_filter(feat, pos, B, n, D, *p, nc, label, n_clusters, rho, delta2, parent, workspace, workspace_bytes, s);
 }
 
 int vitcop_similarity_rows(const void* feat, int B, int n, int D, int metric, int row_begin, int row_end, float* out,

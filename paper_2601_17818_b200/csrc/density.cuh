@@ -45,13 +45,29 @@ __host__ __device__ inline size_t gram_block_offset(int rb, int cb) {
 // instruction.
 __host__ __device__ inline int gram_elem_offset(int r, int c) { return ((c >> 2) * kBlk + r) * 4 + (c & 3); }
 
-// Samples whose Gram values are kept at one time: the sweep and the search run group by group, so that the workspace
-// stays bounded whatever the batch.
-constexpr size_t kKeptTilesBytes = (size_t)3 << 29;       // 1.5 GB: two samples of 16384 tokens take 1.1 GB
-inline int sweep_group_samples(int B, int n) {
-    const size_t per = (size_t)make_sweep_tiling(n).tiles_per_b * kSweepTileFloats * sizeof(float);
-    const size_t fit = per > 0 ? kKeptTilesBytes / per : (size_t)B;
-    return (int)(fit < 1 ? 1 : fit < (size_t)B ? fit : (size_t)B);
+// What the sweep and the search keep of a group of samples: count and list of the search's leftovers, the tokens as the search
+// reads them, block densities, block minima, Gram values (4 bytes per pair of the symmetric half, tile padding included).  They
+// run group by group, so that the workspace stays bounded whatever the batch.
+struct SweepGroupWs {
+    size_t off_left, off_tok, off_blk_rho, off_blk_min, off_gram, total;
+    SweepGroupWs(size_t samples, int n) {
+        const SweepTiling s = make_sweep_tiling(n);
+        size_t o = 0;
+        off_left = o;    o += align_up((samples * n + 1) * 4, 256);
+        off_tok = o;     o += align_up(samples * s.n_pad * sizeof(float4), 256);
+        off_blk_rho = o; o += align_up(samples * s.n_blk() * 4, 256);
+        off_blk_min = o; o += align_up(samples * s.n_blk() * s.n_pad * 4, 256);
+        off_gram = o;    o += align_up(samples * s.tiles_per_b * kSweepTileFloats * 4, 256);
+        total = o;
+    }
+};
+constexpr size_t kSweepGroupBytes = (size_t)3 << 29;      // 1.5 GB: two samples of 16384 tokens take 1.2 GB
+// Samples of a group where it may take `bytes`; 0 if one is too much.
+inline int sweep_group_samples(int B, int n, size_t bytes) {
+    const size_t per = SweepGroupWs(1, n).total;           // (never less than a sample adds)
+    size_t g = bytes / per < (size_t)B ? bytes / per : (size_t)B;
+    while (g < (size_t)B && SweepGroupWs(g + 1, n).total <= bytes) ++g;
+    return (int)g;
 }
 
 struct SweepArgs {

@@ -371,36 +371,36 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
 // host side
 // ------------------------------------------------------------------------------------------------
 // Workspace of the filter: status block | for the one-kernel sweep the tokens' published factors [B, n] | w | a | rho | best |
-// rho partials [B, slots, n_pad] (sized for either sweep) | bounding boxes of the row blocks' positions | and, for
-// problems too large for the one-kernel sweep, of one group of samples: count and list of the search's leftovers, the tokens as the search reads them, block densities, block minima, Gram values of
-// the density sweep (4 bytes per pair of the symmetric half, tile padding included).  The status block and the
-// published factors are zeroed at the start of every call.  Words of the status block: 0 status, 2 grid barrier.
+// rho partials [B, slots, n_pad] | bounding boxes of the row blocks' positions | and, for problems too large for the one-kernel
+// sweep, what is kept of one group of samples (SweepGroupWs).  The status block and the published factors are zeroed at the start
+// of every call.  Words of the status block: 0 status, 2 grid barrier.
+// A group is as large as the workspace allows, so every workspace serves that holds one sample of it; the size asked for holds
+// all samples, or as many as fit 1.5 GB (8 x 2880 tokens take 175 MB: one sample at a time would leave half of the SMs without
+// work).  Neither the size asked for nor the least one ever falls when the batch or the samples grow: a workspace for a larger
+// problem serves a smaller one.
 struct FilterWs {
-    size_t off_ready, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_left, off_tok, off_blk_rho, off_blk_min, off_gram, total;
+    size_t off_ready, off_w, off_a, off_rho, off_best, off_part, off_bbox, off_group, total, least;
+    bool resident;
     FilterWs(int B, int n) {
         size_t o = kStatusBytes;
         const size_t bn = (size_t)B * n;
-        const bool resident = gram_fits_resident(B, n);
+        resident = gram_fits_resident(B, n);
         off_ready = o; o += resident ? align_up(bn * 4, 256) : 0;
         off_w = o;    o += align_up(bn * 4, 256);
         off_a = o;    o += align_up(bn * 4, 256);
         off_rho = o;  o += align_up(bn * 4, 256);
         off_best = o; o += align_up(bn * 8, 256);
-        const GramTiling t = make_gram_tiling(n);           // (two slots per block: never fewer than the density sweep's)
-        const size_t slots = resident && gram_resident_halves(B, n) ? 5 * (size_t)t.TI : (size_t)t.slots();
+        // one-kernel sweep: units of 64 columns take the most slots; density sweep: make_sweep_tiling
+        const GramTiling t = make_gram_tiling(n);
+        const size_t slots = resident ? 5 * (size_t)t.TI : (size_t)make_sweep_tiling(n).slots();
         off_part = o; o += align_up((size_t)B * slots * t.n_pad * 4, 256);
         off_bbox = o;   o += align_up((size_t)B * t.TI * sizeof(float4), 256);
-        off_left = off_tok = off_blk_rho = off_blk_min = off_gram = o;
+        off_group = least = total = o;
         if (B > 0 && n > 0 && !resident) {
-            const SweepTiling s = make_sweep_tiling(n);
-            const size_t group = (size_t)sweep_group_samples(B, n);
-            o += align_up((group * n + 1) * 4, 256);
-            off_tok = o;     o += align_up(group * s.n_pad * sizeof(float4), 256);
-            off_blk_rho = o; o += align_up(group * s.n_blk() * 4, 256);
-            off_blk_min = o; o += align_up(group * s.n_blk() * s.n_pad * 4, 256);
-            off_gram = o;    o += align_up(group * s.tiles_per_b * kSweepTileFloats * 4, 256);
+            const size_t one = SweepGroupWs(1, n).total, all = SweepGroupWs((size_t)B, n).total;
+            least += one;
+            total += all < kSweepGroupBytes ? all : one > kSweepGroupBytes ? one : kSweepGroupBytes;
         }
-        total = o;
     }
 };
 
@@ -425,6 +425,7 @@ size_t filter_workspace_bytes(int B, int n, int D) {
     (void)D;
     return FilterWs(B, n).total;
 }
+size_t filter_workspace_least_bytes(int B, int n) { return FilterWs(B, n).least; }
 size_t similarity_workspace_bytes(int B, int n, int D) {
     (void)D;
     return kStatusBytes + 2 * align_up((size_t)B * n * 4, 256);
@@ -432,8 +433,9 @@ size_t similarity_workspace_bytes(int B, int n, int D) {
 
 int launch_filter(const void* feat, const float* pos, int B, int n, int D, const vitcop_filter_params& p,
                   int n_centers, int32_t* label, int32_t* n_clusters, float* rho_user, float* delta2_user,
-                  int32_t* parent_user, void* workspace, cudaStream_t stream, const KnormJob* knorm) {
-    FilterWs l(B, n);
+                  int32_t* parent_user, void* workspace, size_t workspace_bytes, cudaStream_t stream, const KnormJob* knorm) {
+    const FilterWs l(B, n);
+    if (workspace_bytes < l.least) return VITCOP_ERR_WORKSPACE;
     char* ws = static_cast<char*>(workspace);
     float* w = reinterpret_cast<float*>(ws + l.off_w);
     float* a = reinterpret_cast<float*>(ws + l.off_a);
@@ -453,8 +455,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     // (the producer of the features included) has completed when it starts.
     int rc;
     int knorm_in_sweep = 0;                                // leading samples whose K-norm the Gram sweep computes
-    const bool resident = gram_fits_resident(B, n);
-    if (resident) {
+    if (l.resident) {
         g.rho_out = rho;
         g.rho_user = rho_user;
         g.grid_sync = reinterpret_cast<unsigned int*>(ws) + 2;       // zeroed with the status word at the start of the call
@@ -477,7 +478,9 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
         rc = launch_gram_sweep(GRAM_DIAG, feat, g, stream, false);
         if (rc != VITCOP_OK) return rc;
         const SweepTiling tiling = make_sweep_tiling(n);
-        const int group = sweep_group_samples(B, n);
+        const int group = sweep_group_samples(B, n, (workspace_bytes < l.total ? workspace_bytes : l.total) - l.off_group);
+        const SweepGroupWs kept((size_t)group, n);
+        char* const gws = ws + l.off_group;
         for (int b0 = 0; b0 < B; b0 += group) {
             const size_t at = (size_t)b0 * n;
             SweepArgs s = {};
@@ -487,12 +490,12 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             s.pos = pos ? pos + 2 * at : nullptr;
             s.bbox = g.bbox ? g.bbox + (size_t)b0 * tiling.TI : nullptr;
             s.part = part + (size_t)b0 * tiling.slots() * tiling.n_pad;
-            s.n_left = reinterpret_cast<int32_t*>(ws + l.off_left);
+            s.n_left = reinterpret_cast<int32_t*>(gws + kept.off_left);
             s.left = s.n_left + 1;
-            s.tok = reinterpret_cast<float4*>(ws + l.off_tok);
-            s.blk_rho = reinterpret_cast<uint32_t*>(ws + l.off_blk_rho);
-            s.blk_min = reinterpret_cast<float*>(ws + l.off_blk_min);
-            s.gram = reinterpret_cast<float*>(ws + l.off_gram);
+            s.tok = reinterpret_cast<float4*>(gws + kept.off_tok);
+            s.blk_rho = reinterpret_cast<uint32_t*>(gws + kept.off_blk_rho);
+            s.blk_min = reinterpret_cast<float*>(gws + kept.off_blk_min);
+            s.gram = reinterpret_cast<float*>(gws + kept.off_gram);
             s.status = g.status;
             s.t = tiling;
             rc = launch_density_sweep(static_cast<const uint16_t*>(feat) + at * D, s, p.metric, stream, true);

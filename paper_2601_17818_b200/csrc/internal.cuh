@@ -60,12 +60,14 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
 // do not depend on the selection may be copied while the kernels in front are still running.)
 
 size_t filter_workspace_bytes(int B, int n, int D);
+// The least that launch_filter takes: with less than filter_workspace_bytes the samples go through in smaller groups.
+size_t filter_workspace_least_bytes(int B, int n);
 // Leading bytes of the filter workspace that must be zero when launch_filter starts (status block and published factors).
 size_t filter_zeroed_bytes(int B, int n);
 size_t similarity_workspace_bytes(int B, int n, int D);
 int launch_filter(const void* feat, const float* pos, int B, int n, int D, const vitcop_filter_params& p,
                   int n_centers, int32_t* label, int32_t* n_clusters, float* rho, float* delta2, int32_t* parent,
-                  void* workspace, cudaStream_t stream, const KnormJob* knorm = nullptr);
+                  void* workspace, size_t workspace_bytes, cudaStream_t stream, const KnormJob* knorm = nullptr);
 int launch_similarity_rows(const void* feat, int B, int n, int D, int metric, int row_begin, int row_end,
                            float* out, void* workspace, cudaStream_t stream);
 

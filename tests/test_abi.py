@@ -65,6 +65,17 @@ def test_native_caller_rejects_what_it_cannot_pass(L, arg, error):
         vb._native(vb._address["vitcop_select"], 0.0, *[0] * 40)
 
 
+@pytest.mark.parametrize("op", [vb.OP_FILTER, vb.OP_COLLAB_STEP])
+def test_a_workspace_of_a_larger_problem_serves_a_smaller_one(L, op):
+    sizes = [1, 64, 127, 128, 129, 576, 577, 1408, 1409, 1536, 2048, 2880, 4608, 8191, 8192, 12000, 16384]
+    batches = [1, 2, 3, 5, 8, 11, 12, 16, 40, 149, 300, 6144, 6145]
+    need = [[vb.vitcop_workspace_bytes(op, B=B, Nv=n, D=64) for n in sizes] for B in batches]
+    for i in range(len(batches)):
+        for j in range(len(sizes)):
+            assert i == 0 or need[i][j] >= need[i - 1][j], (batches[i], sizes[j])
+            assert j == 0 or need[i][j] >= need[i][j - 1], (batches[i], sizes[j])
+
+
 @pytest.mark.parametrize("values", [(0, 0.5, 0.6, 0.05, 29), (1, 8.0, 1e300, 0.05, 0), (0, 1e39, -1e39, 2.0, 2 ** 31),
                                     (0, float("inf"), float("nan"), 1e300, -2 ** 40)])
 def test_parameters_are_converted_as_c_does(values):

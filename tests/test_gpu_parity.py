@@ -613,6 +613,42 @@ def test_filter_all_orphans(n, nc):
     assert np.array_equal(np.unique(g.label[0]), np.sort(order[:nc]))
 
 
+def test_filter_in_workspaces_of_other_sizes():
+    """One sized for a longer sample, or with room for fewer samples at a time than the call would like: the same results."""
+    B, n, D = 16, 4000, 64
+    feat = torch.randn((B, n, D), generator=torch.Generator(device=DEV).manual_seed(2), device=DEV).to(torch.bfloat16)
+
+    def run(ws):
+        o = [torch.zeros((B, n), dtype=t, device=DEV) for t in (torch.int32, torch.float32, torch.float32, torch.int32)]
+        vb.vitcop_redundancy_filter(feat, None, o[0], torch.zeros(B, dtype=torch.int32, device=DEV), ws, n_centers=200,
+                                    rho=o[1], delta2=o[2], parent=o[3])
+        assert vb.vitcop_poll_status(ws) == vb.OK
+        return o
+
+    own = vb.alloc_workspace(vb.OP_FILTER, B=B, Nv=n, D=D)
+    want = run(own)
+    one = vb.vitcop_workspace_bytes(vb.OP_FILTER, B=1, Nv=8000, D=D)       # of which one sample's pairs take a quarter
+    assert one < own.numel() // 3
+    # (the guard behind the smaller ones: nothing may be written past what the call was given)
+    for part in (vb.vitcop_workspace_bytes(vb.OP_FILTER, B=B, Nv=16384, D=D), own.numel() // 2, one):
+        ws = torch.full((part + 4096,), 0x5A, dtype=torch.uint8, device=DEV)
+        assert all(torch.equal(a, b) for a, b in zip(run(ws[:part]), want)), part
+        assert bool((ws[part:] == 0x5A).all())
+    with pytest.raises(vb.VitcopError) as e:
+        run(own[: 16 << 20])
+    assert e.value.status == vb.ERR_WORKSPACE
+
+
+@pytest.mark.parametrize("op", [vb.OP_FILTER, vb.OP_COLLAB_STEP])
+def test_workspace_never_shrinks_with_the_problem(op):
+    """Across the line between the one-kernel sweep and the others, which only a device knows."""
+    lens = list(range(1, 2200, 37)) + [576, 1408, 1409, 1536, 2880]
+    for B in (1, 2, 3, 5, 16, 40, 148, 296):
+        need = [vb.vitcop_workspace_bytes(op, B=B, Nv=n, D=64) for n in sorted(lens)]
+        more = [vb.vitcop_workspace_bytes(op, B=B + 1, Nv=n, D=64) for n in sorted(lens)]
+        assert all(a <= b for a, b in zip(need, need[1:])) and all(a <= b for a, b in zip(need, more)), B
+
+
 def test_filter_sample_groups():
     """More Gram values than the workspace keeps at a time: the samples go through the sweep and the search in groups, and
     give what each gives by itself."""
