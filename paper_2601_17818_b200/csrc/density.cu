@@ -622,8 +622,9 @@ int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cu
         return VITCOP_ERR_CUDA;
     const int smem = metric == 1 ? smem_bytes<1>() : smem_bytes<0>();
     auto kern = metric == 1 ? density_sweep_kernel<1> : density_sweep_kernel<0>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return record_cuda(e);
+    static DoneOnDevice attr_done[2];
+    const int arc = allow_dynamic_smem(kern, smem, attr_done[metric == 1]);
+    if (arc != VITCOP_OK) return arc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * (k.n_items < pairs ? k.n_items : pairs)));
     cfg.blockDim = dim3(kThreads);

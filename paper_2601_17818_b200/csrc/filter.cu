@@ -114,6 +114,7 @@ constexpr int kFinRankLanes = 4;
 constexpr int kFinRank = kFinThreads / kFinRankLanes;      // bins of up to this many keys are ranked by counting
 
 // Dynamic shared memory: nxt[n] (uint16), isc[n] (uint8), centre list[nc] (uint16; surplus orphans).  E: tokens per thread.
+constexpr size_t finalize_smem(int n, int nc) { return (((size_t)n + 15) & ~(size_t)15) * 3 + (size_t)(nc > 0 ? nc : 1) * 2 + 16; }
 template <int E>
 __global__ void __launch_bounds__(kFinThreads)
 vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_centers, const float* rho, const unsigned long long* best,
@@ -514,14 +515,15 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     }
 
     const int nc = n_centers < n ? n_centers : n;
-    const size_t smem = (((size_t)n + 15) & ~(size_t)15) * 3 + (size_t)(nc > 0 ? nc : 1) * 2 + 16;
-    auto fin = n <= kFinThreads       ? vic_finalize_kernel<1>
-               : n <= 4 * kFinThreads ? vic_finalize_kernel<4>
-               : n <= 8 * kFinThreads ? vic_finalize_kernel<8> : vic_finalize_kernel<16>;
+    const size_t smem = finalize_smem(n, nc);
+    const int v = n <= kFinThreads ? 0 : n <= 4 * kFinThreads ? 1 : n <= 8 * kFinThreads ? 2 : 3;
+    auto fin = v == 0 ? vic_finalize_kernel<1> : v == 1 ? vic_finalize_kernel<4> : v == 2 ? vic_finalize_kernel<8> : vic_finalize_kernel<16>;
     static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kFinThreads, "tokens of the longest sample");
-    if (smem > 16 * 1024) {                                // (the kernel's static arrays take part of the default 48 KB)
-        cudaError_t e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return record_cuda(e);
+    if (v > 0) {                                           // (up to 1024 tokens 5 KB)
+        static DoneOnDevice attr_done[4];
+        const int most = (v == 1 ? 4 : v == 2 ? 8 : 16) * kFinThreads;
+        rc = allow_dynamic_smem(fin, finalize_smem(most, most), attr_done[v]);
+        if (rc != VITCOP_OK) return rc;
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];

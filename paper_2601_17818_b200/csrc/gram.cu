@@ -1182,13 +1182,6 @@ bool make_feat_map(CUtensorMap* map, const void* feat, int B, int n, int D, int 
 std::atomic<unsigned long long> g_wait_ns{kWaitLimitNs};
 std::atomic<int> g_expire_roles{0};
 
-// What the launchers remember is remembered per device: one process may drive several.
-constexpr int kMaxDevices = 64;
-int current_device() {
-    int dev = 0;
-    return (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) ? dev : 0;
-}
-
 int num_sms() {
     static std::atomic<int> sms[kMaxDevices];
     const int dev = current_device();
@@ -1200,21 +1193,10 @@ int num_sms() {
     return v;
 }
 
-// Raises a kernel's dynamic shared-memory limit once per device.
-template <typename Kernel>
-int allow_dynamic_smem(Kernel kern, int bytes, std::atomic<unsigned long long>& done) {
-    const unsigned long long bit = 1ull << current_device();
-    if (done.load(std::memory_order_relaxed) & bit) return VITCOP_OK;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return record_cuda(e);
-    done.fetch_or(bit, std::memory_order_relaxed);
-    return VITCOP_OK;
-}
-
 template <int BN, int MODE, int METRIC>
 int launch_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream, bool pdl) {
     using S = GemmSmem<BN>;
-    static std::atomic<unsigned long long> attr_done{0};
+    static DoneOnDevice attr_done;
     auto kern = gram_tc_kernel<BN, MODE, METRIC>;
     const int arc = allow_dynamic_smem(kern, S::kTotal, attr_done);
     if (arc != VITCOP_OK) return arc;
@@ -1235,7 +1217,7 @@ int launch_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k
 template <int METRIC, bool SPATIAL, int BN>
 int launch_resident_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream) {
     using S = GemmSmem<kResidentBN>;
-    static std::atomic<unsigned long long> attr_done{0};
+    static DoneOnDevice attr_done;
     auto kern = gram_resident_kernel<METRIC, SPATIAL, BN>;
     constexpr int kSmem = S::kTotal + (BN == 64 ? HalfUnitSmem::kEpiBytes - S::kEpiBytes : 0);
     const int arc = allow_dynamic_smem(kern, kSmem, attr_done);

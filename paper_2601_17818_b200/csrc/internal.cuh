@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "vitcop.h"
 
 namespace vitcop {
@@ -15,6 +17,26 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Records the first failing CUDA runtime error of the calling thread.
 int record_cuda(cudaError_t e);
+
+// What the launchers remember is remembered per device: one process may drive several.
+constexpr int kMaxDevices = 64;
+inline int current_device() {
+    int dev = 0;
+    return (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) ? dev : 0;
+}
+
+// Raises a kernel's dynamic shared-memory limit once per device: to the most the kernel is ever launched with, because another
+// thread may launch it between this call and the launch behind it.
+typedef std::atomic<unsigned long long> DoneOnDevice;      // a bit per device
+template <typename Kernel>
+inline int allow_dynamic_smem(Kernel kern, size_t most_bytes, DoneOnDevice& done) {
+    const unsigned long long bit = 1ull << current_device();
+    if (done.load(std::memory_order_relaxed) & bit) return VITCOP_OK;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_bytes);
+    if (e != cudaSuccess) return record_cuda(e);
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return VITCOP_OK;
+}
 
 // Diagnostic per-kernel timing (vitcop_kernel_timing_begin / _end).  While it is on, a KernelTimeScope
 // around a launch records one CUDA event before and one after the kernel on its stream, and launchers

@@ -340,8 +340,9 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
         return VITCOP_ERR_CUDA;
     const bool rope = cos_tab != nullptr;
     auto kern = rope ? kproj_kernel<true> : kproj_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return record_cuda(e);
+    static DoneOnDevice attr_done[2];
+    const int arc = allow_dynamic_smem(kern, kSmemBytes, attr_done[rope]);
+    if (arc != VITCOP_OK) return arc;
     cudaLaunchConfig_t cfg = {};
     const long long pairs = gram_num_sms() / 2 > 0 ? gram_num_sms() / 2 : 1;
     if (2 * total > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;

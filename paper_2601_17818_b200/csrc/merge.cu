@@ -450,6 +450,12 @@ merge_rows_kernel(const uint4* __restrict__ hidden, int B, int N, int dh8, int s
     }
 }
 
+// Dynamic shared memory of the planner: the counting pass, or the sort's two buffers and counters.
+size_t plan_smem(int Nv_cap) {
+    const size_t sort_bytes = 2 * (size_t)((Nv_cap + 3) & ~3) * sizeof(uint32_t) + (size_t)kCntEntries * sizeof(uint16_t);
+    return sort_bytes > plan_count_bytes(Nv_cap) ? sort_bytes : plan_count_bytes(Nv_cap);
+}
+
 // Workspace: status | members uint16 [B, Nv_cap] | headers [B, Mcap]
 struct MergeWs {
     size_t off_members, off_headers, total;
@@ -478,14 +484,13 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     {
-        const size_t sort_bytes = 2 * (size_t)((Nv_cap + 3) & ~3) * sizeof(uint32_t) + (size_t)kCntEntries * sizeof(uint16_t);
-        const size_t smem = sort_bytes > plan_count_bytes(Nv_cap) ? sort_bytes : plan_count_bytes(Nv_cap);
-        auto kern = Nv_cap <= kPlanThreads       ? merge_plan_kernel<1>
-                    : Nv_cap <= 4 * kPlanThreads ? merge_plan_kernel<4>
-                    : Nv_cap <= 8 * kPlanThreads ? merge_plan_kernel<8> : merge_plan_kernel<16>;
-        if (smem > 40 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return record_cuda(e);
+        const int v = Nv_cap <= kPlanThreads ? 0 : Nv_cap <= 4 * kPlanThreads ? 1 : Nv_cap <= 8 * kPlanThreads ? 2 : 3;
+        auto kern = v == 0 ? merge_plan_kernel<1> : v == 1 ? merge_plan_kernel<4> : v == 2 ? merge_plan_kernel<8> : merge_plan_kernel<16>;
+        const size_t smem = plan_smem(Nv_cap);
+        if (v > 0) {                                       // (up to 1024 tokens 19 KB)
+            static DoneOnDevice attr_done[4];
+            const int rc = allow_dynamic_smem(kern, plan_smem((v == 1 ? 4 : v == 2 ? 8 : 16) * kPlanThreads), attr_done[v]);
+            if (rc != VITCOP_OK) return rc;
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(B);

@@ -221,14 +221,17 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
     // CTAs per sequence: one up to 2048 tokens (the others would be done preparing when the first is done), four, and eight
     // beyond 8192
     const int R = Nv_cap <= 2 * kSelThreads ? 1 : Nv_cap <= 8 * kSelThreads ? 4 : 8;
-    auto kern = Nv_cap <= kSelThreads ? select_quota_kernel<1, 1>
-                : R == 1              ? select_quota_kernel<1, 2>
-                : Nv_cap <= 4 * kSelThreads ? select_quota_kernel<4, 4>
-                : R == 4              ? select_quota_kernel<4, 8> : select_quota_kernel<8, 16>;
+    const int E = Nv_cap <= kSelThreads ? 1 : Nv_cap <= 2 * kSelThreads ? 2 : Nv_cap <= 4 * kSelThreads ? 4 : Nv_cap <= 8 * kSelThreads ? 8 : 16;
+    auto kern = E == 1   ? select_quota_kernel<1, 1>
+                : E == 2 ? select_quota_kernel<1, 2>
+                : E == 4 ? select_quota_kernel<4, 4>
+                : E == 8 ? select_quota_kernel<4, 8> : select_quota_kernel<8, 16>;
     static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kSelThreads, "tokens of the longest sample");
-    if (smem > 40 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return record_cuda(e);
+    {
+        static DoneOnDevice attr_done[17];
+        int most_p = 0;
+        const int rc = allow_dynamic_smem(kern, select_quota_smem(E * kSelThreads, &most_p), attr_done[E]);
+        if (rc != VITCOP_OK) return rc;
     }
     cudaLaunchAttribute attrs[2];
     attrs[0] = attr[0];

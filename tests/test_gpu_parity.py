@@ -804,3 +804,38 @@ def test_collaborative_step_replays_from_a_cuda_graph():
             assert torch.equal(got[key], ref[key]), key
         for key in ("ho", "Ko", "Vo"):
             assert torch.equal(got[key].view(torch.int16), ref[key].view(torch.int16)), key
+
+
+# The same kernels with other amounts of shared memory, called by several threads at once: each launch has what it needs, whatever
+# another thread asked for just before.
+def test_calls_from_several_threads():
+    import threading
+    failed = []
+
+    def worker(n, seed):
+        try:
+            g = torch.Generator(device=DEV).manual_seed(seed)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                score = torch.rand((1, n), generator=g, device=DEV)
+                label = torch.randint(0, n // 20, (1, n), generator=g, device=DEV, dtype=torch.int32)
+                keep, nk = torch.zeros((1, n), dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+                mask = torch.zeros((1, n), dtype=torch.uint8, device=DEV)
+                hid = torch.zeros((1, n, 64), dtype=torch.bfloat16, device=DEV)
+                ml, mc = torch.zeros((1, n), dtype=torch.int32, device=DEV), torch.zeros((1, n), dtype=torch.int32, device=DEV)
+                ws, wm = vb.alloc_workspace(vb.OP_SELECT, B=1, Nv=n), vb.alloc_workspace(vb.OP_MERGE, B=1, Nv=n, N=n)
+                for _ in range(400):
+                    vb.vitcop_select(score, n, n // 4, keep, nk, ws, label=label, keep_mask=mask)
+                    vb.vitcop_merge_clusters(hid, 0, n, label, mask, ml, mc, nk, wm)
+                got = [x.clone() for x in (keep, mask, ml, mc)]
+                torch.cuda.current_stream().synchronize()
+                vb.vitcop_select(score, n, n // 4, keep, nk, ws, label=label, keep_mask=mask)
+                assert torch.equal(keep, got[0]) and torch.equal(mask, got[1])
+        except Exception as e:
+            failed.append(repr(e))
+
+    threads = [threading.Thread(target=worker, args=(n, n)) for n in (16384, 9000, 12345, 8200)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
