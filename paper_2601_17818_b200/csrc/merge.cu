@@ -3,14 +3,15 @@
 //
 // Two kernels on one stream:
 //   merge_plan_kernel   one CTA per sample: lays every cluster's non-elite tokens out contiguously in ascending token order,
-//                       clusters in ascending label order.  Up to 256 clusters by one stable counting pass over dense cluster
-//                       numbers; more by a stable radix sort of the labels in shared memory.
+//                       clusters in ascending label order.  Up to 256 to 1024 clusters, by the sample's length, by one stable
+//                       counting pass over dense cluster numbers; more by a stable radix sort of the labels in shared memory.
 //   merge_rows_kernel   one CTA per (merged row, sample, 1024-byte slice of the hidden row): its four warps stream
 //                       the members' row slices with 128-bit loads (member r goes to warp r mod 4) and the four
 //                       fp32 partial sums are added in warp order, a fixed order (bit-reproducible).  Only rows
 //                       that are averaged are read.
 #include <cuda_bf16.h>
 
+#include "gram.cuh"
 #include "internal.cuh"
 
 namespace vitcop {
@@ -19,7 +20,6 @@ namespace {
 constexpr int kPlanThreads = 1024;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr int kRowsThreads = 128;
-constexpr int kRowsPieces = 2;                             // 16-byte pieces of a row per lane
 constexpr int kPlanItems = VITCOP_MAX_VISUAL_TOKENS / kPlanThreads;   // rows of 32 entries a warp walks at most
 constexpr int kDigitBits = 7, kDigits = 1 << kDigitBits;
 static_assert(kDigits * kPlanWarps == 4 * kPlanThreads, "four counters per thread in the scan");
@@ -36,6 +36,7 @@ struct __align__(16) MergeHeader {
     uint16_t first[4][4];                                 // member r < 16 at [r % 4][r / 4]
 };
 constexpr int kManyMembers = 32;
+__host__ __device__ constexpr int member_stride(int Nv_cap) { return (Nv_cap + 7) & ~7; }     // a sample's member list
 static_assert(sizeof(MergeHeader) == 48, "three 16-byte words");
 
 // Every array of the planner is walked the same way: warp w owns the entries [w * 32 E, (w + 1) * 32 E), E =
@@ -107,40 +108,127 @@ __device__ uint32_t* sort_by_label(uint32_t* a, uint32_t* b, int m, int label_bi
     return a;
 }
 
-// The plan by one stable counting pass, for samples with up to kCountSeg clusters that have non-elite tokens: labels get dense
-// numbers (presence flags, one scan), every warp ranks its tokens inside their cluster (one match per 32 tokens and a counter
-// per (warp, cluster)), one scan over the counters turns ranks into positions.  Returns false, nothing written, when there are
-// more clusters.  E: rows of 32 tokens per warp.  smem: uint32 flags / numbers packed as uint16 [n], counters uint16
-// [32][kCountStride].
-constexpr int kCountSeg = 256, kCountStride = kCountSeg + 2;
-__host__ __device__ constexpr size_t plan_count_bytes(int Nv_cap) {
-    return ((size_t)((Nv_cap + 7) & ~7) + (size_t)kPlanWarps * kCountStride) * sizeof(uint16_t);
+// The plan by one stable counting pass: labels get dense numbers (presence flags, one scan), every warp ranks its tokens inside
+// their cluster (one match per 32 tokens and a counter per (warp, cluster)), one scan over the counters turns ranks into
+// positions.  Taken up to count_seg(E) clusters that have non-elite tokens: 5 % of the tokens that E stands for, rounded up to
+// what divides the threads.  E: rows of 32 tokens per warp.  lab, take: this thread's tokens (labels; bit e: not an elite).
+// smem: flags / numbers uint16 [n rounded up to 8], counters uint16 [32][clusters + 2].
+__host__ __device__ constexpr int count_seg(int E) { return E <= 4 ? 256 : E <= 8 ? 512 : 1024; }
+__host__ __device__ constexpr size_t plan_count_bytes(int Nv_cap, int E) {
+    return ((size_t)((Nv_cap + 7) & ~7) + (size_t)kPlanWarps * (count_seg(E) + 2)) * sizeof(uint16_t);
 }
-template <int E>
-__device__ __forceinline__ bool plan_by_count(const int32_t* label, const uint8_t* keep_mask, int n, int Mcap,
-                                              int32_t* merged_label, int32_t* merged_count, int32_t* n_merged_b,
-                                              uint16_t* members, MergeHeader* headers, uint16_t* smem, uint32_t* warp_sums) {
-    __shared__ uint16_t seg_start[kCountSeg], seg_slot[kCountSeg];   // slot: place of the cluster's header
+__device__ __forceinline__ void zero_counters(uint16_t* cnt, int clusters) {
+    for (int i = threadIdx.x; i < kPlanWarps * (clusters + 2) / 2; i += kPlanThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0u;
+}
+// The first sixteen of a run's members (the low halves of the entries) into its header.
+template <typename Entry>
+__device__ __forceinline__ void store_first(const Entry* run, int count, MergeHeader* h) {
+    uint32_t w[8];
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int r = 8 * k + g;                       // first[g][2 k], first[g][2 k + 1]: members r and r + 4
+            w[2 * g + k] = (r < count ? (uint32_t)run[r] & 0xFFFFu : 0u) | (r + 4 < count ? (uint32_t)run[r + 4] << 16 : 0u);
+        }
+    uint4* const to = reinterpret_cast<uint4*>(h->first);
+    to[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    to[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+// Behind the dense numbers, for up to SEG clusters; the counters are zero.
+template <int E, int SEG>
+__device__ __forceinline__ void plan_positions(const uint32_t (&lab)[E], uint32_t take, int n, int n_seg, int Mcap,
+                                               int32_t* merged_count, uint16_t* members, MergeHeader* headers,
+                                               uint16_t* id_of, uint16_t* cnt, uint16_t* seg_start, uint16_t* seg_slot,
+                                               uint32_t* warp_sums) {
+    constexpr int kStride = SEG + 2, kPer = kPlanThreads / SEG, kOf = kPlanWarps / kPer;     // threads per cluster, counters of one
+    static_assert(kPer * SEG == kPlanThreads && kPer * kOf == kPlanWarps && kPer <= 32, "threads and counters of a cluster");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
+    const int rows = (n + kPlanThreads - 1) / kPlanThreads;
+    const int bits = n_seg > 1 ? 32 - __clz(n_seg - 1) : 0;
+    uint32_t at[E];                                        // cluster << 16 | rank among the warp's tokens of the cluster
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        at[e] = 0;
+        if (e < rows) {                                    // (uniform)
+            const bool mine = (take >> e & 1u) != 0;
+            const uint32_t c = mine ? id_of[lab[e]] : 0u;
+            // the lanes of the same cluster: a ballot per bit of its number (a match takes as many steps as the row has different
+            // clusters: 16384 tokens in 820 clusters 50.4 us, so 45.7)
+            const uint32_t all = __ballot_sync(0xffffffffu, mine);
+            uint32_t peers = mine ? all : 0u;
+#pragma unroll 1
+            for (int k = 0; k < bits; ++k) {
+                const uint32_t bk = __ballot_sync(0xffffffffu, c >> k & 1u);
+                peers &= (c >> k & 1u) ? bk : ~bk;
+            }
+            uint32_t before = 0;
+            if (mine) before = cnt[warp * kStride + c];
+            __syncwarp();
+            if (mine && lane == __ffs(peers) - 1) cnt[warp * kStride + c] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            at[e] = (c << 16) | (before + __popc(peers & lt));
+        }
+    }
+    __syncthreads();
+    uint32_t m;
+    {
+        // counters in (cluster, warp) order -> positions
+        const int c = tid / kPer, w0 = tid % kPer * kOf;
+        uint32_t sum = 0;
+#pragma unroll
+        for (int q = 0; q < kOf; ++q) sum += cnt[(w0 + q) * kStride + c];
+        uint32_t pos = block_exclusive_sum(sum, warp_sums, m);
+        const uint32_t start = __shfl_sync(0xffffffffu, pos, lane & ~(kPer - 1));
+        const uint32_t end = __shfl_sync(0xffffffffu, pos + sum, lane | (kPer - 1));
+        const bool row = tid % kPer == 0 && c < n_seg && c < Mcap, many = row && end - start >= (uint32_t)kManyMembers;
+        uint32_t totals;
+        const uint32_t before = block_exclusive_sum((row ? 1u : 0u) | (many ? 0x10000u : 0u), warp_sums, totals);
+        if (row) {
+            const uint32_t many_before = before >> 16, few_before = (before & 0xFFFFu) - many_before;
+            const uint32_t slot = many ? many_before : (totals >> 16) + few_before;
+            seg_slot[c] = (uint16_t)slot;
+            seg_start[c] = (uint16_t)start;
+            *reinterpret_cast<int4*>(headers + slot) = make_int4((int)(end - start), (int)start, c, 0);
+            merged_count[c] = (int32_t)(end - start);
+        }
+#pragma unroll
+        for (int q = 0; q < kOf; ++q) {
+            const uint32_t v = cnt[(w0 + q) * kStride + c];
+            cnt[(w0 + q) * kStride + c] = (uint16_t)pos;
+            pos += v;
+        }
+    }
+    __syncthreads();
+    // the member list is put together in shared memory and leaves in words of eight: tokens of a warp go to as many places as they
+    // have clusters (16384 tokens in 820 clusters: 45.7 us with scattered two-byte stores, 27.3 so; 4608 in 231: 18.7, 14.6)
+    uint16_t* const sorted = id_of;                        // (the numbers have been read)
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (take >> e & 1u)
+            sorted[cnt[warp * kStride + (at[e] >> 16)] + (at[e] & 0xFFFFu)] = (uint16_t)((warp * rows + e) * 32 + lane);
+    __syncthreads();
+    for (int q = tid; q < ((int)m + 7) / 8; q += kPlanThreads) reinterpret_cast<uint4*>(members)[q] = reinterpret_cast<const uint4*>(sorted)[q];
+    if (tid < min(n_seg, Mcap)) {
+        const int start = seg_start[tid], end = tid + 1 < min(n_seg, Mcap) ? seg_start[tid + 1] : start + 16;
+        store_first(sorted + start, min(end, (int)m) - start, headers + seg_slot[tid]);
+    }
+    for (int c = n_seg + tid; c < Mcap; c += kPlanThreads) headers[c].count = 0;
+}
+// Returns false, nothing written, when there are more clusters than that.
+template <int E>
+__device__ __forceinline__ bool plan_by_count(const uint32_t (&lab)[E], uint32_t take, int n, int Mcap,
+                                              int32_t* merged_label, int32_t* merged_count, int32_t* n_merged_b,
+                                              uint16_t* members, MergeHeader* headers, uint16_t* smem, uint32_t* warp_sums) {
+    constexpr int kSeg = count_seg(E), kNarrow = 256;
+    __shared__ uint16_t seg_start[kSeg], seg_slot[kSeg];   // slot: place of the cluster's header
+    const int tid = threadIdx.x;
     const int n_al = (n + 7) & ~7;
     uint16_t* const id_of = smem;                          // by label: 1 = present, then its dense number
     uint16_t* const cnt = smem + n_al;
     for (int i = tid; i < n_al / 8; i += kPlanThreads) reinterpret_cast<uint4*>(id_of)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = tid; i < kPlanWarps * kCountStride / 2; i += kPlanThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0u;
-    // warp w owns the tokens [w * 32 rows, (w + 1) * 32 rows), row by row: entry order is (warp, row, lane) order
-    const int rows = (n + kPlanThreads - 1) / kPlanThreads;
-    uint32_t lab[E], take = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = (warp * rows + e) * 32 + lane;
-        lab[e] = 0;
-        if (e < rows && i < n) {
-            const uint32_t l = (uint32_t)label[i];
-            lab[e] = l >= (uint32_t)n ? (uint32_t)n - 1 : l;       // out-of-range labels are clamped, never indexed
-            if (!keep_mask[i]) take |= 1u << e;
-        }
-    }
+    zero_counters(cnt, kNarrow);
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < E; ++e)
@@ -158,7 +246,7 @@ __device__ __forceinline__ bool plan_by_count(const int32_t* label, const uint8_
             c += __popc(w[v].x) + __popc(w[v].y) + __popc(w[v].z) + __popc(w[v].w);
         }
         uint32_t next = block_exclusive_sum(c, warp_sums, n_seg);
-        if (n_seg > (uint32_t)kCountSeg) return false;     // uniform
+        if (n_seg > (uint32_t)kSeg) return false;          // uniform
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
             const int l = (tid * words + v) * 8;
@@ -175,72 +263,15 @@ __device__ __forceinline__ bool plan_by_count(const int32_t* label, const uint8_
             }
         }
     }
+    if (kSeg > kNarrow && n_seg > (uint32_t)kNarrow) zero_counters(cnt, kSeg);
     __syncthreads();
-    uint32_t at[E];                                        // cluster << 16 | rank among the warp's tokens of the cluster
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        at[e] = 0;
-        if (e < rows) {                                    // (uniform)
-            const bool mine = (take >> e & 1u) != 0;
-            const uint32_t c = mine ? id_of[lab[e]] : 0xFFFFu;
-            const uint32_t peers = __match_any_sync(0xffffffffu, c);
-            uint32_t before = 0;
-            if (mine) before = cnt[warp * kCountStride + c];
-            __syncwarp();
-            if (mine && lane == __ffs(peers) - 1) cnt[warp * kCountStride + c] = (uint16_t)(before + __popc(peers));
-            __syncwarp();
-            at[e] = (c << 16) | (before + __popc(peers & lt));
-        }
-    }
-    __syncthreads();
-    {
-        // counters in (cluster, warp) order -> positions: four threads per cluster, eight warps each
-        const int c = tid >> 2, w0 = (tid & 3) * 8;
-        uint32_t v[8], sum = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            v[q] = cnt[(w0 + q) * kCountStride + c];
-            sum += v[q];
-        }
-        uint32_t m;
-        uint32_t pos = block_exclusive_sum(sum, warp_sums, m);
-        const uint32_t start = __shfl_sync(0xffffffffu, pos, lane & ~3);
-        const uint32_t end = __shfl_sync(0xffffffffu, pos + sum, lane | 3);
-        const bool row = (tid & 3) == 0 && c < (int)n_seg && c < Mcap, many = row && end - start >= (uint32_t)kManyMembers;
-        uint32_t totals;
-        const uint32_t before = block_exclusive_sum((row ? 1u : 0u) | (many ? 0x10000u : 0u), warp_sums, totals);
-        if ((tid & 3) == 0) {
-            seg_start[c] = (uint16_t)start;
-            seg_slot[c] = 0xFFFFu;
-            if (row) {
-                const uint32_t many_before = before >> 16, few_before = (before & 0xFFFFu) - many_before;
-                const uint32_t slot = many ? many_before : (totals >> 16) + few_before;
-                seg_slot[c] = (uint16_t)slot;
-                *reinterpret_cast<int4*>(headers + slot) = make_int4((int)(end - start), (int)start, c, 0);
-                merged_count[c] = (int32_t)(end - start);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            cnt[(w0 + q) * kCountStride + c] = (uint16_t)pos;
-            pos += v[q];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        if (take >> e & 1u) {
-            const uint32_t c = at[e] >> 16, p = cnt[warp * kCountStride + c] + (at[e] & 0xFFFFu), r = p - seg_start[c];
-            const uint16_t i = (uint16_t)((warp * rows + e) * 32 + lane);
-            members[p] = i;
-            if (r < 16 && seg_slot[c] != 0xFFFFu) headers[seg_slot[c]].first[r & 3][r >> 2] = i;
-        }
-    }
-    for (int c = (int)n_seg + tid; c < Mcap; c += kPlanThreads) headers[c].count = 0;
+    if (kSeg > kNarrow && n_seg > (uint32_t)kNarrow)
+        plan_positions<E, kSeg>(lab, take, n, (int)n_seg, Mcap, merged_count, members, headers, id_of, cnt, seg_start, seg_slot, warp_sums);
+    else
+        plan_positions<E, kNarrow>(lab, take, n, (int)n_seg, Mcap, merged_count, members, headers, id_of, cnt, seg_start, seg_slot, warp_sums);
     if (tid == 0) *n_merged_b = (int32_t)n_seg;
     return true;
 }
-static_assert(kPlanThreads == 4 * kCountSeg && kPlanWarps == 32, "four threads per cluster, eight warps each");
 
 template <int E>
 __global__ void __launch_bounds__(kPlanThreads)
@@ -265,38 +296,42 @@ merge_plan_kernel(const int32_t* label, const uint8_t* keep_mask,
     keep_mask += (size_t)b * Nv_cap;
     merged_label += (size_t)b * Mcap;
     merged_count += (size_t)b * Mcap;
-    members += (size_t)b * Nv_cap;
+    members += (size_t)b * member_stride(Nv_cap);
     headers += (size_t)b * Mcap;
 
-    if (plan_by_count<E>(label, keep_mask, n, Mcap, merged_label, merged_count, n_merged + b, members, headers,
+    // this thread's tokens: warp w owns [w * 32 rows, (w + 1) * 32 rows), row by row, so that entry order is (warp, row, lane) order
+    uint32_t it[E], take = 0;
+    {
+        const int rows = (n + kPlanThreads - 1) / kPlanThreads;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = (warp * rows + e) * 32 + lane;
+            it[e] = 0;
+            if (e < rows && i < n) {
+                const uint32_t lab = (uint32_t)label[i];
+                it[e] = lab >= (uint32_t)n ? (uint32_t)n - 1 : lab;        // out-of-range labels are clamped, never indexed
+                if (!keep_mask[i]) take |= 1u << e;
+            }
+        }
+    }
+    if (plan_by_count<E>(it, take, n, Mcap, merged_label, merged_count, n_merged + b, members, headers,
                          reinterpret_cast<uint16_t*>(smem_items), warp_sums)) {
         grid_dependency_launch_dependents();
         return;
     }
     __syncthreads();
-    // ---- more clusters than that.  The non-elite tokens, in token order: count per warp, one scan, then place.  (Unrolled, unlike the walks
-    //      over shared memory: all of a thread's global loads are in flight together.)
+    // ---- more clusters than that: the non-elite tokens, in token order (count per warp, one scan, then place)
     uint32_t m;
     {
         const int rows = (n + kPlanThreads - 1) / kPlanThreads;
-        uint32_t it[kPlanItems], take = 0, mine = 0;
+        uint32_t mine = 0;
 #pragma unroll
-        for (int e = 0; e < kPlanItems; ++e) {
-            const int i = (warp * rows + e) * 32 + lane;
-            if (e < rows && i < n) {
-                uint32_t lab = (uint32_t)label[i];
-                if (lab >= (uint32_t)n) lab = (uint32_t)n - 1;     // out-of-range labels are clamped, never indexed
-                it[e] = (lab << 16) | (uint32_t)i;
-                if (!keep_mask[i]) take |= 1u << e;
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < kPlanItems; ++e) mine += __popc(__ballot_sync(0xffffffffu, take >> e & 1u));
+        for (int e = 0; e < E; ++e) mine += __popc(__ballot_sync(0xffffffffu, take >> e & 1u));
         uint32_t pos = warp_totals_scan(mine, warp_sums, m);
 #pragma unroll
-        for (int e = 0; e < kPlanItems; ++e) {
+        for (int e = 0; e < E; ++e) {
             const uint32_t bal = __ballot_sync(0xffffffffu, take >> e & 1u);
-            if (take >> e & 1u) buf0[pos + __popc(bal & lt)] = it[e];
+            if (take >> e & 1u) buf0[pos + __popc(bal & lt)] = (it[e] << 16) | (uint32_t)((warp * rows + e) * 32 + lane);
             pos += __popc(bal);
         }
     }
@@ -347,15 +382,14 @@ merge_plan_kernel(const int32_t* label, const uint8_t* keep_mask,
     }
     __syncthreads();
     for (int mm = tid; mm < Mcap; mm += kPlanThreads) {
-        int count = 0;
+        int count = 0, start = 0;
         if (mm < (int)heads) {
-            const int start = headers[mm].start;
+            start = headers[mm].start;
             count = merged_count[mm] - start + 1;
             merged_count[mm] = count;
-            for (int r = 0; r < min(count, 16); ++r) headers[mm].first[r & 3][r >> 2] = (uint16_t)(items[start + r] & 0xFFFFu);
+            store_first(items + start, count, headers + mm);
         }
-        headers[mm].count = count;
-        headers[mm].row = mm;
+        *reinterpret_cast<int4*>(headers + mm) = make_int4(count, start, mm, 0);
     }
     if (tid == 0) n_merged[b] = (int32_t)heads;
     grid_dependency_launch_dependents();
@@ -380,13 +414,15 @@ __device__ __forceinline__ void add8(unsigned long long (&a)[4], const uint4& v)
 // A CTA lives for its trips to memory, so the planner leaves, beside the member list, a header per merged row that holds the
 // run and its first sixteen members, four for each warp: one trip leads to the data.  (Run, member list and rows in three
 // dependent trips: 36 us for 121 MB of rows, 4 x 4608 tokens x 4096.)
+// P: 16-byte pieces of a row per lane; R: members a warp has in flight.
+template <int P, int R>
 __global__ void __launch_bounds__(kRowsThreads)
 merge_rows_kernel(const uint4* __restrict__ hidden, int B, int N, int dh8, int slices, int vis_start, int Nv_cap, int Mcap,
                   const MergeHeader* headers, const uint16_t* members,
                   void* __restrict__ merged_bf16, float* __restrict__ merged_f32) {
     constexpr int G = kRowsThreads / 32;                  // warps sharing the members
     static_assert(G == 4, "a header lists members for four warps");
-    __shared__ unsigned long long partial[kRowsPieces][G][32][5];      // padded against bank conflicts
+    __shared__ unsigned long long partial[P][G][32][5];      // padded against bank conflicts
     grid_dependency_wait();
     // slices of a row side by side, then the samples, then the rows in header order: the long ones of all samples come first
     const int tid = threadIdx.x, g = tid >> 5, lane = tid & 31;
@@ -397,41 +433,43 @@ merge_rows_kernel(const uint4* __restrict__ hidden, int B, int N, int dh8, int s
     const uint2 four = __ldcg(reinterpret_cast<const uint2*>(h->first[g]));
     const int count = run.x, m = run.z;
     if (count == 0) return;                               // no such merged row
-    const uint16_t* mem = members + (size_t)b * Nv_cap + run.y;
-    const int piece = slice * (32 * kRowsPieces) + lane;      // 16-byte pieces of the hidden row this lane owns: + 32 p
-    unsigned long long acc[kRowsPieces][4];               // pairs of fp32 sums
+    const uint16_t* mem = members + (size_t)b * member_stride(Nv_cap) + run.y;
+    const int piece = slice * (32 * P) + lane;      // 16-byte pieces of the hidden row this lane owns: + 32 p
+    unsigned long long acc[P][4];               // pairs of fp32 sums
 #pragma unroll
-    for (int p = 0; p < kRowsPieces; ++p)
+    for (int p = 0; p < P; ++p)
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc[p][u] = 0ull;
     {
         const uint4* src = hidden + ((size_t)b * N + vis_start) * dh8 + piece;
         uint32_t idx[4] = {four.x & 0xFFFFu, four.x >> 16, four.y & 0xFFFFu, four.y >> 16};
-        for (int r = g; r < count; r += 4 * G) {
-            uint4 v[4][kRowsPieces];
+        for (int r = g; r < count; r += R * G) {
+            uint4 v[R][P];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < R; ++u)
 #pragma unroll
-                for (int p = 0; p < kRowsPieces; ++p)
+                for (int p = 0; p < P; ++p)
                     if (r + u * G < count && piece + 32 * p < dh8) v[u][p] = ld_stream(src + (size_t)idx[u] * dh8 + 32 * p);
 #pragma unroll
-            for (int u = 0; u < 4; ++u)                   // the next four travel with the data
-                if (r + (4 + u) * G < count) idx[u] = __ldcg(mem + r + (4 + u) * G);
+            for (int u = 0; u < 4; ++u) {                 // the header's list, then the next ones, which travel with the data
+                if (R < 4 && u < 4 - R) idx[u] = idx[u + R];
+                else if (r + (4 + (u - (4 - R))) * G < count) idx[u] = __ldcg(mem + r + (4 + (u - (4 - R))) * G);
+            }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < R; ++u)
 #pragma unroll
-                for (int p = 0; p < kRowsPieces; ++p)
+                for (int p = 0; p < P; ++p)
                     if (r + u * G < count && piece + 32 * p < dh8) add8(acc[p], v[u][p]);
         }
     }
 #pragma unroll
-    for (int p = 0; p < kRowsPieces; ++p)
+    for (int p = 0; p < P; ++p)
 #pragma unroll
         for (int u = 0; u < 4; ++u) partial[p][g][lane][u] = acc[p][u];
     __syncthreads();
     // each thread finishes a pair of elements of its lane's pieces: g, so that a row is written in 4- and 8-byte words
 #pragma unroll
-    for (int p = 0; p < kRowsPieces; ++p) {
+    for (int p = 0; p < P; ++p) {
         if (piece + 32 * p >= dh8) break;
         float sum[2] = {0.f, 0.f};
 #pragma unroll
@@ -451,17 +489,18 @@ merge_rows_kernel(const uint4* __restrict__ hidden, int B, int N, int dh8, int s
 }
 
 // Dynamic shared memory of the planner: the counting pass, or the sort's two buffers and counters.
-size_t plan_smem(int Nv_cap) {
+size_t plan_smem(int Nv_cap, int E) {
     const size_t sort_bytes = 2 * (size_t)((Nv_cap + 3) & ~3) * sizeof(uint32_t) + (size_t)kCntEntries * sizeof(uint16_t);
-    return sort_bytes > plan_count_bytes(Nv_cap) ? sort_bytes : plan_count_bytes(Nv_cap);
+    const size_t count_bytes = plan_count_bytes(Nv_cap, E);
+    return sort_bytes > count_bytes ? sort_bytes : count_bytes;
 }
 
-// Workspace: status | members uint16 [B, Nv_cap] | headers [B, Mcap]
+// Workspace: status | members uint16 [B, Nv_cap rounded up to 8] | headers [B, Mcap]
 struct MergeWs {
     size_t off_members, off_headers, total;
     MergeWs(int B, int Nv_cap, int Mcap) {
         size_t o = kStatusBytes;
-        off_members = o; o += align_up((size_t)B * Nv_cap * sizeof(uint16_t), 256);
+        off_members = o; o += align_up((size_t)B * member_stride(Nv_cap) * sizeof(uint16_t), 256);
         off_headers = o; o += align_up((size_t)B * Mcap * sizeof(MergeHeader), 256);
         total = o;
     }
@@ -486,10 +525,11 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
     {
         const int v = Nv_cap <= kPlanThreads ? 0 : Nv_cap <= 4 * kPlanThreads ? 1 : Nv_cap <= 8 * kPlanThreads ? 2 : 3;
         auto kern = v == 0 ? merge_plan_kernel<1> : v == 1 ? merge_plan_kernel<4> : v == 2 ? merge_plan_kernel<8> : merge_plan_kernel<16>;
-        const size_t smem = plan_smem(Nv_cap);
+        const int E = v == 0 ? 1 : v == 1 ? 4 : v == 2 ? 8 : 16;
+        const size_t smem = plan_smem(Nv_cap, E);
         if (v > 0) {                                       // (up to 1024 tokens 19 KB)
             static DoneOnDevice attr_done[4];
-            const int rc = allow_dynamic_smem(kern, plan_smem((v == 1 ? 4 : v == 2 ? 8 : 16) * kPlanThreads), attr_done[v]);
+            const int rc = allow_dynamic_smem(kern, plan_smem(E * kPlanThreads, E), attr_done[v]);
             if (rc != VITCOP_OK) return rc;
         }
         cudaLaunchConfig_t cfg = {};
@@ -508,7 +548,14 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
     if (Mcap <= 0 || Dh <= 0 || (!merged_bf16 && !merged_f32)) return VITCOP_OK;
     const int dh8 = Dh / 8;
     cudaLaunchConfig_t cfg = {};
-    const int slices = (dh8 + 32 * kRowsPieces - 1) / (32 * kRowsPieces);
+    // Two pieces a lane halve the CTAs and their trips to the plan; a few rows keep the chip better busy cut into more CTAs.  With
+    // many CTAs and few members a row, two members in flight a warp instead of four let more CTAs share an SM.  (Pieces, members in
+    // flight; us of the kernel under event brackets.  240 CTAs of 400 members: 1,4 123, 2,4 142.  2304 of 18: 1,4 60, 2,4 70.  3712 of 16:
+    // 1,4 21, 2,4 19, 2,2 21.  7392 of 16: 1,4 35, 2,4 31, 2,2 29.  20000 of 3: 2,4 50, 2,2 39.  9600 of 44: 2,4 76, 2,2 95.)
+    const long long wide = (long long)Mcap * B * ((dh8 + 63) / 64), sms = gram_num_sms();
+    const bool few = wide < 16 * sms, shorter = !few && wide >= 28 * sms && Nv_cap <= 24LL * Mcap;
+    const int pieces = few ? 1 : 2, slices = (dh8 + 32 * pieces - 1) / (32 * pieces);
+    auto kern = few ? merge_rows_kernel<1, 4> : shorter ? merge_rows_kernel<2, 2> : merge_rows_kernel<2, 4>;
     const long long ctas = (long long)Mcap * B * slices;
     if (ctas > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
     cfg.gridDim = dim3((unsigned)ctas);
@@ -517,7 +564,7 @@ int launch_merge(const void* hidden, int B, int N, int Dh, int vis_start, const 
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
     KernelTimeScope timed("merge_rows_kernel", stream);
-    return record_cuda(cudaLaunchKernelEx(&cfg, merge_rows_kernel, static_cast<const uint4*>(hidden), B, N, dh8, slices,
+    return record_cuda(cudaLaunchKernelEx(&cfg, kern, static_cast<const uint4*>(hidden), B, N, dh8, slices,
                                           vis_start, Nv_cap, Mcap, (const MergeHeader*)headers, (const uint16_t*)members, merged_bf16,
                                           merged_f32));
 }

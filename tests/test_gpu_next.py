@@ -103,6 +103,21 @@ def test_merge_planner_cluster_line(n, clusters):
     _check_merge(hid, vs, np.array([n, n, 0], dtype=np.int32), label, keep, min(n, 900))
 
 
+# The same line for longer samples (512 and 1024 clusters), and rows enough for the kernel that has two members in flight a warp,
+# with fewer merged rows than clusters and with ragged slices of the hidden row.
+@pytest.mark.parametrize("n,clusters,Dh,Mcap", [(4097, 512, 64, 600), (5000, 513, 520, 900), (8200, 1024, 64, 1100),
+                                                (9000, 1025, 520, 1100), (8200, 900, 520, 700)])
+def test_merge_planner_cluster_line_long(n, clusters, Dh, Mcap):
+    rng = np.random.default_rng(n + clusters)
+    B, vs = 3, 2
+    hid = W.f32_to_bf16_bits(rng.standard_normal((B, n + vs, Dh)).astype(np.float32))
+    ids = np.sort(rng.choice(n, size=clusters, replace=False)).astype(np.int32)
+    label = np.concatenate([np.broadcast_to(ids, (B, clusters)), ids[rng.integers(0, clusters, size=(B, n - clusters))]], 1)
+    label = rng.permuted(label, axis=1).astype(np.int32)
+    keep = (rng.random((B, n)) < 0.02).astype(np.uint8)
+    _check_merge(hid, vs, np.array([n, n - 3, 0], dtype=np.int32), np.minimum(label, n - 4), keep, Mcap)
+
+
 def test_merge_label_out_of_range_is_clamped():
     rng = np.random.default_rng(11)
     n, Dh = 100, 64
