@@ -189,6 +189,51 @@ select_quota_kernel(const float* score, const int32_t* label,
                          keep_mask, status_word, blockIdx.x / R);
 }
 
+typedef void (*QuotaKernel)(const float*, const int32_t*, const int32_t*, int, int, int, int, int32_t*, int, int32_t*, uint8_t*, int*);
+QuotaKernel quota_kernel(int R, int E) {
+    return E == 1   ? select_quota_kernel<1, 1>
+           : E == 2 ? select_quota_kernel<1, 2>
+           : E == 4 ? (R == 1 ? select_quota_kernel<1, 4> : select_quota_kernel<4, 4>)
+           : E == 8 ? (R == 1 ? select_quota_kernel<1, 8> : select_quota_kernel<4, 8>)
+           : R == 1 ? select_quota_kernel<1, 16> : R == 4 ? select_quota_kernel<4, 16> : select_quota_kernel<8, 16>;
+}
+size_t quota_most_smem(int E) {
+    int p = 0;
+    return select_quota_smem(E * kSelThreads, &p);
+}
+int quota_allow_smem(int R, int E) {
+    static DoneOnDevice attr_done[9][17];
+    return allow_dynamic_smem(quota_kernel(R, E), quota_most_smem(E), attr_done[R][E]);
+}
+// How many clusters of R CTAs (an SM each) the device runs at a time: not SMs / R, because a cluster stays inside a group of SMs.
+// Beyond that the clusters behind wait for a whole selection: 16 x 16384 tokens 45 us on clusters of eight, 26 on clusters of four;
+// 40 x 2880 20 us on clusters of four, 13 on single CTAs.  0 if it cannot be told.
+int quota_clusters_at_once(int R, int E) {
+    static std::atomic<int> known[kMaxDevices][9][17];     // number + 1
+    std::atomic<int>& k = known[current_device()][R][E];
+    int v = k.load(std::memory_order_relaxed);
+    if (v == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)R);
+        cfg.blockDim = dim3(kSelThreads);
+        cfg.dynamicSmemBytes = quota_most_smem(E);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)R;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (quota_allow_smem(R, E) != VITCOP_OK || cudaOccupancyMaxActiveClusters(&n, quota_kernel(R, E), &cfg) != cudaSuccess || n < 0) {
+            cudaGetLastError();
+            n = 0;
+        }
+        v = n + 1;
+        k.store(v, std::memory_order_relaxed);
+    }
+    return v - 1;
+}
+
 }  // namespace
 
 int launch_select(const float* score, const int32_t* label, int B, const int32_t* vis_len, int vis_len_uniform,
@@ -218,19 +263,14 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
     }
     int P = 0;
     const size_t smem = select_quota_smem(Nv_cap, &P);
-    // CTAs per sequence: one up to 2048 tokens (the others would be done preparing when the first is done), four, and eight
-    // beyond 8192
-    const int R = Nv_cap <= 2 * kSelThreads ? 1 : Nv_cap <= 8 * kSelThreads ? 4 : 8;
     const int E = Nv_cap <= kSelThreads ? 1 : Nv_cap <= 2 * kSelThreads ? 2 : Nv_cap <= 4 * kSelThreads ? 4 : Nv_cap <= 8 * kSelThreads ? 8 : 16;
-    auto kern = E == 1   ? select_quota_kernel<1, 1>
-                : E == 2 ? select_quota_kernel<1, 2>
-                : E == 4 ? select_quota_kernel<4, 4>
-                : E == 8 ? select_quota_kernel<4, 8> : select_quota_kernel<8, 16>;
-    static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kSelThreads, "tokens of the longest sample");
+    // CTAs per sequence: one up to 2048 tokens (the others would be done preparing when the first is done), four, and eight
+    // beyond 8192; fewer where the batch would not be on the chip at once
+    int R = E <= 2 ? 1 : E <= 8 ? 4 : 8;
+    while (R > 1 && B > quota_clusters_at_once(R, E)) R = R == 8 ? 4 : 1;
+    auto kern = quota_kernel(R, E);
     {
-        static DoneOnDevice attr_done[17];
-        int most_p = 0;
-        const int rc = allow_dynamic_smem(kern, select_quota_smem(E * kSelThreads, &most_p), attr_done[E]);
+        const int rc = quota_allow_smem(R, E);
         if (rc != VITCOP_OK) return rc;
     }
     cudaLaunchAttribute attrs[2];

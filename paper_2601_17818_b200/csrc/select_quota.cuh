@@ -76,8 +76,15 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
 //             whole histogram bin is wanted, the loop when all clusters have stopped.
 constexpr int kMaxSeg = 1024;
 constexpr uint32_t kSegDone = 0xFFFFFFFFu;
-constexpr int kRankWork = 64;                             // rank search when sum |C_c|^2 <= kRankWork * n per CTA ...
-constexpr int kRankMaxSize = 2048;                        // ... and no searched cluster is larger than this
+// The rank search is taken when no searched cluster is larger than kRankMaxSize and the comparisons of the busiest CTA are few enough:
+// a million of them take 28 us, and the other searches on 2880 / 4608 / 8192 / 16384 tokens 18 / 8 / 10 / 20 us longer than what is
+// left of the rank search.  (Counting all comparisons against 64 n per CTA of the cluster, as if they were shared out evenly, took
+// uneven clusters to the rank search: 8 x 8192 tokens 47 us instead of 27, 32 x 16384 160 instead of 47.)  A CTA of several ranks the
+// segments that start in its n / R positions, so it has at most (n / R + largest) * largest, and at most all of them.
+constexpr int kRankWork = 64;                             // of one CTA, times n
+constexpr int kRankPart = 64;                             // of one of several, times n ...
+constexpr int kRankPartSort = 3 << 18;                    // ... on samples that would be sorted otherwise this
+constexpr int kRankMaxSize = 2048;
 constexpr int kRadixMinTokens = 4096;                     // below this a sort beats the radix passes (fewer barriers)
 
 // Writes the tokens whose flag is set in keepf[0..n) to keep_idx in ascending order (every thread scans a run of
@@ -144,7 +151,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
     uint32_t* quota = reinterpret_cast<uint32_t*>(smem + L.off_quota);
     uint32_t* csize = reinterpret_cast<uint32_t*>(smem + L.off_csize);
     uint32_t* offs = reinterpret_cast<uint32_t*>(smem + L.off_offs);
-    uint32_t* misc = reinterpret_cast<uint32_t*>(smem + L.off_misc);   // min key, max key, rank work, rank veto
+    uint32_t* misc = reinterpret_cast<uint32_t*>(smem + L.off_misc);   // min key, max key, comparisons, largest searched cluster
     uint16_t* id_of = reinterpret_cast<uint16_t*>(smem + L.off_id);
     uint8_t* keepf = smem + L.off_keep;
     const int tid = threadIdx.x;
@@ -242,7 +249,7 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
         return true;
     }
     {
-        uint32_t size = 0, work = 0, veto = 0;
+        uint32_t size = 0, work = 0, largest = 0;
         if (tid < (int)n_seg) {
             size = csize[tid];
             // (a budget of n or more keeps every cluster whole, as n does: the product fits 32 bits)
@@ -251,21 +258,28 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
             const bool searched = q > 0 && q < size;                 // none or all of a cluster: nothing to search
             krem[tid] = searched ? q : kSegDone;
             if (searched) {
-                veto = size > (uint32_t)kRankMaxSize ? 1u : 0u;
-                work = veto ? 0u : size * size;
+                largest = size;
+                work = size > (uint32_t)kRankMaxSize ? 0u : size * size;
             }
         }
         work = __reduce_add_sync(0xffffffffu, work);
-        veto = __reduce_or_sync(0xffffffffu, veto);
-        if ((tid & 31) == 0 && (work | veto)) {
+        largest = __reduce_max_sync(0xffffffffu, largest);
+        if ((tid & 31) == 0 && largest) {
             atomicAdd(&misc[2], min(work, 0x0FFFFFFFu));             // 32 sizes of at most 2048: below 2^27
-            atomicOr(&misc[3], veto);
+            atomicMax(&misc[3], largest);
         }
         uint32_t total;
         const uint32_t o = block_exclusive_sum(size, warp_sums, total);   // its barriers publish misc as well
         if (tid < (int)n_seg) offs[tid] = o;
     }
-    const bool by_rank = misc[3] == 0 && (unsigned long long)misc[2] <= (unsigned long long)(kRankWork * R) * (unsigned)n;
+    const uint32_t largest = misc[3], all = misc[2];
+    bool by_rank = largest <= (uint32_t)kRankMaxSize;
+    if (R == 1) {
+        by_rank = by_rank && all <= (uint32_t)kRankWork * (uint32_t)n;
+    } else {
+        const uint32_t part = min(all, ((uint32_t)(n / R) + largest) * min(largest, (uint32_t)kRankMaxSize));
+        by_rank = by_rank && part <= (n <= kRadixMinTokens ? (uint32_t)kRankPartSort : (uint32_t)kRankPart * (uint32_t)n);
+    }
     const uint32_t range_lo = misc[0], range_hi = misc[1];
     if (!by_rank && n <= kRadixMinTokens) return false;    // uniform; nothing has been written yet
     if (!by_rank && part != 0) return true;

@@ -157,6 +157,18 @@ def test_select_quota_span_edges(n):
             assert np.array_equal(keeps[b], want), (n, ncl, skew)
 
 
+# Batches that leave a sequence one CTA, four or eight; even and uneven clusters (searched by rank, by radix or sorted).
+@pytest.mark.parametrize("n,B", [(2500, 40), (5000, 40), (9000, 3), (9000, 20), (9000, 40)])
+def test_select_quota_batches(n, B):
+    score = W.make_scores(n, B, n, "ties")
+    label = np.concatenate([W.make_labels(n + b, 1, n, max(2, n // (20 if b % 2 else 100)), skew=0.3 * (b % 4)) for b in range(B)])
+    keeps, nk, _, status = gpu_select(score, n // 4, label=label)
+    assert status == vb.OK
+    for b in range(B):
+        want, _, _ = oracle.select_quota(score[b].astype(np.float64), label[b], n // 4)
+        assert np.array_equal(keeps[b], want), b
+
+
 # Spans around the numbers of tokens per thread; more than 256 scores equal to the one at the cut, on either side of it.
 @pytest.mark.parametrize("n", [1023, 1024, 1025, 4096, 4097, 8192, 8193, 16384])
 def test_select_plain_span_edges(n):
