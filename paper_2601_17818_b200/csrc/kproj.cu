@@ -4,23 +4,25 @@
 // that a stand-alone K-norm costs (the largest byte term of a pruning step) disappears.
 //
 //   A = hidden [B * N, Dh] (rows = tokens), B = W_k [H * d, Dh] (rows = output features, as a linear layer stores its
-//   weight): both K-major, so D = A * B^T needs no transposition.  Output tile 256 tokens x 256 features.
+//   weight): both K-major, so D = A * B^T needs no transposition.  Output tile 256 tokens x 256 features, or 128 x 256.
 //
-// Bound by the tensor cores at the clock that the power limit leaves.  Persistent clusters of two CTAs, one CTA per SM, each cluster on one tile at a time (tcgen05 cta_group::2): a CTA stages
-// its 128 token rows and its half of the weight rows, 32 KB per k-block where two CTAs working apart would each stage 48 KB,
-// so six k-blocks fit and a third of the operand traffic from the L2 goes (16 x 640 tokens x 4096 -> 4096 back to back,
-// rotary on: 304 us with CTAs working apart, 275 us so; cuBLAS in a sustained loop: 253).  Warp-specialised like the Gram sweep: warp 0
-// loads, one thread of the leader's warp 1 issues the MMAs into one of two accumulators, 8 epilogue warps of each CTA drain
-// the other: a thread owns one token row (its TMEM lane), the two warps of a lane quarter share the row's 256 columns.  Per
-// 32-column chunk a thread rounds the values to bf16 (round to nearest even), stores them (64 contiguous bytes of
-// K[b, h, t, :]) and adds their squares -- of the ROUNDED values, i.e. Eq. 4 of the K cache as written -- to the row's fp32
-// partial sum.  With rotary embedding the chunks holding the two halves of a head are taken together and turned first.
-// Partial sums go to one slot per 128 columns and are added by a second, tiny kernel in slot order (the same bits on every
-// run).
+// Bound by the tensor cores at the clock that the power limit leaves.  Persistent clusters of two CTAs, one CTA per SM, each
+// cluster on one tile at a time (tcgen05 cta_group::2): a CTA stages its 128 token rows and its half of the weight rows, 32 KB
+// per k-block where two CTAs working apart would each stage 48 KB, so six k-blocks fit and a third of the operand traffic from
+// the L2 goes (16 x 640 tokens x 4096 -> 4096 back to back, rotary on: 304 us with CTAs working apart, 275 us so; cuBLAS in a
+// sustained loop: 253).  CTAs working apart, on 128 x 256 tiles, where that is the shorter way (the rule is in
+// launch_kproj_knorm).
+// Warp-specialised like the Gram sweep: warp 0 loads, one thread of the leader's warp 1 issues the MMAs into one of two
+// accumulators, 8 epilogue warps of each CTA drain the other: a thread owns one token row (its TMEM lane), the two warps of a lane
+// quarter share the row's 256 columns.  Per 32-column chunk a thread rounds the values to bf16 (round to nearest even), stores
+// them (64 contiguous bytes of K[b, h, t, :]) and adds their squares -- of the ROUNDED values, i.e. Eq. 4 of the K cache as
+// written -- to the row's fp32 partial sum.  With rotary embedding the chunks holding the two halves of a head are taken together
+// and turned first.  Partial sums go to one slot per 128 columns and are added by a second, tiny kernel in slot order (the same
+// bits on every run and with either tile).
 // When the last round of tiles would occupy at most half of the clusters, its tiles are cut into two of 128 features each
 // (the MMA keeps its rate at N = 128 with two CTAs), so that the round takes half as long
-// (2 x 16512 tokens x 3584 -> 512: 3.5 rounds instead of 4; 121 us before, 113 now).
-// Every wait is bounded; on expiry both CTAs of the cluster leave in order and the call reports VITCOP_ERR_TIMEOUT.
+// (2 x 16512 tokens x 3584 -> 512: 3.5 rounds instead of 4; 121 us before, 117 now).
+// Every wait is bounded; on expiry all CTAs of the cluster leave in order and the call reports VITCOP_ERR_TIMEOUT.
 #include "async_copy.cuh"
 #include "gram.cuh"
 #include "tcgen05.cuh"
@@ -29,16 +31,17 @@ namespace vitcop {
 namespace {
 
 constexpr int BM = 128, BN = 256;                 // rows of one CTA, columns of the cluster's tile
-constexpr int kStages = 6;
-constexpr int kBoxRows = 64;                      // weight rows per load: a CTA stages one or two boxes
-constexpr int kABytes = BM * BK * 2, kBBytes = BN / 2 * BK * 2, kStageBytes = kABytes + kBBytes;
+constexpr int kABytes = BM * BK * 2;
+__host__ __device__ constexpr int stages(int ctas) { return ctas == 2 ? 6 : 4; }      // (192 KB either way)
+__host__ __device__ constexpr int stage_bytes(int ctas) { return kABytes + BN / ctas * BK * 2; }
 constexpr int kEpiWarps = 8, kEpiThreads = kEpiWarps * 32, kThreads = 64 + kEpiThreads;
-constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 256;
+constexpr int kSmemBytes = 1024 + stages(2) * stage_bytes(2) + 256;
+static_assert(stages(1) * stage_bytes(1) == stages(2) * stage_bytes(2), "shared memory of either form");
 
 struct KprojArgs {
     int B, N, Dh, H, d;
     int M, NO;                      // rows of A (B * N), output features (H * d)
-    int TI, TJ;                     // tiles of 256 rows, of 256 columns
+    int TI, TJ;                     // tiles of 128 rows per CTA of a cluster, of 256 columns
     int n_full;                     // tiles taken whole; the others are cut into two column halves
     uint16_t* K_out;                // bf16 [B, H, N, d]
     float* part;                    // [2 TJ, M] sum of squares of a token's values inside 128 columns
@@ -92,10 +95,13 @@ __device__ __forceinline__ KprojItem decode_item(const KprojArgs& k, int t) {
     return it;
 }
 
-template <bool ROPE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const KprojArgs k,
-             const int n_items) {
+// CTAS: CTAs of a cluster, 2 or 1 (one form of the tcgen05 instructions per kernel).
+template <bool ROPE, int CTAS>
+__global__ void __launch_bounds__(kThreads, 1)
+kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+             const __grid_constant__ CUtensorMap map_half, const KprojArgs k, const int n_items) {
+    constexpr bool kPair = CTAS == 2;
+    constexpr int kStages = stages(CTAS), kStageBytes = stage_bytes(CTAS);
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;
@@ -110,8 +116,8 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     const uint32_t abort_addr = smem_u32(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t kTmemCols = 2 * BN;
-    const uint32_t rank = cluster_ctarank();
-    const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
+    const uint32_t rank = kPair ? cluster_ctarank() : 0u;
+    const int cluster = blockIdx.x / CTAS, n_clusters = gridDim.x / CTAS;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -120,7 +126,7 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(bar_tfull + 8 * a, 1);
-            mbar_init(bar_tempty + 8 * a, 2 * kEpiWarps);
+            mbar_init(bar_tempty + 8 * a, CTAS * kEpiWarps);
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
@@ -128,10 +134,13 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
     }
-    if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+    if (warp == 1) {
+        if constexpr (kPair) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+        else tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+    }
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();                                    // both CTAs' barriers and tensor memory are ready
+    if constexpr (kPair) cluster_sync_all();               // both CTAs' barriers and tensor memory are ready
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
@@ -148,17 +157,22 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             bool ok = true;
             for (int t = cluster; ok && t < n_items; t += n_clusters) {
                 const KprojItem it = decode_item(k, t);
-                const int row = (it.ti * 2 + (int)rank) * BM;
-                const int col = it.col0 + (int)rank * it.halves * kBoxRows;
-                const uint32_t bytes = 2u * (uint32_t)(kABytes + it.halves * (kBBytes / 2));      // both CTAs
+                const int row = (it.ti * CTAS + (int)rank) * BM;
+                const int cols = it.halves * (BN / 2 / CTAS), col = it.col0 + (int)rank * cols;       // weight rows that this CTA stages
+                const CUtensorMap* const mb = it.halves == 2 ? &map_b : &map_half;         // (one load whatever their number)
+                const uint32_t bytes = (uint32_t)(CTAS * (kABytes + cols * BK * 2));       // of all CTAs
                 for (int kb = 0; kb < KB; ++kb) {
                     if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
                     const uint32_t sa = tiles + stage * kStageBytes;
-                    const uint32_t full = cluster_map(bar_full + 8 * stage, 0);
                     if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, bytes);    // rows outside the tensors arrive as zeros
-                    tma_load_3d_pair(sa, &map_a, full, kb * BK, row, 0);
-                    tma_load_3d_pair(sa + kABytes, &map_b, full, kb * BK, col, 0);
-                    if (it.halves == 2) tma_load_3d_pair(sa + kABytes + kBBytes / 2, &map_b, full, kb * BK, col + kBoxRows, 0);
+                    if constexpr (kPair) {
+                        const uint32_t full = cluster_map(bar_full + 8 * stage, 0);
+                        tma_load_3d_pair(sa, &map_a, full, kb * BK, row, 0);
+                        tma_load_3d_pair(sa + kABytes, mb, full, kb * BK, col, 0);
+                    } else {
+                        tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, row, 0);
+                        tma_load_3d(sa + kABytes, mb, bar_full + 8 * stage, kb * BK, col, 0);
+                    }
                     issued |= 1u << stage;
                     issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -169,12 +183,16 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim);
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) raise_abort_pair(abort_addr, rank);
+            if (kPair && !ok) raise_abort_pair(abort_addr, rank);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
-            constexpr uint32_t idesc_full = umma_idesc_bf16(2 * BM, BN), idesc_half = umma_idesc_bf16(2 * BM, BN / 2);
+            constexpr uint32_t idesc_full = umma_idesc_bf16(CTAS * BM, BN), idesc_half = umma_idesc_bf16(CTAS * BM, BN / 2);
             const unsigned long long lim = k.limit_of(2);
+            auto commit = [](uint32_t bar) {
+                if constexpr (kPair) tc_commit_pair(bar);
+                else tc_commit(bar);
+            };
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
             for (int t = cluster; ok && t < n_items; t += n_clusters) {
@@ -188,18 +206,20 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                     const uint32_t sa = tiles + stage * kStageBytes;
                     const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + kABytes);
 #pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        tc_mma_bf16_pair(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
-                                         (kb > 0 || kk > 0) ? 1u : 0u);
-                    tc_commit_pair(bar_empty + 8 * stage);
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk) {
+                        const uint32_t add = (kb > 0 || kk > 0) ? 1u : 0u;
+                        if constexpr (kPair) tc_mma_bf16_pair(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc, add);
+                        else tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc, add);
+                    }
+                    commit(bar_empty + 8 * stage);
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                tc_commit_pair(bar_tfull + 8 * acc);
+                commit(bar_tfull + 8 * acc);
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-            if (!ok) raise_abort_pair(abort_addr, rank);
-            tc_commit_pair(bar_drain);                     // (waited for below)
+            if (kPair && !ok) raise_abort_pair(abort_addr, rank);
+            commit(bar_drain);                     // (waited for below)
         }
     } else {
         // ------------------------------------------------------------------ epilogue
@@ -210,7 +230,7 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         bool ok = true;
         for (int t = cluster; ok && t < n_items; t += n_clusters) {
             const KprojItem it = decode_item(k, t);
-            const int m = (it.ti * 2 + (int)rank) * BM + rl;       // token row of this thread
+            const int m = (it.ti * CTAS + (int)rank) * BM + rl;       // token row of this thread
             const bool row_valid = m < k.M;
             const int b = row_valid ? m / k.N : 0, tok = row_valid ? m - b * k.N : 0;
             ok = mbar_wait(bar_tfull + 8 * acc, acc_phase, abort_flag, k.limit_of(4));
@@ -268,10 +288,13 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(cluster_map(bar_tempty + 8 * acc, 0));
+            if (lane == 0) {
+                if constexpr (kPair) mbar_arrive_cluster(cluster_map(bar_tempty + 8 * acc, 0));
+                else mbar_arrive(bar_tempty + 8 * acc);
+            }
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-        if (!ok && lane == 0) raise_abort_pair(abort_addr, rank);
+        if (kPair && !ok && lane == 0) raise_abort_pair(abort_addr, rank);
     }
 
     __syncthreads();
@@ -292,10 +315,11 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();                                    // neither CTA leaves while the other may reach into it
+    if constexpr (kPair) cluster_sync_all();               // neither CTA leaves while the other may reach into it
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc_pair(tmem_base, kTmemCols);
+        if constexpr (kPair) tmem_dealloc_pair(tmem_base, kTmemCols);
+        else tmem_dealloc(tmem_base, kTmemCols);
     }
     grid_dependency_launch_dependents();
 }
@@ -313,6 +337,24 @@ __global__ void kproj_score_kernel(const float* __restrict__ part, int M, int sl
     score[(size_t)b * Nv + i] = sqrtf(s);
 }
 
+// Tiles of 128 rows per CTA x 256 columns on clusters of `ctas` CTAs, those of a last round that would occupy at most half of the
+// clusters cut in two.
+struct TileSplit {
+    int TI, units;                  // row tiles; clusters at work together
+    long long total, cut;
+    double rounds;                  // until the last is done, a cut tile counting half
+};
+TileSplit split_tiles(int M, int TJ, int ctas, bool may_cut) {
+    TileSplit s;
+    s.TI = (int)(((long long)M + ctas * BM - 1) / (ctas * BM));
+    s.units = gram_num_sms() / ctas > 0 ? gram_num_sms() / ctas : 1;
+    s.total = (long long)s.TI * TJ;
+    const long long last = s.total % s.units;
+    s.cut = 2 * last <= s.units && may_cut ? last : 0;
+    s.rounds = (double)(s.total / s.units) + (last == 0 ? 0.0 : s.cut ? 0.5 : 1.0);
+    return s;
+}
+
 }  // namespace
 
 size_t kproj_workspace_bytes(int B, int N, int H, int d) {
@@ -326,39 +368,51 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     KprojArgs k = {};
     k.B = B; k.N = N; k.Dh = Dh; k.H = H; k.d = d;
     k.M = B * N; k.NO = H * d;
-    k.TI = (k.M + 2 * BM - 1) / (2 * BM); k.TJ = (k.NO + BN - 1) / BN;
+    k.TJ = (k.NO + BN - 1) / BN;
     k.K_out = static_cast<uint16_t*>(K_out);
     k.part = reinterpret_cast<float*>(static_cast<char*>(workspace) + kStatusBytes);
     k.cos_tab = cos_tab; k.sin_tab = sin_tab; k.position = position; k.n_pos = n_pos;
     k.status = static_cast<int*>(workspace);
     k.wait_ns = gram_wait_limit_ns();
     k.expire_roles = pair_expire_roles();
-    const long long total = (long long)k.TI * k.TJ;
-    if (total <= 0) return VITCOP_OK;
-    CUtensorMap ma, mb;
-    if (!make_rowmajor_bf16_map(&ma, hidden, 1, k.M, Dh, BM) || !make_rowmajor_bf16_map(&mb, W, 1, k.NO, Dh, kBoxRows))
-        return VITCOP_ERR_CUDA;
+    if (k.M <= 0 || k.NO <= 0) return VITCOP_OK;
     const bool rope = cos_tab != nullptr;
-    auto kern = rope ? kproj_kernel<true> : kproj_kernel<false>;
-    static DoneOnDevice attr_done[2];
-    const int arc = allow_dynamic_smem(kern, kSmemBytes, attr_done[rope]);
+    // (a rotated head of 256 columns cannot be cut: its halves are turned together)
+    const bool may_cut = !(rope && d > BN / 2);
+    const TileSplit two = split_tiles(k.M, k.TJ, 2, may_cut), one = split_tiles(k.M, k.TJ, 1, may_cut);
+    // CTAs apart take a tenth longer for a full round, but their rounds are finer: 1152 tokens x 4096 -> 4096 are 144 tiles of 128
+    // rows, one round, and 80 of 256 rows, one and a half (30.9 and 48.6 us).  Inside one round they are done sooner up to
+    // Dh = 4096 (9000 tokens x 3584 -> 512: 28.7 and 30.8 us; 640 x 8192 -> 4096: 53 and 47): pairs start and stop 2 us slower.
+    const bool pair = !(one.rounds * 1.1 < two.rounds || (one.rounds == two.rounds && two.rounds <= 1.0 && Dh <= 4096));
+    const TileSplit& split = pair ? two : one;
+    if (split.total + split.cut > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
+    k.TI = split.TI;
+    k.n_full = (int)(split.total - split.cut);
+    const int n_items = (int)(split.total + split.cut), units = split.units;
+    const int ctas = pair ? 2 : 1;
+    CUtensorMap ma, mb, mh;
+    if (!make_rowmajor_bf16_map(&ma, hidden, 1, k.M, Dh, BM) || !make_rowmajor_bf16_map(&mb, W, 1, k.NO, Dh, BN / ctas) ||
+        !make_rowmajor_bf16_map(&mh, W, 1, k.NO, Dh, BN / 2 / ctas))
+        return VITCOP_ERR_CUDA;
+    auto kern = pair ? (rope ? kproj_kernel<true, 2> : kproj_kernel<false, 2>) : (rope ? kproj_kernel<true, 1> : kproj_kernel<false, 1>);
+    static DoneOnDevice attr_done[2][2];
+    const int arc = allow_dynamic_smem(kern, kSmemBytes, attr_done[pair][rope]);
     if (arc != VITCOP_OK) return arc;
     cudaLaunchConfig_t cfg = {};
-    const long long pairs = gram_num_sms() / 2 > 0 ? gram_num_sms() / 2 : 1;
-    if (2 * total > 0x7fffffffLL) return VITCOP_ERR_UNSUPPORTED;
-    // (a rotated head of 256 columns cannot be cut: its halves are turned together)
-    const long long last = total % pairs;
-    const long long cut = (2 * last <= pairs && !(rope && d > BN / 2)) ? last : 0;
-    k.n_full = (int)(total - cut);
-    const int n_items = (int)(total + cut);
-    cfg.gridDim = dim3((unsigned)(2 * (n_items < pairs ? n_items : pairs)));
+    cfg.gridDim = dim3((unsigned)(ctas * (n_items < units ? n_items : units)));
+    cudaLaunchAttribute shape[1];
+    shape[0].id = cudaLaunchAttributeClusterDimension;
+    shape[0].val.clusterDim.x = (unsigned)ctas;
+    shape[0].val.clusterDim.y = shape[0].val.clusterDim.z = 1;
+    cfg.attrs = shape;
+    cfg.numAttrs = pair ? 1 : 0;
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
     int rc;
     {
         KernelTimeScope timed("kproj_kernel", stream);
-        rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k, n_items));
+        rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, mh, k, n_items));
     }
     if (rc != VITCOP_OK || Nv <= 0 || !score) return rc;
     cudaLaunchAttribute attr[1];

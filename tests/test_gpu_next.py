@@ -272,6 +272,14 @@ def test_kproj_knorm_tile_split(B, N, Dh, H, d, rope):
     _kproj_case(B, N, Dh, H, d, rope, vis_start=7, Nv=N - 19, rows=40, seed=N)
 
 
+# CTAs apart (one round of tiles of 128 rows: all cut, whole, with a ragged last row block) and in pairs, on the same sizes where
+# only the length of a row differs.
+@pytest.mark.parametrize("B,N,Dh,H,d,rope", [(1, 130, 64, 2, 64, False), (3, 1500, 64, 12, 64, True), (1, 1152, 128, 8, 256, True),
+                                              (1, 1100, 128, 32, 128, True), (1, 130, 4160, 2, 64, True), (1, 700, 4160, 32, 64, False)])
+def test_kproj_knorm_cluster_sizes(B, N, Dh, H, d, rope):
+    _kproj_case(B, N, Dh, H, d, rope, vis_start=3, Nv=N - 11, rows=40, seed=N)
+
+
 def test_kproj_knorm_identity_weights_and_text_only_span():
     # W = I: K is the hidden row cut into heads, bit for bit, and the score is Eq. 4 of the input
     rng = np.random.default_rng(3)
