@@ -36,6 +36,13 @@ EXPORTS = [
     "vitcop_collaborative_step", "vitcop_set_wait_limit", "vitcop_kproj_knorm",
 ]
 
+# the calls of a pruning step, which go through _call.so
+NATIVE = [
+    "vitcop_redundancy_filter", "vitcop_similarity_rows", "vitcop_knorm_score", "vitcop_select", "vitcop_compact_kv",
+    "vitcop_prune_step", "vitcop_prune_step_static", "vitcop_merge_clusters", "vitcop_cls_saliency",
+    "vitcop_collaborative_step", "vitcop_kproj_knorm",
+]
+
 
 class VitcopError(RuntimeError):
     def __init__(self, status: int, where: str):
@@ -61,7 +68,7 @@ class SelectParams(C.Structure):
 
 _lib: Optional[C.CDLL] = None
 _native = None                                   # _call.so's function
-_address: dict = {}                              # entry point -> address
+_address: dict = {}                              # entry point -> its handle there
 _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
@@ -127,12 +134,14 @@ def lib() -> C.CDLL:
         L.vitcop_kernel_timing_begin.argtypes = []
         L.vitcop_kernel_timing_end.argtypes = [C.POINTER(KernelTime), i32, C.POINTER(C.c_int)]
         for name in EXPORTS:
-            _address[name] = C.cast(getattr(L, name), C.c_void_p).value
+            getattr(L, name)
         if not os.path.exists(CALL_PATH):
             raise ImportError(f"{CALL_PATH} is missing: run `python -m paper_2601_17818_b200.build` first")
         loader = importlib.machinery.ExtensionFileLoader("_call", CALL_PATH)
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_call", loader))
         loader.exec_module(module)
+        for name in NATIVE:
+            _address[name] = module.bind(name, C.cast(getattr(L, name), C.c_void_p).value)
         _native = module.call
         _lib = L
     return _lib

@@ -44,7 +44,7 @@ def _build_caller() -> None:
     libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
     tmp = CALL + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           *inc, os.path.join(CSRC, "call.cpp"), "-o", tmp, "-L", libdir, "-lc10", "-ltorch_cpu", "-ltorch_python"]
+           *inc, "-I", INCLUDE, os.path.join(CSRC, "call.cpp"), "-o", tmp, "-L", libdir, "-lc10", "-ltorch_cpu", "-ltorch_python"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode:
         sys.stderr.write(f"$ {' '.join(cmd)}\n{r.stdout}{r.stderr}")

@@ -65,6 +65,25 @@ def test_native_caller_rejects_what_it_cannot_pass(L, arg, error):
         vb._native(vb._address["vitcop_select"], 0.0, *[0] * 40)
 
 
+def test_native_caller_calls_every_entry_point_by_its_type(L):
+    """Each with as many words as it has parameters (the float of the saliency travels apart), neither more nor fewer, and
+    whatever the host's calling convention."""
+    text = open(os.path.join(ROOT, "include", "vitcop.h")).read()
+    text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+    for name in vb.NATIVE:
+        params = re.search(r"\bint\s+" + name + r"\s*\(([^)]*)\)", text).group(1).split(",")
+        words = sum(not p.strip().startswith("float scale") for p in params)
+        refused = (vb.ERR_INVALID_ARG, vb.ERR_CUDA) if name == "vitcop_prune_step_static" else (vb.ERR_INVALID_ARG,)
+        assert vb._native(vb._address[name], 0.5, *[0] * words) in refused, name       # (the static step looks its scratch up first)
+        for wrong in (words - 1, words + 1):
+            with pytest.raises(TypeError):
+                vb._native(vb._address[name], 0.5, *[0] * wrong)
+    source = open(os.path.join(ROOT, "paper_2601_17818_b200", "csrc", "call.cpp")).read()
+    assert "__x86_64__" not in source and "#error" not in source
+    with pytest.raises(ValueError):
+        vb._native(len(vb.NATIVE), 0.0)
+
+
 @pytest.mark.parametrize("op", [vb.OP_FILTER, vb.OP_COLLAB_STEP])
 def test_a_workspace_of_a_larger_problem_serves_a_smaller_one(L, op):
     sizes = [1, 64, 127, 128, 129, 576, 577, 1408, 1409, 1536, 2048, 2880, 4608, 8191, 8192, 12000, 16384]
