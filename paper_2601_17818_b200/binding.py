@@ -4,7 +4,7 @@ Argument marshalling only: every function takes torch CUDA tensors (or ``None``)
 data pointers and the current CUDA stream to the C ABI and raises ``VitcopError`` on a non-zero
 status.  No arithmetic of the method happens here, and there is no fallback: if the shared
 library is missing or fails to load, importing the functions raises.  The calls of a pruning step
-go through ``_call.so`` (csrc/call.cpp), the diagnostic and host-only ones through ctypes.
+go through a CPython extension (csrc/call.cpp), the diagnostic and host-only ones through ctypes.
 """
 from __future__ import annotations
 
@@ -18,9 +18,10 @@ from typing import Optional
 
 import torch
 
+from . import build
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libvitcop.so")
-CALL_PATH = os.path.join(_PKG, "_call.so")
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_BUDGET, ERR_CUDA, ERR_TIMEOUT = range(7)
 (OP_FILTER, OP_KNORM, OP_SELECT, OP_COMPACT, OP_PRUNE_STEP, OP_SIMILARITY, OP_SALIENCY, OP_MERGE, OP_COLLAB_STEP,
@@ -36,7 +37,7 @@ EXPORTS = [
     "vitcop_collaborative_step", "vitcop_set_wait_limit", "vitcop_kproj_knorm",
 ]
 
-# the calls of a pruning step, which go through _call.so
+# the calls of a pruning step, which go through the extension
 NATIVE = [
     "vitcop_redundancy_filter", "vitcop_similarity_rows", "vitcop_knorm_score", "vitcop_select", "vitcop_compact_kv",
     "vitcop_prune_step", "vitcop_prune_step_static", "vitcop_merge_clusters", "vitcop_cls_saliency",
@@ -67,7 +68,7 @@ class SelectParams(C.Structure):
 
 
 _lib: Optional[C.CDLL] = None
-_native = None                                   # _call.so's function
+_native = None                                   # the extension's function
 _address: dict = {}                              # entry point -> its handle there
 _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
@@ -135,9 +136,10 @@ def lib() -> C.CDLL:
         L.vitcop_kernel_timing_end.argtypes = [C.POINTER(KernelTime), i32, C.POINTER(C.c_int)]
         for name in EXPORTS:
             getattr(L, name)
-        if not os.path.exists(CALL_PATH):
-            raise ImportError(f"{CALL_PATH} is missing: run `python -m paper_2601_17818_b200.build` first")
-        loader = importlib.machinery.ExtensionFileLoader("_call", CALL_PATH)
+        path = build.caller_path()
+        if not os.path.exists(path):
+            raise ImportError(f"{path} is missing: run `python -m paper_2601_17818_b200.build` with this interpreter and torch")
+        loader = importlib.machinery.ExtensionFileLoader("_call", path)
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_call", loader))
         loader.exec_module(module)
         for name in NATIVE:

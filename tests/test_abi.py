@@ -184,6 +184,20 @@ def test_argument_validation_of_the_wider_entry_points(L):
     assert vb.vitcop_workspace_bytes(vb.OP_SALIENCY, B=2, H=4, N=33) >= 2 * 4 * 33 * 4
 
 
+def test_the_caller_belongs_to_one_torch_and_one_interpreter(monkeypatch):
+    """The extension is compiled against torch's and Python's headers: with another version of either it is neither taken for
+    up to date nor found."""
+    from paper_2601_17818_b200 import build
+    path, digest = build.caller_path(), build._caller_digest()
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    assert build.caller_path() != path and build._caller_digest() != digest
+    monkeypatch.setattr(vb, "_lib", None)
+    with pytest.raises(ImportError):
+        vb.lib()
+    monkeypatch.undo()
+    assert build.caller_path() == path and os.path.exists(path)
+
+
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(vb, "_lib", None)
     monkeypatch.setattr(vb, "LIB_PATH", str(tmp_path / "nope.so"))
