@@ -70,7 +70,8 @@ class SelectParams(C.Structure):
 _lib: Optional[C.CDLL] = None
 _native = None                                   # the extension's function
 _address: dict = {}                              # entry point -> its handle there
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# (a torch without CUDA has neither; the host-only entry points work there)
+_raw_stream, _device = (getattr(torch._C, name, None) for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
 
 
 # the parameter structs as bytes, laid out as the compiler does; values that a field cannot hold are converted as C does (a
@@ -100,6 +101,7 @@ def lib() -> C.CDLL:
         L.vitcop_status_string.restype = C.c_char_p
         L.vitcop_status_string.argtypes = [C.c_int]
         L.vitcop_last_cuda_error.restype = C.c_int
+        # (the types of the native calls too: whoever calls them through ctypes, as the checks of the C ABI do, needs them)
         vp, i32, i64, sz = C.c_void_p, C.c_int, C.c_int64, C.c_size_t
         L.vitcop_workspace_bytes.argtypes = [i32] * 8 + [C.POINTER(sz)]
         L.vitcop_poll_status.argtypes = [vp, vp, C.POINTER(C.c_int)]

@@ -198,6 +198,15 @@ def test_the_caller_belongs_to_one_torch_and_one_interpreter(monkeypatch):
     assert build.caller_path() == path and os.path.exists(path)
 
 
+def test_host_only_calls_need_no_cuda_in_torch():
+    import subprocess
+    import sys
+    code = ("import torch\nfor name in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n    delattr(torch._C, name)\n"
+            "from paper_2601_17818_b200 import binding as vb\nassert vb.vitcop_stage_count(576, 0.5) == 288\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-800:]
+
+
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(vb, "_lib", None)
     monkeypatch.setattr(vb, "LIB_PATH", str(tmp_path / "nope.so"))
