@@ -26,15 +26,16 @@ namespace {
 // ------------------------------------------------------------------------------------------------
 // rho[b,i] = sum of the partials of the density sweep in a fixed order (reproducible bits): first the later tokens, 256 at a
 // time (a tile's columns: the sum of its two 128-token blocks), then the earlier ones, one 128-token block after the other, to
-// the end of the token's tile (blocks that hold none of them count as zero).  Up to 64 entries are added one by one; longer
-// lists (up to 192 on the longest samples) in four equal parts, whose sums are then added.  One CTA per 32 tokens: its warps
-// fetch the entries, all of them in one trip to memory, and the sums are taken from shared memory.  (One thread per token
-// walking its list paid a trip for every sixteen entries.)
+// the end of the token's tile (blocks that hold none of them count as zero).  On samples with T + TI <= 64 tiles and blocks (up to
+// 5376 tokens) the entries are added one by one; on longer ones in four equal parts, whose sums are then added.  One CTA per 32
+// tokens: its warps fetch the entries, all of them in one trip to memory, and the sums are taken from shared memory.  (One thread
+// per token walking its list paid a trip for every sixteen entries.)
 // blk_rho[b,k]: bits of the largest density among the tokens of block k (densities are not negative, their bit patterns order
 // like the values).  tok[b,i]: what the search needs of a token, in one 16-byte load.
 constexpr int kRhoThreads = 256;
 constexpr int kRhoOneByOne = 64;
-constexpr int kRhoEntries = 3 * VITCOP_MAX_VISUAL_TOKENS / kSweepTile;       // longest list
+// the longest list: (T - tile) + min(TI, 2 (tile + 1)) entries, most at the last tile
+constexpr int kRhoEntries = VITCOP_MAX_VISUAL_TOKENS / kGramBM + 1;
 __global__ void __launch_bounds__(kRhoThreads)
 rho_reduce_kernel(const __grid_constant__ SweepArgs g, int metric, float* __restrict__ rho_user) {
     constexpr int kWarps = kRhoThreads / 32;
