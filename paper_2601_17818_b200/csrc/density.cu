@@ -18,13 +18,15 @@
 // stands between two tiles.
 //
 // Measured: 8 x 2880 x 1024 75 us (60 us with an empty epilogue), 2 x 16384 x 1280 519 us (433 us with an empty epilogue:
-// 0.69 Tflop at the rate cuBLAS reaches in a burst; the stores of the Gram values are about 30 of the rest).  Sixteen warps of one role: 70 and 517 us, but another order of the sums.  A sweep of single SMs on 128 x 256 tiles,
-// without the minima: 68 and 549 us.
+// 0.69 Tflop at the rate cuBLAS reaches in a burst; the stores of the Gram values are about 30 of the rest).  Sixteen warps of
+// one role: 70 and 517 us, but another order of the sums.  A sweep of single SMs on 128 x 256 tiles, without the minima: 68 and
+// 549 us.
 //
 // A last round of tiles that would occupy at most half of the clusters is cut into tiles of 128 columns.
 // Every wait is bounded; on expiry both CTAs of the cluster leave in order and the call reports VITCOP_ERR_TIMEOUT.
 #include "async_copy.cuh"
 #include "density.cuh"
+#include "f32x2.cuh"
 #include "tcgen05.cuh"
 
 namespace vitcop {
@@ -88,40 +90,6 @@ __device__ __forceinline__ Item decode_item(const KernelArgs& k, int t) {
     it.tj = q;
     it.tp = r - q * (q + 1) / 2;
     return it;
-}
-
-// Two fp32 operations in one instruction (each half rounded like the scalar instruction).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-    float2 o;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(v));
-    return o;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-// 2^x for x <= 0 (results below the normal range flush to zero); relative error about 2^-22.
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
 }
 
 // Smallest of the values, or NaN if one of them is none.

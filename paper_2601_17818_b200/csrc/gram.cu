@@ -21,6 +21,7 @@
 #include <atomic>
 
 #include "async_copy.cuh"
+#include "f32x2.cuh"
 #include "gram.cuh"
 #include "tcgen05.cuh"
 #include "knorm.cuh"
@@ -33,44 +34,6 @@ constexpr int BM = kGramBM;
 // TMEM lane quarter).
 constexpr int kEpiSlices = 2;
 constexpr int kGemmThreads = 64 + kEpiSlices * 128;
-
-// ------------------------------------------------------------------------------------------------
-// PTX wrappers
-// ------------------------------------------------------------------------------------------------
-// 2^x for x <= 0 (results below the normal range flush to zero); relative error about 2^-22.
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Two fp32 operations in one instruction (each half rounded like the scalar instruction): the epilogues are bound
-// by instruction issue, and a pair of neighbouring columns shares every step of the distance arithmetic.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long v) {
-    float2 o;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(v));
-    return o;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 // ------------------------------------------------------------------------------------------------
 // tile numbering
@@ -323,7 +286,7 @@ __device__ __forceinline__ bool epi_tile(const KernelArgs& k, const EpiSmem& sm,
         rho_i = sm.rowrho[rl];
         if (SPATIAL) { x_i = sm.rowx[rl]; y_i = sm.rowy[rl]; }
     }
-    // the row's constants, twice each, for the paired arithmetic
+    // the row's constants, twice each, for the paired arithmetic (the epilogues are bound by instruction issue)
     const unsigned long long m2w2 = pack2(m2w_i, m2w_i), ai2 = pack2(a_i, a_i), two2 = pack2(2.f, 2.f);
     const unsigned long long nxi2 = pack2(-x_i, -x_i), nyi2 = pack2(-y_i, -y_i), c22 = pack2(g.c2, g.c2);
     if (ok && call.wait_bar) ok = mbar_wait(call.wait_bar, call.wait_parity, call.abort_flag, call.limit_ns);
