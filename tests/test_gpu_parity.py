@@ -490,14 +490,12 @@ def test_filter_resident_shapes(B, n, metric, check):
         check_vic_sample(f[b], p[b], metric, d_c, w.tau, nc, g.rho[b], g.delta2[b], g.parent[b], g.label[b])
 
 
-# Long samples (8192 tokens and more) keep the Gram tiles of the density sweep and run Eq. 3 as a separate pass over
-# them: a ragged length (tiles that straddle the diagonal and the end of the sample), both metrics, with and
-# without the spatial test.  Small feature width: the oracle's pairwise work stays cheap.
-# With a radius, the tiles whose row block lies beyond it from their column blocks are neither kept nor read: 0.25 and
-# 0.02 drop most of them (0.02: nearly all but the tiles on the diagonal).
+# Long samples: a ragged length (tiles that straddle the diagonal and the end of the sample), both metrics, with and without the
+# spatial test.  Small feature width: the oracle's pairwise work stays cheap.  With a radius, the blocks beyond it are neither kept
+# nor looked into: 0.25 and 0.02 drop most of them (0.02: nearly all but those on the diagonal).
 @pytest.mark.parametrize("n,metric,tau", [(8200, 0, 0.6), (8321, 1, 0.6), (8200, 0, -1.0), (8192, 0, 0.25),
                                           (8250, 0, 0.02), (8200, 1, 0.25)])
-def test_filter_long_sample_delta_pass(n, metric, tau):
+def test_filter_long_sample(n, metric, tau):
     w = dataclasses.replace(W.workload("c4"), B=1, D=64, dup_rate=0.3)
     f = W.make_features(w, n=n, B=1)
     p = W.make_positions(w, n)[:1]
@@ -546,7 +544,7 @@ def test_filter_search_shared_tokens(metric):
 # Too many tiles for the one-kernel sweep: pairs of CTAs on 256 x 256 tiles (ragged ends, an odd number of 128-token blocks, the
 # last tiles cut into column halves or not), block minima, the search.  Half of the last sample's tokens are one token plus
 # noise (plain copies would tie in every distance, and the oracle's report excuses ties): the densest of them have neighbours
-# in half of the blocks and none is denser, so the search hands them to the whole CTA.
+# in half of the blocks and none is denser, so the search leaves them to its second kernel, several warps a token.
 @pytest.mark.parametrize("B,n,metric,tau", [(16, 1153, 0, 0.6), (16, 1279, 1, -1.0), (17, 1281, 0, 0.1), (300, 127, 0, 0.6),
                                              (80, 257, 1, 0.3)])
 def test_filter_sweep_and_search_edges(B, n, metric, tau):
