@@ -79,11 +79,13 @@ constexpr uint32_t kSegDone = 0xFFFFFFFFu;
 // The rank search is taken when no searched cluster is larger than kRankMaxSize and the comparisons of the busiest CTA are few enough:
 // a million of them take 28 us, and the other searches on 2880 / 4608 / 8192 / 16384 tokens 18 / 8 / 10 / 20 us longer than what is
 // left of the rank search.  (Counting all comparisons against 64 n per CTA of the cluster, as if they were shared out evenly, took
-// uneven clusters to the rank search: 8 x 8192 tokens 47 us instead of 27, 32 x 16384 160 instead of 47.)  A CTA of several ranks the
-// segments that start in its n / R positions, so it has at most (n / R + largest) * largest, and at most all of them.
+// uneven clusters to the rank search: 8 x 8192 tokens 47 us instead of 27, 32 x 16384 160 instead of 47.)  A CTA of several ranks
+// the segments that start in its n / R positions, so it has at most (n / R + largest) * largest, and at most all of them; where
+// that bound leaves it open, the CTAs' parts are added up (a third of a microsecond).
 constexpr int kRankWork = 64;                             // of one CTA, times n
-constexpr int kRankPart = 64;                             // of one of several, times n ...
-constexpr int kRankPartSort = 3 << 18;                    // ... on samples that would be sorted otherwise this
+__host__ __device__ constexpr uint32_t rank_part(int n, bool sorted_otherwise) {         // of one of several
+    return sorted_otherwise ? 600000u : 40u * (uint32_t)n + 100000u;
+}
 constexpr int kRankMaxSize = 2048;
 constexpr int kRadixMinTokens = 4096;                     // below this a sort beats the radix passes (fewer barriers)
 
@@ -276,9 +278,23 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
     bool by_rank = largest <= (uint32_t)kRankMaxSize;
     if (R == 1) {
         by_rank = by_rank && all <= (uint32_t)kRankWork * (uint32_t)n;
-    } else {
-        const uint32_t part = min(all, ((uint32_t)(n / R) + largest) * min(largest, (uint32_t)kRankMaxSize));
-        by_rank = by_rank && part <= (n <= kRadixMinTokens ? (uint32_t)kRankPartSort : (uint32_t)kRankPart * (uint32_t)n);
+    } else if (by_rank) {
+        const uint32_t most = rank_part(n, n <= kRadixMinTokens);
+        if (min(all, ((uint32_t)(n / R) + largest) * largest) > most) {       // (uniform over the CTAs)
+            __shared__ uint32_t part_work[R];
+            if (tid < R) part_work[tid] = 0u;
+            __syncthreads();
+            const bool searched = tid < (int)n_seg && krem[tid] != kSegDone;
+            const uint32_t size = searched ? csize[tid] : 0u, to = searched ? offs[tid] / (uint32_t)((n + R - 1) / R) : 0u;
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const uint32_t w = __reduce_add_sync(0xffffffffu, to == (uint32_t)u ? size * size : 0u);
+                if ((tid & 31) == u && w) atomicAdd(&part_work[u], w);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < R; ++u) by_rank = by_rank && part_work[u] <= most;
+        }
     }
     const uint32_t range_lo = misc[0], range_hi = misc[1];
     if (!by_rank && n <= kRadixMinTokens) return false;    // uniform; nothing has been written yet
