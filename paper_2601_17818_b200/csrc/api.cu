@@ -375,9 +375,10 @@ int vitcop_collaborative_step(const void* feat, const float* pos, int D, const v
     float* score = score_out ? score_out : reinterpret_cast<float*>(ws2 + lay.off_score);
     int32_t* keep = keep_idx_out ? keep_idx_out : reinterpret_cast<int32_t*>(ws2 + lay.off_keep);
     int32_t* nkeep = n_keep_out ? n_keep_out : reinterpret_cast<int32_t*>(ws2 + lay.off_nkeep);
-    rc = record_cuda(cudaMemsetAsync(workspace, 0, filter_zeroed_bytes(B, Nv), s));
-    if (rc != VITCOP_OK) return rc;
-    if (B == 0) return VITCOP_OK;
+    if (B == 0 || Nv == 0) {
+        rc = reset_status(workspace, s);
+        if (rc != VITCOP_OK || B == 0) return rc;
+    }
     if (Nv > 0) {
         const KnormJob job = {K, B, H, N, d, vis_start, Nv, score};
         rc = launch_filter(feat, pos, B, Nv, D, *fp, nc, label_out, n_clusters_out, rho_out, delta2_out, parent_out,
@@ -436,9 +437,7 @@ int vitcop_kproj_knorm(const void* hidden, const void* W_k, int B, int N, int Dh
     if (!workspace || workspace_bytes < kproj_workspace_bytes(B, N, H, d) || !aligned256(workspace))
         return VITCOP_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int rc = reset_status(workspace, s);
-    if (rc != VITCOP_OK) return rc;
-    if (B == 0 || N == 0 || H == 0 || d == 0 || Dh == 0) return VITCOP_OK;
+    if (B == 0 || N == 0 || H == 0 || d == 0 || Dh == 0) return reset_status(workspace, s);
     return launch_kproj_knorm(hidden, W_k, B, N, Dh, H, d, rope_cos, rope_sin, position_ids, n_pos, K_out, vis_start,
                               score ? Nv : 0, score, workspace, s);
 }
@@ -475,9 +474,7 @@ int vitcop_redundancy_filter(const void* feat, const float* pos, int B, int n, i
     }
     if (nc > n) nc = n;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int rc = record_cuda(cudaMemsetAsync(workspace, 0, filter_zeroed_bytes(B, n), s));
-    if (rc != VITCOP_OK) return rc;
-    if (B == 0 || n == 0) return VITCOP_OK;
+    if (B == 0 || n == 0) return reset_status(workspace, s);
     return launch_filter(feat, pos, B, n, D, *p, nc, label, n_clusters, rho, delta2, parent, workspace, workspace_bytes, s);
 }
 

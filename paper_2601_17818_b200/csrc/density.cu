@@ -558,7 +558,8 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             const unsigned long long t0 = global_ns();
             while (global_ns() - t0 < kDrainLimitNs) {}
         }
-        if (g.status) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
+        grid_dependency_wait();                            // (the kernel in front clears the word)
+        atomicMax(g.status, VITCOP_ERR_TIMEOUT);
     }
     tc_fence_before();
     __syncthreads();

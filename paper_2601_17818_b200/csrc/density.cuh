@@ -90,6 +90,7 @@ struct SweepArgs {
     int32_t* n_left;
     unsigned long long* best;   // [B, n] packed (d^2 bits << 32 | index) of the nearest denser token, ~0 = none
     int* status;                // device status word
+    int diag_reports;           // CTAs of the diagonal in front that reported whether they gave up, 0: they set the word themselves
     SweepTiling t;
 };
 

@@ -58,6 +58,7 @@ rho_reduce_kernel(const __grid_constant__ SweepArgs g, int metric, float* __rest
         }
     }
     if (blk == 0 && b == 0 && threadIdx.x == 0) *g.n_left = 0;       // for the search behind this kernel
+    if (blk == 0 && b == 0 && warp == 1 && any_gave_up(g.status, g.diag_reports) && lane == 0) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
     const int own = blk * kBlk / kGramBM, tile = own / 2;
     const int rows = t.T - tile;                           // entries on the row side, then min(TI, 2 (tile + 1)) more
     const int entries = rows + min(t.TI, 2 * (tile + 1));
@@ -374,8 +375,8 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
 // ------------------------------------------------------------------------------------------------
 // Workspace of the filter: status block | for the one-kernel sweep the tokens' published factors [B, n] | w | a | rho | best |
 // rho partials [B, slots, n_pad] | bounding boxes of the row blocks' positions | and, for problems too large for the one-kernel
-// sweep, what is kept of one group of samples (SweepGroupWs).  The status block and the published factors are zeroed at the start
-// of every call.  Words of the status block: 0 status, 2 grid barrier.
+// sweep, what is kept of one group of samples (SweepGroupWs).  The first kernel of a call clears the status block, the
+// one-kernel sweep the published factors too.  Words of the status block: 0 status, 2 grid barrier.
 // A group is as large as the workspace allows, so every workspace serves that holds one sample of it; the size asked for holds
 // all samples, or as many as fit 1.5 GB (8 x 2880 tokens take 175 MB: one sample at a time would leave half of the SMs without
 // work).  Neither the size asked for nor the least one ever falls when the batch or the samples grow: a workspace for a larger
@@ -421,8 +422,6 @@ void pdl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 grid, d
 
 }  // namespace
 
-size_t filter_zeroed_bytes(int B, int n) { return FilterWs(B, n).off_w; }
-
 size_t filter_workspace_bytes(int B, int n, int D) {
     (void)D;
     return FilterWs(B, n).total;
@@ -460,12 +459,11 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     if (l.resident) {
         g.rho_out = rho;
         g.rho_user = rho_user;
-        g.grid_sync = reinterpret_cast<unsigned int*>(ws) + 2;       // zeroed with the status word at the start of the call
+        g.grid_sync = reinterpret_cast<unsigned int*>(ws) + 2;
         g.ready = reinterpret_cast<uint32_t*>(ws + l.off_ready);
         if (knorm && gram_resident_takes_knorm(knorm->H, knorm->d)) {
-            // The sweep's two idle warps take the K-norm of the first samples, about as many as they finish while
-            // the epilogue warps work on the accumulators; the other samples follow beside vic_finalize_kernel.
-            knorm_in_sweep = (5 * knorm->B + 8) / 16;
+            // The sweep's side warps take the K-norm of the first samples; the others follow beside vic_finalize_kernel.
+            knorm_in_sweep = gram_resident_knorm_samples(B, n, knorm->Nv);
             if (knorm_in_sweep > 0) {
                 g.kn_K = knorm->K; g.kn_score = knorm->score; g.kn_B = knorm_in_sweep;
                 g.kn_H = knorm->H; g.kn_N = knorm->N; g.kn_d = knorm->d; g.kn_vis_start = knorm->vis_start; g.kn_Nv = knorm->Nv;
@@ -477,9 +475,15 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
         // with a spatial radius, blocks beyond it are neither kept nor looked into (density.cuh: blocks_outside_radius)
         g.bbox = g.tau2 >= 0.f ? reinterpret_cast<float4*>(ws + l.off_bbox) : nullptr;
         g.best = nullptr;                                  // (the search writes every token's entry)
+        const SweepTiling tiling = make_sweep_tiling(n);
+        const int diag_ctas = (long long)B * tiling.TI < gram_num_sms() ? B * tiling.TI : gram_num_sms();
+        g.reports = diag_ctas <= kMaxReports;
+        if (!g.reports) {
+            rc = record_cuda(cudaMemsetAsync(workspace, 0, kStatusBytes, stream));
+            if (rc != VITCOP_OK) return rc;
+        }
         rc = launch_gram_sweep(GRAM_DIAG, feat, g, stream, false);
         if (rc != VITCOP_OK) return rc;
-        const SweepTiling tiling = make_sweep_tiling(n);
         const int group = sweep_group_samples(B, n, (workspace_bytes < l.total ? workspace_bytes : l.total) - l.off_group);
         const SweepGroupWs kept((size_t)group, n);
         char* const gws = ws + l.off_group;
@@ -499,6 +503,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             s.blk_min = reinterpret_cast<float*>(gws + kept.off_blk_min);
             s.gram = reinterpret_cast<float*>(gws + kept.off_gram);
             s.status = g.status;
+            s.diag_reports = g.reports ? diag_ctas : 0;
             s.t = tiling;
             rc = launch_density_sweep(static_cast<const uint16_t*>(feat) + at * D, s, p.metric, stream, true);
             if (rc != VITCOP_OK) return rc;

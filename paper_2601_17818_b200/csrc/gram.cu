@@ -16,9 +16,11 @@
 //   warps 2..   epilogue: warp w reads TMEM lanes 32 * (w % 4) .. + 31 (its rows) and one slice of the columns
 // Every wait is bounded; on expiry the CTA raises an abort flag, all roles leave, TMEM is released and
 // VITCOP_ERR_TIMEOUT is written to the status word.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include <atomic>
+#include <utility>
 
 #include "async_copy.cuh"
 #include "f32x2.cuh"
@@ -46,6 +48,7 @@ struct KernelArgs {
     int unit_w;                    // resident sweep: column blocks of a unit, 1 or 2
     unsigned long long wait_ns;    // time limit of every bounded wait
     int expire_roles;              // roles whose waits give up at once: 1 load warp, 2 MMA warp, 4 epilogue warps
+    int reports;                   // diagonal: every CTA reports (internal.cuh); rho_reduce_kernel sets the status word
     __device__ __forceinline__ unsigned long long limit_of(int role) const {
         return (expire_roles & role) ? 0ull : wait_ns;
     }
@@ -615,6 +618,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // The kernels that follow on the stream may be scheduled from here on; they wait for this grid to complete
     // before they touch anything it writes.
     grid_dependency_launch_dependents();
+    if (k.reports && blockIdx.x == 0 && threadIdx.x == 0) *g.status = VITCOP_OK;
 
     const long long total_tiles = k.total_tiles;
     const int KB = g.D / BK;
@@ -710,8 +714,9 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // flight into this CTA's shared memory time to land before the CTA goes away.
         for (int s = 0; s < S::kStages; ++s)
             if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
-        if (g.status) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
+        if (!k.reports) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
     }
+    if (threadIdx.x == 0 && k.reports) report_gave_up(g.status, *abort_flag != 0);
 }
 
 
@@ -739,13 +744,16 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 // The grid (at most one CTA per SM) is launched cooperatively, so all CTAs are resident together; factors and barrier
 // are words in global memory with bounded waits.  No wait can form a cycle: a factor is published by a CTA that has
 // waited for nothing but its own tensor-core work.
-// The load warp and the MMA warp are idle once the CTA's last MMA is issued, and so are, a little later, the
+// The load warp and the MMA warp are idle once the CTA's last MMA is issued (warp 0, which only speaks for the CTA at the barriers
+// of the launch, before that), and so are, a little later, the
 // operand buffers and -- for the rest of the kernel, which is arithmetic on the accumulators -- the memory system:
-// if the caller has a K-norm (Eq. 4) to compute, these two warps stream K through the operand buffers with bulk
+// if the caller has a K-norm (Eq. 4) to compute, these warps and two more stream K through the operand buffers with bulk
 // copies and reduce it there (resident_knorm).
 constexpr int kResidentUnits = 2;
 constexpr int kResidentBN = 2 * BM;                       // columns of a unit
 constexpr int kResidentEpiThreads = 512;
+constexpr int kResidentThreads = 64 + kResidentEpiThreads + 64;
+constexpr int kKnThreads = 128;                           // of the four warps in front of and behind the epilogue's
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
     unsigned int v;
@@ -834,53 +842,43 @@ __device__ __forceinline__ ResidentUnit decode_resident_unit(const KernelArgs& k
 constexpr int kKnChunkTokens = 8;                          // tokens per chunk: 8 threads each
 constexpr int kKnBuffers = 3;
 
-// K-norm (Eq. 4) by the 64 threads of warps 0 and 1, after the CTA's last MMA has completed.  Chunks of eight
-// consecutive tokens of one sample are copied head by head (one contiguous run per head) into the operand
-// buffers, up to three chunks in flight; eight threads reduce one token, each standing in for lanes s and s + 8
-// of the sixteen-lane reduction of the stand-alone kernel, so that both give the same bits.
-__device__ __forceinline__ void resident_knorm(const GramArgs& g, const uint8_t* buf_gen, uint32_t buf_smem,
+// K-norm (Eq. 4) by the warps beside the epilogue's, after the CTA's last MMA has completed.  Chunks of eight consecutive
+// tokens of one sample, all heads, are copied into the operand buffers, up to three chunks in flight; sixteen threads
+// reduce one token as in the stand-alone kernel, so that both give the same bits.  One tensor copy per chunk: as bulk copies, one
+// per head, they took a warp 1.3 us to issue where the arithmetic takes 1.0 (32 heads).
+__device__ __forceinline__ void resident_knorm(const GramArgs& g, const CUtensorMap* map_k, const uint8_t* buf_gen, uint32_t buf_smem,
                                                uint32_t buf_bytes, uint32_t bar_kn, uint32_t bar_last_mma,
                                                volatile int* abort_flag, unsigned long long limit_ns) {
-    const int tid = threadIdx.x;                           // 0 .. 63
+    const int tid = threadIdx.x < 64 ? threadIdx.x : threadIdx.x - kResidentEpiThreads;        // 0 .. 127
     auto all_ok = [](bool ok) {
         uint32_t out;
         asm volatile(
             "{\n\t.reg .pred p, q;\n\t"
             "setp.eq.b32 p, %1, 0;\n\t"
-            "bar.red.or.pred q, 2, 64, p;\n\t"
+            "bar.red.or.pred q, 2, %2, p;\n\t"
             "selp.u32 %0, 0, 1, q;\n\t}"
-            : "=r"(out) : "r"((uint32_t)ok) : "memory");
+            : "=r"(out) : "r"((uint32_t)ok), "n"(kKnThreads) : "memory");
         return out != 0;
     };
     // the tensor cores read the operand buffers until the last MMA completes
     if (!all_ok(mbar_wait(bar_last_mma, 0, abort_flag, limit_ns))) return;
 
     const int H = g.kn_H, d8 = g.kn_d / 8, Nv = g.kn_Nv;
-    const uint32_t row_bytes = (uint32_t)d8 * 16u;
-    const uint32_t head_bytes = kKnChunkTokens * row_bytes;         // one head of a chunk
-    const uint32_t chunk_bytes = (uint32_t)H * head_bytes;
+    const uint32_t chunk_bytes = (uint32_t)(H * kKnChunkTokens * d8) * 16u;
     const int nbuf = min(kKnBuffers, (int)(buf_bytes / chunk_bytes));   // >= 1 (gram_resident_takes_knorm)
     const int chunks_per_b = (Nv + kKnChunkTokens - 1) / kKnChunkTokens;
     const long long total = (long long)g.kn_B * chunks_per_b;
-    const uint8_t* Kb = static_cast<const uint8_t*>(g.kn_K);
-    const size_t head_stride = (size_t)g.kn_N * row_bytes;
-
     auto issue = [&](long long c, int buf) {               // thread 0
-        const int b = (int)(c / chunks_per_b);
-        const int i0 = (int)(c - (long long)b * chunks_per_b) * kKnChunkTokens;
-        const int cnt = min(kKnChunkTokens, Nv - i0);
-        const uint32_t run = (uint32_t)cnt * row_bytes;
-        mbar_expect_tx(bar_kn + 8 * buf, (uint32_t)H * run);
-        const uint8_t* src = Kb + ((size_t)b * H * g.kn_N + (size_t)(g.kn_vis_start + i0)) * row_bytes;
-        const uint32_t dst = buf_smem + (uint32_t)buf * chunk_bytes;
-        for (int h = 0; h < H; ++h) bulk_load(dst + (uint32_t)h * head_bytes, src + (size_t)h * head_stride, run, bar_kn + 8 * buf);
+        const int b = (int)(c / chunks_per_b), i0 = (int)(c - (long long)b * chunks_per_b) * kKnChunkTokens;
+        mbar_expect_tx(bar_kn + 8 * buf, chunk_bytes);     // (rows past the sequence arrive as zeros)
+        tma_load_4d(buf_smem + (uint32_t)buf * chunk_bytes, map_k, bar_kn + 8 * buf, 0, g.kn_vis_start + i0, 0, b);
     };
     long long issued = 0;                                  // chunks this CTA has requested (thread 0)
     if (tid == 0)
         for (; issued < nbuf && blockIdx.x + issued * gridDim.x < total; ++issued)
             issue(blockIdx.x + issued * gridDim.x, (int)issued);
 
-    const int tk = tid >> 3, s = tid & 7;
+    const int tk = tid >> 4, s = tid & 15;
     long long it = 0;
     bool ok = true;
     for (long long c = blockIdx.x; c < total; c += gridDim.x, ++it) {
@@ -892,22 +890,18 @@ __device__ __forceinline__ void resident_knorm(const GramArgs& g, const uint8_t*
         const int cnt = min(kKnChunkTokens, Nv - i0);
         const uint4* rows = reinterpret_cast<const uint4*>(buf_gen + (size_t)buf * chunk_bytes) + (size_t)tk * d8;
         const int head16 = kKnChunkTokens * d8;            // uint4 per head of a chunk
-        float part = 0.f;
+        float a0 = 0.f, a1 = 0.f;
         if (tk < cnt) {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                float a0 = 0.f, a1 = 0.f;
-                for (int piece = s + 8 * q; piece < d8; piece += 16) {
+            for (int piece = s; piece < d8; piece += 16) {
 #pragma unroll 8
-                    for (int h = 0; h < H; ++h) knorm_sq_acc(rows[(size_t)h * head16 + piece], a0, a1);
-                }
-                part += a0 + a1;
+                for (int h = 0; h < H; ++h) knorm_sq_acc(rows[(size_t)h * head16 + piece], a0, a1);
             }
         }
+        float part = a0 + a1;
 #pragma unroll
-        for (int off = 4; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+        for (int off = 8; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
         if (tk < cnt && s == 0) g.kn_score[(size_t)b * Nv + i0 + tk] = sqrtf(part);
-        asm volatile("bar.sync 2, 64;" ::: "memory");      // the buffer has been read by everyone
+        asm volatile("bar.sync 2, %0;" ::"n"(kKnThreads) : "memory");      // the buffer has been read by everyone
         if (tid == 0) {
             const long long cn = blockIdx.x + issued * gridDim.x;
             if (cn < total) {
@@ -925,10 +919,11 @@ __device__ __forceinline__ void resident_knorm(const GramArgs& g, const uint8_t*
 
 // BN: columns of the epilogue's tiles: 128, or 64 for units of half a tile.
 template <int METRIC, bool SPATIAL, int BN>
-__global__ void __launch_bounds__(64 + kResidentEpiThreads, 1)
+__global__ void __launch_bounds__(kResidentThreads, 1)
 gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                     const KernelArgs k) {
+                     const __grid_constant__ CUtensorMap map_k, const KernelArgs k) {
     constexpr bool HALF = BN == 64;
+    constexpr int kLoadThread = 32, kMmaThread = 64 + kResidentEpiThreads;
     constexpr int NS = 4;
     using S = GemmSmem<kResidentBN>;                       // stages of 128 + 256 operand rows
     constexpr uint32_t kStages = HALF ? HalfUnitSmem::kStages : S::kStages;
@@ -971,79 +966,81 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    grid_dependency_wait();                                // (whatever was queued before the call has completed)
 
     const long long total_units = k.total_tiles;          // <= kResidentUnits * gridDim.x (checked by the launcher)
     const int KB = g.D / BK;
-    uint32_t issued = 0, issued_parity = 0;               // thread 0, per stage: a load was issued / parity of its phase
-
-    if (warp == 0) {
-        // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            const unsigned long long lim = k.limit_of(kRoleLoad);
-            uint32_t stage = 0, phase = 0;
-            bool ok = true;
-            for (long long t = blockIdx.x; ok && t < total_units; t += gridDim.x) {
-                const ResidentUnit u = unit_of(t);
-                const int I0 = u.ti * BM, J0 = u.tj0 * BN;
-                for (int kb = 0; kb < KB; ++kb) {
-                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
-                    const uint32_t sa = tiles + stage * kStageBytes;
-                    // rows of the box past the sample's last token are zero-filled and still count as received
-                    mbar_expect_tx(bar_full + 8 * stage, HALF ? kStageBytes : S::kABytes + (uint32_t)k.unit_w * S::kABytes);
-                    tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, I0, u.b);
-                    tma_load_3d(sa + S::kABytes, &map_b, bar_full + 8 * stage, kb * BK, J0, u.b);
-                    issued |= 1u << stage;
-                    issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                }
-            }
+    uint32_t issued = 0, issued_parity = 0;               // load thread, per stage: a load was issued / parity of its phase
+    uint32_t stage = 0, phase = 0;                         // load and MMA warp
+    bool ok = true;
+    auto load_unit = [&](long long t) {
+        const unsigned long long lim = k.limit_of(kRoleLoad);
+        const ResidentUnit u = unit_of(t);
+        const int I0 = u.ti * BM, J0 = u.tj0 * BN;
+        for (int kb = 0; kb < KB; ++kb) {
+            if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
+            const uint32_t sa = tiles + stage * kStageBytes;
+            // rows of the box past the sample's last token are zero-filled and still count as received
+            mbar_expect_tx(bar_full + 8 * stage, HALF ? kStageBytes : S::kABytes + (uint32_t)k.unit_w * S::kABytes);
+            tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, I0, u.b);
+            tma_load_3d(sa + S::kABytes, &map_b, bar_full + 8 * stage, kb * BK, J0, u.b);
+            issued |= 1u << stage;
+            issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer: unit s of this CTA -> columns 256 s ..
-        if (lane == 0) {
-            const uint32_t idesc = !HALF && k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BN);
-            const unsigned long long lim = k.limit_of(kRoleMma);
-            uint32_t stage = 0, phase = 0;
-            uint32_t slot = 0;
-            bool ok = true;
-            for (long long t = blockIdx.x; ok && t < total_units; t += gridDim.x, ++slot) {
-                const uint32_t d_tmem = tmem_base + slot * kResidentBN;
-                for (int kb = 0; kb < KB; ++kb) {
-                    if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t sa = tiles + stage * kStageBytes;
-                    const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + S::kABytes);
+    };
+    // Status word, barrier counter and factors are cleared here, a slice per CTA; no CTA touches them before all have arrived at
+    // the cooperative launch's own barrier.  (A memset in front of the kernel stood before the first loads.)
+    if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) g.status[threadIdx.x] = 0;
+    const uint32_t n_ready = (uint32_t)g.B * (uint32_t)g.n;       // (a wave of tiles: below 2^23)
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_ready; i += gridDim.x * blockDim.x) g.ready[i] = 0u;
+    tc_fence_before();
+    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    auto cleared = grid.barrier_arrive();                  // (begins with a barrier of the CTA)
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    auto mma_unit = [&](uint32_t slot) {                   // this CTA's unit number `slot` -> columns 256 slot ..
+        const uint32_t idesc = !HALF && k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BN);
+        const unsigned long long lim = k.limit_of(kRoleMma);
+        const uint32_t d_tmem = tmem_base + slot * kResidentBN;
+        for (int kb = 0; kb < KB; ++kb) {
+            if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; return; }
+            tc_fence_after();
+            const uint32_t sa = tiles + stage * kStageBytes;
+            const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + S::kABytes);
 #pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
-                                    (kb > 0 || kk > 0) ? 1u : 0u);
-                    tc_commit(bar_empty + 8 * stage);
-                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                }
-                if (!ok) break;
-                tc_commit(bar_tfull + 8 * slot);
-            }
-            tc_commit(bar_drain);                          // (as in gram_tc_kernel)
-            mbar_drain(bar_drain, 0);
+            for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+            tc_commit(bar_empty + 8 * stage);
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
+        tc_commit(bar_tfull + 8 * slot);
+    };
+    // The first unit's loads and MMAs need nothing from another CTA: the warps meet behind them, by when the other CTAs have
+    // arrived too.  (Thread 0 speaks for the CTA, so warp 0 has no other role: its release waits for the stores above, and it
+    // has seen the others arrive before the first MMA completes.)
+    static_assert(kResidentUnits == 2, "a first unit and a second one");
+    const long long second = (long long)blockIdx.x + gridDim.x;
+    if (threadIdx.x == kLoadThread) load_unit(blockIdx.x);
+    if (threadIdx.x == kMmaThread) mma_unit(0);
+    grid.barrier_wait(std::move(cleared));                 // (unbounded, but all CTAs are resident and arrive whatever happens)
+    if (threadIdx.x == kLoadThread && ok && second < total_units) load_unit(second);
+    if (threadIdx.x == kMmaThread) {
+        if (ok && second < total_units) mma_unit(1);
+        tc_commit(bar_drain);                              // (as in gram_tc_kernel)
+        mbar_drain(bar_drain, 0);
     }
-    if (warp < 2) {
+    if (warp < 2 || warp >= 2 + kResidentEpiThreads / 32) {
         __syncwarp();
         if (g.kn_K) {
             const long long my_units = (total_units - blockIdx.x + gridDim.x - 1) / gridDim.x;   // >= 1
-            resident_knorm(g, gen, tiles, (uint32_t)S::kTileBytes, bar_kn, bar_tfull + 8 * (uint32_t)(my_units - 1),
+            resident_knorm(g, &map_k, gen, tiles, (uint32_t)S::kTileBytes, bar_kn, bar_tfull + 8 * (uint32_t)(my_units - 1),
                            abort_flag, k.limit_of(kRoleLoad | kRoleMma));
         }
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..17)
-        bool ok = true;
         bool stop = false;
         const unsigned long long lim = k.limit_of(kRoleEpi);
-        grid_dependency_wait();
         // tile s (0 or 1) of this CTA's unit number `slot`
         auto tile_call = [&](const ResidentUnit& u, uint32_t slot, int s, bool wait_mma) {
             EpiCall c;
@@ -1098,11 +1095,11 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         tc_fence_after();
         tmem_dealloc(tmem_base, kTmemCols);
     }
-    if (threadIdx.x == 0 && *abort_flag) {
+    if (threadIdx.x == kLoadThread && *abort_flag) {
         // (see gram_tc_kernel: unconsumed operand loads must have landed before the CTA goes away)
         for (uint32_t s = 0; s < kStages; ++s)
             if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
-        if (g.status) atomicMax(g.status, VITCOP_ERR_TIMEOUT);
+        atomicMax(g.status, VITCOP_ERR_TIMEOUT);
     }
     grid_dependency_launch_dependents();
 }
@@ -1175,28 +1172,34 @@ int launch_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k
     return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
 }
 
+// As many CTAs as there are SMs (never fewer than the units need): the shortest chain of units per CTA.
+long long resident_ctas(long long units) {
+    const long long least = (units + kResidentUnits - 1) / kResidentUnits, sms = num_sms();
+    return units < sms ? units : least > sms ? least : sms;
+}
+
 template <int METRIC, bool SPATIAL, int BN>
-int launch_resident_one(const CUtensorMap& ma, const CUtensorMap& mb, const KernelArgs& k, cudaStream_t stream) {
+int launch_resident_one(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mk, const KernelArgs& k, cudaStream_t stream) {
     using S = GemmSmem<kResidentBN>;
     static DoneOnDevice attr_done;
     auto kern = gram_resident_kernel<METRIC, SPATIAL, BN>;
     constexpr int kSmem = S::kTotal + (BN == 64 ? HalfUnitSmem::kEpiBytes - S::kEpiBytes : 0);
     const int arc = allow_dynamic_smem(kern, kSmem, attr_done);
     if (arc != VITCOP_OK) return arc;
-    const long long ctas = (k.total_tiles + kResidentUnits - 1) / kResidentUnits;
     cudaLaunchConfig_t cfg = {};
-    // as many CTAs as there are SMs (never fewer than the units need): the shortest chain of units per CTA
-    cfg.gridDim = dim3((unsigned)(k.total_tiles < num_sms() ? k.total_tiles : (ctas > num_sms() ? ctas : num_sms())));
-    cfg.blockDim = dim3(64 + kResidentEpiThreads);
+    cfg.gridDim = dim3((unsigned)resident_ctas(k.total_tiles));
+    cfg.blockDim = dim3(kResidentThreads);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;          // all CTAs resident together: they wait for one another
     attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl_allowed(true) ? 2 : 1;
     KernelTimeScope timed("gram_resident_kernel", stream);
-    return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
+    return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, mk, k));
 }
 
 }  // namespace
@@ -1205,6 +1208,18 @@ int gram_num_sms() { return num_sms(); }
 
 bool make_rowmajor_bf16_map(CUtensorMap* map, const void* base, int batches, int rows, int cols, int box_rows) {
     return make_feat_map(map, base, batches, rows, cols, box_rows);
+}
+
+bool make_keys_map(CUtensorMap* map, const void* K, int B, int H, int N, int d, int box_tokens, int box_heads) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t row = (cuuint64_t)d * 2;
+    cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)N, (cuuint64_t)H, (cuuint64_t)B};
+    cuuint64_t strides[3] = {row, row * N, row * N * H};
+    cuuint32_t box[4] = {(cuuint32_t)d, (cuuint32_t)box_tokens, (cuuint32_t)box_heads, 1};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(K), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 unsigned long long gram_wait_limit_ns() { return g_wait_ns.load(); }
@@ -1237,6 +1252,7 @@ int launch_gram_sweep(int mode, const void* feat, const GramArgs& args, cudaStre
     k.unit_w = 0;
     k.wait_ns = g_wait_ns.load();
     k.expire_roles = g_expire_roles.load() & 7;
+    k.reports = args.reports;
     if (k.total_tiles <= 0) return VITCOP_OK;
     CUtensorMap ma, mb;
     if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) || !make_feat_map(&mb, feat, args.B, args.n, args.D, BM))
@@ -1272,11 +1288,34 @@ bool gram_resident_halves(int B, int n) {
     return (long long)B * units <= num_sms();
 }
 
+// How a problem is cut into units.
+struct ResidentCut {
+    bool halves;                                           // units of 64 columns
+    int unit_w, extra_per_b;                               // column blocks of a unit; units of a sample that hold no diagonal tile
+    long long total;
+    ResidentCut(int B, int n) {
+        const int TI = (n + BM - 1) / BM, TJ = (n + 63) / 64;
+        halves = gram_resident_halves(B, n);
+        unit_w = (long long)B * TI * (TI + 1) / 2 <= num_sms() ? 1 : 2;
+        const int units = halves ? resident_half_units(TI, TJ) : TI + resident_extra_units(TI, unit_w);
+        extra_per_b = units - (halves ? TJ : TI);
+        total = (long long)B * units;
+    }
+};
+
 bool gram_resident_takes_knorm(int H, int d) {
-    // sixteen or more 16-byte pieces per row (the lane layout of the stand-alone kernel's widest variant), and at
-    // least one chunk of eight tokens must fit the operand buffers
-    if (H <= 0 || d <= 0 || d % 8 || d / 8 < 16) return false;
+    // eight 16-byte pieces per row, or sixteen and more (the lane layouts of the stand-alone kernel that sixteen lanes a token
+    // reproduce), a copy's box of at most 256 elements a side, and at least one chunk of eight tokens must fit the operand buffers
+    if (H <= 0 || H > 256 || d % 8 || d > 256 || (d != 64 && d < 128)) return false;
     return (long long)H * kKnChunkTokens * d * 2 <= (long long)GemmSmem<kResidentBN>::kTileBytes;
+}
+
+// As many chunks of tokens to a CTA as it has buffers for (16 x 576 tokens: 6 samples; all of them hold up the barrier and the
+// searches of the sweep by what the rest takes beside vic_finalize_kernel; 1 x 576: all, one kernel less, 34.8 -> 33.5 us).
+int gram_resident_knorm_samples(int B, int n, int Nv) {
+    const ResidentCut cut(B, n);
+    const long long chunks = (Nv + kKnChunkTokens - 1) / kKnChunkTokens, samples = chunks ? kKnBuffers * resident_ctas(cut.total) / chunks : B;
+    return samples < B ? (int)samples : B;
 }
 
 int launch_gram_resident(const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream) {
@@ -1285,33 +1324,31 @@ int launch_gram_resident(const void* feat, const GramArgs& args, const GramTilin
     k.t = tiling;
     k.g.row0 = 0;
     k.g.row_end = args.n;
-    const bool halves = gram_resident_halves(args.B, args.n);
-    k.unit_w = (long long)args.B * k.t.TI * (k.t.TI + 1) / 2 <= num_sms() ? 1 : 2;
-    k.extra_units_per_b = resident_extra_units(k.t.TI, k.unit_w);
-    k.total_tiles = (long long)args.B * (k.t.TI + k.extra_units_per_b);
-    if (halves) {
-        const int TJ = (args.n + 63) / 64, units = resident_half_units(k.t.TI, TJ);
-        k.extra_units_per_b = units - TJ;
-        k.total_tiles = (long long)args.B * units;
-    }
+    const ResidentCut cut(args.B, args.n);
+    const bool halves = cut.halves;
+    k.unit_w = cut.unit_w;
+    k.extra_units_per_b = cut.extra_per_b;
+    k.total_tiles = cut.total;
     k.wait_ns = g_wait_ns.load();
     k.expire_roles = g_expire_roles.load() & 7;
+    k.reports = 0;
     if (k.total_tiles <= 0) return VITCOP_OK;
     if (k.total_tiles > (long long)kResidentUnits * num_sms()) return VITCOP_ERR_INVALID_ARG;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mk = {};
     if (!make_feat_map(&ma, feat, args.B, args.n, args.D, BM) ||
         !make_feat_map(&mb, feat, args.B, args.n, args.D, halves ? 64 : BM * k.unit_w))
         return VITCOP_ERR_CUDA;
+    if (args.kn_K && !make_keys_map(&mk, args.kn_K, args.kn_B, args.kn_H, args.kn_N, args.kn_d, kKnChunkTokens, args.kn_H)) return VITCOP_ERR_CUDA;
     const bool euclid = args.metric == 1;
     const bool spatial = args.tau2 >= 0.f && args.pos != nullptr;
     if (halves) {
         if (spatial)
-            return euclid ? launch_resident_one<1, true, 64>(ma, mb, k, stream) : launch_resident_one<0, true, 64>(ma, mb, k, stream);
-        return euclid ? launch_resident_one<1, false, 64>(ma, mb, k, stream) : launch_resident_one<0, false, 64>(ma, mb, k, stream);
+            return euclid ? launch_resident_one<1, true, 64>(ma, mb, mk, k, stream) : launch_resident_one<0, true, 64>(ma, mb, mk, k, stream);
+        return euclid ? launch_resident_one<1, false, 64>(ma, mb, mk, k, stream) : launch_resident_one<0, false, 64>(ma, mb, mk, k, stream);
     }
     if (spatial)
-        return euclid ? launch_resident_one<1, true, BM>(ma, mb, k, stream) : launch_resident_one<0, true, BM>(ma, mb, k, stream);
-    return euclid ? launch_resident_one<1, false, BM>(ma, mb, k, stream) : launch_resident_one<0, false, BM>(ma, mb, k, stream);
+        return euclid ? launch_resident_one<1, true, BM>(ma, mb, mk, k, stream) : launch_resident_one<0, true, BM>(ma, mb, mk, k, stream);
+    return euclid ? launch_resident_one<1, false, BM>(ma, mb, mk, k, stream) : launch_resident_one<0, false, BM>(ma, mb, mk, k, stream);
 }
 
 }  // namespace vitcop

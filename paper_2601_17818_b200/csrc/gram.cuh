@@ -52,10 +52,10 @@ struct GramArgs {
     float* a_out;               // [B, n]
     float* rho_out;             // [B, n] written by the resident sweep (same memory as rho)
     float* rho_user;            // [B, n] optional copy of rho for the caller
-    unsigned int* grid_sync;    // zeroed counter for the resident sweep's grid-wide barrier
-    uint32_t* ready;            // resident sweep, zeroed [B, n]: a token's factor (w, or for euclid a) once it is known, as its
-                                // bits + 1
-    // Optional K-norm (Eq. 4) for the resident sweep's load and MMA warps to stream once their own work is issued:
+    unsigned int* grid_sync;    // counter of the resident sweep's grid-wide barrier (a word of the status block)
+    uint32_t* ready;            // resident sweep [B, n]: a token's factor (w, or for euclid a) once it is known, as its bits + 1
+                                // (the sweep clears both before it uses them)
+    // Optional K-norm (Eq. 4) for the resident sweep's warps beside the epilogue's to stream once the MMAs are done:
     // K bf16 [kn_B, kn_H, kn_N, kn_d] dense, span [kn_vis_start, kn_vis_start + kn_Nv), score [kn_B, kn_Nv].
     // Only shapes gram_resident_takes_knorm accepts.
     const void* kn_K;
@@ -64,6 +64,7 @@ struct GramArgs {
     float4* bbox;               // [B, ceil(n / 128)] bounding box (min x, min y, max x, max y) of every row block's
                                 // positions, or nullptr: written by GRAM_DIAG
     int* status;                // device status word
+    int reports;                // GRAM_DIAG: clear the status word; CTAs that give up report it (internal.cuh) to rho_reduce_kernel
 };
 
 // rho of token i of one sample from the partial sums of the tiles that hold it, in a fixed order (reproducible
@@ -125,6 +126,9 @@ bool gram_fits_resident(int B, int n);
 
 // True when the resident sweep can compute the K-norm of keys with H heads of d elements on the side.
 bool gram_resident_takes_knorm(int H, int d);
+
+// How many leading samples' K-norm, over spans of Nv tokens, the resident sweep of [B, n] finishes without being held up.
+int gram_resident_knorm_samples(int B, int n, int Nv);
 
 // One kernel for the norms, Eq. 2 and Eq. 3 on small problems: every CTA keeps the accumulators of its tiles in
 // tensor memory; the diagonal tiles publish the per-token factors, which the density epilogues of the other tiles wait for

@@ -12,6 +12,10 @@ namespace vitcop {
 
 // Device status word lives in the first 256 bytes of every workspace.
 constexpr size_t kStatusBytes = 256;
+// A kernel that nothing of its call precedes finds the status word as the last call left it, and none of its CTAs can clear it for
+// the others.  Its CTAs report in a byte each whether they gave up, and a later kernel of the call sets the word.  (A memset
+// in front of the first kernel is 1.2 us of its own and another 1.5 until the kernel behind it starts.)
+constexpr int kReportsAt = 64, kMaxReports = (int)kStatusBytes - kReportsAt;
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -84,8 +88,6 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
 size_t filter_workspace_bytes(int B, int n, int D);
 // The least that launch_filter takes: with less than filter_workspace_bytes the samples go through in smaller groups.
 size_t filter_workspace_least_bytes(int B, int n);
-// Leading bytes of the filter workspace that must be zero when launch_filter starts (status block and published factors).
-size_t filter_zeroed_bytes(int B, int n);
 size_t similarity_workspace_bytes(int B, int n, int D);
 int launch_filter(const void* feat, const float* pos, int B, int n, int D, const vitcop_filter_params& p,
                   int n_centers, int32_t* label, int32_t* n_clusters, float* rho, float* delta2, int32_t* parent,
@@ -118,6 +120,17 @@ __device__ __forceinline__ float bf16hi(uint32_t u) { return __uint_as_float(u &
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void report_gave_up(int* status, bool gave_up) {
+    reinterpret_cast<volatile uint8_t*>(status)[kReportsAt + blockIdx.x] = gave_up ? 1 : 0;
+}
+// Called by a warp, behind the kernel whose `ctas` CTAs reported.
+__device__ __forceinline__ bool any_gave_up(const int* status, int ctas) {
+    bool any = false;
+    for (int c = threadIdx.x & 31; c < ctas; c += 32)
+        any |= reinterpret_cast<const volatile uint8_t*>(status)[kReportsAt + c] != 0;
+    return __any_sync(0xffffffffu, any);
 }
 
 // Exclusive prefix count of `flag` over a CTA of 1024 threads, in thread order; `total` receives the CTA-wide

@@ -50,6 +50,7 @@ struct KprojArgs {
     const int32_t* position;        // [B, N] or null (token index)
     int n_pos;
     int* status;
+    int reports;                    // every CTA reports (internal.cuh) to the kernel behind this one, which sets the status word
     unsigned long long wait_ns;
     int expire_roles;               // roles whose waits give up at once: 1 load warp, 2 MMA warp, 4 epilogue warps
     __device__ __forceinline__ unsigned long long limit_of(int role) const { return (expire_roles & role) ? 0ull : wait_ns; }
@@ -311,8 +312,9 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             const unsigned long long t0 = global_ns();
             while (global_ns() - t0 < kDrainLimitNs) {}
         }
-        if (k.status) atomicMax(k.status, VITCOP_ERR_TIMEOUT);
+        if (!k.reports) atomicMax(k.status, VITCOP_ERR_TIMEOUT);
     }
+    if (threadIdx.x == 0 && k.reports) report_gave_up(k.status, *abort_flag != 0);
     tc_fence_before();
     __syncthreads();
     if constexpr (kPair) cluster_sync_all();               // neither CTA leaves while the other may reach into it
@@ -326,8 +328,13 @@ kproj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 
 // score[b, i] = sqrt( sum over the slots, in order, of the partial sums of token vis_start + i ).
 __global__ void kproj_score_kernel(const float* __restrict__ part, int M, int slots, int N, int vis_start, int Nv,
-                                   float* __restrict__ score) {
+                                   float* __restrict__ score, int* __restrict__ status, int reports) {
+    grid_dependency_launch_dependents();
     grid_dependency_wait();
+    if (reports > 0 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
+        const bool gave_up = any_gave_up(status, reports);
+        if (threadIdx.x == 0) *status = gave_up ? VITCOP_ERR_TIMEOUT : VITCOP_OK;
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (i >= Nv) return;
     const size_t m = (size_t)b * N + vis_start + i;
@@ -375,7 +382,12 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     k.status = static_cast<int*>(workspace);
     k.wait_ns = gram_wait_limit_ns();
     k.expire_roles = pair_expire_roles();
-    if (k.M <= 0 || k.NO <= 0) return VITCOP_OK;
+    const bool scores = Nv > 0 && score;
+    k.reports = scores && gram_num_sms() <= kMaxReports;
+    if (!k.reports) {
+        const int rc = record_cuda(cudaMemsetAsync(workspace, 0, kStatusBytes, stream));
+        if (rc != VITCOP_OK) return rc;
+    }
     const bool rope = cos_tab != nullptr;
     // (a rotated head of 256 columns cannot be cut: its halves are turned together)
     const bool may_cut = !(rope && d > BN / 2);
@@ -400,12 +412,20 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     if (arc != VITCOP_OK) return arc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ctas * (n_items < units ? n_items : units)));
-    cudaLaunchAttribute shape[1];
-    shape[0].id = cudaLaunchAttributeClusterDimension;
-    shape[0].val.clusterDim.x = (unsigned)ctas;
-    shape[0].val.clusterDim.y = shape[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute shape[2];
+    int n_shape = 0;
+    if (pdl_allowed(k.reports)) {                          // (a memset is no kernel to overlap with)
+        shape[n_shape].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        shape[n_shape++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (pair) {
+        shape[n_shape].id = cudaLaunchAttributeClusterDimension;
+        shape[n_shape].val.clusterDim.x = (unsigned)ctas;
+        shape[n_shape].val.clusterDim.y = shape[n_shape].val.clusterDim.z = 1;
+        ++n_shape;
+    }
     cfg.attrs = shape;
-    cfg.numAttrs = pair ? 1 : 0;
+    cfg.numAttrs = n_shape;
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
@@ -414,7 +434,7 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
         KernelTimeScope timed("kproj_kernel", stream);
         rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, mh, k, n_items));
     }
-    if (rc != VITCOP_OK || Nv <= 0 || !score) return rc;
+    if (rc != VITCOP_OK || !scores) return rc;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -426,7 +446,7 @@ int launch_kproj_knorm(const void* hidden, const void* W, int B, int N, int Dh, 
     c2.numAttrs = pdl_allowed(true) ? 1 : 0;
     KernelTimeScope timed("kproj_score_kernel", stream);
     return record_cuda(cudaLaunchKernelEx(&c2, kproj_score_kernel, (const float*)k.part, k.M, 2 * k.TJ, N, vis_start, Nv,
-                                          score));
+                                          score, k.status, k.reports ? (int)cfg.gridDim.x : 0));
 }
 
 }  // namespace vitcop

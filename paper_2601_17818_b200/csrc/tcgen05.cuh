@@ -18,7 +18,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
-
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
                  : "memory");
@@ -152,5 +157,9 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
 // 3-D tensor map (cols, rows, batches) of a row-major bf16 tensor with a (64, box_rows, 1) box and the 128-byte
 // swizzle (host; gram.cu).  Rows past `rows` read as zero.
 bool make_rowmajor_bf16_map(CUtensorMap* map, const void* base, int batches, int rows, int cols, int box_rows);
+
+// 4-D tensor map (d, N, H, B) of dense bf16 keys with a (d, box_tokens, box_heads, 1) box (host; gram.cu).  What lies past the
+// sequence or the heads reads as zero.
+bool make_keys_map(CUtensorMap* map, const void* K, int B, int H, int N, int d, int box_tokens, int box_heads);
 
 }  // namespace vitcop
