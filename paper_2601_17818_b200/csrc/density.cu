@@ -17,6 +17,11 @@
 // next tile's tokens and join the column warps' parts of the previous one, so that neither the trip to the L2 nor the joining
 // stands between two tiles.
 //
+// The sweep leaves the HBM mostly idle, so four warps more may compute a K-norm (Eq. 4) meanwhile, fed by tensor copies through the
+// shared memory of one of the six stages.  (With plain loads the warps have too few of them in flight: 112 us for 188 MB of keys beside a sweep
+// of 70; one warp with the copies, in the place of an auxiliary one, takes 126.  With more than five warps to a quarter of the SM a
+// thread has 80 registers instead of 96.)
+//
 // Measured: 8 x 2880 x 1024 75 us (60 us with an empty epilogue), 2 x 16384 x 1280 519 us (433 us with an empty epilogue:
 // 0.69 Tflop at the rate cuBLAS reaches in a burst; the stores of the Gram values are about 30 of the rest).  Sixteen warps of
 // one role: 70 and 517 us, but another order of the sums.  A sweep of single SMs on 128 x 256 tiles, without the minima: 68 and
@@ -27,6 +32,7 @@
 #include "async_copy.cuh"
 #include "density.cuh"
 #include "f32x2.cuh"
+#include "knorm.cuh"
 #include "tcgen05.cuh"
 
 namespace vitcop {
@@ -37,8 +43,10 @@ constexpr int kBoxRows = 64;                      // column tokens per load: a C
 constexpr int kABytes = BM * BK * 2, kBBytes = BN / 2 * BK * 2, kStageBytes = kABytes + kBBytes;
 constexpr int kHalfBlks = BM / kBlk;              // blocks of a warp: 128 columns
 constexpr int kEpiWarps = 16, kEpiThreads = kEpiWarps * 32, kAuxThreads = 64;
-constexpr int kThreads = 64 + kEpiThreads + kAuxThreads;
 constexpr int kTileThreads = kEpiThreads + kAuxThreads;   // meet once per tile
+// A K-norm on the side has four warps more, and one of the six stages is its buffers.
+constexpr int kKnWarps = 4, kKnHeads = 4, kKnBufBytes = 64 * kKnHeads * 16;
+__host__ __device__ constexpr int threads(bool knorm) { return 64 + kTileThreads + (knorm ? kKnWarps * 32 : 0); }
 constexpr float kInf = __builtin_huge_valf();
 constexpr int kRoleLoad = 1, kRoleMma = 2, kRoleEpi = 4;
 
@@ -52,9 +60,11 @@ struct EpiSmem {
     float rowmin[2][BM][4];
     int far[2][4];
 };
-constexpr int kStages = 6;
+constexpr int kMaxStages = 6;
+__host__ __device__ constexpr int stages(bool knorm) { return knorm ? kMaxStages - 1 : kMaxStages; }
+static_assert(kKnWarps * 2 * kKnBufBytes == kStageBytes, "the K-norm's buffers");
 template <int METRIC>
-__host__ __device__ constexpr int smem_bytes() { return 1024 + kStages * kStageBytes + (int)sizeof(EpiSmem<METRIC>) + 256; }
+__host__ __device__ constexpr int smem_bytes() { return 1024 + kMaxStages * kStageBytes + (int)sizeof(EpiSmem<METRIC>) + 256; }
 static_assert(smem_bytes<0>() <= 227 * 1024 && smem_bytes<1>() <= 227 * 1024, "shared memory of an SM");
 
 struct KernelArgs {
@@ -144,22 +154,101 @@ __device__ __forceinline__ int column_of(int lane) {
     return 8 * (((lane >> 4) & 1) * 2 + ((lane >> 3) & 1)) + 2 * (lane & 3) + ((lane >> 2) & 1);
 }
 
-template <int METRIC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+// The K-norm (Eq. 4) of the job's samples, shared out over the side warps of all CTAs.  A warp takes 64 16-byte lanes of tokens at a time
+// (4 tokens of d = 128, 8 of d = 64), kKnHeads heads per copy into one of its two buffers; a lane carries two of the tokens, so
+// that two chains of sums are under way, with the arithmetic and the order of the stand-alone kernel (LPR lanes a token).
+template <int LPR>
+__device__ __forceinline__ void side_knorm(const KnormJob& kn, const CUtensorMap* map_k, const uint8_t* buf_gen, uint32_t buf_smem, uint32_t bars,
+                                           int slot, int slots, volatile int* abort_flag, unsigned long long limit_ns) {
+    constexpr int kTok = 2 * (32 / LPR);                   // tokens of a unit
+    const int lane = threadIdx.x & 31, sub = lane % LPR, tk = lane / LPR;
+    const int per_b = (kn.Nv + kTok - 1) / kTok, units = kn.B * per_b, parts = (kn.H + kKnHeads - 1) / kKnHeads;
+    const int copies = units > slot ? (units - slot + slots - 1) / slots * parts : 0;
+    struct Unit {
+        int b, r;                                          // sample, unit of it
+        __device__ __forceinline__ void advance(int by, int per) {
+            for (r += by; r >= per; r -= per) ++b;
+        }
+    };
+    Unit next = {0, 0}, now = {0, 0};                      // of the next copy (lane 0); of the sums
+    now.advance(slot, per_b);
+    next = now;
+    int part = 0, issued = 0;
+    auto issue = [&]() {
+        const uint32_t buf = (uint32_t)issued & 1u;
+        mbar_expect_tx(bars + 8 * buf, kKnBufBytes);
+        tma_load_4d_once(buf_smem + buf * kKnBufBytes, map_k, bars + 8 * buf, 0, kn.vis_start + next.r * kTok, part * kKnHeads, next.b);
+        if (++part == parts) { part = 0; next.advance(slots, per_b); }
+        ++issued;
+    };
+    if (lane == 0)
+        while (issued < copies && issued < 2) issue();
+    int p = 0;
+    bool ok = true;
+    float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
+    int c = 0;
+#pragma unroll 1
+    for (; c < copies; ++c) {
+        const uint32_t buf = (uint32_t)c & 1u;
+        ok = __all_sync(0xffffffffu, mbar_wait(bars + 8 * buf, (uint32_t)(c >> 1) & 1u, abort_flag, limit_ns));
+        if (!ok) break;
+        const uint4* rows = reinterpret_cast<const uint4*>(buf_gen + buf * kKnBufBytes) + lane;
+        uint4 x[kKnHeads], y[kKnHeads];                    // (heads past the last are zeros: their squares change nothing)
+#pragma unroll
+        for (int h = 0; h < kKnHeads; ++h) {
+            x[h] = rows[h * 64];
+            y[h] = rows[h * 64 + 32];
+        }
+#pragma unroll
+        for (int h = 0; h < kKnHeads; ++h) {
+            knorm_sq_acc(x[h], a0, a1);
+            knorm_sq_acc(y[h], b0, b1);
+        }
+        __syncwarp();                                      // the buffer has been read by everyone
+        if (lane == 0 && issued < copies) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            issue();
+        }
+        if (++p < parts) continue;
+        float s0 = a0 + a1, s1 = b0 + b1;
+#pragma unroll
+        for (int off = LPR / 2; off > 0; off >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        }
+        const int i = now.r * kTok + tk;
+        if (sub == 0) {
+            float* const out = kn.score + (int64_t)now.b * kn.Nv;
+            if (i < kn.Nv) out[i] = sqrtf(s0);
+            if (i + kTok / 2 < kn.Nv) out[i + kTok / 2] = sqrtf(s1);
+        }
+        p = 0;
+        a0 = a1 = b0 = b1 = 0.f;
+        now.advance(slots, per_b);
+    }
+    if (!ok && lane == 0)                                  // the copies still in flight land before the CTA's shared memory goes away
+        for (int j = c; j < issued; ++j) mbar_drain(bars + 8 * (j & 1), (uint32_t)(j >> 1) & 1u);
+}
+
+template <int METRIC, bool KNORM>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads(KNORM), 1)
 density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                     const __grid_constant__ KernelArgs k) {
+                     const __grid_constant__ CUtensorMap map_k, const __grid_constant__ KernelArgs k) {
+    constexpr int kStages = stages(KNORM);
     const SweepArgs& g = k.g;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;                 // 1024-byte aligned for the 128B swizzle
     uint8_t* gen = smem_raw + (tiles - raw);
-    EpiSmem<METRIC>& sm = *reinterpret_cast<EpiSmem<METRIC>*>(gen + kStages * kStageBytes);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + kStages * kStageBytes + sizeof(EpiSmem<METRIC>));
+    EpiSmem<METRIC>& sm = *reinterpret_cast<EpiSmem<METRIC>*>(gen + kMaxStages * kStageBytes);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gen + kMaxStages * kStageBytes + sizeof(EpiSmem<METRIC>));
     // The leader's full barriers count the bytes of both CTAs and its tempty barriers the epilogue warps of both; empty and
     // tfull are signalled in both CTAs by the leader's commits.
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kStages;
     const uint32_t bar_tfull = bar_empty + 8 * kStages, bar_tempty = bar_tfull + 16, bar_drain = bar_tempty + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
+    const uint32_t bar_kn = bar_drain + 8;
+    static_assert((2 * kStages + 5 + 2 * kKnWarps) * 8 + 8 <= 256, "barriers");
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5 + 2 * kKnWarps);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const uint32_t abort_addr = smem_u32(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -177,6 +266,7 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             mbar_init(bar_tempty + 8 * a, 2 * kEpiWarps);
         }
         mbar_init(bar_drain, 1);
+        for (int a = 0; a < 2 * kKnWarps; ++a) mbar_init(bar_kn + 8 * a, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
@@ -266,6 +356,12 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             if (!ok) raise_abort_pair(abort_addr, rank);
             tc_commit_pair(bar_drain);                     // (waited for below)
         }
+    } else if (KNORM && warp >= 2 + kTileThreads / 32) {
+        // ------------------------------------------------------------------ K-norm (keys are an input of the whole call, as the features)
+        const int w = warp - (2 + kTileThreads / 32), at = kStages * kStageBytes + w * 2 * kKnBufBytes;
+        const int slot = (int)blockIdx.x * kKnWarps + w, slots = (int)gridDim.x * kKnWarps;
+        if (g.kn.d == 64) side_knorm<8>(g.kn, &map_k, gen + at, tiles + at, bar_kn + 16 * w, slot, slots, abort_flag, k.limit_of(0));
+        else side_knorm<16>(g.kn, &map_k, gen + at, tiles + at, bar_kn + 16 * w, slot, slots, abort_flag, k.limit_of(0));
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2 .. 17), auxiliary warps
         const int TI = g.t.TI, nb = g.t.n_blk();
@@ -572,6 +668,19 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
 
 }  // namespace
 
+// In microseconds.  The sweep runs at 0.9 PFLOP/s or more and has room for 2.6 MB of keys in each (four warps of every SM, 5 us
+// slower by them and the missing stage); the stand-alone kernel reads 6.2 MB, the first 4 + n / 600 of them beside
+// vic_finalize_kernel.  So worth it where that leaves 8 to be gained: 8 x 2880 tokens x 32 heads 193 -> 178 (whole call), 4 x 4608 203 ->
+// 200; not for 2 x 16384 x 4, whose keys all fit beside vic_finalize_kernel.
+int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D) {
+    if (!job.K || job.B <= 0 || job.H <= 0 || job.Nv <= 0 || (job.d != 64 && job.d != 128)) return 0;
+    const double mb = 2e-6 * job.H * job.d * job.Nv, sweep = 1e-9 / 0.9 * samples * n * (double)n * D;
+    const double fits = 2.6 * sweep / mb, hidden = 4.0 + n / 600.0;
+    const int s = fits < job.B ? (int)fits : job.B;
+    auto left = [&](int b) { return b * mb / 6.2 > hidden ? b * mb / 6.2 - hidden : 0.0; };
+    return left(job.B) - left(job.B - s) >= 8.0 ? s : 0;
+}
+
 int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cudaStream_t stream, bool pdl) {
     KernelArgs k;
     k.g = args;
@@ -585,18 +694,21 @@ int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cu
     k.n_full = (int)(total - cut);
     k.n_items = (int)(total + cut);
     k.inv_tiles = 1.f / (float)args.t.tiles_per_b;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mk = {};
+    const bool kn = k.g.kn.K != nullptr;
     if (!make_rowmajor_bf16_map(&ma, feat, args.B, args.n, args.D, BM) ||
         !make_rowmajor_bf16_map(&mb, feat, args.B, args.n, args.D, kBoxRows))
         return VITCOP_ERR_CUDA;
+    if (kn && !make_keys_map(&mk, k.g.kn.K, k.g.kn.B, k.g.kn.H, k.g.kn.N, k.g.kn.d, 512 / k.g.kn.d, kKnHeads)) return VITCOP_ERR_CUDA;
     const int smem = metric == 1 ? smem_bytes<1>() : smem_bytes<0>();
-    auto kern = metric == 1 ? density_sweep_kernel<1> : density_sweep_kernel<0>;
-    static DoneOnDevice attr_done[2];
-    const int arc = allow_dynamic_smem(kern, smem, attr_done[metric == 1]);
+    auto kern = metric == 1 ? (kn ? density_sweep_kernel<1, true> : density_sweep_kernel<1, false>)
+                            : (kn ? density_sweep_kernel<0, true> : density_sweep_kernel<0, false>);
+    static DoneOnDevice attr_done[2][2];
+    const int arc = allow_dynamic_smem(kern, smem, attr_done[metric == 1][kn]);
     if (arc != VITCOP_OK) return arc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * (k.n_items < pairs ? k.n_items : pairs)));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads(kn));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -605,7 +717,7 @@ int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cu
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(pdl) ? 1 : 0;
     KernelTimeScope timed("density_sweep_kernel", stream);
-    return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, k));
+    return record_cuda(cudaLaunchKernelEx(&cfg, kern, ma, mb, mk, k));
 }
 
 }  // namespace vitcop

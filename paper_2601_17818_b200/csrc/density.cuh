@@ -92,6 +92,7 @@ struct SweepArgs {
     int* status;                // device status word
     int diag_reports;           // CTAs of the diagonal in front that reported whether they gave up, 0: they set the word themselves
     SweepTiling t;
+    KnormJob kn;                // K-norm that the sweep computes on the side (kn.K null: none); d = 64 or 128
 };
 
 // Eq. 3 only pairs tokens within the spatial radius, so blocks of 128 x 128 pairs whose row tokens all lie farther than the
@@ -104,6 +105,9 @@ __device__ __forceinline__ bool blocks_outside_radius(const float4& r, const flo
     const float dy = fmaxf(0.f, fmaxf(r.y - c.w, c.y - r.w));
     return fmaf(dx, dx, dy * dy) > tau2;
 }
+
+// How many leading samples' K-norm a sweep over `samples` samples of n tokens should compute on the side.
+int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D);
 
 // Eq. 2: rho partials, Gram values and block minima (metric: 0 cosine, 1 euclid).
 int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cudaStream_t stream, bool pdl);

@@ -505,6 +505,10 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             s.status = g.status;
             s.diag_reports = g.reports ? diag_ctas : 0;
             s.t = tiling;
+            if (knorm && b0 == 0 && (knorm_in_sweep = sweep_knorm_samples(*knorm, s.B, n, D)) > 0) {
+                s.kn = *knorm;
+                s.kn.B = knorm_in_sweep;
+            }
             rc = launch_density_sweep(static_cast<const uint16_t*>(feat) + at * D, s, p.metric, stream, true);
             if (rc != VITCOP_OK) return rc;
             {
@@ -544,8 +548,8 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     if (knorm && knorm_in_sweep < knorm->B) {
         // vic_finalize_kernel runs one CTA per sample and releases its dependents when it starts: the K-norm, which
         // does not depend on the clustering, streams K from HBM on the other SMs meanwhile and waits for the
-        // finalize kernel before it ends.  (Beside the Gram sweep it would not fit: that kernel's CTAs hold most
-        // of each SM's registers.)
+        // finalize kernel before it ends.  (Beside a Gram sweep it would not fit: those kernels' CTAs hold most of each SM's
+        // registers.)
         const int64_t stride_b = (int64_t)knorm->H * knorm->N * knorm->d;
         rc = launch_knorm(static_cast<const uint16_t*>(knorm->K) + (size_t)knorm_in_sweep * stride_b,
                           knorm->B - knorm_in_sweep, knorm->H, knorm->d, stride_b, (int64_t)knorm->N * knorm->d, knorm->d,

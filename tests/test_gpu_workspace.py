@@ -1,4 +1,4 @@
-"""What a call finds in its workspace does not matter, and the K-norm computed beside the one-kernel sweep has the bits of the
+"""What a call finds in its workspace does not matter, and the K-norm computed beside a sweep has the bits of the
 stand-alone one (``-m gpu``).
 
 The filter and the key projection are not preceded by a memset: their kernels clear what they need themselves, so a workspace full of
@@ -68,8 +68,12 @@ def test_kproj_whatever_the_workspace_holds(N, fill):
 @pytest.mark.parametrize("H,d", [(1, 64), (5, 64), (32, 128), (3, 128), (40, 136), (17, 256), (6, 96), (2, 512)])
 @pytest.mark.parametrize("B,n,T", [(1, 1, 1), (2, 9, 0), (3, 129, 9), (1, 577, 3), (16, 200, 2)])
 def test_norms_beside_the_sweep_are_the_stand_alone_ones(B, n, T, H, d):
+    _compare_norms(B, n, T, H, d, 64)
+
+
+def _compare_norms(B, n, T, H, d, D):
     N, budget, nc = n + T, max(1, n // 2), max(1, n // 20)
-    feat = _randn(n, B, n, 64).to(torch.bfloat16)
+    feat = _randn(n, B, n, D).to(torch.bfloat16)
     K = (_randn(d, B, H, N, d) * torch.exp(0.5 * _randn(H, B, 1, N, 1))).to(torch.bfloat16)
     vis_start = T // 2
     ref = torch.zeros((B, n), dtype=torch.float32, device=DEV)
@@ -78,8 +82,16 @@ def test_norms_beside_the_sweep_are_the_stand_alone_ones(B, n, T, H, d):
     score, cap = torch.zeros_like(ref), T + budget
     hidden, hidden_out = torch.zeros((B, N, 8), dtype=torch.bfloat16, device=DEV), torch.zeros((B, cap, 8), dtype=torch.bfloat16, device=DEV)
     K_out, V_out = (torch.zeros((B, H, cap, d), dtype=torch.bfloat16, device=DEV) for _ in range(2))
-    ws = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=64)
+    ws = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=D)
     vb.vitcop_collaborative_step(feat, None, hidden, K, K, vis_start, budget, hidden_out, K_out, V_out, i32(B), i32(B, n), i32(B), ws,
                                  n_centers=nc, score_out=score)
     torch.cuda.synchronize()
     assert torch.equal(score, ref)
+
+
+# Beside the density sweep: all of the samples or, where the sweep is over before, the first ones of them; units of four and eight
+# tokens that end inside a copy, heads that end inside one.
+@pytest.mark.parametrize("B,n,T,H,d,D", [(8, 2881, 3, 31, 128, 1024), (9, 2879, 0, 62, 64, 1024), (20, 1501, 1, 32, 128, 1024),
+                                         (4, 4606, 2, 33, 128, 1024)])
+def test_norms_beside_the_density_sweep_are_the_stand_alone_ones(B, n, T, H, d, D):
+    _compare_norms(B, n, T, H, d, D)
