@@ -1310,12 +1310,12 @@ bool gram_resident_takes_knorm(int H, int d) {
     return (long long)H * kKnChunkTokens * d * 2 <= (long long)GemmSmem<kResidentBN>::kTileBytes;
 }
 
-// As many chunks of tokens to a CTA as it has buffers for (16 x 576 tokens: 6 samples; all of them hold up the barrier and the
-// searches of the sweep by what the rest takes beside vic_finalize_kernel; 1 x 576: all, one kernel less, 34.8 -> 33.5 us).
+// All of them where a CTA has a buffer for each of its chunks of tokens: one kernel less (1 x 576 tokens 34.8 -> 33.5 us).  Otherwise two
+// and a half chunks to a CTA: more hold up the sweep's barrier and searches by as much as they take beside vic_finalize_kernel
+// (16 x 576 tokens, inputs that change: 62.0 us with 5 of the samples, 62.6 with 6).
 int gram_resident_knorm_samples(int B, int n, int Nv) {
-    const ResidentCut cut(B, n);
-    const long long chunks = (Nv + kKnChunkTokens - 1) / kKnChunkTokens, samples = chunks ? kKnBuffers * resident_ctas(cut.total) / chunks : B;
-    return samples < B ? (int)samples : B;
+    const long long ctas = resident_ctas(ResidentCut(B, n).total), chunks = (Nv + kKnChunkTokens - 1) / kKnChunkTokens;
+    return chunks * B <= kKnBuffers * ctas ? B : (int)(5 * ctas / (2 * chunks));
 }
 
 int launch_gram_resident(const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream) {
