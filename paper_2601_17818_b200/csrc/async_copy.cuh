@@ -1,4 +1,4 @@
-// Shared-memory barriers (mbarrier), bounded waits on them and bulk asynchronous copies into shared memory: the
+// Thread-block clusters, shared-memory barriers (mbarrier) and bounded waits on them: the
 // plumbing shared by the kernels that stage data through shared memory with the copy engine (gram.cu, density.cu, kproj.cu).
 // Every wait is bounded: when the limit runs out the caller's CTA-wide abort flag is raised and the wait returns
 // false; the kernel then leaves in an orderly way and reports VITCOP_ERR_TIMEOUT.
@@ -78,11 +78,5 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
     const unsigned long long t0 = global_ns();
     while (!mbar_try_wait(bar, parity))
         if (global_ns() - t0 > kDrainLimitNs) break;
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
-                 : "memory");
 }
 }  // namespace vitcop

@@ -1,5 +1,5 @@
-// Per-token arithmetic of the K-norm (Eq. 4), shared by the stand-alone kernel (knorm.cu) and the resident Gram
-// kernel (gram.cu), whose epilogue warps run it while they wait for the tensor cores.
+// Per-token arithmetic of the K-norm (Eq. 4), shared by the stand-alone kernel (knorm.cu) and the two sweeps (gram.cu, density.cu),
+// which run it in warps beside their epilogues.
 #pragma once
 
 #include "internal.cuh"
