@@ -370,12 +370,26 @@ vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_cente
     if (tid == 0) n_clusters[b] = nc;
 }
 
+// In front of the one-kernel sweep: status word, barrier counter and published factors.  The sweep's CTAs have nothing to meet by
+// until these are cleared, and the launch's own barrier has no time limit.  Latency: the sweep starts beside this kernel and waits
+// for it behind its first MMAs, so 1 x 576 tokens (whole call) take 30.8 us where a memset takes 32.2 and clearing inside the sweep,
+// behind the launch's barrier, 32.7; 16 x 576 56.1, 57.2 and 55.2.
+// It lets the sweep go only behind its own wait: the sweep's loads, its K-norm and the early parts of the kernels behind it rest on
+// everything queued before the call being complete by then.
+constexpr int kClearThreads = 256;
+__global__ void __launch_bounds__(kClearThreads) clear_kernel(uint4* __restrict__ words, unsigned pieces) {
+    grid_dependency_wait();
+    grid_dependency_launch_dependents();
+    const unsigned i = blockIdx.x * kClearThreads + threadIdx.x;
+    if (i < pieces) words[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
 // Workspace of the filter: status block | for the one-kernel sweep the tokens' published factors [B, n] | w | a | rho | best |
 // rho partials [B, slots, n_pad] | bounding boxes of the row blocks' positions | and, for problems too large for the one-kernel
-// sweep, what is kept of one group of samples (SweepGroupWs).  The first kernel of a call clears the status block, the
+// sweep, what is kept of one group of samples (SweepGroupWs).  The first kernel of a call clears the status block, in front of the
 // one-kernel sweep the published factors too.  Words of the status block: 0 status, 2 grid barrier.
 // A group is as large as the workspace allows, so every workspace serves that holds one sample of it; the size asked for holds
 // all samples, or as many as fit 1.5 GB (8 x 2880 tokens take 175 MB: one sample at a time would leave half of the SMs without
@@ -452,8 +466,9 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     g.w_out = w; g.a_out = a;
     g.sim_out = nullptr; g.status = reinterpret_cast<int*>(ws);
 
-    // The first kernel of the call is launched without programmatic overlap, so everything queued before the call
-    // (the producer of the features included) has completed when it starts.
+    // Everything queued before the call (the producers of features and keys included) has completed before a kernel of the call
+    // other than the first can start: the diagonal is launched without programmatic overlap, and clear_kernel waits
+    // before it releases the one-kernel sweep.
     int rc;
     int knorm_in_sweep = 0;                                // leading samples whose K-norm the Gram sweep computes
     if (l.resident) {
@@ -468,6 +483,15 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
                 g.kn_K = knorm->K; g.kn_score = knorm->score; g.kn_B = knorm_in_sweep;
                 g.kn_H = knorm->H; g.kn_N = knorm->N; g.kn_d = knorm->d; g.kn_vis_start = knorm->vis_start; g.kn_Nv = knorm->Nv;
             }
+        }
+        {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attr[1];
+            const unsigned pieces = (unsigned)(l.off_w / sizeof(uint4));
+            pdl_config(cfg, attr, dim3((pieces + kClearThreads - 1) / kClearThreads), dim3(kClearThreads), 0, stream, true);
+            KernelTimeScope timed("clear_kernel", stream);
+            rc = record_cuda(cudaLaunchKernelEx(&cfg, clear_kernel, static_cast<uint4*>(workspace), pieces));
+            if (rc != VITCOP_OK) return rc;
         }
         rc = launch_gram_resident(feat, g, make_gram_tiling(n), stream);
         if (rc != VITCOP_OK) return rc;

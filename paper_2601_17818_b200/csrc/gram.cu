@@ -10,17 +10,15 @@
 // rows of the tile: inside each warp a shuffle butterfly for the sums of Eq. 2 and one redux.sync per column for
 // the minima of Eq. 3, then a fixed-order combination of the four warps that share a column range).
 //
-// One persistent CTA per SM, warp-specialised:
+// One persistent CTA per SM, warp-specialised (the one-kernel sweep has two warps more behind these):
 //   warp 0      TMA producer: feature tiles [128 x 64] (128-byte swizzle) into a ring of stages
 //   warp 1      one thread issues tcgen05.mma into one of two TMEM accumulators
 //   warps 2..   epilogue: warp w reads TMEM lanes 32 * (w % 4) .. + 31 (its rows) and one slice of the columns
 // Every wait is bounded; on expiry the CTA raises an abort flag, all roles leave, TMEM is released and
 // VITCOP_ERR_TIMEOUT is written to the status word.
-#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include <atomic>
-#include <utility>
 
 #include "async_copy.cuh"
 #include "f32x2.cuh"
@@ -742,12 +740,11 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 //   2. delta epilogue of every tile, re-reading the accumulators; rho of the tile's rows and columns is summed
 //      from the partials on the way (the diagonal tiles publish it)
 // The grid (at most one CTA per SM) is launched cooperatively, so all CTAs are resident together; factors and barrier
-// are words in global memory with bounded waits.  No wait can form a cycle: a factor is published by a CTA that has
-// waited for nothing but its own tensor-core work.
-// The load warp and the MMA warp are idle once the CTA's last MMA is issued (warp 0, which only speaks for the CTA at the barriers
-// of the launch, before that), and so are, a little later, the
+// are words in global memory, cleared by clear_kernel (filter.cu) in front, with bounded waits.  No wait can form a cycle: a factor
+// is published by a CTA that has waited for nothing but its own tensor-core work and that kernel.
+// The load warp and the MMA warp are idle once the CTA's last MMA is issued, and so are, a little later, the
 // operand buffers and -- for the rest of the kernel, which is arithmetic on the accumulators -- the memory system:
-// if the caller has a K-norm (Eq. 4) to compute, these warps and two more stream K through the operand buffers with bulk
+// if the caller has a K-norm (Eq. 4) to compute, these two warps and two more stream K through the operand buffers with tensor
 // copies and reduce it there (resident_knorm).
 constexpr int kResidentUnits = 2;
 constexpr int kResidentBN = 2 * BM;                       // columns of a unit
@@ -839,7 +836,7 @@ __device__ __forceinline__ ResidentUnit decode_resident_unit(const KernelArgs& k
     return u;
 }
 
-constexpr int kKnChunkTokens = 8;                          // tokens per chunk: 8 threads each
+constexpr int kKnChunkTokens = 8;                          // tokens per chunk: 16 threads each
 constexpr int kKnBuffers = 3;
 
 // K-norm (Eq. 4) by the warps beside the epilogue's, after the CTA's last MMA has completed.  Chunks of eight consecutive
@@ -923,7 +920,6 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
 gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      const __grid_constant__ CUtensorMap map_k, const KernelArgs k) {
     constexpr bool HALF = BN == 64;
-    constexpr int kLoadThread = 32, kMmaThread = 64 + kResidentEpiThreads;
     constexpr int NS = 4;
     using S = GemmSmem<kResidentBN>;                       // stages of 128 + 256 operand rows
     constexpr uint32_t kStages = HALF ? HalfUnitSmem::kStages : S::kStages;
@@ -966,69 +962,65 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-    grid_dependency_wait();                                // (whatever was queued before the call has completed)
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
 
     const long long total_units = k.total_tiles;          // <= kResidentUnits * gridDim.x (checked by the launcher)
     const int KB = g.D / BK;
-    uint32_t issued = 0, issued_parity = 0;               // load thread, per stage: a load was issued / parity of its phase
-    uint32_t stage = 0, phase = 0;                         // load and MMA warp
-    bool ok = true;
-    auto load_unit = [&](long long t) {
-        const unsigned long long lim = k.limit_of(kRoleLoad);
-        const ResidentUnit u = unit_of(t);
-        const int I0 = u.ti * BM, J0 = u.tj0 * BN;
-        for (int kb = 0; kb < KB; ++kb) {
-            if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
-            const uint32_t sa = tiles + stage * kStageBytes;
-            // rows of the box past the sample's last token are zero-filled and still count as received
-            mbar_expect_tx(bar_full + 8 * stage, HALF ? kStageBytes : S::kABytes + (uint32_t)k.unit_w * S::kABytes);
-            tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, I0, u.b);
-            tma_load_3d(sa + S::kABytes, &map_b, bar_full + 8 * stage, kb * BK, J0, u.b);
-            issued |= 1u << stage;
-            issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    uint32_t issued = 0, issued_parity = 0;               // thread 0, per stage: a load was issued / parity of its phase
+
+    if (warp == 0) {
+        // ------------------------------------------------------------------ TMA producer
+        if (lane == 0) {
+            const unsigned long long lim = k.limit_of(kRoleLoad);
+            uint32_t stage = 0, phase = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x; ok && t < total_units; t += gridDim.x) {
+                const ResidentUnit u = unit_of(t);
+                const int I0 = u.ti * BM, J0 = u.tj0 * BN;
+                for (int kb = 0; kb < KB; ++kb) {
+                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, lim)) { ok = false; break; }
+                    const uint32_t sa = tiles + stage * kStageBytes;
+                    // rows of the box past the sample's last token are zero-filled and still count as received
+                    mbar_expect_tx(bar_full + 8 * stage, HALF ? kStageBytes : S::kABytes + (uint32_t)k.unit_w * S::kABytes);
+                    tma_load_3d(sa, &map_a, bar_full + 8 * stage, kb * BK, I0, u.b);
+                    tma_load_3d(sa + S::kABytes, &map_b, bar_full + 8 * stage, kb * BK, J0, u.b);
+                    issued |= 1u << stage;
+                    issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                }
+            }
         }
-    };
-    // Status word, barrier counter and factors are cleared here, a slice per CTA; no CTA touches them before all have arrived at
-    // the cooperative launch's own barrier.  (A memset in front of the kernel stood before the first loads.)
-    if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) g.status[threadIdx.x] = 0;
-    const uint32_t n_ready = (uint32_t)g.B * (uint32_t)g.n;       // (a wave of tiles: below 2^23)
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_ready; i += gridDim.x * blockDim.x) g.ready[i] = 0u;
-    tc_fence_before();
-    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
-    auto cleared = grid.barrier_arrive();                  // (begins with a barrier of the CTA)
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    auto mma_unit = [&](uint32_t slot) {                   // this CTA's unit number `slot` -> columns 256 slot ..
-        const uint32_t idesc = !HALF && k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BN);
-        const unsigned long long lim = k.limit_of(kRoleMma);
-        const uint32_t d_tmem = tmem_base + slot * kResidentBN;
-        for (int kb = 0; kb < KB; ++kb) {
-            if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; return; }
-            tc_fence_after();
-            const uint32_t sa = tiles + stage * kStageBytes;
-            const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + S::kABytes);
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer: unit s of this CTA -> columns 256 s ..
+        if (lane == 0) {
+            const uint32_t idesc = !HALF && k.unit_w == 2 ? umma_idesc_bf16(BM, kResidentBN) : umma_idesc_bf16(BM, BN);
+            const unsigned long long lim = k.limit_of(kRoleMma);
+            uint32_t stage = 0, phase = 0;
+            uint32_t slot = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x; ok && t < total_units; t += gridDim.x, ++slot) {
+                const uint32_t d_tmem = tmem_base + slot * kResidentBN;
+                for (int kb = 0; kb < KB; ++kb) {
+                    if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag, lim)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t sa = tiles + stage * kStageBytes;
+                    const uint64_t da = umma_desc_k128(sa), db = umma_desc_k128(sa + S::kABytes);
 #pragma unroll
-            for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(bar_empty + 8 * stage);
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                        tc_mma_bf16(d_tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
+                                    (kb > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(bar_empty + 8 * stage);
+                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                }
+                if (!ok) break;
+                tc_commit(bar_tfull + 8 * slot);
+            }
+            tc_commit(bar_drain);                          // (as in gram_tc_kernel)
+            mbar_drain(bar_drain, 0);
         }
-        tc_commit(bar_tfull + 8 * slot);
-    };
-    // The first unit's loads and MMAs need nothing from another CTA: the warps meet behind them, by when the other CTAs have
-    // arrived too.  (Thread 0 speaks for the CTA, so warp 0 has no other role: its release waits for the stores above, and it
-    // has seen the others arrive before the first MMA completes.)
-    static_assert(kResidentUnits == 2, "a first unit and a second one");
-    const long long second = (long long)blockIdx.x + gridDim.x;
-    if (threadIdx.x == kLoadThread) load_unit(blockIdx.x);
-    if (threadIdx.x == kMmaThread) mma_unit(0);
-    grid.barrier_wait(std::move(cleared));                 // (unbounded, but all CTAs are resident and arrive whatever happens)
-    if (threadIdx.x == kLoadThread && ok && second < total_units) load_unit(second);
-    if (threadIdx.x == kMmaThread) {
-        if (ok && second < total_units) mma_unit(1);
-        tc_commit(bar_drain);                              // (as in gram_tc_kernel)
-        mbar_drain(bar_drain, 0);
     }
     if (warp < 2 || warp >= 2 + kResidentEpiThreads / 32) {
         __syncwarp();
@@ -1039,8 +1031,9 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         }
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..17)
-        bool stop = false;
+        bool ok = true, stop = false;
         const unsigned long long lim = k.limit_of(kRoleEpi);
+        grid_dependency_wait();                            // clear_kernel has cleared status word, factors and barrier counter
         // tile s (0 or 1) of this CTA's unit number `slot`
         auto tile_call = [&](const ResidentUnit& u, uint32_t slot, int s, bool wait_mma) {
             EpiCall c;
@@ -1095,7 +1088,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         tc_fence_after();
         tmem_dealloc(tmem_base, kTmemCols);
     }
-    if (threadIdx.x == kLoadThread && *abort_flag) {
+    if (threadIdx.x == 0 && *abort_flag) {
         // (see gram_tc_kernel: unconsumed operand loads must have landed before the CTA goes away)
         for (uint32_t s = 0; s < kStages; ++s)
             if (issued >> s & 1u) mbar_drain(bar_full + 8 * s, issued_parity >> s & 1u);
@@ -1194,6 +1187,7 @@ int launch_resident_one(const CUtensorMap& ma, const CUtensorMap& mb, const CUte
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;          // all CTAs resident together: they wait for one another
     attr[0].val.cooperative = 1;
+    // (Of its own stream only clear_kernel can still be running when the grid starts, and that waits for nothing any more.)
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;

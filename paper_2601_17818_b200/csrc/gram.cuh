@@ -54,7 +54,7 @@ struct GramArgs {
     float* rho_user;            // [B, n] optional copy of rho for the caller
     unsigned int* grid_sync;    // counter of the resident sweep's grid-wide barrier (a word of the status block)
     uint32_t* ready;            // resident sweep [B, n]: a token's factor (w, or for euclid a) once it is known, as its bits + 1
-                                // (the sweep clears both before it uses them)
+                                // (both cleared by the kernel in front)
     // Optional K-norm (Eq. 4) for the resident sweep's warps beside the epilogue's to stream once the MMAs are done:
     // K bf16 [kn_B, kn_H, kn_N, kn_d] dense, span [kn_vis_start, kn_vis_start + kn_Nv), score [kn_B, kn_Nv].
     // Only shapes gram_resident_takes_knorm accepts.
@@ -130,7 +130,7 @@ bool gram_resident_takes_knorm(int H, int d);
 // How many leading samples' K-norm, over spans of Nv tokens, the resident sweep of [B, n] finishes without being held up.
 int gram_resident_knorm_samples(int B, int n, int Nv);
 
-// One kernel for the norms, Eq. 2 and Eq. 3 on small problems: every CTA keeps the accumulators of its tiles in
+// One kernel for the norms, Eq. 2 and Eq. 3 on small problems, behind one that has cleared grid_sync, ready and the status word: every CTA keeps the accumulators of its tiles in
 // tensor memory; the diagonal tiles publish the per-token factors, which the density epilogues of the other tiles wait for
 // value by value, the grid synchronises once (bounded waits) after the density
 // partials; the delta epilogue sums the partials it needs itself and re-reads the same accumulators.

@@ -23,7 +23,8 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
-}// (as above; what it brings into the L2 is the first to leave it)
+}
+// (as above; what it brings into the L2 is the first to leave it)
 __device__ __forceinline__ void tma_load_4d_once(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
     asm volatile(
         "{\n\t.reg .b64 pol;\n\t"

@@ -772,8 +772,8 @@ def test_collaborative_step_equals_filter_then_prune_step(name):
 
 
 def test_collaborative_step_replays_from_a_cuda_graph():
-    """The one-call step only enqueues work on the caller's stream (one memset, cooperative and programmatically
-    dependent launches): it can be captured once and replayed, with the same results as direct calls."""
+    """The one-call step only enqueues work on the caller's stream (cooperative and programmatically dependent
+    launches): it can be captured once and replayed, with the same results as direct calls."""
     w = W.workload("c0")
     B, n = 2, w.Nv
     feat = vb.bf16_tensor(W.make_features(w, B=B))

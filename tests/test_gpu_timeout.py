@@ -88,6 +88,32 @@ def test_density_sweep_reports_timeout_and_recovers(B, n, roles):
     assert status == vb.OK and all(torch.equal(a, b) for a, b in zip(got, ref))
 
 
+def test_sweeps_of_several_streams_end_together():
+    """One-kernel sweeps that each want every SM, from three streams of two priorities at once: the CTAs of each wait for one
+    another, so they may not keep one another from starting."""
+    B, n, D, calls = 16, 576, 256, 12                      # 208 units: 148 CTAs with one or two
+    feat = torch.randn((B, n, D), generator=torch.Generator(device=DEV).manual_seed(5), device=DEV).to(torch.bfloat16)
+    streams = [torch.cuda.Stream(priority=p) for p in (0, -1, 0)]
+    ws = [[vb.alloc_workspace(vb.OP_FILTER, B=B, Nv=n, D=D) for _ in range(calls)] for _ in range(4)]
+    z = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
+    label, ncl = [[z(B, n) for _ in range(calls)] for _ in range(4)], z(B)
+
+    def call(s, i):
+        vb.vitcop_redundancy_filter(feat, None, label[s][i], ncl, ws[s][i], n_centers=29)
+
+    call(3, 0)
+    torch.cuda.synchronize()
+    for i in range(calls):
+        for s, stream in enumerate(streams):
+            with torch.cuda.stream(stream):
+                call(s, i)
+    torch.cuda.synchronize()
+    for s in range(3):
+        for i in range(calls):
+            assert vb.vitcop_poll_status(ws[s][i]) == vb.OK
+            assert torch.equal(label[s][i], label[3][0])
+
+
 def test_similarity_rows_reports_timeout_and_recovers():
     w = W.workload("tiny")
     f = W.make_features(w)
@@ -107,7 +133,7 @@ def test_similarity_rows_reports_timeout_and_recovers():
 
 
 def test_one_call_step_reports_timeout_and_recovers():
-    """The one-kernel sweep with its K-norm side work (bulk copies streamed by the load and MMA warps)."""
+    """The one-kernel sweep with its K-norm side work (tensor copies streamed by the warps beside the epilogue)."""
     w = W.workload("tiny")
     B, n = w.B, w.Nv
     feat = vb.bf16_tensor(W.make_features(w))
