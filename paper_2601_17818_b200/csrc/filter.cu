@@ -478,7 +478,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
         g.ready = reinterpret_cast<uint32_t*>(ws + l.off_ready);
         if (knorm && gram_resident_takes_knorm(knorm->H, knorm->d)) {
             // The sweep's side warps take the K-norm of the first samples; the others follow beside vic_finalize_kernel.
-            knorm_in_sweep = gram_resident_knorm_samples(B, n, knorm->Nv);
+            knorm_in_sweep = gram_resident_knorm_samples(B, n, knorm->H, knorm->d, knorm->Nv);
             if (knorm_in_sweep > 0) {
                 g.kn_K = knorm->K; g.kn_score = knorm->score; g.kn_B = knorm_in_sweep;
                 g.kn_H = knorm->H; g.kn_N = knorm->N; g.kn_d = knorm->d; g.kn_vis_start = knorm->vis_start; g.kn_Nv = knorm->Nv;

@@ -838,13 +838,17 @@ __device__ __forceinline__ ResidentUnit decode_resident_unit(const KernelArgs& k
 
 constexpr int kKnChunkTokens = 8;                          // tokens per chunk: 16 threads each
 constexpr int kKnBuffers = 3;
+__host__ __device__ constexpr int knorm_buffers(int H, int d) {         // 0: a chunk does not fit
+    const long long fit = (long long)GemmSmem<kResidentBN>::kTileBytes / ((long long)H * kKnChunkTokens * d * 2);
+    return fit < kKnBuffers ? (int)fit : kKnBuffers;
+}
 
 // K-norm (Eq. 4) by the warps beside the epilogue's, after the CTA's last MMA has completed.  Chunks of eight consecutive
 // tokens of one sample, all heads, are copied into the operand buffers, up to three chunks in flight; sixteen threads
 // reduce one token as in the stand-alone kernel, so that both give the same bits.  One tensor copy per chunk: as bulk copies, one
 // per head, they took a warp 1.3 us to issue where the arithmetic takes 1.0 (32 heads).
 __device__ __forceinline__ void resident_knorm(const GramArgs& g, const CUtensorMap* map_k, const uint8_t* buf_gen, uint32_t buf_smem,
-                                               uint32_t buf_bytes, uint32_t bar_kn, uint32_t bar_last_mma,
+                                               uint32_t bar_kn, uint32_t bar_last_mma,
                                                volatile int* abort_flag, unsigned long long limit_ns) {
     const int tid = threadIdx.x < 64 ? threadIdx.x : threadIdx.x - kResidentEpiThreads;        // 0 .. 127
     auto all_ok = [](bool ok) {
@@ -862,7 +866,7 @@ __device__ __forceinline__ void resident_knorm(const GramArgs& g, const CUtensor
 
     const int H = g.kn_H, d8 = g.kn_d / 8, Nv = g.kn_Nv;
     const uint32_t chunk_bytes = (uint32_t)(H * kKnChunkTokens * d8) * 16u;
-    const int nbuf = min(kKnBuffers, (int)(buf_bytes / chunk_bytes));   // >= 1 (gram_resident_takes_knorm)
+    const int nbuf = knorm_buffers(H, g.kn_d);             // >= 1 (gram_resident_takes_knorm)
     const int chunks_per_b = (Nv + kKnChunkTokens - 1) / kKnChunkTokens;
     const long long total = (long long)g.kn_B * chunks_per_b;
     auto issue = [&](long long c, int buf) {               // thread 0
@@ -1026,7 +1030,7 @@ gram_resident_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         __syncwarp();
         if (g.kn_K) {
             const long long my_units = (total_units - blockIdx.x + gridDim.x - 1) / gridDim.x;   // >= 1
-            resident_knorm(g, &map_k, gen, tiles, (uint32_t)S::kTileBytes, bar_kn, bar_tfull + 8 * (uint32_t)(my_units - 1),
+            resident_knorm(g, &map_k, gen, tiles, bar_kn, bar_tfull + 8 * (uint32_t)(my_units - 1),
                            abort_flag, k.limit_of(kRoleLoad | kRoleMma));
         }
     } else {
@@ -1301,15 +1305,19 @@ bool gram_resident_takes_knorm(int H, int d) {
     // eight 16-byte pieces per row, or sixteen and more (the lane layouts of the stand-alone kernel that sixteen lanes a token
     // reproduce), a copy's box of at most 256 elements a side, and at least one chunk of eight tokens must fit the operand buffers
     if (H <= 0 || H > 256 || d % 8 || d > 256 || (d != 64 && d < 128)) return false;
-    return (long long)H * kKnChunkTokens * d * 2 <= (long long)GemmSmem<kResidentBN>::kTileBytes;
+    return knorm_buffers(H, d) > 0;
 }
 
-// All of them where a CTA has a buffer for each of its chunks of tokens: one kernel less (1 x 576 tokens 34.8 -> 33.5 us).  Otherwise two
-// and a half chunks to a CTA: more hold up the sweep's barrier and searches by as much as they take beside vic_finalize_kernel
-// (16 x 576 tokens, inputs that change: 62.0 us with 5 of the samples, 62.6 with 6).
-int gram_resident_knorm_samples(int B, int n, int Nv) {
+// All of them where no CTA has more than three chunks of tokens: one kernel less (1 x 576 tokens x 8 heads of 128 30.8 -> 29.6 us, 4 x 576
+// x 2 of 64 30.9 -> 29.1).  Not with a single buffer, where each chunk waits for the one before (48 heads of 256: 1 x 576 35.2 us with
+// all against 34.6 without, 2 x 576 37.2 / 35.2 with half).  Otherwise two and a half chunks to a CTA, whatever their size: more
+// hold up the sweep's barrier and searches by as much as they take beside vic_finalize_kernel (16 x 576 x 32 of 128 61.7 us with 5 of
+// the samples, 64.3 / 62.6 / 63.5 with 0 / 7 / 16; 3 x 1000 x 48 of 256 48.0 with 2, 61.7 with none), and over 16 problems x 9 forms of
+// keys no share was found that is better throughout (times come in steps of 2 us).
+int gram_resident_knorm_samples(int B, int n, int H, int d, int Nv) {
     const long long ctas = resident_ctas(ResidentCut(B, n).total), chunks = (Nv + kKnChunkTokens - 1) / kKnChunkTokens;
-    return chunks * B <= kKnBuffers * ctas ? B : (int)(5 * ctas / (2 * chunks));
+    const long long share = 5 * ctas / (2 * chunks);
+    return share >= B || (knorm_buffers(H, d) > 1 && chunks * B <= 3 * ctas) ? B : (int)share;
 }
 
 int launch_gram_resident(const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream) {

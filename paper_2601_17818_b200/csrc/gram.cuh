@@ -127,8 +127,9 @@ bool gram_fits_resident(int B, int n);
 // True when the resident sweep can compute the K-norm of keys with H heads of d elements on the side.
 bool gram_resident_takes_knorm(int H, int d);
 
-// How many leading samples' K-norm, over spans of Nv tokens, the resident sweep of [B, n] finishes without being held up.
-int gram_resident_knorm_samples(int B, int n, int Nv);
+// How many leading samples' K-norm (H heads of d elements, spans of Nv tokens) the resident sweep of [B, n] finishes without being
+// held up.
+int gram_resident_knorm_samples(int B, int n, int H, int d, int Nv);
 
 // One kernel for the norms, Eq. 2 and Eq. 3 on small problems, behind one that has cleared grid_sync, ready and the status word: every CTA keeps the accumulators of its tiles in
 // tensor memory; the diagonal tiles publish the per-token factors, which the density epilogues of the other tiles wait for

@@ -65,7 +65,7 @@ def test_kproj_whatever_the_workspace_holds(N, fill):
 
 # Chunks of eight tokens, eight or sixteen lanes a token, boxes that reach past the sequence; head counts that fill the buffers
 # once, twice and three times; row lengths that the sweep leaves to the stand-alone kernel (96, 512).
-@pytest.mark.parametrize("H,d", [(1, 64), (5, 64), (32, 128), (3, 128), (40, 136), (17, 256), (6, 96), (2, 512)])
+@pytest.mark.parametrize("H,d", [(1, 64), (5, 64), (32, 128), (3, 128), (40, 136), (17, 256), (48, 256), (6, 96), (2, 512)])
 @pytest.mark.parametrize("B,n,T", [(1, 1, 1), (2, 9, 0), (3, 129, 9), (1, 577, 3), (16, 200, 2)])
 def test_norms_beside_the_sweep_are_the_stand_alone_ones(B, n, T, H, d):
     _compare_norms(B, n, T, H, d, 64)
