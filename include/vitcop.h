@@ -206,7 +206,8 @@ int vitcop_select(const float* score, const int32_t* label, int B,
  *   hidden      bf16 [B, N, Dh]      (any of hidden / K / V may be NULL together with its output)
  *   K, V        bf16 [B, H, N, d]
  *   seq_len     int32 [B] or NULL (= N for every sample)
- *   keep_idx    int32 [B, keep_stride], ascending, as written by vitcop_select;  n_keep int32 [B]
+ *   keep_idx    int32 [B, keep_stride], ascending, as written by vitcop_select;  n_keep int32 [B] (more than keep_stride
+ *               counts as keep_stride; with keep_stride 0 all samples read one list, of any length)
  *   hidden_out  bf16 [B, Ncap, Dh];  K_out, V_out bf16 [B, H, Ncap, d]; must not overlap the inputs
  *   kept_pos    int32 [B, Ncap] out, optional: input position of each output row, -1 past out_len
  *   out_len     int32 [B] out

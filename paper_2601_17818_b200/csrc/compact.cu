@@ -101,12 +101,14 @@ compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, co
         if (r != 0) return;                                // row 0 still reports the sample's new length
     }
     grid_dependency_wait();
-    // (the row's entry in the list travels with the list's length, whether there is one or not)
+    // (the row's entry in the list travels with the list's length, whether there is one or not; of one list for all samples,
+    // stride 0, nobody knows the end but the length)
     const int slot = r - vis_start;
-    int ki = slot >= 0 && slot < keep_stride ? __ldcg(keep_idx + (int64_t)b * keep_stride + slot) : 0;
+    const int32_t* const entry = keep_idx + (int64_t)b * keep_stride + slot;
+    int ki = slot >= 0 && slot < keep_stride ? __ldcg(entry) : 0;
     int nv = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
     nv = max(0, min(nv, L - vis_start));
-    const int nk = max(0, min(min(__ldcg(n_keep + b), keep_stride), nv));
+    const int nk = max(0, min(min(__ldcg(n_keep + b), keep_stride > 0 ? keep_stride : nv), nv));
     const int olen = L - nv + nk;
     if (r == 0 && lane == 0) out_len[b] = olen;
     if (r >= Ncap || prefix_row) return;
@@ -117,6 +119,7 @@ compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, co
     int src_row;
     if (r < vis_start) src_row = r;
     else if (r < vis_start + nk) {
+        if (keep_stride == 0) ki = __ldcg(entry);
         ki = max(0, min(ki, nv - 1));                     // a corrupt index can never leave the span
         src_row = vis_start + ki;
     } else src_row = r - nk + nv;

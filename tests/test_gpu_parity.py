@@ -265,6 +265,28 @@ def test_compact_row_lengths(pieces):
         assert np.all(ho[b, L:] == 0)
 
 
+@pytest.mark.parametrize("B", [1, 3])
+def test_compact_list_without_a_stride(B):
+    """keep_stride 0: one list for all samples, through the C ABI; a length past a positive stride ends with the row of the list."""
+    rng = np.random.default_rng(B)
+    N, Dh, vs, nv = 50, 16, 3, 41
+    hid = _rand_bits(rng, (B, N, Dh))
+    keep = np.sort(rng.permutation(nv)[:17]).astype(np.int32)
+    th, ki, nk = vb.bf16_tensor(hid), dev_i32(np.tile(keep, B)), dev_i32([17 - 4 * b for b in range(B)])
+    for stride in (0, 17, 5):
+        ho = torch.zeros((B, N, Dh), dtype=torch.bfloat16, device=DEV)
+        olen = torch.zeros((B,), dtype=torch.int32, device=DEV)
+        rc = vb.lib().vitcop_compact_kv(th.data_ptr(), None, None, B, 0, N, 0, Dh, None, vs, None, nv, ki.data_ptr(), stride, nk.data_ptr(),
+                                        ho.data_ptr(), None, None, N, None, olen.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert rc == vb.OK
+        for b in range(B):
+            row = np.tile(keep, B)[b * stride:][: min(17 - 4 * b, stride or N)]
+            o = oracle.compact(hid[b], None, None, N, vs, nv, row, N)
+            L = o["out_len"]
+            assert int(olen[b]) == L and np.array_equal(vb.bf16_bits(ho)[b, :L], o["hidden"][:L]), (stride, b)
+
+
 def test_compact_ragged_partial_tensors_and_small_capacity():
     rng = np.random.default_rng(3)
     B, H, N, d, Dh, vs = 3, 2, 40, 16, 32, 4
