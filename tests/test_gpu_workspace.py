@@ -2,7 +2,8 @@
 stand-alone one (``-m gpu``).
 
 The filter and the key projection are not preceded by a memset: their kernels clear what they need themselves, so a workspace full of
-anything must give the results and the status of a fresh one, also right behind a call of another size in the same memory.
+anything must give the results and the status of a fresh one, also right behind a call of another size in the same memory.  Their first
+kernels are launched ahead of time and wait on the device for what precedes them.
 """
 import pytest
 import torch
@@ -71,9 +72,11 @@ def test_norms_beside_the_sweep_are_the_stand_alone_ones(B, n, T, H, d):
     _compare_norms(B, n, T, H, d, 64)
 
 
-def _compare_norms(B, n, T, H, d, D):
+def _compare_norms(B, n, T, H, d, D, metric=0, spatial=False, ws=None):
+    """Scores of the one-call step against the stand-alone K-norm; returns its labels and cluster counts, and the step itself."""
     N, budget, nc = n + T, max(1, n // 2), max(1, n // 20)
     feat = _randn(n, B, n, D).to(torch.bfloat16)
+    pos = torch.rand((B, n, 2), generator=torch.Generator(device=DEV).manual_seed(n), device=DEV) if spatial else None
     K = (_randn(d, B, H, N, d) * torch.exp(0.5 * _randn(H, B, 1, N, 1))).to(torch.bfloat16)
     vis_start = T // 2
     ref = torch.zeros((B, n), dtype=torch.float32, device=DEV)
@@ -82,16 +85,121 @@ def _compare_norms(B, n, T, H, d, D):
     score, cap = torch.zeros_like(ref), T + budget
     hidden, hidden_out = torch.zeros((B, N, 8), dtype=torch.bfloat16, device=DEV), torch.zeros((B, cap, 8), dtype=torch.bfloat16, device=DEV)
     K_out, V_out = (torch.zeros((B, H, cap, d), dtype=torch.bfloat16, device=DEV) for _ in range(2))
-    ws = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=D)
-    vb.vitcop_collaborative_step(feat, None, hidden, K, K, vis_start, budget, hidden_out, K_out, V_out, i32(B), i32(B, n), i32(B), ws,
-                                 n_centers=nc, score_out=score)
-    torch.cuda.synchronize()
+    if ws is None:
+        ws = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=D)
+    label, ncl, olen = i32(B, n), i32(B), i32(B)
+    how = dict(metric=metric, d_c=0.5 if metric == 0 else 16.0, n_centers=nc)
+
+    def step(ws=ws):
+        vb.vitcop_collaborative_step(feat, pos, hidden, K, K, vis_start, budget, hidden_out, K_out, V_out, olen, label, ncl, ws,
+                                     score_out=score, **how)
+        return vb.vitcop_poll_status(ws)
+
+    assert step() == vb.OK
     assert torch.equal(score, ref)
+    got = label.clone(), ncl.clone()
+    if D > 64:                                             # the sweep that has keys on the side is another one
+        fws = vb.alloc_workspace(vb.OP_FILTER, B=B, Nv=n, D=D)
+        vb.vitcop_redundancy_filter(feat, pos, label, ncl, fws, **how)
+        assert vb.vitcop_poll_status(fws) == vb.OK and torch.equal(got[0], label) and torch.equal(got[1], ncl)
+    return step, (K_out, V_out, olen, label, ncl, score)
+
+
+def _kernels(step):
+    vb.vitcop_kernel_timing_begin()
+    assert step() == vb.OK
+    return vb.vitcop_kernel_timing_end()
 
 
 # Beside the density sweep: all of the samples or, where the sweep is over before, the first ones of them; units of four and eight
-# tokens that end inside a copy, heads that end inside one.
-@pytest.mark.parametrize("B,n,T,H,d,D", [(8, 2881, 3, 31, 128, 1024), (9, 2879, 0, 62, 64, 1024), (20, 1501, 1, 32, 128, 1024),
-                                         (4, 4606, 2, 33, 128, 1024)])
-def test_norms_beside_the_density_sweep_are_the_stand_alone_ones(B, n, T, H, d, D):
-    _compare_norms(B, n, T, H, d, D)
+# tokens that end inside a copy, heads that end inside one (also before its first four).
+@pytest.mark.parametrize("B,n,T,H,d,D,alone", [(8, 2881, 3, 31, 128, 1024, False), (9, 2879, 0, 62, 64, 1024, False),
+                                               (20, 1501, 1, 32, 128, 1024, True), (4, 4606, 2, 33, 128, 1024, False),
+                                               (340, 1000, 1, 1, 128, 256, False), (340, 1000, 1, 2, 64, 256, False),
+                                               (115, 999, 2, 3, 128, 512, False)])
+def test_norms_beside_the_density_sweep_are_the_stand_alone_ones(B, n, T, H, d, D, alone):
+    step, _ = _compare_norms(B, n, T, H, d, D)
+    names = _kernels(step)
+    assert "density_sweep_kernel" in names and ("knorm_kernel" in names) == alone
+
+
+@pytest.mark.parametrize("metric,spatial", [(0, True), (1, False), (1, True)])
+@pytest.mark.parametrize("B,n,T,H,d,D", [(8, 2881, 3, 31, 128, 512), (9, 2879, 0, 62, 64, 512)])
+def test_norms_beside_the_density_sweep_with_either_metric(B, n, T, H, d, D, metric, spatial):
+    _compare_norms(B, n, T, H, d, D, metric, spatial)
+
+
+def test_norms_beside_the_density_sweep_of_a_group():
+    """With the least workspace that is taken the samples go through one by one; the first sweep takes norms of others along."""
+    B, n, T, H, d, D = 30, 5000, 4, 4, 128, 1024
+    full = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=D)
+    step, _ = _compare_norms(B, n, T, H, d, D, ws=full)
+
+    def taken(units):
+        try:
+            return step(full[:256 * units]) == vb.OK
+        except RuntimeError:
+            return False
+
+    lo, hi = 1, full.numel() // 256                        # lo is refused
+    assert not taken(lo)
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if taken(mid) else (mid, hi)
+    step, _ = _compare_norms(B, n, T, H, d, D, ws=full[:256 * hi])
+    names = _kernels(step)
+    assert names["density_sweep_kernel"][0] == B and names["knorm_kernel"][0] == 1
+
+
+@pytest.mark.parametrize("metric", [0, 1])
+@pytest.mark.parametrize("roles", [1, 2, 4])
+def test_density_sweep_with_keys_reports_timeout_and_recovers(roles, metric):
+    """A role of the sweep's pairs of CTAs gives up while copies of keys are in flight (8: the kernels on pairs alone)."""
+    step, outputs = _compare_norms(8, 2881, 3, 31, 128, 512, metric)
+    assert step() == vb.OK
+    ref = [t.clone() for t in outputs]
+    try:
+        vb.vitcop_set_wait_limit(0, 8 * roles)
+        assert step() == vb.ERR_TIMEOUT
+    finally:
+        vb.vitcop_set_wait_limit(0, 0)
+    assert step() == vb.OK and all(torch.equal(a, b) for a, b in zip(outputs, ref))
+
+
+# The first kernels of these calls are launched before what precedes them ends: keys that the projection has just written, without a
+# synchronisation in between (one-kernel sweep; diagonal and density sweep).
+@pytest.mark.parametrize("B,n", [(1, 576), (4, 1800)])
+def test_step_right_behind_the_projection_of_its_keys(B, n):
+    H, d, Dh, D, T, budget, times = 4, 128, 256, 256, 16, n // 3, 6
+    N, cap = n + T, T + n // 3
+    W = _randn(1, H * d, Dh).to(torch.bfloat16)
+    hidden = [_randn(10 + i, B, N, Dh).to(torch.bfloat16) for i in range(times)]
+    feat = [_randn(30 + i, B, n, D).to(torch.bfloat16) for i in range(times)]
+    z = lambda *s, dt=torch.bfloat16: torch.zeros(s, dtype=dt, device=DEV)
+    i32 = lambda *s: z(*s, dt=torch.int32)
+
+    def run(wait):
+        K, out = z(B, H, N, d), []
+        wk, ws = vb.alloc_workspace(vb.OP_KPROJ, B=B, H=H, N=N, d=d), vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=D)
+        wp = vb.alloc_workspace(vb.OP_PRUNE_STEP, B=B, Nv=n)
+        for h, f in zip(hidden, feat):
+            o = [z(B, cap, Dh), z(B, H, cap, d), z(B, H, cap, d), i32(B), i32(B, n), i32(B), z(B, n, dt=torch.float32)]
+            q = [z(B, cap, Dh), z(B, H, cap, d), z(B, H, cap, d), i32(B), z(B, n, dt=torch.float32)]
+            mid = z(B, n, dt=torch.float32)
+            vb.vitcop_kproj_knorm(h, W, H, d, K, wk, vis_start=5, score=mid)
+            if wait:
+                torch.cuda.synchronize()
+            vb.vitcop_collaborative_step(f, None, h, K, K, 5, budget, *o[:6], ws, n_centers=n // 20, score_out=o[6])
+            if wait:
+                torch.cuda.synchronize()
+            vb.vitcop_kproj_knorm(o[0][:, :1].expand(B, N, Dh).contiguous(), W, H, d, K, wk, vis_start=5, score=mid)
+            if wait:
+                torch.cuda.synchronize()
+            vb.vitcop_prune_step(h, K, K, 5, n, n, budget, *q[:4], wp, score_out=q[4])
+            if wait:
+                torch.cuda.synchronize()
+            out += o + q
+        torch.cuda.synchronize()
+        return out
+
+    assert all(torch.equal(a, b) for a, b in zip(run(False), run(True)))
