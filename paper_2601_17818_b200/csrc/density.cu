@@ -670,8 +670,11 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
 
 // In microseconds.  The sweep runs at 0.9 PFLOP/s or more and has room for 2.6 MB of keys in each (four warps of every SM, 5 us
 // slower by them and the missing stage); the stand-alone kernel reads 6.2 MB, the first 4 + n / 600 of them beside
-// vic_finalize_kernel.  So worth it where that leaves 8 to be gained: 8 x 2880 tokens x 32 heads 193 -> 178 (whole call), 4 x 4608 203 ->
-// 200; not for 2 x 16384 x 4, whose keys all fit beside vic_finalize_kernel.
+// vic_finalize_kernel.  So worth it where that leaves 8 to be gained.  Whole calls without and with, 32 heads of 128: 8 x 2880 tokens
+// 204 -> 193, 4 x 4608 222 -> 212, 16 x 1152 132.6 -> 128.3, 20 x 1500 207 -> 193; not for 2 x 16384 x 4 heads (868 / 896), whose keys
+// all fit beside vic_finalize_kernel.  Over 14 problems x 6 forms of keys no call with keys beside the sweep was slower than
+// without.  The line is a careful one: with all of the samples, which saves a kernel, calls below it measured up to 9 less too (4 x
+// 2880 x 768 features, 32 heads of 64: 111 / 106).
 int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D) {
     if (!job.K || job.B <= 0 || job.H <= 0 || job.Nv <= 0 || (job.d != 64 && job.d != 128)) return 0;
     const double mb = 2e-6 * job.H * job.d * job.Nv, sweep = 1e-9 / 0.9 * samples * n * (double)n * D;
