@@ -379,16 +379,19 @@ int vitcop_collaborative_step(const void* feat, const float* pos, int D, const v
         rc = reset_status(workspace, s);
         if (rc != VITCOP_OK || B == 0) return rc;
     }
+    QuotaJob quota = {score, budget, keep, nkeep, false};
     if (Nv > 0) {
         const KnormJob job = {K, B, H, N, d, vis_start, Nv, score};
         rc = launch_filter(feat, pos, B, Nv, D, *fp, nc, label_out, n_clusters_out, rho_out, delta2_out, parent_out,
-                           workspace, filter_bytes, s, &job);
+                           workspace, filter_bytes, s, &job, &quota);
         if (rc != VITCOP_OK) return rc;
     }
-    // (plain stream order when the filter was skipped: see vitcop_prune_step)
-    rc = launch_select(score, label_out, B, nullptr, Nv, Nv, 1, 0, budget, keep, Nv, nkeep, nullptr,
-                       reinterpret_cast<int*>(ws), s, Nv > 0);
-    if (rc != VITCOP_OK) return rc;
+    if (!quota.taken) {
+        // (plain stream order when the filter was skipped: see vitcop_prune_step)
+        rc = launch_select(score, label_out, B, nullptr, Nv, Nv, 1, 0, budget, keep, Nv, nkeep, nullptr,
+                           reinterpret_cast<int*>(ws), s, Nv > 0);
+        if (rc != VITCOP_OK) return rc;
+    }
     return launch_compact(hidden, K, V, B, H, N, d, Dh, nullptr, vis_start, nullptr, Nv, keep, Nv, nkeep, hidden_out,
                           K_out, V_out, Ncap, kept_pos, out_len, s, true);
 }

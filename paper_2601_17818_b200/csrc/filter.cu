@@ -17,6 +17,8 @@
 // tensor memory.
 #include "density.cuh"
 #include "gram.cuh"
+#include "select_rank.cuh"
+#include "vic_labels.cuh"
 
 namespace vitcop {
 namespace {
@@ -103,271 +105,96 @@ rho_reduce_kernel(const __grid_constant__ SweepArgs g, int metric, float* __rest
 }
 
 // ------------------------------------------------------------------------------------------------
-// Centres, forest roots and labels: one CTA per sample.
+// Centres, forest roots and labels (vic_labels.cuh): R CTAs per sample, E tokens per thread.  SELECT: right behind them the
+// cluster-quota selection of a pruning step (select_rank.cuh) whose scores are there by then: the labels stay in registers, and a launch and a
+// trip to memory go (1 x 576 tokens, whole call, 31.5 -> 29.0 us).
 // ------------------------------------------------------------------------------------------------
-// The CTA runs alone on its SM, so what counts is the number of dependent steps, not throughput: every thread holds its tokens'
-// keys in registers, all global loads are in flight together, the cut among the keys is found with one or two histogram
-// passes of 11 bits that start at the highest bit in which two keys differ, and what is left in the cut's bin is ranked by
-// counting.  (8-bit passes over the whole 64-bit key with ordered scans for ties and for the list of centres: 9.2 us on 576
-// tokens, 14 on 2880, 38 on 16384; the list is needed for surplus orphans only and is built when there are any.)
-constexpr int kFinThreads = 1024;
-constexpr int kFinBits = 11, kFinBins = 1 << kFinBits;
-constexpr int kFinRankLanes = 4;
-constexpr int kFinRank = kFinThreads / kFinRankLanes;      // bins of up to this many keys are ranked by counting
-
-// Dynamic shared memory: nxt[n] (uint16), isc[n] (uint8), centre list[nc] (uint16; surplus orphans).  E: tokens per thread.
-constexpr size_t finalize_smem(int n, int nc) { return (((size_t)n + 15) & ~(size_t)15) * 3 + (size_t)(nc > 0 ? nc : 1) * 2 + 16; }
-template <int E>
-__global__ void __launch_bounds__(kFinThreads)
-vic_finalize_kernel(const uint16_t* __restrict__ feat, int n, int D, int n_centers, const float* rho, const unsigned long long* best,
-                    const float* w, const float* a, int32_t* __restrict__ label, int32_t* __restrict__ n_clusters,
-                    float* __restrict__ delta2_user, int32_t* __restrict__ parent_user) {
-    extern __shared__ __align__(16) uint8_t fin_smem[];
-    const int n_al = (n + 15) & ~15;
-    uint16_t* nxt = reinterpret_cast<uint16_t*>(fin_smem);
-    uint8_t* isc = fin_smem + (size_t)n_al * 2;
-    uint16_t* centres = reinterpret_cast<uint16_t*>(fin_smem + (size_t)n_al * 3);
-    __shared__ uint32_t hist[kFinBins];
-    __shared__ unsigned long long cand_key[kFinRank];
-    __shared__ uint16_t cand_idx[kFinRank];
-    __shared__ uint32_t warp_sums[32];
-    __shared__ uint32_t s_lo, s_hi, s_digit, s_krem, s_count, s_cands;
-    __shared__ unsigned long long orph_best[kFinThreads];
-    __shared__ int orph_list[kFinThreads];
-    __shared__ int orph_cnt, centre_cnt;
-
-    const int tid = threadIdx.x, lane = tid & 31;
-    hist[tid] = 0;
-    hist[tid + kFinThreads] = 0;
-    if (tid == 0) { s_lo = 0xFFFFFFFFu; s_hi = 0u; s_cands = 0u; centre_cnt = 0; }
-    static_assert(kFinBins == 2 * kFinThreads, "two bins per thread");
+struct QuotaArgs {
+    QuotaJob job;
+    int P_cap;
+    int* status;
+};
+template <int R, int E, bool SELECT>
+__global__ void __launch_bounds__(kGroupThreads)
+vic_finalize_kernel(const __grid_constant__ VicArgs v, const __grid_constant__ QuotaArgs q) {
+    extern __shared__ __align__(16) uint8_t fin_dyn[];
+    __shared__ VicShared<R> sh;
     grid_dependency_launch_dependents();
+    sh.init();
     grid_dependency_wait();
-    const int b = blockIdx.x;
-    rho += (size_t)b * n;
-    best += (size_t)b * n;
-    w += (size_t)b * n;
-    a += (size_t)b * n;
-    label += (size_t)b * n;
-    feat += (size_t)b * n * D;
-    if (delta2_user) delta2_user += (size_t)b * n;
-    if (parent_user) parent_user += (size_t)b * n;
-    const int nc = min(n_centers, n);
+    const int b = blockIdx.x / R;
+    int lab[E];
+    if constexpr (SELECT) {
+        static_assert(R == 1 && kGroupThreads == kSelThreads, "one CTA, its tokens spread as the selection has them");
+        const int n = v.n;
+        const float* const score = q.job.score + (size_t)b * n;
+        uint32_t key[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {                      // (on their way while the labels are worked out)
+            const int i = e * kSelThreads + threadIdx.x;
+            key[e] = i < n ? __float_as_uint(__ldcg(score + i)) : 0u;
+        }
+        vic_labels<R, E>(v, b, sh, fin_dyn, lab);
+#pragma unroll
+        for (int e = 0; e < E; ++e) key[e] = order_key(__uint_as_float(key[e]), 0);
+        __shared__ RankShared rs;
+        int32_t *const keep = q.job.keep + (size_t)b * n, *const n_keep = q.job.n_keep + b;
+        __syncthreads();                                   // (the table is no longer needed, and all labels are written)
+        if (!select_by_rank<E>(lab, key, n, q.job.budget, rs, fin_dyn, keep, n, n_keep, nullptr, q.status))
+            select_by_sort(score, v.label + (size_t)b * n, n, n, q.P_cap, q.job.budget, keep, n, n_keep, nullptr, q.status, fin_dyn, rs.warp_sums);
+    } else {
+        vic_labels<R, E>(v, b, sh, fin_dyn, lab);
+    }
+}
 
-    // (Loads of what the preceding kernels wrote: pointers without __restrict__, so that nothing lets the compiler move one in
-    // front of the wait.)
-    // rank key, ascending = better centre candidate: ( ~( orphan ? 0xFFFFFFFF : gamma ), ~rho, index )
-    uint32_t hi[E];
-    {
-        unsigned long long p[E];
-        float r[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int i = e * kFinThreads + tid;
-            p[e] = i < n ? __ldcg(best + i) : 0ull;
-            r[e] = i < n ? __ldcg(rho + i) : 0.f;
+typedef void (*FinalizeKernel)(VicArgs, QuotaArgs);
+FinalizeKernel finalize_kernel(int R, int E, bool select) {
+    return select   ? (E == 1 ? vic_finalize_kernel<1, 1, true> : vic_finalize_kernel<1, 2, true>)
+           : R == 8 ? vic_finalize_kernel<8, 2, false>
+           : E == 1 ? vic_finalize_kernel<1, 1, false>
+           : E == 2 ? vic_finalize_kernel<1, 2, false>
+           : E == 4 ? vic_finalize_kernel<1, 4, false>
+           : E == 8 ? vic_finalize_kernel<1, 8, false> : vic_finalize_kernel<1, 16, false>;
+}
+size_t finalize_smem(int R, int n, int nc, bool select, int* P_cap) {
+    const size_t labels = R == 1 ? vic_smem<1>(n, nc) : vic_smem<8>(n, nc), quota = select ? rank_or_sort_smem(n, P_cap) : 0;
+    return labels > quota ? labels : quota;
+}
+size_t finalize_most_smem(int R, int E, bool select) {
+    int p = 0;
+    return finalize_smem(R, R * E * kGroupThreads, R * E * kGroupThreads, select, &p);
+}
+int finalize_allow_smem(int R, int E, bool select) {
+    static DoneOnDevice attr_done[2][9][17];
+    return allow_dynamic_smem(finalize_kernel(R, E, select), finalize_most_smem(R, E, select), attr_done[select][R][E]);
+}
+// How many clusters of eight CTAs (an SM each) the device runs at a time: not SMs / 8, because a cluster stays inside a group of
+// SMs.  0 if it cannot be told.
+int finalize_clusters_at_once() {
+    static std::atomic<int> known[kMaxDevices];            // number + 1
+    std::atomic<int>& k = known[current_device()];
+    int v = k.load(std::memory_order_relaxed);
+    if (v == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(8);
+        cfg.blockDim = dim3(kGroupThreads);
+        cfg.dynamicSmemBytes = finalize_most_smem(8, 2, false);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 8;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (finalize_allow_smem(8, 2, false) != VITCOP_OK ||
+            cudaOccupancyMaxActiveClusters(&n, finalize_kernel(8, 2, false), &cfg) != cudaSuccess || n < 0) {
+            cudaGetLastError();
+            n = 0;
         }
-        uint32_t lo_k = 0xFFFFFFFFu, hi_k = 0u;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int i = e * kFinThreads + tid;
-            if (i < n) {
-                const bool orphan = p[e] == ~0ull;
-                const float d2 = orphan ? __int_as_float(0x7f800000) : __uint_as_float((uint32_t)(p[e] >> 32));
-                const int par = orphan ? -1 : (int)(uint32_t)(p[e] & 0xFFFFFFFFull);
-                if (delta2_user) delta2_user[i] = d2;
-                if (parent_user) parent_user[i] = par;
-                nxt[i] = (uint16_t)((par < 0 || par >= n) ? i : par);
-                hi[e] = ~(orphan ? 0xFFFFFFFFu : __float_as_uint(r[e] * sqrtf(d2)));
-                lo_k = min(lo_k, hi[e]);
-                hi_k = max(hi_k, hi[e]);
-            }
-        }
-        lo_k = __reduce_min_sync(0xffffffffu, lo_k);
-        hi_k = __reduce_max_sync(0xffffffffu, hi_k);
-        __syncthreads();                                   // (s_lo, s_hi and the histogram are set)
-        if (lane == 0 && lo_k <= hi_k) {
-            atomicMin(&s_lo, lo_k);
-            atomicMax(&s_hi, hi_k);
-        }
+        v = n + 1;
+        k.store(v, std::memory_order_relaxed);
     }
-    __syncthreads();
-
-    // ---- the nc smallest keys.  `in`: tokens of this thread (bit e) that still are on the cut; `sel`: chosen ones.
-    uint32_t in = 0, sel = 0, ranked = 0;                  // ranked: how many of the listed candidates are wanted
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (e * kFinThreads + tid < n) in |= 1u << e;
-    if (nc >= n) {
-        sel = in;
-    } else if (nc > 0) {
-        uint32_t krem = (uint32_t)nc;
-        int word = 0, top = 32 - __clz(s_lo ^ s_hi);       // word of the key, bits of it not yet looked at
-        for (;;) {
-            while (top == 0) top = ++word == 2 ? 14 : 32;  // (indices differ: the last word settles everything)
-            const int shift = top > kFinBits ? top - kFinBits : 0;
-            auto digit = [&](int e) {
-                const int i = e * kFinThreads + tid;
-                const uint32_t k = word == 0 ? hi[e] : word == 1 ? ~__float_as_uint(__ldcg(rho + i)) : (uint32_t)i;
-                return (k >> shift) & ((1u << (top - shift)) - 1u);
-            };
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                if (in >> e & 1u) atomicAdd(&hist[digit(e)], 1u);
-            __syncthreads();
-            const uint32_t h0 = hist[2 * tid], h1 = hist[2 * tid + 1];
-            uint32_t total;
-            const uint32_t before = block_exclusive_sum(h0 + h1, warp_sums, total);
-            if (before < krem && krem <= before + h0 + h1) {
-                const bool second = krem > before + h0;
-                s_digit = 2 * tid + (second ? 1 : 0);
-                s_krem = krem - before - (second ? h0 : 0u);
-                s_count = second ? h1 : h0;
-            }
-            hist[2 * tid] = 0;                             // for the next pass
-            hist[2 * tid + 1] = 0;
-            __syncthreads();
-            const uint32_t cut = s_digit, count = s_count;
-            krem = s_krem;
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                if (in >> e & 1u) {
-                    const uint32_t d = digit(e);
-                    if (d < cut) sel |= 1u << e;
-                    if (d != cut) in &= ~(1u << e);
-                }
-            }
-            top = shift;
-            if (count == krem) {                           // the whole bin is wanted
-                sel |= in;
-                break;
-            }
-            if (count <= (uint32_t)kFinRank) {
-                // few left: listed, and ranked below
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    if (in >> e & 1u) {
-                        const int i = e * kFinThreads + tid;
-                        const uint32_t at = atomicAdd(&s_cands, 1u);
-                        cand_key[at] = ((unsigned long long)hi[e] << 32) | (unsigned long long)~__float_as_uint(__ldcg(rho + i));
-                        cand_idx[at] = (uint16_t)i;
-                    }
-                }
-                ranked = krem;
-                break;
-            }
-            __syncthreads();                               // (s_digit .. are rewritten)
-        }
-    }
-    // ---- centres are roots; an orphan is one already
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = e * kFinThreads + tid;
-        if (i < n) {
-            const bool f = (sel >> e & 1u) != 0;
-            isc[i] = f ? 1 : 0;
-            if (f) nxt[i] = (uint16_t)i;
-        }
-    }
-    __syncthreads();
-    if (ranked > 0) {                                      // (uniform) four threads per candidate count the better ones
-        const int c = tid / kFinRankLanes, cands = (int)s_cands;
-        uint32_t rank = 0;
-        unsigned long long mine = 0ull;
-        int idx = 0;
-        if (c < cands) {
-            mine = cand_key[c];
-            idx = cand_idx[c];
-            for (int o = tid % kFinRankLanes; o < cands; o += kFinRankLanes)
-                rank += (cand_key[o] < mine || (cand_key[o] == mine && cand_idx[o] < idx)) ? 1u : 0u;
-        }
-#pragma unroll
-        for (int off = 1; off < kFinRankLanes; off <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
-        if (c < cands && tid % kFinRankLanes == 0 && rank < ranked) {
-            isc[idx] = 1;
-            nxt[idx] = (uint16_t)idx;
-        }
-        __syncthreads();
-    }
-    // ---- forest roots by pointer jumping: any value read is an ancestor, roots are fixed points
-    for (int round = 0; round < 16; ++round) {
-        int changed = 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int i = e * kFinThreads + tid;
-            if (i < n) {
-                int p = nxt[i];
-                const int q = nxt[p];
-                if (q != p) {
-                    p = nxt[q];
-                    nxt[i] = nxt[p];
-                    changed = 1;
-                }
-            }
-        }
-        if (!__syncthreads_or(changed)) break;
-    }
-    // ---- a root that is an orphan but not a centre joins the nearest centre (feature distance)
-    int any_surplus = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = e * kFinThreads + tid;
-        if (i < n && !isc[i] && nxt[i] == i) any_surplus = 1;
-    }
-    if (nc > 0 && __syncthreads_or(any_surplus)) {
-        // Surplus orphans are rare but each needs its distance to every centre: they are listed, kFinThreads tokens at a time,
-        // and the (orphan, centre) pairs are spread over all warps; the nearest centre wins through a packed minimum
-        // (distance bits, then the lower centre).
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int i = e * kFinThreads + tid;
-            if (i < n && isc[i]) centres[atomicAdd(&centre_cnt, 1)] = (uint16_t)i;
-        }
-        for (int base = 0; base < n; base += kFinThreads) {
-            __syncthreads();                                        // the previous round's list has been consumed
-            if (tid == 0) orph_cnt = 0;
-            __syncthreads();
-            const int o = base + tid;
-            if (o < n && !isc[o] && nxt[o] == o) {
-                const int at = atomicAdd(&orph_cnt, 1);
-                orph_list[at] = o;
-                orph_best[at] = ~0ull;
-            }
-            __syncthreads();
-            const int pairs = orph_cnt * nc;
-            for (int pr = tid >> 5; pr < pairs; pr += kFinThreads / 32) {
-                const int e = pr / nc, q = pr - e * nc;
-                const int oo = orph_list[e], c = centres[q];
-                const uint16_t* fo = feat + (size_t)oo * D;
-                const uint16_t* fc = feat + (size_t)c * D;
-                float dot = 0.f;
-                for (int k = lane * 2; k < D; k += 64) {
-                    const uint32_t u = *reinterpret_cast<const uint32_t*>(fo + k);
-                    const uint32_t v = *reinterpret_cast<const uint32_t*>(fc + k);
-                    dot = fmaf(bf16lo(u), bf16lo(v), dot);
-                    dot = fmaf(bf16hi(u), bf16hi(v), dot);
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-                const float d2 = fmaxf(0.f, fmaf(-2.f, (dot * w[oo]) * w[c], a[oo] + a[c]));
-                if (lane == 0)
-                    atomicMin(&orph_best[e], ((unsigned long long)__float_as_uint(d2) << 32) | (unsigned long long)(uint32_t)c);
-            }
-            __syncthreads();
-            if (tid < orph_cnt) nxt[orph_list[tid]] = (uint16_t)(orph_best[tid] & 0xFFFFFFFFull);   // the adopted centre
-        }
-        __syncthreads();
-    }
-    // ---- labels
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = e * kFinThreads + tid;
-        if (i < n) {
-            const int root = nxt[i];
-            label[i] = isc[root] ? root : (int)nxt[root];           // (a surplus orphan's entry is the centre that adopted it)
-        }
-    }
-    if (tid == 0) n_clusters[b] = nc;
+    return v - 1;
 }
 
 // In front of the one-kernel sweep: status word, barrier counter and published factors.  The sweep's CTAs have nothing to meet by
@@ -448,7 +275,8 @@ size_t similarity_workspace_bytes(int B, int n, int D) {
 
 int launch_filter(const void* feat, const float* pos, int B, int n, int D, const vitcop_filter_params& p,
                   int n_centers, int32_t* label, int32_t* n_clusters, float* rho_user, float* delta2_user,
-                  int32_t* parent_user, void* workspace, size_t workspace_bytes, cudaStream_t stream, const KnormJob* knorm) {
+                  int32_t* parent_user, void* workspace, size_t workspace_bytes, cudaStream_t stream, const KnormJob* knorm,
+                  QuotaJob* quota) {
     const FilterWs l(B, n);
     if (workspace_bytes < l.least) return VITCOP_ERR_WORKSPACE;
     char* ws = static_cast<char*>(workspace);
@@ -549,24 +377,34 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
     }
 
     const int nc = n_centers < n ? n_centers : n;
-    const size_t smem = finalize_smem(n, nc);
-    const int v = n <= kFinThreads ? 0 : n <= 4 * kFinThreads ? 1 : n <= 8 * kFinThreads ? 2 : 3;
-    auto fin = v == 0 ? vic_finalize_kernel<1> : v == 1 ? vic_finalize_kernel<4> : v == 2 ? vic_finalize_kernel<8> : vic_finalize_kernel<16>;
-    static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kFinThreads, "tokens of the longest sample");
-    if (v > 0) {                                           // (up to 1024 tokens 5 KB)
-        static DoneOnDevice attr_done[4];
-        const int most = (v == 1 ? 4 : v == 2 ? 8 : 16) * kFinThreads;
-        rc = allow_dynamic_smem(fin, finalize_smem(most, most), attr_done[v]);
-        if (rc != VITCOP_OK) return rc;
-    }
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    pdl_config(cfg, attr, dim3(B), dim3(kFinThreads), smem, stream, true);
+    // CTAs per sample: one up to 8192 tokens, eight beyond where the batch is on the chip at once (2 x 16384 tokens 28 us on one, 15
+    // on eight; 4 x 4608 9 on one, 12 on eight, which meet a dozen times).
+    const int R = n > 8 * kGroupThreads && B <= finalize_clusters_at_once() ? 8 : 1;
+    int E = 1;
+    while (R * E * kGroupThreads < n) E *= 2;
+    static_assert(VITCOP_MAX_VISUAL_TOKENS <= 16 * kGroupThreads, "tokens of the longest sample");
+    // With all scores there by then the selection of up to 2048 tokens follows in the same kernel.
+    const bool select = quota && n <= kRankTokens && knorm && knorm_in_sweep == knorm->B;
+    if (quota) quota->taken = select;
     {
+        const VicArgs v = {static_cast<const uint16_t*>(feat), n, D, nc, rho, best, w, a, label, n_clusters, delta2_user, parent_user};
+        QuotaArgs q = {};
+        if (select) q.job = *quota;
+        q.status = g.status;
+        const size_t smem = finalize_smem(R, n, nc, select, &q.P_cap);
+        rc = finalize_allow_smem(R, E, select);
+        if (rc != VITCOP_OK) return rc;
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[2];
+        pdl_config(cfg, attr, dim3((unsigned)B * (unsigned)R), dim3(kGroupThreads), smem, stream, true);
+        if (R > 1) {
+            attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+            attr[cfg.numAttrs].val.clusterDim.x = (unsigned)R;
+            attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+            ++cfg.numAttrs;
+        }
         KernelTimeScope timed("vic_finalize_kernel", stream);
-        rc = record_cuda(cudaLaunchKernelEx(&cfg, fin, static_cast<const uint16_t*>(feat), n, D, nc,
-                                            (const float*)rho, (const unsigned long long*)best, (const float*)w,
-                                            (const float*)a, label, n_clusters, delta2_user, parent_user));
+        rc = record_cuda(cudaLaunchKernelEx(&cfg, finalize_kernel(R, E, select), v, q));
         if (rc != VITCOP_OK) return rc;
     }
     if (knorm && knorm_in_sweep < knorm->B) {

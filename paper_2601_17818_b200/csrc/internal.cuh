@@ -72,6 +72,14 @@ struct KnormJob {
     float* score;
 };
 
+// Cluster-quota selection to follow the labels in the same kernel where the scores are there by then (`taken`).
+struct QuotaJob {
+    const float* score;                                    // [B, Nv]
+    int budget;
+    int32_t *keep, *n_keep;                                // [B, Nv], [B]
+    bool taken;
+};
+
 int launch_select(const float* score, const int32_t* label, int B, const int32_t* vis_len, int vis_len_uniform,
                   int Nv_cap, int mode, int largest, int budget, int32_t* keep_idx, int keep_stride,
                   int32_t* n_keep, uint8_t* keep_mask, int* status_word, cudaStream_t stream, bool pdl,
@@ -91,7 +99,8 @@ size_t filter_workspace_least_bytes(int B, int n);
 size_t similarity_workspace_bytes(int B, int n, int D);
 int launch_filter(const void* feat, const float* pos, int B, int n, int D, const vitcop_filter_params& p,
                   int n_centers, int32_t* label, int32_t* n_clusters, float* rho, float* delta2, int32_t* parent,
-                  void* workspace, size_t workspace_bytes, cudaStream_t stream, const KnormJob* knorm = nullptr);
+                  void* workspace, size_t workspace_bytes, cudaStream_t stream, const KnormJob* knorm = nullptr,
+                  QuotaJob* quota = nullptr);
 int launch_similarity_rows(const void* feat, int B, int n, int D, int metric, int row_begin, int row_end,
                            float* out, void* workspace, cudaStream_t stream);
 

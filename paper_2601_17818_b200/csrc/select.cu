@@ -4,8 +4,8 @@
 //    found with one or two histogram passes of 11 bits that start at the highest bit in which two keys differ; the pairs left in
 //    the cut's bin are ranked by counting.  The kept indices leave in ascending order: a ballot ranks a token inside its warp,
 //    one scan over the warps' counts the rest.
-//  quota mode (Eq. 5 / Algorithm 3 up to the elite set): select_quota.cuh.
-#include "select_quota.cuh"
+//  quota mode (Eq. 5 / Algorithm 3 up to the elite set): select_rank.cuh up to 2048 tokens, select_quota.cuh beyond.
+#include "select_rank.cuh"
 
 namespace vitcop {
 namespace {
@@ -185,8 +185,30 @@ select_quota_kernel(const float* score, const int32_t* label,
                     uint8_t* __restrict__ keep_mask, int* __restrict__ status_word) {
     grid_dependency_launch_dependents();                  // see select_plain_kernel
     grid_dependency_wait();
-    select_quota_body<R, E>(score, label, vis_len, vis_len_uniform, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep,
-                         keep_mask, status_word, blockIdx.x / R);
+    if constexpr (E * kSelThreads <= kRankTokens) {
+        extern __shared__ __align__(16) uint8_t rank_dyn[];
+        __shared__ RankShared sh;
+        const int b = blockIdx.x, n = max(0, min(vis_len ? __ldcg(vis_len + b) : vis_len_uniform, Nv_cap));
+        score += (int64_t)b * Nv_cap;
+        label += (int64_t)b * Nv_cap;
+        keep_idx += (int64_t)b * keep_stride;
+        if (keep_mask) keep_mask += (int64_t)b * Nv_cap;
+        int lab[E];
+        uint32_t key[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = e * kSelThreads + threadIdx.x;
+            lab[e] = i < n ? __ldcg(label + i) : 0;
+            key[e] = i < n ? order_key(__ldcg(score + i), 0) : 0u;
+            if ((uint32_t)lab[e] >= (uint32_t)n) lab[e] = max(n - 1, 0);     // out-of-range labels are clamped, never indexed
+        }
+        if (select_by_rank<E>(lab, key, n, budget, sh, rank_dyn, keep_idx, keep_stride, n_keep + b, keep_mask, status_word)) return;
+        select_by_sort(score, label, n, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word, rank_dyn,
+                       sh.warp_sums);
+    } else {
+        select_quota_body<R, E>(score, label, vis_len, vis_len_uniform, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep,
+                                keep_mask, status_word, blockIdx.x / R);
+    }
 }
 
 typedef void (*QuotaKernel)(const float*, const int32_t*, const int32_t*, int, int, int, int, int32_t*, int, int32_t*, uint8_t*, int*);
@@ -197,9 +219,12 @@ QuotaKernel quota_kernel(int R, int E) {
            : E == 8 ? (R == 1 ? select_quota_kernel<1, 8> : select_quota_kernel<4, 8>)
            : R == 1 ? select_quota_kernel<1, 16> : R == 4 ? select_quota_kernel<4, 16> : select_quota_kernel<8, 16>;
 }
+size_t quota_smem(int E, int Nv_cap, int* P_cap) {
+    return E * kSelThreads <= kRankTokens ? rank_or_sort_smem(Nv_cap, P_cap) : select_quota_smem(Nv_cap, P_cap);
+}
 size_t quota_most_smem(int E) {
     int p = 0;
-    return select_quota_smem(E * kSelThreads, &p);
+    return quota_smem(E, E * kSelThreads, &p);
 }
 int quota_allow_smem(int R, int E) {
     static DoneOnDevice attr_done[9][17];
@@ -262,8 +287,8 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
                                               largest, budget, keep_idx, keep_stride, n_keep, keep_mask, clear_status));
     }
     int P = 0;
-    const size_t smem = select_quota_smem(Nv_cap, &P);
     const int E = Nv_cap <= kSelThreads ? 1 : Nv_cap <= 2 * kSelThreads ? 2 : Nv_cap <= 4 * kSelThreads ? 4 : Nv_cap <= 8 * kSelThreads ? 8 : 16;
+    const size_t smem = quota_smem(E, Nv_cap, &P);
     // CTAs per sequence: one up to 2048 tokens (the others would be done preparing when the first is done), four, and eight
     // beyond 8192; fewer where the batch would not be on the chip at once
     int R = E <= 2 ? 1 : E <= 8 ? 4 : 8;

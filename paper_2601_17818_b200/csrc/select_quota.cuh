@@ -1,5 +1,5 @@
 // Cluster-quota selection (Eq. 5 / Algorithm 3 up to the elite set) as a device routine of one to eight CTAs, called by
-// select_quota_kernel (select.cu).
+// select_quota_kernel (select.cu) for more than 2048 tokens (select_rank.cuh: up to there).
 #pragma once
 
 #include "async_copy.cuh"
@@ -50,9 +50,9 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
         const int i = t * E + e;
         unsigned long long c = ~0ull;
         if (t < T && i < n) {
-            uint32_t lab = (uint32_t)label[i];
+            uint32_t lab = (uint32_t)__ldcg(label + i);
             if (lab >= (uint32_t)n) lab = (uint32_t)n - 1;          // out-of-range labels are clamped, never indexed
-            c = ((unsigned long long)lab << 48) | ((unsigned long long)order_key(score[i], 0) << 16) |
+            c = ((unsigned long long)lab << 48) | ((unsigned long long)order_key(__ldcg(score + i), 0) << 16) |
                 (unsigned long long)i;
         }
         r[e] = c;
@@ -454,38 +454,18 @@ __device__ __forceinline__ bool select_quota_by_cluster(const float* score, cons
     return true;
 }
 
-// ------------------------------------------------------------------------------------------ quota
-// Shared memory: comp[P] (uint64), cstart[n] and csize[n] (uint16, indexed by label value), keep[n] (uint8).
-// Cluster-quota selection of sample b by R whole CTAs (kSelThreads threads each); uses the dynamic shared memory.
-template <int R, int E>
-__device__ __forceinline__ void select_quota_body(const float* score, const int32_t* label,
-                                                  const int32_t* vis_len, int vis_len_uniform,
-                                                  int Nv_cap, int P_cap, int budget, int32_t* __restrict__ keep_idx,
-                                                  int keep_stride, int32_t* __restrict__ n_keep,
-                                                  uint8_t* __restrict__ keep_mask, int* __restrict__ status_word,
-                                                  int b) {
-    extern __shared__ __align__(16) uint32_t quota_smem[];
-    unsigned long long* comp = reinterpret_cast<unsigned long long*>(quota_smem);
+// ------------------------------------------------------------------------------------------ quota by a sort
+// For more clusters than the per-cluster searches handle, or a short sample with very uneven clusters: the composites (label, score
+// key, index) sorted by one CTA.  Shared memory: comp[P] (uint64), cstart[n] and csize[n] (uint16, indexed by label value), keep[n]
+// (uint8).
+__device__ __forceinline__ void select_by_sort(const float* score, const int32_t* label, int n, int Nv_cap, int P_cap, int budget,
+                                               int32_t* keep_idx, int keep_stride, int32_t* n_keep_b, uint8_t* keep_mask,
+                                               int* status_word, uint8_t* smem, uint32_t* warp_sums) {
+    unsigned long long* comp = reinterpret_cast<unsigned long long*>(smem);
     uint16_t* cstart = reinterpret_cast<uint16_t*>(comp + P_cap);
     uint16_t* csize = cstart + Nv_cap;
     uint8_t* keepf = reinterpret_cast<uint8_t*>(csize + Nv_cap);
-    __shared__ uint32_t warp_sums[kSelWarps];
-
     const int tid = threadIdx.x;
-    int n = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
-    n = max(0, min(n, Nv_cap));
-    score += (int64_t)b * Nv_cap;
-    label += (int64_t)b * Nv_cap;
-    keep_idx += (int64_t)b * keep_stride;
-    if (keep_mask) keep_mask += (int64_t)b * Nv_cap;
-
-    if (select_quota_by_cluster<R, E>(score, label, n, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
-                                   reinterpret_cast<uint8_t*>(quota_smem), warp_sums))
-        return;
-    if (R > 1 && cluster_ctarank() != 0) return;
-    __syncthreads();
-    // more clusters than the per-cluster searches handle, or a short sample with very uneven clusters: sort the
-    // composites (label, score key, index)
     int P = 256;                                          // at least one warp of 8 keys per thread
     while (P < n) P <<= 1;
     for (int i = tid; i < n; i += kSelThreads) keepf[i] = 0;
@@ -531,7 +511,35 @@ __device__ __forceinline__ void select_quota_body(const float* score, const int3
     __syncthreads();
     const uint32_t kept =
         emit_ascending(n, [&](int i) { return keepf[i] != 0; }, keep_idx, keep_stride, keep_mask, warp_sums);
-    if (tid == 0) n_keep[b] = (int32_t)kept;
+    if (tid == 0) *n_keep_b = (int32_t)kept;
+}
+
+// ------------------------------------------------------------------------------------------ quota
+// Cluster-quota selection of sample b by R whole CTAs (kSelThreads threads each); uses the dynamic shared memory.
+template <int R, int E>
+__device__ __forceinline__ void select_quota_body(const float* score, const int32_t* label,
+                                                  const int32_t* vis_len, int vis_len_uniform,
+                                                  int Nv_cap, int P_cap, int budget, int32_t* __restrict__ keep_idx,
+                                                  int keep_stride, int32_t* __restrict__ n_keep,
+                                                  uint8_t* __restrict__ keep_mask, int* __restrict__ status_word,
+                                                  int b) {
+    extern __shared__ __align__(16) uint32_t quota_smem[];
+    __shared__ uint32_t warp_sums[kSelWarps];
+
+    int n = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
+    n = max(0, min(n, Nv_cap));
+    score += (int64_t)b * Nv_cap;
+    label += (int64_t)b * Nv_cap;
+    keep_idx += (int64_t)b * keep_stride;
+    if (keep_mask) keep_mask += (int64_t)b * Nv_cap;
+
+    if (select_quota_by_cluster<R, E>(score, label, n, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
+                                   reinterpret_cast<uint8_t*>(quota_smem), warp_sums))
+        return;
+    if (R > 1 && cluster_ctarank() != 0) return;
+    __syncthreads();
+    select_by_sort(score, label, n, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
+                   reinterpret_cast<uint8_t*>(quota_smem), warp_sums);
 }
 
 
