@@ -16,15 +16,15 @@
 // from block to block and the warp exchanges only the bound; the place of a value is one add and one select away from the
 // token's.  Measured on 8 x 2880 tokens, caches warm: 19.7 -> 15.1 us and 18.3 -> 13.9 us against a warp-wide minimum and ballot
 // per block and four separate loads per token.  Passing over blocks without a denser token in the first kernel too: 6 us less on
-// 4 x 4096 tokens.  Four rounds instead of three: 1 us less there, 20 us more on 2 x 16384 tokens.
+// 4 x 4096 tokens.  Four rounds there: three, five and six take as long on 8 x 2880 and 4 x 4608 tokens and up to 3 us longer on 2 x 16384.
 #include "density.cuh"
 
 namespace vitcop {
 namespace {
 
 constexpr int kNdThreads = 256, kNdWarps = kNdThreads / 32;
-constexpr int kNdRounds = 3;                               // rounds of two blocks that a warp does for its own token
-constexpr int kNdAhead = 4;                                // blocks a warp of the second kernel looks into at a time
+constexpr int kNdRounds = 4;                               // rounds of two blocks that a warp does for its own token
+constexpr int kNdAhead = 3;                                // blocks a warp of the second kernel looks into at a time
 constexpr uint32_t kInfBits = 0x7f800000u;
 // A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, above it
 // one bit that marks a stand-in; i.e. a bound up to 2^-13 too low.
@@ -162,8 +162,10 @@ nearest_denser_kernel(const __grid_constant__ SweepArgs g) {
 // The tokens left over, each shared out over `slices` warps: warp w of a token takes the blocks w, w + slices, .. that are
 // still open and hold a denser token.  (Those the first kernel has looked into already cannot improve on its result.)
 // Each warp in ascending order of its blocks' minima: in the order of their numbers it looked into more of them (2 x 16384 tokens
-// of no structure 128.6 -> 117.5 us; 4 x 4608 of a video, whole call, 212 -> 209).  Two or four times as many blocks per warp measured
-// the same or worse.
+// of no structure 128.6 -> 117.5 us; 4 x 4608 of a video, whole call, 212 -> 209).  Two or four times as many or as few blocks per warp
+// measured the same or worse.  What one warp finds it tells the token's others at once, and what they have found travels with its blocks,
+// three at a time instead of four: alone, a warp goes on below a bound that another one has lowered long since (2 x 16384 tokens 41 -> 25 us;
+// of no structure, whole call, 1000 -> 754).
 template <int METRIC, bool SPATIAL>
 __global__ void __launch_bounds__(kNdThreads)
 nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
@@ -179,8 +181,7 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
         Search<METRIC, SPATIAL> s(g, b, i, lane);
         // (other warps may be lowering it: a stale one is only looser, but all lanes must go by the same one, as it decides which of
         // them meet in the reductions below)
-        const unsigned long long known = __shfl_sync(0xffffffffu, lane == 0 ? __ldcg(g.best + at) : 0ull, 0);
-        unsigned long long best = known;
+        unsigned long long best = __shfl_sync(0xffffffffu, lane == 0 ? __ldcg(g.best + at) : 0ull, 0);
         // Can block k, with minimum `lo`, hold a token below `best`?  (An equal distance at a lower index would win.)
         auto can = [&](uint32_t lo, int k) {
             return lo < kInfBits && (((unsigned long long)lo << 32) | (unsigned long long)(uint32_t)(k * kBlk)) < best;
@@ -211,14 +212,20 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
                     }
                 }
                 if (cnt == 0) break;
+                // (what the token's other warps have found by now travels with the blocks)
+                const unsigned long long others = lane == 0 ? __ldcg(g.best + at) : 0ull;
 #pragma unroll
                 for (int u = 0; u < kNdAhead; ++u)
                     if (u < cnt) s.look(p[u], blk[u]);
                 const unsigned long long found = s.packed(s.bound());
-                best = found < best ? found : best;
+                if (found < best) {
+                    best = found;
+                    if (lane == 0) atomicMin(g.best + at, best);
+                }
+                const unsigned long long theirs = __shfl_sync(0xffffffffu, others, 0);
+                best = theirs < best ? theirs : best;
             }
         }
-        if (lane == 0 && best < known) atomicMin(g.best + at, best);
     }
 }
 
