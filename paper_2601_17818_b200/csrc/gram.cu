@@ -1308,16 +1308,20 @@ bool gram_resident_takes_knorm(int H, int d) {
     return knorm_buffers(H, d) > 0;
 }
 
-// All of them where no CTA has more than three chunks of tokens: one kernel less (1 x 576 tokens x 8 heads of 128 30.8 -> 29.6 us, 4 x 576
-// x 2 of 64 30.9 -> 29.1).  Not with a single buffer, where each chunk waits for the one before (48 heads of 256: 1 x 576 35.2 us with
-// all against 34.6 without, 2 x 576 37.2 / 35.2 with half).  Otherwise two and a half chunks to a CTA, whatever their size: more
-// hold up the sweep's barrier and searches by as much as they take beside vic_finalize_kernel (16 x 576 x 32 of 128 61.7 us with 5 of
-// the samples, 64.3 / 62.6 / 63.5 with 0 / 7 / 16; 3 x 1000 x 48 of 256 48.0 with 2, 61.7 with none), and over 16 problems x 9 forms of
-// keys no share was found that is better throughout (times come in steps of 2 us).
+// All of them where the copies are double buffered, for samples of more than one row tile: one kernel less, and with all of them the
+// selection follows within the labels' kernel.  Two and a half chunks of eight tokens to a CTA in the sweep and the other samples
+// beside vic_finalize_kernel / all in the sweep, us: 1 x 300 tokens x 32 heads of 128 28.7 / 26.8, 7 x 700 x 32 of 128 47.1 / 44.0, 16 x 576 x
+// 32 of 128 66.9 / 57.5 (8 chunks), 16 x 576 x 4 of 64 50.1 / 47.4, 32 x 576 x 32 of 128 119.1 / 101.8 (16 chunks), 148 x 256 x 32 of 128
+// 226.2 / 208.9 (32); 1 x 182 x 32 of 128 26.9 / 28.5 was the one loss of 60 problems.  Short chunks are held up by their waits: above
+// 24 of them rows of 2 KB at least (140 x 256 x 4 of 64 91.6 / 94.8 with 30, 120 x 256 x 8 of 128 101.3 / 92.2 with 26).
+// Samples of one row tile have one CTA each, whose sweep ends when its keys do: three chunks (1 x 64 x 32 of 128 26.8 / 30.8 with all
+// 8, 64 x 64 x 16 of 128 43.5 / 44.9; more only pays where they fill the chip, 100 x 128 x 32 of 128 108.6 / 100.3).  With a single buffer
+// each chunk waits for the one before (48 heads of 256: 2 x 576 35.0 / 36.0, 16 x 200 63.6 / 70.8): two and a half chunks to a CTA.
 int gram_resident_knorm_samples(int B, int n, int H, int d, int Nv) {
     const long long ctas = resident_ctas(ResidentCut(B, n).total), chunks = (Nv + kKnChunkTokens - 1) / kKnChunkTokens;
     const long long share = 5 * ctas / (2 * chunks);
-    return share >= B || (knorm_buffers(H, d) > 1 && chunks * B <= 3 * ctas) ? B : (int)share;
+    const bool all = n > BM ? chunks * B <= 24 * ctas || H * d >= 1024 : chunks * B <= 3 * ctas;
+    return share >= B || (knorm_buffers(H, d) > 1 && all) ? B : (int)share;
 }
 
 int launch_gram_resident(const void* feat, const GramArgs& args, const GramTiling& tiling, cudaStream_t stream) {

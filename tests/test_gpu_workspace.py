@@ -123,6 +123,16 @@ def test_norms_beside_the_density_sweep_are_the_stand_alone_ones(B, n, T, H, d, 
     assert "density_sweep_kernel" in names and ("knorm_kernel" in names) == alone
 
 
+# Keys of all samples beside a sweep, on either side of the lines: one and two row tiles, 24 chunks to a CTA, a single buffer; 8 MB.
+@pytest.mark.parametrize("B,n,T,H,d,D,alone", [(1, 128, 1, 3, 128, 128, True), (1, 129, 1, 3, 128, 128, False),
+                                               (147, 249, 2, 1, 64, 64, True), (147, 249, 0, 16, 64, 64, False),
+                                               (32, 576, 3, 3, 256, 64, False), (8, 577, 0, 48, 256, 64, True),
+                                               (7, 1921, 5, 32, 64, 768, False), (7, 1921, 0, 4, 64, 768, True)])
+def test_norms_of_all_samples_beside_a_sweep(B, n, T, H, d, D, alone):
+    step, _ = _compare_norms(B, n, T, H, d, D)
+    assert ("knorm_kernel" in _kernels(step)) == alone
+
+
 @pytest.mark.parametrize("metric,spatial", [(0, True), (1, False), (1, True)])
 @pytest.mark.parametrize("B,n,T,H,d,D", [(8, 2881, 3, 31, 128, 512), (9, 2879, 0, 62, 64, 512)])
 def test_norms_beside_the_density_sweep_with_either_metric(B, n, T, H, d, D, metric, spatial):
