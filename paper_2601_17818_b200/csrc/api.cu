@@ -334,6 +334,11 @@ int vitcop_prune_step(const void* hidden, const void* K, const void* V, int B, i
     // in front of the span before its own wait: that is safe only behind a kernel of this call that has itself
     // waited for everything queued before the call.  With an empty span there is no such kernel, so the selection
     // is then launched in plain stream order.
+    if (have_knorm && !label && compact_selects(hidden != nullptr, V != nullptr, B, H, d, Dh, Nv_cap, Ncap)) {
+        const SmallestJob smallest = {score, budget, keep, nkeep};
+        return launch_compact(hidden, K, V, B, H, N, d, Dh, seq_len, vis_start, vis_len, vis_len_uniform, nullptr, Nv_cap,
+                              nullptr, hidden_out, K_out, V_out, Ncap, kept_pos, out_len, s, true, &smallest);
+    }
     rc = launch_select(score, label, B, vis_len, vis_len_uniform, Nv_cap, label ? 1 : 0, 0, budget, keep, Nv_cap,
                        nkeep, nullptr, reinterpret_cast<int*>(ws), s, have_knorm);
     if (rc != VITCOP_OK) return rc;

@@ -86,10 +86,19 @@ int launch_select(const float* score, const int32_t* label, int B, const int32_t
                   int* clear_status = nullptr);
 // (`clear_status`: plain mode sets this status word to VITCOP_OK on the way, in place of a memset in front of the kernel.)
 
+// Plain selection (smallest scores) inside the copy, in place of a list; where compact_selects says that this is the faster way.
+struct SmallestJob {
+    const float* score;                                    // [B, keep_stride]
+    int budget;
+    int32_t *keep, *n_keep;                                // the list, written: [B, keep_stride], [B]
+};
+bool compact_selects(bool hidden, bool V, int B, int H, int d, int Dh, int Nv_cap, int Ncap);
+
 int launch_compact(const void* hidden, const void* K, const void* V, int B, int H, int N, int d, int Dh,
                    const int32_t* seq_len, int vis_start, const int32_t* vis_len, int vis_len_uniform,
                    const int32_t* keep_idx, int keep_stride, const int32_t* n_keep, void* hidden_out, void* K_out,
-                   void* V_out, int Ncap, int32_t* kept_pos, int32_t* out_len, cudaStream_t stream, bool early);
+                   void* V_out, int Ncap, int32_t* kept_pos, int32_t* out_len, cudaStream_t stream, bool early,
+                   const SmallestJob* smallest = nullptr);
 // (`early`: the tensors are inputs of a whole call whose first kernel has waited for everything queued before it, so rows that
 // do not depend on the selection may be copied while the kernels in front are still running.)
 
