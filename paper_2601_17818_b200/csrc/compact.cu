@@ -128,17 +128,14 @@ __device__ __forceinline__ void warp_smallest(const float* score, int n, int k, 
     }
 }
 
-// TOKENS > 0: the rows are chosen here, from the scores of at most so many tokens a sample, and the first CTA of a sample writes the
-// list (keep_out, n_keep_out).
-template <int G, int TOKENS>
+template <int G>
 __global__ void __launch_bounds__(kCompactThreads, G == kCompactThreads ? 4 : 3)
 compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, const uint4* __restrict__ V, int B, int H, int N,
                int d8, int dh8, int d8_shift, const int32_t* seq_len, int vis_start,
                const int32_t* vis_len, int vis_len_uniform, const int32_t* keep_idx,
                int keep_stride, const int32_t* n_keep, uint4* __restrict__ hidden_out,
                uint4* __restrict__ K_out, uint4* __restrict__ V_out, int Ncap, int32_t* __restrict__ kept_pos,
-               int32_t* __restrict__ out_len, int early, const float* score, int budget,
-               int32_t* __restrict__ keep_out, int32_t* __restrict__ n_keep_out) {
+               int32_t* __restrict__ out_len, int early) {
     // A copy that stands alone reads rows that the kernel in front may still be writing, so only its launch overlaps (a
     // selection and a copy of 16 x 576 rows: 23.7 -> 19.1 us with both launched this way).
     if (!early) grid_dependency_wait();
@@ -151,39 +148,6 @@ compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, co
     const int lane = G == kCompactThreads ? threadIdx.x : threadIdx.x % G;
     const int L = seq_len ? min(__ldcg(seq_len + b), N) : N;
     const int64_t head_in = (int64_t)N * d8, head_out = (int64_t)Ncap * d8;
-    if constexpr (TOKENS > 0) {
-        const auto copy_row = [&](int from) {
-            copy_token<G>(lane, hidden ? hidden + ((int64_t)b * N + from) * dh8 : nullptr, hidden_out + ((int64_t)b * Ncap + r) * dh8,
-                          dh8, K ? K + ((int64_t)b * H * N + from) * d8 : nullptr, K_out + ((int64_t)b * H * Ncap + r) * d8,
-                          V ? V + ((int64_t)b * H * N + from) * d8 : nullptr, V_out + ((int64_t)b * H * Ncap + r) * d8, H, d8,
-                          d8_shift, head_in, head_out);
-            if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = from;
-        };
-        // How many tokens stay follows from the lengths: rows behind the span have their place as early as those in front of it.
-        __shared__ uint16_t list[TOKENS];
-        const int len = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
-        const int n = max(0, min(len, keep_stride)), k = max(0, min(budget, n));
-        const int nv = max(0, min(len, L - vis_start)), nk = min(k, nv), olen = L - nv + nk;
-        const bool chosen = r >= vis_start && r < vis_start + nk;
-        if (r < Ncap && !chosen) {
-            if (r < olen) copy_row(r < vis_start ? r : r - nk + nv);
-            else if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = -1;
-        }
-        constexpr int kRows = kCompactThreads / G;
-        if (rg != 0 && (rg * kRows >= vis_start + nk || rg * kRows + kRows <= vis_start)) return;      // (uniform over the CTA)
-        grid_dependency_wait();
-        if (threadIdx.x < 32) warp_smallest<TOKENS / 32>(score + (int64_t)b * keep_stride, n, k, list);
-        __syncthreads();
-        if (rg == 0) {
-            if ((int)threadIdx.x < k) keep_out[(int64_t)b * keep_stride + threadIdx.x] = (int32_t)list[threadIdx.x];
-            if (threadIdx.x == 0) {
-                n_keep_out[b] = k;
-                out_len[b] = olen;
-            }
-        }
-        if (r < Ncap && chosen) copy_row(vis_start + min((int)list[r - vis_start], nv - 1));
-        return;
-    }
     // A row in front of the visual span keeps its place whatever the selection turns out to be: it is copied
     // before this kernel waits for the selection, while the kernels that produce it are still running.  (The
     // tensors copied here are inputs of the whole call, complete before its first kernel started.)
@@ -227,10 +191,51 @@ compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, co
                d8_shift, head_in, head_out);
 }
 
-typedef decltype(&compact_kernel<32, 0>) CompactKernel;
-template <int G>
-CompactKernel compact_of(int tokens) {
-    return tokens == 0 ? compact_kernel<G, 0> : tokens <= 128 ? compact_kernel<G, 128> : compact_kernel<G, 256>;
+// The same with the selection inside, from the scores of at most TOKENS tokens a sample; the first CTA of a sample writes the list.  (A
+// kernel of its own: four more parameters cost each launch of the other one 0.4 us of the caller's time.)
+template <int G, int TOKENS>
+__global__ void __launch_bounds__(kCompactThreads, G == kCompactThreads ? 4 : 3)
+select_compact_kernel(const uint4* __restrict__ hidden, const uint4* __restrict__ K, const uint4* __restrict__ V, int B, int H, int N,
+                      int d8, int dh8, int d8_shift, const int32_t* seq_len, int vis_start, const int32_t* vis_len, int vis_len_uniform,
+                      const float* score, int keep_stride, int budget, int32_t* __restrict__ keep_out, int32_t* __restrict__ n_keep_out,
+                      uint4* __restrict__ hidden_out, uint4* __restrict__ K_out, uint4* __restrict__ V_out, int Ncap,
+                      int32_t* __restrict__ kept_pos, int32_t* __restrict__ out_len) {
+    const int rg = (int)(blockIdx.x / (unsigned)B);
+    const int b = (int)(blockIdx.x - (unsigned)rg * (unsigned)B);
+    const int r = G == kCompactThreads ? rg : rg * (kCompactThreads / G) + (int)threadIdx.x / G;
+    const int lane = G == kCompactThreads ? threadIdx.x : threadIdx.x % G;
+    const int L = seq_len ? min(__ldcg(seq_len + b), N) : N;
+    const int64_t head_in = (int64_t)N * d8, head_out = (int64_t)Ncap * d8;
+    const auto copy_row = [&](int from) {
+        copy_token<G>(lane, hidden ? hidden + ((int64_t)b * N + from) * dh8 : nullptr, hidden_out + ((int64_t)b * Ncap + r) * dh8,
+                      dh8, K ? K + ((int64_t)b * H * N + from) * d8 : nullptr, K_out + ((int64_t)b * H * Ncap + r) * d8,
+                      V ? V + ((int64_t)b * H * N + from) * d8 : nullptr, V_out + ((int64_t)b * H * Ncap + r) * d8, H, d8,
+                      d8_shift, head_in, head_out);
+        if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = from;
+    };
+    // How many tokens stay follows from the lengths: rows behind the span have their place as early as those in front of it.
+    __shared__ uint16_t list[TOKENS];
+    const int len = vis_len ? __ldcg(vis_len + b) : vis_len_uniform;
+    const int n = max(0, min(len, keep_stride)), k = max(0, min(budget, n));
+    const int nv = max(0, min(len, L - vis_start)), nk = min(k, nv), olen = L - nv + nk;
+    const bool chosen = r >= vis_start && r < vis_start + nk;
+    if (r < Ncap && !chosen) {
+        if (r < olen) copy_row(r < vis_start ? r : r - nk + nv);
+        else if (kept_pos && lane == 0) kept_pos[(int64_t)b * Ncap + r] = -1;
+    }
+    constexpr int kRows = kCompactThreads / G;
+    if (rg != 0 && (rg * kRows >= vis_start + nk || rg * kRows + kRows <= vis_start)) return;      // (uniform over the CTA)
+    grid_dependency_wait();
+    if (threadIdx.x < 32) warp_smallest<TOKENS / 32>(score + (int64_t)b * keep_stride, n, k, list);
+    __syncthreads();
+    if (rg == 0) {
+        if ((int)threadIdx.x < k) keep_out[(int64_t)b * keep_stride + threadIdx.x] = (int32_t)list[threadIdx.x];
+        if (threadIdx.x == 0) {
+            n_keep_out[b] = k;
+            out_len[b] = olen;
+        }
+    }
+    if (r < Ncap && chosen) copy_row(vis_start + min((int)list[r - vis_start], nv - 1));
 }
 
 // How many threads move a row of so many pieces, and how many CTAs that makes.
@@ -279,16 +284,22 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
     KernelTimeScope timed("compact_kernel", stream);
-    const SmallestJob job = smallest ? *smallest : SmallestJob{};
-    const int tokens = !smallest ? 0 : keep_stride <= 128 ? 128 : 256;
-    auto kern = G == 256   ? compact_of<256>(tokens)
-                : G == 128 ? compact_of<128>(tokens)
-                : G == 64  ? compact_of<64>(tokens) : compact_of<32>(tokens);
-    return record_cuda(cudaLaunchKernelEx(
-        &cfg, kern, static_cast<const uint4*>(hidden), static_cast<const uint4*>(K),
-        static_cast<const uint4*>(V), B, H, N, d / 8, Dh / 8, d8_shift, seq_len, vis_start, vis_len, vis_len_uniform,
-        keep_idx, keep_stride, n_keep, static_cast<uint4*>(hidden_out), static_cast<uint4*>(K_out), static_cast<uint4*>(V_out),
-        Ncap, kept_pos, out_len, early ? 1 : 0, job.score, job.budget, job.keep, job.n_keep));
+    const uint4 *hid = static_cast<const uint4*>(hidden), *k = static_cast<const uint4*>(K), *v = static_cast<const uint4*>(V);
+    uint4 *const hid_out = static_cast<uint4*>(hidden_out), *const k_out = static_cast<uint4*>(K_out), *const v_out = static_cast<uint4*>(V_out);
+    if (smallest) {
+        const bool few = keep_stride <= 128;
+        auto kern = G == 256   ? (few ? select_compact_kernel<256, 128> : select_compact_kernel<256, 256>)
+                    : G == 128 ? (few ? select_compact_kernel<128, 128> : select_compact_kernel<128, 256>)
+                    : G == 64  ? (few ? select_compact_kernel<64, 128> : select_compact_kernel<64, 256>)
+                               : (few ? select_compact_kernel<32, 128> : select_compact_kernel<32, 256>);
+        return record_cuda(cudaLaunchKernelEx(&cfg, kern, hid, k, v, B, H, N, d8, Dh / 8, d8_shift, seq_len, vis_start, vis_len,
+                                              vis_len_uniform, smallest->score, keep_stride, smallest->budget, smallest->keep,
+                                              smallest->n_keep, hid_out, k_out, v_out, Ncap, kept_pos, out_len));
+    }
+    auto kern = G == 256 ? compact_kernel<256> : G == 128 ? compact_kernel<128> : G == 64 ? compact_kernel<64> : compact_kernel<32>;
+    return record_cuda(cudaLaunchKernelEx(&cfg, kern, hid, k, v, B, H, N, d8, Dh / 8, d8_shift, seq_len, vis_start, vis_len,
+                                          vis_len_uniform, keep_idx, keep_stride, n_keep, hid_out, k_out, v_out, Ncap, kept_pos, out_len,
+                                          early ? 1 : 0));
 }
 
 }  // namespace vitcop
