@@ -254,7 +254,7 @@ struct Split {
 }  // namespace
 
 // A copy of few rows is the end of a chain of short kernels: one link less outweighs that every CTA selects (whole calls by
-// themselves / in a graph, selection as a kernel -> in the copy, us: 1 x 128 tokens x 32 heads of 128 8.9 -> 7.1 / 7.5 -> 6.5, 1 x 256
+// themselves / in a graph, selection as a kernel -> in the copy, us: 1 x 128 tokens x 32 heads of 128 9.1 -> 6.8 / 7.5 -> 6.5, 1 x 256
 // 9.4 -> 8.6 / 8.6 -> 8.6, 4 x 256 12.1 -> 11.4 / 11.6 -> 11.3).  Not where the copy fills the chip (8 x 256: 22.1 -> 23.2, 16 x 256 x 4 of 128
 // 16.9 -> 21.4), and not for longer lists (1 x 576 11.2 -> 12.7).
 bool compact_selects(bool hidden, bool V, int B, int H, int d, int Dh, int Nv_cap, int Ncap) {
