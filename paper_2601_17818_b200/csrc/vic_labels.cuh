@@ -19,7 +19,10 @@ template <int R>
 constexpr int kVicBinsPer = (1 << kVicBits<R>) / kGroupThreads;              // of a thread
 constexpr int kVicRank = 256;                              // bins of up to this many keys are ranked by counting
 constexpr uint32_t kVicIndex = VITCOP_MAX_VISUAL_TOKENS - 1, kVicCentre = 0x8000u;         // an entry of the table: parent; the token is a centre
-constexpr int kChase = 64;
+// Steps of a round and rounds of the chase.  Tokens d steps from their root need one round below 64, two below 4033, four at the 16383 of the
+// longest sample.  The rest is the limit: parents are denser than their children and form no cycle, but behind a sweep that gave up they
+// are whatever the workspace held (two negative densities one step apart are each other's), and then too the kernel has to end.
+constexpr int kChase = 64, kChaseRounds = 8;
 static_assert((kVicIndex & (kVicIndex + 1)) == 0 && kVicIndex < kVicCentre, "indices and the mark of a centre share 16 bits");
 
 struct VicArgs {
@@ -48,14 +51,14 @@ struct VicShared {
     uint16_t cand_idx[kVicRank], all_idx[R == 1 ? 1 : kVicRank];
     uint32_t warp_sums[32];
     uint32_t lo, hi, digit, krem, count, cands;
-    uint32_t flags[8];                                     // per round of the chase: 1 a chain goes on, 2 a root is no centre
+    uint32_t flags[kChaseRounds];                          // per round of the chase: 1 a chain goes on, 2 a root is no centre
     int orph_cnt, centre_cnt;
 
     // All CTAs, before any of them calls vic_labels.
     __device__ __forceinline__ void init() {
         const int tid = threadIdx.x;
         for (int k = tid; k < 2 * kVicBinsPer<R> * kGroupThreads; k += kGroupThreads) hist[0][k] = 0u;
-        if (tid < 8) flags[tid] = 0u;
+        if (tid < kChaseRounds) flags[tid] = 0u;
         if (tid == 0) { lo = 0xFFFFFFFFu; hi = 0u; cands = 0u; centre_cnt = 0; }
         group_sync<R>();
     }
@@ -295,7 +298,7 @@ __device__ __forceinline__ void vic_labels(const VicArgs& v, int b, VicShared<R>
 #pragma unroll
         for (int e = 0; e < E; ++e)
             if (e * kGroupThreads + tid < own) open |= 1u << e;
-        for (int round = 0;; ++round) {
+        for (int round = 0; round < kChaseRounds; ++round) {
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 if (!(open >> e & 1u)) continue;
@@ -314,9 +317,9 @@ __device__ __forceinline__ void vic_labels(const VicArgs& v, int b, VicShared<R>
             }
             // (bits of the warp, to every CTA)
             const uint32_t say = __reduce_or_sync(0xffffffffu, (open ? 1u : 0u) | found);
-            if (say && lane < R) or_cluster(at_cta<R>(&sh.flags[round & 7], lane), say);
+            if (say && lane < R) or_cluster(at_cta<R>(&sh.flags[round], lane), say);
             group_sync<R>();
-            flags = sh.flags[round & 7];
+            flags = sh.flags[round];
             if (!(flags & 1u)) break;
             // chains go on: what was found so far goes into the tables (an ancestor in the place of another)
 #pragma unroll
@@ -326,6 +329,10 @@ __device__ __forceinline__ void vic_labels(const VicArgs& v, int b, VicShared<R>
             tell_others();
             group_sync<R>();
         }
+        // (the limit: an ancestor stands in for the root, as above)
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (open >> e & 1u) at[e] = table[at[e]];
     }
     // ---- a root that is an orphan but not a centre joins the nearest centre (feature distance)
     if ((flags & 2u) && nc > 0) {

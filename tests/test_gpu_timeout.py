@@ -88,6 +88,31 @@ def test_density_sweep_reports_timeout_and_recovers(B, n, roles):
     assert status == vb.OK and all(torch.equal(a, b) for a, b in zip(got, ref))
 
 
+# Beyond 8192 tokens the labels follow the parents in rounds.  The sweep gives up in a workspace that holds 0.5 and -1.5 by turns: every
+# other token has the same negative density, the blocks' minima let the search look at them, and they are one another's parents.
+@pytest.mark.parametrize("roles", [ROLE_EPILOGUE, ROLE_LOAD])
+def test_long_samples_report_timeout_and_recover(roles):
+    B, n = 2, 9000
+    feat = torch.randn((B, n, 64), generator=torch.Generator(device=DEV).manual_seed(n), device=DEV).to(torch.bfloat16)
+    ws = vb.alloc_workspace(vb.OP_FILTER, B=B, Nv=n, D=64)
+
+    def run():
+        label = torch.full((B, n), -1, dtype=torch.int32, device=DEV)
+        ws.view(torch.float32)[0::2] = 0.5
+        ws.view(torch.float32)[1::2] = -1.5
+        vb.vitcop_redundancy_filter(feat, None, label, torch.zeros(B, dtype=torch.int32, device=DEV), ws, n_centers=n // 20)
+        return vb.vitcop_poll_status(ws), label
+
+    status, ref = run()
+    assert status == vb.OK
+    vb.vitcop_set_wait_limit(0, roles * 8)
+    status, label = run()
+    assert status == vb.ERR_TIMEOUT and int(label.min()) >= 0 and int(label.max()) < n
+    vb.vitcop_set_wait_limit(0, 0)
+    status, got = run()
+    assert status == vb.OK and torch.equal(got, ref)
+
+
 def test_sweeps_of_several_streams_end_together():
     """One-kernel sweeps that each want every SM, from three streams of two priorities at once: the CTAs of each wait for one
     another, so they may not keep one another from starting."""
