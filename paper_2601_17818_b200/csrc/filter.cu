@@ -115,7 +115,7 @@ struct QuotaArgs {
     int* status;
 };
 // (One CTA an SM, said aloud: left to itself ptxas went for two of the form up to 1024 tokens, 32 registers a thread and spills, and the
-// filter of 8 x 203 tokens took 21.5 us with the caches flushed; 20.0 so.)
+// filter of 8 x 203 tokens took 21.5 us with the caches flushed; 19.5 so.)
 template <int R, int E, bool SELECT>
 __global__ void __launch_bounds__(kGroupThreads, 1)
 vic_finalize_kernel(const __grid_constant__ VicArgs v, const __grid_constant__ QuotaArgs q) {

@@ -224,19 +224,24 @@ __device__ __forceinline__ void vic_labels(const VicArgs& v, int b, VicShared<R>
             idx_of = sh.all_idx;
             __syncthreads();
         }
-        // a warp per candidate of this CTA
+        // all candidates of this CTA at once, on a warp each or on as many lanes as there are for them (at least four)
+        static_assert(kVicRank * 4 <= kGroupThreads, "four lanes a candidate");
         const int mine = (int)sh.cands;
-        for (int c = tid / 32; c < mine; c += kGroupThreads / 32) {
+        int log_lanes = 5;
+        while (mine << log_lanes > kGroupThreads) --log_lanes;
+        const int lanes = 1 << log_lanes, c = tid >> log_lanes, sub = tid & (lanes - 1);
+        uint32_t better = 0;
+        int idx = 0;
+        if (c < mine) {
             const unsigned long long k = sh.cand_key[c];
-            const int idx = sh.cand_idx[c];
-            uint32_t better = 0;
-            for (int o = lane; o < cands; o += 32) {
+            idx = sh.cand_idx[c];
+            for (int o = sub; o < cands; o += lanes) {
                 const unsigned long long x = key[o];
                 better += (uint32_t)(x < k) | ((uint32_t)(x == k) & (uint32_t)(idx_of[o] < idx));
             }
-            better = __reduce_add_sync(0xffffffffu, better);
-            if (lane == 0 && better < ranked) won[idx - s.base] = 1;
         }
+        for (int off = 1; off < lanes; off <<= 1) better += __shfl_xor_sync(0xffffffffu, better, off);
+        if (c < mine && sub == 0 && better < ranked) won[idx - s.base] = 1;
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < E; ++e)

@@ -82,6 +82,17 @@ def _labels(r, b, n_centers, feat):
     return at, depth
 
 
+# The tokens left in the cut's bin are ranked on as many lanes each as there are for all of them, four to 32.  The densest token has no
+# parent, so the first histogram is a coarse one, and tokens that are much alike all fall into one bin.
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 34, 64, 65, 66, 127, 129, 130, 200, 255, 256, 257, 300])
+def test_centres_among_few_candidates(n):
+    feat = torch.randn((2, n, 64), generator=torch.Generator(device=DEV).manual_seed(n), device=DEV).to(torch.bfloat16)
+    for n_centers in {1, n // 2, n - 1}:
+        r = gpu_filter(vb.bf16_bits(feat), None, 0, 0.5, -1.0, n_centers)
+        for b in range(2):
+            assert r.status == vb.OK and np.array_equal(r.label[b], _labels(r, b, n_centers, None)[0])
+
+
 # every token an orphan (radius zero): all but the centres join the nearest one; a few centres, many, all of them
 @pytest.mark.parametrize("n,n_centers", [(8193, 3), (8200, 411), (16384, 820), (8193, 8193)])
 @pytest.mark.parametrize("tau", [-1.0, 0.0])
