@@ -50,9 +50,9 @@ __device__ void sort_composites(const float* score, const int32_t* label, int n,
         const int i = t * E + e;
         unsigned long long c = ~0ull;
         if (t < T && i < n) {
-            uint32_t lab = (uint32_t)__ldcg(label + i);
+            uint32_t lab = (uint32_t)label[i];
             if (lab >= (uint32_t)n) lab = (uint32_t)n - 1;          // out-of-range labels are clamped, never indexed
-            c = ((unsigned long long)lab << 48) | ((unsigned long long)order_key(__ldcg(score + i), 0) << 16) |
+            c = ((unsigned long long)lab << 48) | ((unsigned long long)order_key(score[i], 0) << 16) |
                 (unsigned long long)i;
         }
         r[e] = c;
