@@ -1312,15 +1312,22 @@ bool gram_resident_takes_knorm(int H, int d) {
 // selection follows within the labels' kernel.  Two and a half chunks of eight tokens to a CTA in the sweep and the other samples
 // beside vic_finalize_kernel / all in the sweep, us: 1 x 300 tokens x 32 heads of 128 28.7 / 26.8, 7 x 700 x 32 of 128 47.1 / 44.0, 16 x 576 x
 // 32 of 128 66.9 / 57.5 (8 chunks), 16 x 576 x 4 of 64 50.1 / 47.4, 32 x 576 x 32 of 128 119.1 / 101.8 (16 chunks), 148 x 256 x 32 of 128
-// 226.2 / 208.9 (32); 1 x 182 x 32 of 128 26.9 / 28.5 was the one loss of 60 problems.  Short chunks are held up by their waits: above
-// 24 of them rows of 2 KB at least (140 x 256 x 4 of 64 91.6 / 94.8 with 30, 120 x 256 x 8 of 128 101.3 / 92.2 with 26).
+// 226.2 / 208.9 (32).  Short chunks are held up by their waits: above 24 of them rows of 2 KB at least (140 x 256 x 4 of 64 91.6 / 94.8
+// with 30, 120 x 256 x 8 of 128 101.3 / 92.2 with 26).
+// Not where a CTA has many keys and all of them together are few: short samples have few CTAs for them (129 to 192 tokens four), and below
+// 16 MB the other kernel ends beside vic_finalize_kernel.  A chunk takes a time of its own and one for each piece of 16 lanes, so
+// pieces are counted: beyond 170 to a CTA calls one behind the other are 1.5 % faster in two parts (112 of 520 problems of 129 to 640 tokens,
+// B 1 to 16; 1 x 182 x 32 of 128 with 768 features 27.9 / 28.9, 8 x 182 x 32 of 128 29.6 / 31.0, 1 x 256 x 48 of 128 27.6 / 30.6), the others
+// 4.4 % less with all.  (With the L2 flushed in front all of them is the faster form on either side, by 5 %: the line is drawn for calls that
+// follow the layer that wrote their keys.)
 // Samples of one row tile have one CTA each, whose sweep ends when its keys do: three chunks (1 x 64 x 32 of 128 26.8 / 30.8 with all
 // 8, 64 x 64 x 16 of 128 43.5 / 44.9; more only pays where they fill the chip, 100 x 128 x 32 of 128 108.6 / 100.3).  With a single buffer
 // each chunk waits for the one before (48 heads of 256: 2 x 576 35.0 / 36.0, 16 x 200 63.6 / 70.8): two and a half chunks to a CTA.
 int gram_resident_knorm_samples(int B, int n, int H, int d, int Nv) {
     const long long ctas = resident_ctas(ResidentCut(B, n).total), chunks = (Nv + kKnChunkTokens - 1) / kKnChunkTokens;
     const long long share = 5 * ctas / (2 * chunks);
-    const bool all = n > BM ? chunks * B <= 24 * ctas || H * d >= 1024 : chunks * B <= 3 * ctas;
+    const bool few = 2.0 * B * Nv * H * d < 16e6 && chunks * B * H * ((d + 127) / 128) > 170 * ctas;
+    const bool all = n > BM && !few ? chunks * B <= 24 * ctas || H * d >= 1024 : chunks * B <= 3 * ctas;
     return share >= B || (knorm_buffers(H, d) > 1 && all) ? B : (int)share;
 }
 
