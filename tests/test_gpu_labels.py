@@ -116,3 +116,20 @@ def test_long_chains_of_parents():
     want, depth = _labels(r, 0, 2, None)
     assert r.status == vb.OK and depth > 256
     assert np.array_equal(r.label[0], want)
+
+
+# More samples than the device runs clusters of eight for have one CTA each, with sixteen tokens a thread; and a few samples on clusters.
+# Ordinary parents, and every token an orphan; single calls (clusters) have the same labels.
+@pytest.mark.parametrize("B,n,n_centers", [(20, 8200, 411), (40, 8193, 3), (2, 9001, 450), (3, 16384, 819)])
+@pytest.mark.parametrize("tau", [-1.0, 0.0])
+def test_labels_of_many_long_samples(B, n, n_centers, tau):
+    rng = np.random.default_rng(B)
+    bits = _bits(rng.standard_normal((B, n, 64), dtype=np.float32))
+    pos = np.repeat(np.stack([np.arange(n) / n, np.zeros(n)], -1)[None].astype(np.float32), B, 0)
+    r = gpu_filter(bits, pos, 0, 0.5, tau, n_centers)
+    assert r.status == vb.OK and (r.n_clusters == n_centers).all()
+    for b in {0, B // 2, B - 1}:
+        feat = (bits[b].astype(np.uint32) << 16).view(np.float32)
+        assert np.array_equal(r.label[b], _labels(r, b, n_centers, feat)[0])
+        one = gpu_filter(bits[b: b + 1], pos[b: b + 1], 0, 0.5, tau, n_centers)
+        assert np.array_equal(one.rho[0], r.rho[b]) and np.array_equal(one.parent[0], r.parent[b]) and np.array_equal(one.label[0], r.label[b])
