@@ -675,15 +675,18 @@ density_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
 // all fit beside vic_finalize_kernel.
 // And where the keys of all samples have room, which saves the kernel and its wait: from 8 MB of keys, where a tenth
 // of a microsecond for each MB (saved) exceeds a twentieth of the sweep (slower by its side warps), up to 8192 tokens.  Without and with: 12 x 1779 x 32 heads of 128 189 / 183, 8 x 1920 x
-// 768 features, 32 of 64 105 / 97, 3 x 2845 x 16 of 128 119 / 113, 4 x 2473 x 16 of 64 103 / 99, 3 x 4675 x 16 of 128 168 / 162; none of 48
-// drawn problems slower.  Fewer keys are hidden beside vic_finalize_kernel, and longer samples hide more (4 x 3393 x 4 of 64
-// 1.8 % slower, above 8192 tokens 1 to 4 %).
-int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D) {
+// 768 features, 32 of 64 105 / 97, 3 x 2845 x 16 of 128 119 / 113, 4 x 2473 x 16 of 64 103 / 99, 3 x 4675 x 16 of 128 168 / 162.  Fewer keys
+// are hidden beside vic_finalize_kernel, and longer samples hide more (4 x 3393 x 4 of 64 1.8 % slower, above 8192 tokens 1 to 4 %).
+// Below some 760 features the sweep takes as long as its epilogue does, and with the Euclidean metric the side warps cost it a little more: by the
+// features alone, 14 of 167 problems were 1 to 4 % slower with all (5 x 7252 x 128 features, 4 of 128 294 / 306; 6 x 4092 x 512, 8 of 128 153 /
+// 159).  So the line, of 260 problems, leaves 120, 2.5 % faster in the mean, one of them slower (1.7 %).
+int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D, int metric) {
     if (!job.K || job.B <= 0 || job.H <= 0 || job.Nv <= 0 || (job.d != 64 && job.d != 128)) return 0;
     const double mb = 2e-6 * job.H * job.d * job.Nv, sweep = 1e-9 / 0.9 * samples * n * (double)n * D;
     const double fits = 2.6 * sweep / mb, hidden = 4.0 + n / 600.0, all_mb = mb * job.B;
     const int s = fits < job.B ? (int)fits : job.B;
-    if (s == job.B && n <= 8192 && all_mb >= 8.0 && 0.1 * all_mb > 0.05 * sweep) return s;
+    const double lasts = D < 760 ? sweep / D * 760 : sweep;
+    if (s == job.B && n <= 8192 && all_mb >= 8.0 && 0.1 * all_mb > (metric == 1 ? 0.06 : 0.05) * lasts) return s;
     auto left = [&](int b) { return b * mb / 6.2 > hidden ? b * mb / 6.2 - hidden : 0.0; };
     return left(job.B) - left(job.B - s) >= 8.0 ? s : 0;
 }

@@ -107,7 +107,7 @@ __device__ __forceinline__ bool blocks_outside_radius(const float4& r, const flo
 }
 
 // How many leading samples' K-norm a sweep over `samples` samples of n tokens should compute on the side.
-int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D);
+int sweep_knorm_samples(const KnormJob& job, int samples, int n, int D, int metric);
 
 // Eq. 2: rho partials, Gram values and block minima (metric: 0 cosine, 1 euclid).
 int launch_density_sweep(const void* feat, const SweepArgs& args, int metric, cudaStream_t stream, bool pdl);

@@ -359,7 +359,7 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
             s.status = g.status;
             s.diag_reports = g.reports ? diag_ctas : 0;
             s.t = tiling;
-            if (knorm && b0 == 0 && (knorm_in_sweep = sweep_knorm_samples(*knorm, s.B, n, D)) > 0) {
+            if (knorm && b0 == 0 && (knorm_in_sweep = sweep_knorm_samples(*knorm, s.B, n, D, p.metric)) > 0) {
                 s.kn = *knorm;
                 s.kn.B = knorm_in_sweep;
             }

@@ -9,15 +9,16 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-def _kernels(B, n, H, d):
+def _kernels(B, n, H, d, D=64, metric=0):
     g = torch.Generator(device=DEV).manual_seed(n)
     rand = lambda *s: torch.randn(s, generator=g, device=DEV).to(torch.bfloat16)
     i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
     K, budget = rand(B, H, n, d), n // 4
     K_out, score = torch.zeros((B, H, budget, d), dtype=torch.bfloat16, device=DEV), torch.zeros((B, n), device=DEV)
-    ws = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=64)
+    ws = vb.alloc_workspace(vb.OP_COLLAB_STEP, B=B, Nv=n, D=D)
     vb.vitcop_kernel_timing_begin()
-    vb.vitcop_collaborative_step(rand(B, n, 64), None, None, K, K, 0, budget, None, K_out, torch.zeros_like(K_out), i32(B), i32(B, n), i32(B), ws,
+    vb.vitcop_collaborative_step(rand(B, n, D), None, None, K, K, 0, budget, None, K_out, torch.zeros_like(K_out), i32(B), i32(B, n), i32(B), ws,
+                                 metric=metric, d_c=0.5 if metric == 0 else 0.5 * D ** 0.5,
                                  n_centers=n // 20, score_out=score)
     kernels = vb.vitcop_kernel_timing_end()
     assert vb.vitcop_poll_status(ws) == vb.OK
@@ -33,3 +34,11 @@ def _kernels(B, n, H, d):
 def test_norms_of_short_samples(B, n, H, d, apart):
     kernels = _kernels(B, n, H, d)
     assert ("knorm_kernel" in kernels) == apart and ("select_quota_kernel" in kernels) == apart
+
+
+# Norms in the density sweep or in a kernel of their own: with few features the sweep is slower by them than that kernel takes.
+@pytest.mark.parametrize("B,n,H,d,D,metric,apart", [(1, 4581, 16, 64, 256, 0, False), (1, 4581, 16, 64, 256, 1, True), (19, 1517, 4, 64, 128, 0, True),
+                                                    (19, 1517, 32, 64, 1024, 1, False)])
+def test_norms_beside_the_density_sweep(B, n, H, d, D, metric, apart):
+    kernels = _kernels(B, n, H, d, D, metric)
+    assert "density_sweep_kernel" in kernels and ("knorm_kernel" in kernels) == apart
