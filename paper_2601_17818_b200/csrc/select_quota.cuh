@@ -514,6 +514,18 @@ __device__ __forceinline__ void select_by_sort(const float* score, const int32_t
     if (tid == 0) *n_keep_b = (int32_t)kept;
 }
 
+// For more than 2048 tokens a function of its own: in the middle of the kernel the searches in front of it came out with fewer registers or
+// more spills (8 x 16384 tokens in even clusters 24.4 us, 22.7 so; 1 x 9000 18.1, 17.0; uneven clusters 5 x 4372 26.3, 24.7, 2 x 7508 32.9, 31.0).
+// Not so with four CTAs and sixteen tokens a thread, which spills more that way (32 x 16345 in uneven clusters 47.3, 48.8).
+static __device__ __noinline__ void select_by_sort_apart(const float* score, const int32_t* label, int n, int Nv_cap, int P_cap, int budget,
+                                                         int32_t* __restrict__ keep_idx, int keep_stride, int32_t* __restrict__ n_keep_b,
+                                                         uint8_t* __restrict__ keep_mask, int* __restrict__ status_word) {
+    extern __shared__ __align__(16) uint32_t quota_smem[];
+    __shared__ uint32_t warp_sums[kSelWarps];
+    select_by_sort(score, label, n, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep_b, keep_mask, status_word,
+                   reinterpret_cast<uint8_t*>(quota_smem), warp_sums);
+}
+
 // ------------------------------------------------------------------------------------------ quota
 // Cluster-quota selection of sample b by R whole CTAs (kSelThreads threads each); uses the dynamic shared memory.
 template <int R, int E>
@@ -538,8 +550,11 @@ __device__ __forceinline__ void select_quota_body(const float* score, const int3
         return;
     if (R > 1 && cluster_ctarank() != 0) return;
     __syncthreads();
-    select_by_sort(score, label, n, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
-                   reinterpret_cast<uint8_t*>(quota_smem), warp_sums);
+    if constexpr (R == 4 && E == 16)
+        select_by_sort(score, label, n, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word,
+                       reinterpret_cast<uint8_t*>(quota_smem), warp_sums);
+    else
+        select_by_sort_apart(score, label, n, Nv_cap, P_cap, budget, keep_idx, keep_stride, n_keep + b, keep_mask, status_word);
 }
 
 
