@@ -170,33 +170,10 @@ int finalize_allow_smem(int R, int E, bool select) {
     static DoneOnDevice attr_done[2][9][17];
     return allow_dynamic_smem(finalize_kernel(R, E, select), finalize_most_smem(R, E, select), attr_done[select][R][E]);
 }
-// How many clusters of eight CTAs (an SM each) the device runs at a time: not SMs / 8, because a cluster stays inside a group of
-// SMs.  0 if it cannot be told.
 int finalize_clusters_at_once() {
-    static std::atomic<int> known[kMaxDevices];            // number + 1
-    std::atomic<int>& k = known[current_device()];
-    int v = k.load(std::memory_order_relaxed);
-    if (v == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(8);
-        cfg.blockDim = dim3(kGroupThreads);
-        cfg.dynamicSmemBytes = finalize_most_smem(8, 2, false);
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 8;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (finalize_allow_smem(8, 2, false) != VITCOP_OK ||
-            cudaOccupancyMaxActiveClusters(&n, finalize_kernel(8, 2, false), &cfg) != cudaSuccess || n < 0) {
-            cudaGetLastError();
-            n = 0;
-        }
-        v = n + 1;
-        k.store(v, std::memory_order_relaxed);
-    }
-    return v - 1;
+    static KnownOnDevice known;
+    return clusters_at_once(finalize_kernel(8, 2, false), 8, kGroupThreads, finalize_most_smem(8, 2, false),
+                            [] { return finalize_allow_smem(8, 2, false); }, known);
 }
 
 // In front of the one-kernel sweep: status word, barrier counter and published factors.  The sweep's CTAs have nothing to meet by
@@ -410,8 +387,8 @@ int launch_filter(const void* feat, const float* pos, int B, int n, int D, const
         if (rc != VITCOP_OK) return rc;
     }
     if (knorm && knorm_in_sweep < knorm->B) {
-        // vic_finalize_kernel runs one CTA per sample and releases its dependents when it starts: the K-norm, which
-        // does not depend on the clustering, streams K from HBM on the other SMs meanwhile and waits for the
+        // vic_finalize_kernel runs one CTA per sample, eight of a long one, and releases its dependents when it starts: the
+        // K-norm, which does not depend on the clustering, streams K from HBM on the other SMs meanwhile and waits for the
         // finalize kernel before it ends.  (Beside a Gram sweep it would not fit: those kernels' CTAs hold most of each SM's
         // registers.)
         const int64_t stride_b = (int64_t)knorm->H * knorm->N * knorm->d;

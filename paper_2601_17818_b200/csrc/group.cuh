@@ -21,7 +21,7 @@ struct Share {
     }
     __device__ __forceinline__ int own() const { return max(0, min(share, n - base)); }       // tokens of this CTA
 };
-// Tokens of a thread where a share holds at most this many: the template argument E.
+// Tokens of a CTA, at most.
 template <int R>
 __host__ __device__ constexpr int share_capacity(int Nv_cap) { return R == 1 ? (Nv_cap + 7) & ~7 : ((Nv_cap + R - 1) / R + 7) & ~7; }
 

@@ -42,6 +42,35 @@ inline int allow_dynamic_smem(Kernel kern, size_t most_bytes, DoneOnDevice& done
     return VITCOP_OK;
 }
 
+// How many clusters of R CTAs (an SM each) the device runs of a kernel at a time: not SMs / R, because a cluster stays inside a group of
+// SMs.  0 if it cannot be told.  `known`: number + 1, per device; `allow` raises the kernel's limit of dynamic shared memory.
+typedef std::atomic<int> KnownOnDevice[kMaxDevices];
+template <typename Kernel, typename Allow>
+inline int clusters_at_once(Kernel kern, int R, int threads, size_t smem, Allow allow, KnownOnDevice& known) {
+    std::atomic<int>& k = known[current_device()];
+    int v = k.load(std::memory_order_relaxed);
+    if (v == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)R);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)R;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (allow() != VITCOP_OK || cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 0) {
+            cudaGetLastError();
+            n = 0;
+        }
+        v = n + 1;
+        k.store(v, std::memory_order_relaxed);
+    }
+    return v - 1;
+}
+
 // Diagnostic per-kernel timing (vitcop_kernel_timing_begin / _end).  While it is on, a KernelTimeScope
 // around a launch records one CUDA event before and one after the kernel on its stream, and launchers
 // drop the programmatic-dependent-launch attribute so that consecutive kernels do not overlap.

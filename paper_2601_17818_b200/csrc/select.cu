@@ -230,33 +230,11 @@ int quota_allow_smem(int R, int E) {
     static DoneOnDevice attr_done[9][17];
     return allow_dynamic_smem(quota_kernel(R, E), quota_most_smem(E), attr_done[R][E]);
 }
-// How many clusters of R CTAs (an SM each) the device runs at a time: not SMs / R, because a cluster stays inside a group of SMs.
-// Beyond that the clusters behind wait for a whole selection: 16 x 16384 tokens 45 us on clusters of eight, 26 on clusters of four;
-// 40 x 2880 20 us on clusters of four, 13 on single CTAs.  0 if it cannot be told.
+// Beyond as many clusters as the device runs at a time the ones behind wait for a whole selection: 16 x 16384 tokens 45 us on clusters of
+// eight, 26 on clusters of four; 40 x 2880 20 us on clusters of four, 13 on single CTAs.
 int quota_clusters_at_once(int R, int E) {
-    static std::atomic<int> known[kMaxDevices][9][17];     // number + 1
-    std::atomic<int>& k = known[current_device()][R][E];
-    int v = k.load(std::memory_order_relaxed);
-    if (v == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)R);
-        cfg.blockDim = dim3(kSelThreads);
-        cfg.dynamicSmemBytes = quota_most_smem(E);
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)R;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (quota_allow_smem(R, E) != VITCOP_OK || cudaOccupancyMaxActiveClusters(&n, quota_kernel(R, E), &cfg) != cudaSuccess || n < 0) {
-            cudaGetLastError();
-            n = 0;
-        }
-        v = n + 1;
-        k.store(v, std::memory_order_relaxed);
-    }
-    return v - 1;
+    static KnownOnDevice known[9][17];
+    return clusters_at_once(quota_kernel(R, E), R, kSelThreads, quota_most_smem(E), [=] { return quota_allow_smem(R, E); }, known[R][E]);
 }
 
 }  // namespace
