@@ -283,7 +283,7 @@ int launch_compact(const void* hidden, const void* K, const void* V, int B, int 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl_allowed(true) ? 1 : 0;
-    KernelTimeScope timed("compact_kernel", stream);
+    KernelTimeScope timed("compact_kernel", stream);       // (either kernel: a selection inside counts as part of the copy)
     const uint4 *hid = static_cast<const uint4*>(hidden), *k = static_cast<const uint4*>(K), *v = static_cast<const uint4*>(V);
     uint4 *const hid_out = static_cast<uint4*>(hidden_out), *const k_out = static_cast<uint4*>(K_out), *const v_out = static_cast<uint4*>(V_out);
     if (smallest) {
