@@ -16,15 +16,20 @@
 // from block to block and the warp exchanges only the bound; the place of a value is one add and one select away from the
 // token's.  Measured on 8 x 2880 tokens, caches warm: 19.7 -> 15.1 us and 18.3 -> 13.9 us against a warp-wide minimum and ballot
 // per block and four separate loads per token.  Passing over blocks without a denser token in the first kernel too: 6 us less on
-// 4 x 4096 tokens.  Four rounds there: three, five and six take as long on 8 x 2880 and 4 x 4608 tokens and up to 3 us longer on 2 x 16384.
+// 4 x 4096 tokens.
 #include "density.cuh"
 
 namespace vitcop {
 namespace {
 
 constexpr int kNdThreads = 256, kNdWarps = kNdThreads / 32;
-constexpr int kNdRounds = 4;                               // rounds of two blocks that a warp does for its own token
-constexpr int kNdAhead = 3;                                // blocks a warp of the second kernel looks into at a time
+// Rounds of two blocks that a warp of the first kernel does for its own token, and blocks that a warp of the second looks into at a time: four and
+// three (three, five and six rounds take as long on 8 x 2880 and 4 x 4608 tokens and up to 3 us longer on 2 x 16384).  Three and four where the
+// tokens' warps are at most one and a half times what the chip holds (64 an SM): the first kernel lasts as long as its longest warps there, and
+// the second has idle SMs for what is left.  64 steps on such calls, four and three / three and four: 44 on videos 1.0 % less, 20 on images 1.2 %
+// (4 x 3420 tokens of a video 125.1 / 122.4 us, 3 x 3143 99.5 / 98.5); filters of more than 15000 tokens in all 1 to 2 % more.  Beyond 8192
+// tokens to a sample four and three are as good or better with few samples too.
+bool few_tokens(long long tokens, int n) { return n <= 8192 && 2 * tokens <= 3 * 64LL * gram_num_sms(); }
 constexpr uint32_t kInfBits = 0x7f800000u;
 // A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, above it
 // one bit that marks a stand-in; i.e. a bound up to 2^-13 too low.
@@ -99,7 +104,7 @@ struct Search {
 
 template <int METRIC, bool SPATIAL>
 __global__ void __launch_bounds__(kNdThreads)
-nearest_denser_kernel(const __grid_constant__ SweepArgs g) {
+nearest_denser_kernel(const __grid_constant__ SweepArgs g, const int rounds) {
     // A kernel queued behind this one that does not depend on it may share the SMs from the start.
     grid_dependency_launch_dependents();
     grid_dependency_wait();                                // densities, factors, Gram values and minima come from the kernels before
@@ -137,7 +142,7 @@ nearest_denser_kernel(const __grid_constant__ SweepArgs g) {
         least = __reduce_min_sync(0xffffffffu, m1);
     };
 #pragma unroll 1
-    for (int round = 0; round < kNdRounds && can(least) && !(least & kStandIn); ++round) {
+    for (int round = 0; round < rounds && can(least) && !(least & kStandIn); ++round) {
         const int b0 = (int)(least & kBlkMask);
         const auto p0 = s.fetch(b0);
         take();
@@ -163,10 +168,10 @@ nearest_denser_kernel(const __grid_constant__ SweepArgs g) {
 // still open and hold a denser token.  (Those the first kernel has looked into already cannot improve on its result.)
 // Each warp in ascending order of its blocks' minima: in the order of their numbers it looked into more of them (2 x 16384 tokens
 // of no structure 128.6 -> 117.5 us; 4 x 4608 of a video, whole call, 212 -> 209).  Two or four times as many or as few blocks per warp
-// measured the same or worse.  What one warp finds it tells the token's others at once, and what they have found travels with its blocks,
-// three at a time instead of four: alone, a warp goes on below a bound that another one has lowered long since (2 x 16384 tokens 41 -> 25 us;
+// measured the same or worse.  What one warp finds it tells the token's others at once, and what they have found travels with its
+// blocks: alone, a warp goes on below a bound that another one has lowered long since (2 x 16384 tokens 41 -> 25 us;
 // of no structure, whole call, 1000 -> 754).
-template <int METRIC, bool SPATIAL>
+template <int METRIC, bool SPATIAL, int AHEAD>
 __global__ void __launch_bounds__(kNdThreads)
 nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
     grid_dependency_launch_dependents();
@@ -197,11 +202,11 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
             // in ascending order of the minima, several at a time: the first ones are the likeliest to hold the answer, and
             // none behind the first that cannot hold it can
             for (;;) {
-                typename Search<METRIC, SPATIAL>::Pair p[kNdAhead];
-                int blk[kNdAhead];
+                typename Search<METRIC, SPATIAL>::Pair p[AHEAD];
+                int blk[AHEAD];
                 int cnt = 0;
 #pragma unroll
-                for (int u = 0; u < kNdAhead; ++u) {
+                for (int u = 0; u < AHEAD; ++u) {
                     const uint32_t m = __reduce_min_sync(0xffffffffu, lo);
                     const int who = __ffs(__ballot_sync(0xffffffffu, lo == m)) - 1;
                     blk[u] = k0 + who * slices;
@@ -215,7 +220,7 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
                 // (what the token's other warps have found by now travels with the blocks)
                 const unsigned long long others = lane == 0 ? __ldcg(g.best + at) : 0ull;
 #pragma unroll
-                for (int u = 0; u < kNdAhead; ++u)
+                for (int u = 0; u < AHEAD; ++u)
                     if (u < cnt) s.look(p[u], blk[u]);
                 const unsigned long long found = s.packed(s.bound());
                 if (found < best) {
@@ -234,7 +239,7 @@ nearest_left_kernel(const __grid_constant__ SweepArgs g, const int slices) {
 int launch_nearest_denser(const SweepArgs& args, int metric, cudaStream_t stream, bool pdl) {
     if (args.B <= 0 || args.n <= 0) return VITCOP_OK;
     if (!args.gram || !args.blk_min || !args.blk_rho || !args.tok || !args.best || !args.left || !args.n_left) return VITCOP_ERR_INVALID_ARG;
-    const bool spatial = args.tau2 >= 0.f && args.pos != nullptr;
+    const bool spatial = args.tau2 >= 0.f && args.pos != nullptr, few = few_tokens((long long)args.B * args.n, args.n);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((args.n + kNdWarps - 1) / kNdWarps), (unsigned)args.B);
     cfg.blockDim = dim3(kNdThreads);
@@ -249,15 +254,18 @@ int launch_nearest_denser(const SweepArgs& args, int metric, cudaStream_t stream
     int rc;
     {
         KernelTimeScope timed("nearest_denser_kernel", stream);
-        rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, args));
+        rc = record_cuda(cudaLaunchKernelEx(&cfg, kern, args, few ? 3 : 4));
         if (rc != VITCOP_OK) return rc;
     }
     int slices = 2;                                        // at most 32 blocks a warp: one per lane
     while (slices * 32 < args.t.n_blk()) slices *= 2;
     const long long most = ((long long)args.B * args.n * slices + kNdWarps - 1) / kNdWarps, ctas = 6LL * gram_num_sms();
     cfg.gridDim = dim3((unsigned)(most < ctas ? most : ctas));
-    auto rest = metric == 1 ? (spatial ? nearest_left_kernel<1, true> : nearest_left_kernel<1, false>)
-                            : (spatial ? nearest_left_kernel<0, true> : nearest_left_kernel<0, false>);
+    auto pick = [&](auto four, auto three) { return few ? four : three; };
+    auto rest = metric == 1 ? (spatial ? pick(nearest_left_kernel<1, true, 4>, nearest_left_kernel<1, true, 3>)
+                                       : pick(nearest_left_kernel<1, false, 4>, nearest_left_kernel<1, false, 3>))
+                            : (spatial ? pick(nearest_left_kernel<0, true, 4>, nearest_left_kernel<0, true, 3>)
+                                       : pick(nearest_left_kernel<0, false, 4>, nearest_left_kernel<0, false, 3>));
     KernelTimeScope timed("nearest_left_kernel", stream);
     return record_cuda(cudaLaunchKernelEx(&cfg, rest, args, slices));
 }
