@@ -25,11 +25,14 @@ namespace {
 constexpr int kNdThreads = 256, kNdWarps = kNdThreads / 32;
 // Rounds of two blocks that a warp of the first kernel does for its own token, and blocks that a warp of the second looks into at a time: four and
 // three (three, five and six rounds take as long on 8 x 2880 and 4 x 4608 tokens and up to 3 us longer on 2 x 16384).  Three and four where the
-// tokens' warps are at most one and a half times what the chip holds (64 an SM): the first kernel lasts as long as its longest warps there, and
-// the second has idle SMs for what is left.  64 steps on such calls, four and three / three and four: 44 on videos 1.0 % less, 20 on images 1.2 %
-// (4 x 3420 tokens of a video 125.1 / 122.4 us, 3 x 3143 99.5 / 98.5); filters of more than 15000 tokens in all 1 to 2 % more.  Beyond 8192
-// tokens to a sample four and three are as good or better with few samples too.
-bool few_tokens(long long tokens, int n) { return n <= 8192 && 2 * tokens <= 3 * 64LL * gram_num_sms(); }
+// chip holds the tokens' warps (64 an SM), up to 4096 tokens to a sample one and a half times as many: the first kernel lasts as long as its longest
+// warps there, and the second has idle SMs for what is left.  64 steps on such calls, four and three / three and four: 44 on videos 1.0 %
+// less, 20 on images 1.2 % (4 x 3420 tokens of a video 125.1 / 122.4 us, 3 x 3143 99.5 / 98.5).  Beyond that line 1 to 2 % more (2 x 5600 to 6800
+// tokens without structure 4 to 5 %), and beyond 8192 tokens to a sample with few samples too.
+bool few_tokens(long long tokens, int n) {
+    const long long held = 64LL * gram_num_sms();
+    return n <= 8192 && (tokens <= held || (n <= 4096 && 2 * tokens <= 3 * held));
+}
 constexpr uint32_t kInfBits = 0x7f800000u;
 // A lane orders its blocks by a key: the bits of the minimum (never negative) with the block's number in the low bits, above it
 // one bit that marks a stand-in; i.e. a bound up to 2^-13 too low.
